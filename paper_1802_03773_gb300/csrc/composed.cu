@@ -553,73 +553,6 @@ __global__ void block_apply_qt_kernel(ComposedView<T> V, FactorOut<T> O, const T
     for (int r = m; r < na; ++r) rhs0[O.red_off[i] + (r - m)] = y[r];
 }
 
-// The s x s triangle R_S is solved by one CTA with a thread per row (s <= kTriMax).
-constexpr int kTriMax = 1024;
-static inline unsigned tri_threads(int s) { return (unsigned)(s <= 32 ? 32 : (s + 31) / 32 * 32); }
-
-template <typename T>
-__device__ __forceinline__ T block_warp_sum(T v) {
-  for (int d = 16; d >= 1; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-  return v;
-}
-
-// R_S x = c (upper triangular, column-major with ld), optionally x += result (x may be c).
-// Columns are eliminated from the last: once x_k is known, every row above subtracts R_ik x_k,
-// so each column is read once, coalesced, and the next one is loaded a step ahead.
-template <typename T>
-__global__ void __launch_bounds__(kTriMax) dense_backsub_kernel(const T* R, int64_t ld, int s, const T* c, T* x,
-                                                                int accumulate, int* status) {
-  __shared__ T xs[2];
-  const int i = threadIdx.x;
-  T yi = i < s ? c[i] : T(0);
-  T rcur = i < s ? R[(int64_t)(s - 1) * ld + i] : T(0);   // column s - 1
-  for (int k = s - 1; k >= 0; --k) {
-    const T rnext = i < k ? R[(int64_t)(k - 1) * ld + i] : T(0);
-    if (i == k) {
-      if (rcur == T(0)) record(status, QRKIT_ESINGULAR);
-      xs[k & 1] = yi / rcur;
-    }
-    __syncthreads();
-    const T xk = xs[k & 1];
-    if (i < k) yi -= rcur * xk;
-    else if (i == k) yi = xk;
-    rcur = rnext;
-  }
-  if (i < s) x[i] = accumulate ? x[i] + yi : yi;
-}
-
-// R_S^T h = g (forward substitution), g given in double: h_k = (g_k - sum_{i<k} R_ik h_i) / R_kk,
-// the sum over column k of R (coalesced, loaded a step ahead) reduced over the CTA.
-template <typename T>
-__global__ void __launch_bounds__(kTriMax) dense_fwdsub_rt_kernel(const T* R, int64_t ld, int s, const double* g,
-                                                                  T* h) {
-  __shared__ T part_s[2][32];
-  __shared__ T hs[2];
-  const int i = threadIdx.x, lane = i & 31, warp = i >> 5, nw = (int)(blockDim.x >> 5);
-  T hi = T(0);
-  T rcur = i < 1 && s > 0 ? R[0] : T(0);                          // column 0
-  T dnext = s > 0 && i == 0 ? R[0] : T(0), gnext = s > 0 && i == 0 ? (T)g[0] : T(0);
-  for (int k = 0; k < s; ++k) {
-    const T rnext = (k + 1 < s && i <= k + 1) ? R[(int64_t)(k + 1) * ld + i] : T(0);
-    const T dk = dnext, gk = gnext;   // thread 0: R_kk and g_k
-    if (i == 0 && k + 1 < s) {
-      dnext = R[(int64_t)(k + 1) * ld + k + 1];
-      gnext = (T)g[k + 1];
-    }
-    const T p = block_warp_sum<T>(i < k ? rcur * hi : T(0));
-    if (lane == 0) part_s[k & 1][warp] = p;
-    __syncthreads();
-    if (warp == 0) {
-      const T q = block_warp_sum<T>(lane < nw ? part_s[k & 1][lane] : T(0));
-      if (lane == 0) hs[k & 1] = (gk - q) / dk;
-    }
-    __syncthreads();
-    if (i == k) hi = hs[k & 1];
-    rcur = rnext;
-  }
-  if (i < s) h[i] = hi;
-}
-
 // Per-block R_i x_i = rhs_i - R12_i x_S; rhs from ctop (T) or from a double vector.  NA > 0:
 // every block has at most NA augmented rows and MM columns (registers only).
 template <typename T, int NA = 0, int MM = 0>
@@ -817,9 +750,7 @@ __device__ __forceinline__ void resid_g_small_f32(const ComposedView<float>& V, 
 #pragma unroll
       for (int j = 0; j < MM; ++j)
         if (j < m) dot2_acc(sh, sl, -J[j * n + r], pj[j]);
-      if (V.coupled == QRKIT_COUPLED_DENSE) {
-        for (int c = 0; c < V.s; ++c) dot2_acc(sh, sl, -V.S[(int64_t)c * V.rows + r0 + r], p[V.nb + c]);
-      } else if (V.coupled == QRKIT_COUPLED_WINDOW) {
+      if (V.coupled == QRKIT_COUPLED_WINDOW) {
         for (int t = 0; t < V.w; ++t)
           if (st + t < V.s) dot2_acc(sh, sl, -V.S[r0 * V.w + (int64_t)t * n + r], p[V.nb + st + t]);
       }
@@ -843,20 +774,7 @@ __device__ __forceinline__ void resid_g_small_f32(const ComposedView<float>& V, 
       g[c0 + j] = ((double)ah + (double)al) - lam * d * d * (double)pj[j];
     }
   }
-  if (V.coupled == QRKIT_COUPLED_DENSE) {
-    for (int c = 0; c < V.s; ++c) {
-      float ah = 0.f, al = 0.f;
-#pragma unroll
-      for (int r = 0; r < NR; ++r)
-        if (r < n) {
-          const float a = V.S[(int64_t)c * V.rows + r0 + r];
-          dot2_acc(ah, al, a, rh[r]);
-          al = __fmaf_rn(a, rl[r], al);
-        }
-      const double acc = (double)ah + (double)al;
-      if (acc != 0.0) atomicAdd(&gS[c], acc);
-    }
-  } else if (V.coupled == QRKIT_COUPLED_WINDOW) {
+  if (V.coupled == QRKIT_COUPLED_WINDOW) {
     for (int t = 0; t < V.w; ++t) {
       float ah = 0.f, al = 0.f;
 #pragma unroll
@@ -1211,6 +1129,17 @@ int small_class(const Plan& P, bool damp) {
     else LAUNCH(ctx, (KERNEL<T><<<grid, threads, smem, stream>>>(__VA_ARGS__)));                \
   } while (0)
 
+// R_i x_i = rhs_i - R12_i x_S for every block.  From 16 shared columns on a warp takes a block (the
+// lanes read its rows of R12 together); below, and for windows of up to 8, a thread per block.
+template <typename T>
+static qrkit_status launch_block_backsub(qrkit_ctx* ctx, const ComposedView<T>& V, const FactorOut<T>& O, const T* rhs,
+                                         const T* xS, T* x, int accumulate) {
+  if (V.coupled == QRKIT_COUPLED_DENSE && V.s >= 16) return dense_block_backsub<T>(ctx, V, O, rhs, xS, x, accumulate);
+  LAUNCH_SHAPED(ctx, small_class(ctx->plan, O.damp), block_backsub_kernel, blocks_for(V.K, 64), 64, 0, ctx->stream, V, O,
+                rhs, xS, x, accumulate);
+  return QRKIT_OK;
+}
+
 // D = column norms of J (Sec. 5.2), zero -> 1, in double; C.sq is the scratch.
 template <typename T>
 static qrkit_status norms_typed(qrkit_ctx* ctx, const ComposedView<T>& V, double* D) {
@@ -1394,8 +1323,8 @@ static qrkit_status solve_typed(qrkit_ctx* ctx, const void* J, const void* S, co
   const T* RS = pan ? (const T*)C.Rs.ptr : (top ? (const T*)top->X.ptr : nullptr);
   const int64_t ldRS = pan ? s : (top ? top->ld : 0);
   if (V.coupled == QRKIT_COUPLED_DENSE) {
-    LAUNCH(ctx, dense_backsub_kernel<T><<<1, tri_threads(s), 0, st>>>(
-                    RS, ldRS, s, pan ? (const T*)C.cs.ptr : (const T*)top->rhs.ptr, x + nb, 0, ctx->d_status));
+    qrkit_status rc = dense_backsub<T>(ctx, RS, ldRS, s, pan ? (const T*)C.cs.ptr : (const T*)top->rhs.ptr, x + nb);
+    if (rc != QRKIT_OK) return rc;
   } else if (V.coupled == QRKIT_COUPLED_WINDOW) {
     // reduced banded block of every segment (Sec. 4.4), rows in P_r order, the shared
     // columns' damping rows interleaved
@@ -1410,8 +1339,8 @@ static qrkit_status solve_typed(qrkit_ctx* ctx, const void* J, const void* S, co
                                  C.damp ? C.lam : 0.0, C.RwS.ptr, C.cS.ptr, x + nb, (double*)C.res2.ptr);
     if (rc != QRKIT_OK) return rc;
   }
-  LAUNCH_SHAPED(ctx, small_class(P, O.damp), block_backsub_kernel, blocks_for(P.K, 64), 64, 0, st, V, O, O.ctop,
-                s ? x + nb : nullptr, x, 0);
+  qrkit_status rc_b = launch_block_backsub<T>(ctx, V, O, (const T*)O.ctop, s ? x + nb : nullptr, x, 0);
+  if (rc_b != QRKIT_OK) return rc_b;
   // refinement (extended-precision residual, corrections through R only)
   for (int it = 0; it < refine_steps; ++it) {
     const int64_t N = nb + s;
@@ -1421,22 +1350,31 @@ static qrkit_status solve_typed(qrkit_ctx* ctx, const void* J, const void* S, co
     double* g = (double*)C.g.ptr;
     T* h = (T*)C.h.ptr;
     double* gS = g + nb;
-    if (s > 0) QRKIT_CUDA_TRY(ctx, cudaMemsetAsync(gS, 0, (size_t)s * sizeof(double), st));
-    // dense S: all s columns per CTA; windowed S: the CTA's column range (up to kWinSumCols),
-    // with larger CTAs so that more blocks share a column sum
-    const bool win = V.coupled == QRKIT_COUPLED_WINDOW;
-    const int rthreads = win ? 256 : 64;
-    const size_t sum_smem = (V.coupled == QRKIT_COUPLED_DENSE && s <= kCtaSumCols) ? (size_t)s * sizeof(double)
-                            : win ? (size_t)kWinSumCols * sizeof(double) : 0;
-    const int win_cols = win ? kWinSumCols : 0;
-    LAUNCH_SHAPED(ctx, small_class(P, O.damp), resid_g_kernel, blocks_for(P.K, rthreads), rthreads, sum_smem, st, V,
-                  (const T*)b, x, O.D, C.lam, g, gS, win_cols);
-    if (s > 0)
-      LAUNCH(ctx, gS_damping_kernel<<<blocks_for(s, 128), 128, 0, st>>>(
-                      gS, sizeof(T) == 4 ? (const float*)x : nullptr,
-                      sizeof(T) == 8 ? (const double*)x : nullptr, O.D, nb, s, C.lam));
-    LAUNCH_SHAPED(ctx, small_class(P, O.damp), block_fwdsub_rt_kernel, blocks_for(P.K, rthreads), rthreads, sum_smem,
-                  st, V, O, g, h, gS, win_cols);
+    bool have_g = false;
+    if constexpr (sizeof(T) == sizeof(float)) {
+      if (V.coupled == QRKIT_COUPLED_DENSE) {   // g_S - R12^T h_B and h_B by row, block and column passes
+        if ((rc = dense_refine_gradient(ctx, V, O, (const float*)b, x, C.lam, C.dref.ptr, h, gS)) != QRKIT_OK) return rc;
+        have_g = true;
+      }
+    }
+    if (!have_g) {
+      if (s > 0) QRKIT_CUDA_TRY(ctx, cudaMemsetAsync(gS, 0, (size_t)s * sizeof(double), st));
+      // dense S: all s columns per CTA; windowed S: the CTA's column range (up to kWinSumCols),
+      // with larger CTAs so that more blocks share a column sum
+      const bool win = V.coupled == QRKIT_COUPLED_WINDOW;
+      const int rthreads = win ? 256 : 64;
+      const size_t sum_smem = (V.coupled == QRKIT_COUPLED_DENSE && s <= kCtaSumCols) ? (size_t)s * sizeof(double)
+                              : win ? (size_t)kWinSumCols * sizeof(double) : 0;
+      const int win_cols = win ? kWinSumCols : 0;
+      LAUNCH_SHAPED(ctx, small_class(P, O.damp), resid_g_kernel, blocks_for(P.K, rthreads), rthreads, sum_smem, st, V,
+                    (const T*)b, x, O.D, C.lam, g, gS, win_cols);
+      if (s > 0)
+        LAUNCH(ctx, gS_damping_kernel<<<blocks_for(s, 128), 128, 0, st>>>(
+                        gS, sizeof(T) == 4 ? (const float*)x : nullptr,
+                        sizeof(T) == 8 ? (const double*)x : nullptr, O.D, nb, s, C.lam));
+      LAUNCH_SHAPED(ctx, small_class(P, O.damp), block_fwdsub_rt_kernel, blocks_for(P.K, rthreads), rthreads, sum_smem,
+                    st, V, O, g, h, gS, win_cols);
+    }
     if (V.coupled == QRKIT_COUPLED_WINDOW && C.cr) {
       // dp_S = R_S^{-1} R_S^{-T} (g_S - R12^T h_B) with the parallel banded factor
       qrkit_status rc = cr_normal_solve(ctx, *C.cr, gS, h + nb);
@@ -1454,15 +1392,11 @@ static qrkit_status solve_typed(qrkit_ctx* ctx, const void* J, const void* S, co
       LAUNCH(ctx, axpy_kernel<T><<<blocks_for(s, 128), 128, 0, st>>>(x + nb, h + nb, s));
     }
     if (V.coupled == QRKIT_COUPLED_DENSE) {
-      // h_S = R_S^{-T} (g_S - R12^T h_B), then dp_S = R_S^{-1} h_S in place
-      LAUNCH(ctx, dense_fwdsub_rt_kernel<T><<<1, tri_threads(s), 0, st>>>(RS, ldRS, s, gS, h + nb));
-      LAUNCH(ctx, dense_backsub_kernel<T><<<1, tri_threads(s), 0, st>>>(RS, ldRS, s, h + nb, h + nb, 0,
-                                                                         ctx->d_status));
-      LAUNCH(ctx, axpy_kernel<T><<<blocks_for(s, 128), 128, 0, st>>>(x + nb, h + nb, s));
+      // dp_S = R_S^{-1} R_S^{-T} (g_S - R12^T h_B), added to p_S and kept in h for the blocks
+      if ((rc = dense_normal<T>(ctx, RS, ldRS, s, gS, h + nb, x + nb)) != QRKIT_OK) return rc;
     }
     // dp_B = R_B^{-1} (h_B - R12 dp_S), accumulated into p
-    LAUNCH_SHAPED(ctx, small_class(P, O.damp), block_backsub_kernel, blocks_for(P.K, 64), 64, 0, st, V, O, h,
-                  s ? h + nb : nullptr, x, 1);
+    if ((rc = launch_block_backsub<T>(ctx, V, O, (const T*)h, s ? h + nb : nullptr, x, 1)) != QRKIT_OK) return rc;
   }
   return QRKIT_OK;
 }
@@ -1526,7 +1460,7 @@ static void release_levels(std::vector<TsqrLevel>& LV) {
 
 void release_composed(Composed& C) {
   release(C.D); release(C.sq); release(C.Fa); release(C.tau); release(C.R12); release(C.ctop);
-  release(C.g); release(C.h);
+  release(C.g); release(C.h); release(C.dref);
   release(C.Xw); release(C.Xstart); release(C.rhs_red); release(C.RwS); release(C.cS);
   release(C.res2); release(C.meta); release(C.dense_ws);
   release(C.sort_tab); release(C.hist); release(C.spos); release(C.order); release(C.Xw_s);
@@ -1675,6 +1609,9 @@ qrkit_status composed_layout(qrkit_ctx* ctx, size_t elem) {
                   "dense shared block: s <= 64, or (float) s a multiple of 32 up to 512");
     const int64_t M0 = C.red_rows + (C.damp ? s : 0);
     if (M0 < s) return fail(ctx, QRKIT_EINVAL, "reduced shared block has fewer rows than columns");
+    if (elem == sizeof(float) &&
+        (rc = ensure(ctx, C.dref, dense_refine_bytes(P.rows, P.cols, s), "refinement sums")) != QRKIT_OK)
+      return rc;
     C.tile_rows = 256;
     // the TSQR levels of a panel of pw columns over M rows, w columns wide (panel + trailing);
     // each level's leading dimension is padded to 16 bytes, and the rows that leave a panel
@@ -1753,12 +1690,11 @@ static qrkit_status solve_r_typed(qrkit_ctx* ctx, const void* qtb, void* p) {
   if (V.coupled == QRKIT_COUPLED_DENSE) {
     const TsqrLevel& top = C.levels.back();
     const bool pan = !C.panels.empty();
-    LAUNCH(ctx, dense_backsub_kernel<T><<<1, tri_threads(s), 0, st>>>(
-                    pan ? (const T*)C.Rs.ptr : (const T*)top.X.ptr, pan ? s : top.ld, s, c + P.cols, x + P.cols, 0,
-                    ctx->d_status));
+    qrkit_status rc = dense_backsub<T>(ctx, pan ? (const T*)C.Rs.ptr : (const T*)top.X.ptr, pan ? s : top.ld, s,
+                                       c + P.cols, x + P.cols);
+    if (rc != QRKIT_OK) return rc;
   }
-  LAUNCH(ctx, block_backsub_kernel<T><<<blocks_for(P.K, 64), 64, 0, st>>>(V, O, c, s ? x + P.cols : nullptr, x, 0));
-  return QRKIT_OK;
+  return launch_block_backsub<T>(ctx, V, O, c, s ? x + P.cols : nullptr, x, 0);
 }
 
 qrkit_status composed_solve_r(qrkit_ctx* ctx, const void* qtb, void* p) {
@@ -1824,9 +1760,7 @@ static qrkit_status solve_blocks_typed(qrkit_ctx* ctx, const void* qtb, void* p)
   ComposedView<T> V = view<T>(ctx, nullptr, nullptr);
   FactorOut<T> O = fout<T>(ctx);
   T* x = (T*)p;
-  LAUNCH(ctx, block_backsub_kernel<T><<<blocks_for(P.K, 64), 64, 0, ctx->stream>>>(
-                  V, O, (const T*)qtb, V.s ? x + P.cols : nullptr, x, 0));
-  return QRKIT_OK;
+  return launch_block_backsub<T>(ctx, V, O, (const T*)qtb, V.s ? x + P.cols : nullptr, x, 0);
 }
 
 qrkit_status composed_solve_blocks(qrkit_ctx* ctx, const void* qtb, void* p) {

@@ -1,0 +1,507 @@
+// Solves with a dense shared part S (Sec. 4.2, Sec. 5.1): the triangle R_S of the reduced block,
+// the block unknowns below it, and the refinement residual of float plans.
+//
+// Every pass over S (column-major, rows of J) or R12 (row-major, one row of s values per block
+// column) is written for the memory system: a warp reads whole 128-byte lines, a CTA's warps split
+// the columns, sums leave through per-chunk partials that are added in a fixed order.  S and R12
+// are read twice and once per refinement step, so those passes are bound by HBM: at 100,000 blocks
+// 4 x 2 with s = 512 (S 819 MB, R12 410 MB) the row pass takes 126 us, the column pass 135 us, the
+// R12 pass 136 us and a block back-substitution 97 us.  A thread per block walking all s columns,
+// with a shared-memory FP64 atomic per column and block, took 4.33 ms for the two passes over S,
+// 4.04 ms for R12^T h and 0.38 ms per back-substitution.
+#include <cuda_runtime.h>
+#include <math.h>
+#include <stdint.h>
+
+#include <algorithm>
+
+#include "device_util.cuh"
+#include "internal.h"
+
+namespace qrkit {
+namespace {
+
+// Compensated float accumulation (Dot2, Ogita-Rump-Oishi): (sh + sl) += a x.
+__device__ __forceinline__ void dot2(float& sh, float& sl, float a, float x) {
+  const float p = __fmul_rn(a, x);
+  const float pe = __fmaf_rn(a, x, -p);
+  float t, e;
+  dev::two_sum(sh, p, t, e);
+  sh = t;
+  sl = __fadd_rn(sl, __fadd_rn(e, pe));
+}
+
+// (sh + sl) += (bh + bl)
+__device__ __forceinline__ void add_pair(float& sh, float& sl, float bh, float bl) {
+  float t, e;
+  dev::two_sum(sh, bh, t, e);
+  sh = t;
+  sl = __fadd_rn(sl, __fadd_rn(e, bl));
+}
+
+template <int V>
+struct Vec;
+template <>
+struct Vec<4> {
+  float v[4];
+  __device__ __forceinline__ void load(const float* p) {
+    const float4 q = *reinterpret_cast<const float4*>(p);
+    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+  }
+};
+template <>
+struct Vec<1> {
+  float v[1];
+  __device__ __forceinline__ void load(const float* p) { v[0] = *p; }
+};
+
+// ---- triangular solves with R_S: one CTA, thread i owns row (or column) i, 32 at a time ----
+// The 32 unknowns of a diagonal block are found by the warp that owns them (broadcasts, no
+// barrier); then every other thread takes their 32 products off its own right-hand side in one
+// go, its 32 values of R fetched while the diagonal block is being solved.  Two barriers per 32
+// columns instead of one or two per column (s = 512: 82 us against 211 us for R_S x = c, 240 us
+// against 465 us for R_S^T and R_S together).
+constexpr int kTriThreads = kMaxDenseS;
+inline unsigned tri_cta(int s) { return (unsigned)((s + 31) / 32 * 32); }
+
+// R x = y (upper triangular, column-major): returns x_i for thread i < s; xs: 32 shared values.
+template <typename T>
+__device__ __forceinline__ T tri_backsub(const T* R, int64_t ld, int s, T y, T* xs, int* status) {
+  const int i = threadIdx.x, lane = i & 31, warp = i >> 5;
+  T r[32];
+  for (int kb = (s - 1) / 32; kb >= 0; --kb) {
+    const int k0 = kb * 32, nk = min(32, s - k0);
+    if (warp <= kb) {
+#pragma unroll
+      for (int j = 0; j < 32; ++j) r[j] = (j < nk && i <= k0 + j) ? R[(int64_t)(k0 + j) * ld + i] : T(0);
+    }
+    if (warp == kb) {
+      T x = T(0);
+#pragma unroll
+      for (int j = 31; j >= 0; --j) {
+        if (j < nk) {
+          if (lane == j) {
+            if (r[j] == T(0)) dev::record(status, QRKIT_ESINGULAR);
+            x = y / r[j];
+          }
+          const T xj = __shfl_sync(0xffffffffu, x, j);
+          if (lane < j) y -= r[j] * xj;
+        }
+      }
+      y = x;
+      xs[lane] = x;
+    }
+    __syncthreads();
+    if (warp < kb) {
+#pragma unroll
+      for (int j = 0; j < 32; ++j)
+        if (j < nk) y -= r[j] * xs[j];
+    }
+    __syncthreads();
+  }
+  return y;
+}
+
+// R^T h = g: returns h_i for thread i < s.
+template <typename T>
+__device__ __forceinline__ T tri_fwdsub(const T* R, int64_t ld, int s, T g, T* xs) {
+  const int i = threadIdx.x, lane = i & 31, warp = i >> 5;
+  T r[32];
+  for (int kb = 0; kb * 32 < s; ++kb) {
+    const int k0 = kb * 32, nk = min(32, s - k0);
+    if (warp >= kb) {
+#pragma unroll
+      for (int j = 0; j < 32; ++j) r[j] = (j < nk && i < s && k0 + j <= i) ? R[(int64_t)i * ld + k0 + j] : T(0);
+    }
+    if (warp == kb) {
+      T x = T(0);
+#pragma unroll
+      for (int j = 0; j < 32; ++j) {
+        if (j < nk) {
+          if (lane == j) x = g / r[j];
+          const T xj = __shfl_sync(0xffffffffu, x, j);
+          if (lane > j) g -= r[j] * xj;
+        }
+      }
+      g = x;
+      xs[lane] = x;
+    }
+    __syncthreads();
+    if (warp > kb) {
+#pragma unroll
+      for (int j = 0; j < 32; ++j)
+        if (j < nk) g -= r[j] * xs[j];
+    }
+    __syncthreads();
+  }
+  return g;
+}
+
+// x = R_S^{-1} c (x may be c).
+template <typename T>
+__global__ void __launch_bounds__(kTriThreads) tri_backsub_kernel(const T* R, int64_t ld, int s, const T* c, T* x,
+                                                                  int* status) {
+  __shared__ T xs[32];
+  const int i = threadIdx.x;
+  const T y = tri_backsub<T>(R, ld, s, i < s ? c[i] : T(0), xs, status);
+  if (i < s) x[i] = y;
+}
+
+// dp = R_S^{-1} R_S^{-T} g (g in double), written to dp and added to x.
+template <typename T>
+__global__ void __launch_bounds__(kTriThreads) tri_normal_kernel(const T* R, int64_t ld, int s, const double* g, T* dp,
+                                                                 T* x, int* status) {
+  __shared__ T xs[32];
+  const int i = threadIdx.x;
+  const T h = tri_fwdsub<T>(R, ld, s, i < s ? (T)g[i] : T(0), xs);
+  const T y = tri_backsub<T>(R, ld, s, h, xs, status);
+  if (i < s) {
+    dp[i] = y;
+    x[i] += y;
+  }
+}
+
+// ---- block unknowns R_i x_i = c_i - R12_i x_S, one warp per block ----
+// The lanes share a row of R12 (s values, contiguous), so that the pass over R12 is coalesced and
+// many loads are in flight; the m_i <= 8 unknowns are then found by every lane alike.
+constexpr int kWarpBackThreads = 256;
+
+template <typename T>
+__global__ void __launch_bounds__(kWarpBackThreads) block_backsub_warp_kernel(ComposedView<T> V, FactorOut<T> O,
+                                                                              const T* rhs, const T* xS, T* x,
+                                                                              int accumulate) {
+  __shared__ __align__(16) T xs[kMaxDenseS];
+  const int s = V.s;
+  for (int t = threadIdx.x; t < s; t += kWarpBackThreads) xs[t] = xS[t];
+  __syncthreads();
+  const int64_t i = ((int64_t)blockIdx.x * kWarpBackThreads + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (i >= V.K) return;
+  const int n = V.n[i], m = V.m[i];
+  const int na = n + (O.damp ? m : 0);
+  const int64_t c0 = V.col_off[i];
+  const T* F = O.Fa + O.aug_off[i];
+  T y[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    y[k] = T(0);
+    if (k < m) {
+      const T* r12 = O.R12 + (c0 + k) * (int64_t)s;
+      T a = T(0);
+      bool done = false;
+      if constexpr (sizeof(T) == 4) {
+        if ((s & 3) == 0) {   // rows of R12 are then 16-byte aligned
+          const float4* r4 = reinterpret_cast<const float4*>(r12);
+          const float4* x4 = reinterpret_cast<const float4*>(xs);
+#pragma unroll 4
+          for (int t = lane; t < s / 4; t += 32) {
+            const float4 q = r4[t], z = x4[t];
+            a += q.x * z.x + q.y * z.y + q.z * z.z + q.w * z.w;
+          }
+          done = true;
+        }
+      }
+      if (!done)
+        for (int t = lane; t < s; t += 32) a += r12[t] * xs[t];
+#pragma unroll
+      for (int d = 16; d >= 1; d >>= 1) a += __shfl_xor_sync(0xffffffffu, a, d);
+      y[k] = rhs[c0 + k] - a;
+    }
+  }
+#pragma unroll
+  for (int k = 7; k >= 0; --k) {
+    if (k < m) {
+      T v = y[k];
+#pragma unroll
+      for (int j = k + 1; j < 8; ++j)
+        if (j < m) v -= F[j * na + k] * y[j];
+      y[k] = v / F[k * na + k];
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    if (k < m && lane == k) x[c0 + k] = accumulate ? x[c0 + k] + y[k] : y[k];
+}
+
+// ---- refinement of float plans: g = J^T (b - J p - S p_S) - lambda D^2 p with the residual and
+// its sums as unevaluated float pairs (Dot2) ----
+
+// 1. rows: b - S p_S as a pair per row.  A CTA takes 32 V rows; its 8 warps split the columns.
+constexpr int kRowWarps = 8;
+
+template <int V>
+__global__ void __launch_bounds__(32 * kRowWarps) dense_rows_kernel(const float* S, int64_t rows, int s, const float* b,
+                                                                    const float* pS, float* rh, float* rl) {
+  __shared__ float sh_s[kRowWarps][32 * V], sl_s[kRowWarps][32 * V];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t row0 = (int64_t)blockIdx.x * (32 * V);
+  const int64_t row = row0 + lane * V;
+  float sh[V], sl[V];
+#pragma unroll
+  for (int q = 0; q < V; ++q) sh[q] = sl[q] = 0.f;
+  if (row < rows) {   // V divides rows
+    const float* src = S + row;
+    int c = warp;
+    for (; c + 3 * kRowWarps < s; c += 4 * kRowWarps) {
+      Vec<V> a[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) a[u].load(src + (int64_t)(c + u * kRowWarps) * rows);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float p = -pS[c + u * kRowWarps];
+#pragma unroll
+        for (int q = 0; q < V; ++q) dot2(sh[q], sl[q], a[u].v[q], p);
+      }
+    }
+    for (; c < s; c += kRowWarps) {
+      Vec<V> a;
+      a.load(src + (int64_t)c * rows);
+      const float p = -pS[c];
+#pragma unroll
+      for (int q = 0; q < V; ++q) dot2(sh[q], sl[q], a.v[q], p);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < V; ++q) {
+    sh_s[warp][lane * V + q] = sh[q];
+    sl_s[warp][lane * V + q] = sl[q];
+  }
+  __syncthreads();
+  const int t = threadIdx.x;
+  if (t < 32 * V && row0 + t < rows) {
+    float h = b[row0 + t], l = 0.f;
+#pragma unroll
+    for (int w = 0; w < kRowWarps; ++w) add_pair(h, l, sh_s[w][t], sl_s[w][t]);
+    rh[row0 + t] = h;
+    rl[row0 + t] = l;
+  }
+}
+
+// 2. blocks (one thread each): r -= J p, g_B = J^T r - lambda D^2 p, h_B = R_i^{-T} g_B.
+__global__ void __launch_bounds__(128) dense_blocks_kernel(ComposedView<float> V, FactorOut<float> O, const float* p,
+                                                           double lam, float* rh, float* rl, float* h) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= V.K) return;
+  const int n = V.n[i], m = V.m[i];
+  const int na = n + (O.damp ? m : 0);
+  const int64_t c0 = V.col_off[i], r0 = V.row_off[i];
+  const float* J = V.J + V.val_off[i];
+  const float* F = O.Fa + O.aug_off[i];
+  float ph[16], pl[16], pj[8], hv[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) pj[j] = j < m ? p[c0 + j] : 0.f;
+#pragma unroll
+  for (int r = 0; r < 16; ++r) {
+    ph[r] = pl[r] = 0.f;
+    if (r < n) {
+      float sh = rh[r0 + r], sl = rl[r0 + r];
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (j < m) dot2(sh, sl, -J[j * n + r], pj[j]);
+      ph[r] = sh;
+      pl[r] = sl;
+      rh[r0 + r] = sh;
+      rl[r0 + r] = sl;
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    hv[k] = 0.f;
+    if (k < m) {
+      float ah = 0.f, al = 0.f;
+#pragma unroll
+      for (int r = 0; r < 16; ++r)
+        if (r < n) {
+          const float a = J[k * n + r];
+          dot2(ah, al, a, ph[r]);
+          al = __fmaf_rn(a, pl[r], al);
+        }
+      const double d = O.D[c0 + k];
+      float v = (float)(((double)ah + (double)al) - lam * d * d * (double)pj[k]);
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (j < k) v -= F[k * na + j] * hv[j];
+      hv[k] = v / F[k * na + k];
+      h[c0 + k] = hv[k];
+    }
+  }
+}
+
+// 3. shared columns, first part: S^T r per chunk of kSumRows rows.  A warp takes a column at a
+// time; the chunk's r pairs are in shared memory.
+constexpr int kSumRows = 2048;
+constexpr int kSumWarps = 8;
+constexpr int kSumCols = 2;    // columns per warp
+
+template <int V>
+__global__ void __launch_bounds__(32 * kSumWarps) dense_cols_kernel(const float* S, int64_t rows, int s, const float* rh,
+                                                                    const float* rl, double* part) {
+  __shared__ __align__(16) float rh_s[kSumRows], rl_s[kSumRows];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t row0 = (int64_t)blockIdx.x * kSumRows;
+  const int nr = (int)(rows - row0 < kSumRows ? rows - row0 : kSumRows);
+  for (int e = threadIdx.x; e < nr; e += 32 * kSumWarps) {
+    rh_s[e] = rh[row0 + e];
+    rl_s[e] = rl[row0 + e];
+  }
+  __syncthreads();
+  for (int u = 0; u < kSumCols; ++u) {
+    const int c = ((int)blockIdx.y * kSumCols + u) * kSumWarps + warp;
+    if (c >= s) return;
+    const float* src = S + (int64_t)c * rows + row0;
+    float sh = 0.f, sl = 0.f;
+#pragma unroll 4
+    for (int e = lane * V; e < nr; e += 32 * V) {   // V divides nr
+      Vec<V> a, h, l;
+      a.load(src + e);
+      h.load(rh_s + e);
+      l.load(rl_s + e);
+#pragma unroll
+      for (int q = 0; q < V; ++q) {
+        dot2(sh, sl, a.v[q], h.v[q]);
+        sl = __fmaf_rn(a.v[q], l.v[q], sl);
+      }
+    }
+    double t = (double)sh + (double)sl;
+#pragma unroll
+    for (int d = 16; d >= 1; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
+    if (lane == 0) part[(int64_t)blockIdx.x * s + c] = t;
+  }
+}
+
+// ... second part: R12^T h per chunk of kR12Rows rows of R12 (row-major, s values each).  A
+// thread takes V adjacent columns; groups of threads take alternate rows.
+constexpr int kR12Rows = 512;
+constexpr int kR12Threads = 256;
+
+template <int V>
+__global__ void __launch_bounds__(kR12Threads) dense_r12_kernel(const float* R12, int64_t nb, int s, const float* h,
+                                                                double* part) {
+  __shared__ float h_s[kR12Rows];
+  __shared__ double sum_s[kR12Threads * V];
+  const int64_t j0 = (int64_t)blockIdx.x * kR12Rows;
+  const int nj = (int)(nb - j0 < kR12Rows ? nb - j0 : kR12Rows);
+  const int units = s / V;                                   // V divides s
+  const int u0 = (int)blockIdx.y * kR12Threads;
+  const int nu = min(kR12Threads, units - u0);               // column units of this CTA
+  const int groups = kR12Threads / nu;
+  const int u = (int)threadIdx.x % nu, g = (int)threadIdx.x / nu;
+  for (int e = threadIdx.x; e < nj; e += kR12Threads) h_s[e] = h[j0 + e];
+  __syncthreads();
+  if (g < groups) {
+    float sh[V], sl[V];
+#pragma unroll
+    for (int q = 0; q < V; ++q) sh[q] = sl[q] = 0.f;
+    const float* src = R12 + j0 * s + (int64_t)(u0 + u) * V;
+#pragma unroll 4
+    for (int j = g; j < nj; j += groups) {
+      Vec<V> a;
+      a.load(src + (int64_t)j * s);
+#pragma unroll
+      for (int q = 0; q < V; ++q) dot2(sh[q], sl[q], a.v[q], h_s[j]);
+    }
+#pragma unroll
+    for (int q = 0; q < V; ++q) sum_s[(g * nu + u) * V + q] = (double)sh[q] + (double)sl[q];
+  }
+  __syncthreads();
+  for (int c = threadIdx.x; c < nu * V; c += kR12Threads) {
+    double t = 0;
+    for (int k = 0; k < groups; ++k) t += sum_s[k * nu * V + c];
+    part[(int64_t)blockIdx.x * s + (int64_t)u0 * V + c] = t;
+  }
+}
+
+// ... and their sum, one warp per column in a fixed order: g_S = S^T r - R12^T h - lambda D^2 p_S.
+__global__ void __launch_bounds__(256) dense_gsum_kernel(const double* part_s, int64_t ns, const double* part_r,
+                                                         int64_t nr, int s, const double* DS, const float* pS,
+                                                         double lam, double* gS) {
+  const int c = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (c >= s) return;
+  double t = 0;
+  for (int64_t k = lane; k < ns; k += 32) t += part_s[k * s + c];
+  for (int64_t k = lane; k < nr; k += 32) t -= part_r[k * s + c];
+#pragma unroll
+  for (int d = 16; d >= 1; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
+  if (lane == 0) {
+    const double d = DS[c];
+    gS[c] = t - lam * d * d * (double)pS[c];
+  }
+}
+
+inline unsigned nblk(int64_t n, int64_t t) { return (unsigned)((n + t - 1) / t); }
+
+}  // namespace
+
+#define DS_LAUNCH(ctx, ...)                         \
+  do {                                              \
+    __VA_ARGS__;                                    \
+    (ctx)->launches += 1;                           \
+    QRKIT_CUDA_TRY(ctx, cudaGetLastError());        \
+  } while (0)
+
+template <typename T>
+qrkit_status dense_backsub(qrkit_ctx* ctx, const T* R, int64_t ld, int s, const T* c, T* x) {
+  DS_LAUNCH(ctx, tri_backsub_kernel<T><<<1, tri_cta(s), 0, ctx->stream>>>(R, ld, s, c, x, ctx->d_status));
+  return QRKIT_OK;
+}
+template qrkit_status dense_backsub<float>(qrkit_ctx*, const float*, int64_t, int, const float*, float*);
+template qrkit_status dense_backsub<double>(qrkit_ctx*, const double*, int64_t, int, const double*, double*);
+
+template <typename T>
+qrkit_status dense_normal(qrkit_ctx* ctx, const T* R, int64_t ld, int s, const double* g, T* dp, T* x) {
+  DS_LAUNCH(ctx, tri_normal_kernel<T><<<1, tri_cta(s), 0, ctx->stream>>>(R, ld, s, g, dp, x, ctx->d_status));
+  return QRKIT_OK;
+}
+template qrkit_status dense_normal<float>(qrkit_ctx*, const float*, int64_t, int, const double*, float*, float*);
+template qrkit_status dense_normal<double>(qrkit_ctx*, const double*, int64_t, int, const double*, double*, double*);
+
+template <typename T>
+qrkit_status dense_block_backsub(qrkit_ctx* ctx, const ComposedView<T>& V, const FactorOut<T>& O, const T* rhs,
+                                 const T* xS, T* x, int accumulate) {
+  DS_LAUNCH(ctx, block_backsub_warp_kernel<T><<<nblk(V.K * 32, kWarpBackThreads), kWarpBackThreads, 0, ctx->stream>>>(
+                     V, O, rhs, xS, x, accumulate));
+  return QRKIT_OK;
+}
+template qrkit_status dense_block_backsub<float>(qrkit_ctx*, const ComposedView<float>&, const FactorOut<float>&,
+                                                 const float*, const float*, float*, int);
+template qrkit_status dense_block_backsub<double>(qrkit_ctx*, const ComposedView<double>&, const FactorOut<double>&,
+                                                  const double*, const double*, double*, int);
+
+size_t dense_refine_bytes(int64_t rows, int64_t nb, int s) {
+  const int64_t chunks = (rows + kSumRows - 1) / kSumRows + (nb + kR12Rows - 1) / kR12Rows;
+  return (size_t)chunks * s * sizeof(double) + 2 * (size_t)((rows + 3) & ~int64_t(3)) * sizeof(float);
+}
+
+qrkit_status dense_refine_gradient(qrkit_ctx* ctx, const ComposedView<float>& V, const FactorOut<float>& O,
+                                   const float* b, const float* p, double lam, void* ws, float* h, double* gS) {
+  cudaStream_t st = ctx->stream;
+  const int s = V.s;
+  const int64_t ns = (V.rows + kSumRows - 1) / kSumRows, nr = (V.nb + kR12Rows - 1) / kR12Rows;
+  double* part_s = (double*)ws;
+  double* part_r = part_s + ns * s;
+  float* rh = (float*)(part_r + nr * s);
+  float* rl = rh + ((V.rows + 3) & ~int64_t(3));
+  // 16-byte loads where every column of the caller's S is 16-byte aligned
+  const bool v4 = (V.rows & 3) == 0 && (reinterpret_cast<uintptr_t>(V.S) & 15) == 0;
+  if (v4)
+    DS_LAUNCH(ctx, dense_rows_kernel<4><<<nblk(V.rows, 128), 32 * kRowWarps, 0, st>>>(V.S, V.rows, s, b, p + V.nb, rh, rl));
+  else
+    DS_LAUNCH(ctx, dense_rows_kernel<1><<<nblk(V.rows, 32), 32 * kRowWarps, 0, st>>>(V.S, V.rows, s, b, p + V.nb, rh, rl));
+  DS_LAUNCH(ctx, dense_blocks_kernel<<<nblk(V.K, 128), 128, 0, st>>>(V, O, p, lam, rh, rl, h));
+  const dim3 gs((unsigned)ns, nblk(s, kSumWarps * kSumCols));
+  if (v4)
+    DS_LAUNCH(ctx, dense_cols_kernel<4><<<gs, 32 * kSumWarps, 0, st>>>(V.S, V.rows, s, rh, rl, part_s));
+  else
+    DS_LAUNCH(ctx, dense_cols_kernel<1><<<gs, 32 * kSumWarps, 0, st>>>(V.S, V.rows, s, rh, rl, part_s));
+  if ((s & 3) == 0)
+    DS_LAUNCH(ctx, dense_r12_kernel<4><<<dim3((unsigned)nr, nblk(s / 4, kR12Threads)), kR12Threads, 0, st>>>(
+                       O.R12, V.nb, s, h, part_r));
+  else
+    DS_LAUNCH(ctx, dense_r12_kernel<1><<<dim3((unsigned)nr, nblk(s, kR12Threads)), kR12Threads, 0, st>>>(
+                       O.R12, V.nb, s, h, part_r));
+  DS_LAUNCH(ctx, dense_gsum_kernel<<<nblk((int64_t)s * 32, 256), 256, 0, st>>>(part_s, ns, part_r, nr, s, O.D + V.nb,
+                                                                             p + V.nb, lam, gS));
+  return QRKIT_OK;
+}
+
+}  // namespace qrkit

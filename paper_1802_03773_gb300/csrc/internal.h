@@ -197,6 +197,7 @@ struct Composed {
   std::vector<TsqrPanel> panels;   // s > 128: the column panels after the first
   int panel0_w = 0;                // columns of the first panel's factor (s, or 128 with panels)
   DevBuf Rs, cs;                   // with panels: R_S (s x s, column-major) and its rhs
+  DevBuf dref;                     // float dense S: residual pairs and column partials of a refinement step
   DevBuf dense_ws;                 // qrkit_dense_lstsq: the copied matrix and rhs
   const void* J = nullptr;         // caller's values recorded at factor time
   const void* S = nullptr;
@@ -330,6 +331,19 @@ qrkit_status tsqr_panel_apply(qrkit_ctx* ctx, const float* X, int64_t ld, int64_
                               int64_t tiles);
 constexpr int kPanelCols = 32;    // column panel width of a (float) dense reduced block wider than that
 constexpr int kMaxDenseS = 512;   // widest dense reduced block (float, column panels)
+// Solves with a dense S (dense_solve.cu): x = R_S^{-1} c; dp = R_S^{-1} R_S^{-T} g, also added to x;
+// R_i x_i = rhs_i - R12_i x_S by a warp per block; and, for float plans, a refinement step's
+// h_B = R_i^{-T} g_B and g_S - R12^T h_B with g = J^T (b - J p) - lambda D^2 p (ws: dense_refine_bytes).
+template <typename T>
+qrkit_status dense_backsub(qrkit_ctx* ctx, const T* R, int64_t ld, int s, const T* c, T* x);
+template <typename T>
+qrkit_status dense_normal(qrkit_ctx* ctx, const T* R, int64_t ld, int s, const double* g, T* dp, T* x);
+template <typename T>
+qrkit_status dense_block_backsub(qrkit_ctx* ctx, const ComposedView<T>& V, const FactorOut<T>& O, const T* rhs,
+                                 const T* xS, T* x, int accumulate);
+size_t dense_refine_bytes(int64_t rows, int64_t nb, int s);
+qrkit_status dense_refine_gradient(qrkit_ctx* ctx, const ComposedView<float>& V, const FactorOut<float>& O,
+                                   const float* b, const float* p, double lam, void* ws, float* h, double* gS);
 qrkit_status reduced_rhs_sort(qrkit_ctx* ctx, const int64_t* spos, const void* rhs, void* rhs_s, int64_t rows);
 void release_band(Band& B);
 qrkit_status launch_block_solve(qrkit_ctx* ctx, const void* J, const void* b, const void* D,
