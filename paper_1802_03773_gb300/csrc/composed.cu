@@ -375,14 +375,15 @@ __global__ void block_factor_kernel(ComposedView<T> V, FactorOut<T> O) {
   }
 }
 
-// Damping rows of the shared columns, appended below the stacked bottoms (dense case).
+// Damping rows of the shared columns (dense case), s rows from row0, and with `damp` false zero rows
+// that pad the first level: `count` rows in all.
 template <typename T>
-__global__ void reduced_damping_kernel(T* X0, int64_t ld0, int64_t row0, int s, const double* D,
+__global__ void reduced_damping_kernel(T* X0, int64_t ld0, int64_t row0, int s, int count, bool damp, const double* D,
                                        int64_t nb, double lam_half) {
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e >= (int64_t)s * s) return;
-  const int j = (int)(e / s), c = (int)(e % s);
-  X0[(int64_t)c * ld0 + row0 + j] = (c == j) ? (T)(lam_half * D[nb + j]) : T(0);
+  if (e >= (int64_t)count * s) return;
+  const int c = (int)(e / count), j = (int)(e % count);
+  X0[(int64_t)c * ld0 + row0 + j] = (damp && c == j) ? (T)(lam_half * D[nb + j]) : T(0);
 }
 
 // ---- TSQR tile factor: one CTA per row tile of a level matrix (column-major, ld) ----
@@ -462,12 +463,11 @@ tsqr_tile_kernel(T* X, int64_t ld, int64_t M, int s, int tile_rows, T* taus, T* 
   }
 }
 
-// Q_tile^T applied to a level's rhs segment; the top min(r, s) entries go to the next level, and
-// with column panels the others to the next panel's first level (row down0 + tile (tile_rows - s)).
+// Q_tile^T applied to a level's rhs segment; the top min(r, s) entries go to the next level.
 template <typename T>
 __global__ void __launch_bounds__(kTileThreads)
 tsqr_apply_qt_kernel(const T* X, int64_t ld, int64_t M, int s, int tile_rows, const T* taus,
-                     T* rhs, T* rhs_next, T* rhs_down, int64_t down0) {
+                     T* rhs, T* rhs_next) {
   __shared__ T red[32];
   const int64_t r0 = (int64_t)blockIdx.x * tile_rows;
   const int r = (int)(M - r0 < (int64_t)tile_rows ? M - r0 : (int64_t)tile_rows);
@@ -495,9 +495,6 @@ tsqr_apply_qt_kernel(const T* X, int64_t ld, int64_t M, int s, int tile_rows, co
   }
   if (rhs_next)
     for (int i = tid; i < kmax; i += blockDim.x) rhs_next[(int64_t)blockIdx.x * s + i] = y[i];
-  if (rhs_down)   // column panels: the rows below the tile's R rows, for the next panel
-    for (int i = kmax + tid; i < r; i += blockDim.x)
-      rhs_down[down0 + (int64_t)blockIdx.x * (tile_rows - s) + (i - kmax)] = y[i];
 }
 
 // Per-block Q_i^T [b_i; 0]: top m -> ctop, bottom -> reduced rhs rows.  NA > 0: every block has
@@ -1085,6 +1082,14 @@ static ComposedView<T> view(qrkit_ctx* ctx, const void* J, const void* S) {
   return V;
 }
 
+// Rows of the dense reduced block before the stacked bottoms.  With column panels the damping rows of
+// the shared columns come first: row c of a tile moves up by 32 with every panel, so each of them is
+// the pivot row of its own column, and a column that is zero but for it stays exactly zero elsewhere.
+static int64_t reduced_head(const qrkit_ctx* ctx) {
+  const Composed& C = ctx->comp;
+  return C.damp && !C.panels.empty() ? ctx->plan.s.shared_cols : 0;
+}
+
 template <typename T>
 static FactorOut<T> fout(qrkit_ctx* ctx) {
   Composed& C = ctx->comp;
@@ -1098,7 +1103,7 @@ static FactorOut<T> fout(qrkit_ctx* ctx) {
   O.ctop = (T*)C.ctop.ptr;
   O.aug_off = (const int64_t*)(C.damp ? C.d_aug_off_d.ptr : C.d_aug_off_u.ptr);
   O.red_off = (const int64_t*)(C.damp ? C.d_red_off_d.ptr : C.d_red_off_u.ptr);
-  O.X0 = C.levels.empty() ? nullptr : (T*)C.levels[0].X.ptr;
+  O.X0 = C.levels.empty() ? nullptr : (T*)C.levels[0].X.ptr + reduced_head(ctx);
   O.ld0 = C.levels.empty() ? 0 : C.levels[0].ld;
   O.Xw = (T*)C.Xw.ptr;
   O.Xstart = (int64_t*)C.Xstart.ptr;
@@ -1174,30 +1179,25 @@ static qrkit_status norms_typed(qrkit_ctx* ctx, const ComposedView<T>& V, double
 // panel width, while the trailing updates do the rest of the arithmetic.
 static qrkit_status factor_panels(qrkit_ctx* ctx, int s) {
   Composed& C = ctx->comp;
-  cudaStream_t st = ctx->stream;
   float* Rs = (float*)C.Rs.ptr;
   const int np = 1 + (int)C.panels.size();
   for (int j = 0; j < np; ++j) {
     std::vector<TsqrLevel>& LV = j == 0 ? C.levels : C.panels[j - 1].levels;
     const int c0 = j * kPanelCols;
-    const int pw = std::min(kPanelCols, s - c0);
-    const int n = s - c0 - pw;   // trailing columns
-    if (pw != kPanelCols) return fail(ctx, QRKIT_EINVAL, "column panels: s must be a multiple of 32");
+    const int n = s - c0 - kPanelCols;   // trailing columns
     for (size_t l = 0; l < LV.size(); ++l) {
       TsqrLevel& L = LV[l];
       const bool top = l + 1 == LV.size();
       float* X = (float*)L.X.ptr;
-      float* Xn = top ? Rs + (int64_t)c0 * s + c0 : (float*)LV[l + 1].X.ptr;
       const int64_t ldn = top ? s : LV[l + 1].ld;
-      qrkit_status rc = tsqr_panel_tile(ctx, X, L.ld, L.M, (float*)L.tau.ptr, Xn, ldn, L.tiles,
-                                        n > 0 ? (float*)L.T.ptr : nullptr);
+      float* Xn = top ? Rs + (int64_t)c0 * s + c0 : (float*)LV[l + 1].X.ptr;
+      qrkit_status rc = tsqr_panel_tile(ctx, X, L.ld, L.M, Xn, ldn, L.tiles, (float*)L.T.ptr,
+                                        (float*)L.tau.ptr);
       if (rc != QRKIT_OK) return rc;
       if (n > 0) {
-        float* upp = top ? Rs + (int64_t)(c0 + pw) * s + c0 : (float*)LV[l + 1].X.ptr + (int64_t)pw * LV[l + 1].ld;
-        const int64_t ldu = top ? s : LV[l + 1].ld;
         TsqrLevel& N0 = C.panels[j].levels[0];
-        rc = tsqr_panel_apply(ctx, X, L.ld, L.M, pw, (const float*)L.T.ptr, n, upp, ldu, (float*)N0.X.ptr, N0.ld,
-                              L.down0, L.tiles);
+        rc = tsqr_panel_apply(ctx, X, L.ld, L.M, (const float*)L.T.ptr, n, Xn + kPanelCols * ldn, ldn,
+                              (float*)N0.X.ptr, N0.ld, L.down0, L.tiles);
         if (rc != QRKIT_OK) return rc;
       }
     }
@@ -1250,10 +1250,15 @@ static qrkit_status factor_typed(qrkit_ctx* ctx, const void* J, const void* S, c
   }
   if (V.coupled == QRKIT_COUPLED_DENSE) {
     const int s = V.s;
+    T* X0 = (T*)C.levels[0].X.ptr;
     if (C.damp)
       LAUNCH(ctx, reduced_damping_kernel<T><<<blocks_for((int64_t)s * s, 256), 256, 0, st>>>(
-                      (T*)C.levels[0].X.ptr, C.levels[0].ld, C.red_rows, s, (const double*)C.D.ptr,
-                      P.cols, C.lam_half));
+                      X0, C.levels[0].ld, C.panels.empty() ? C.red_rows : 0, s, s, true, (const double*)C.D.ptr, P.cols,
+                      C.lam_half));
+    const int64_t used = C.red_rows + (C.damp ? s : 0);
+    if (C.levels[0].M > used)
+      LAUNCH(ctx, reduced_damping_kernel<T><<<blocks_for((C.levels[0].M - used) * s, 256), 256, 0, st>>>(
+                      X0, C.levels[0].ld, used, s, (int)(C.levels[0].M - used), false, nullptr, 0, 0.0));
     if (!C.panels.empty()) return factor_panels(ctx, s);
     for (size_t l = 0; l < C.levels.size(); ++l) {
       TsqrLevel& L = C.levels[l];
@@ -1281,29 +1286,37 @@ static qrkit_status solve_typed(qrkit_ctx* ctx, const void* J, const void* S, co
   const int64_t nb = P.cols;
   T* x = (T*)p;
   // Q^T [b; 0]
-  T* rhs0 = (V.coupled == QRKIT_COUPLED_DENSE) ? (T*)C.levels[0].rhs.ptr
+  T* rhs0 = (V.coupled == QRKIT_COUPLED_DENSE) ? (T*)C.levels[0].rhs.ptr + reduced_head(ctx)
              : (V.coupled == QRKIT_COUPLED_WINDOW ? (T*)C.rhs_red.ptr : nullptr);
   LAUNCH_SHAPED(ctx, small_class(P, O.damp), block_apply_qt_kernel, blocks_for(P.K, 64), 64, 0, st, V, O, (const T*)b,
                 rhs0);
   if (V.coupled == QRKIT_COUPLED_DENSE) {
-    if (C.damp)
-      QRKIT_CUDA_TRY(ctx, cudaMemsetAsync(rhs0 + C.red_rows, 0, (size_t)s * sizeof(T), st));
-    // Q^T of every panel's levels: the top rows of a level go up (the last level's into c_S),
-    // the others, with column panels, into the next panel's first level
-    const int np = 1 + (int)C.panels.size();
-    for (int j = 0; j < np; ++j) {
-      std::vector<TsqrLevel>& LV = j == 0 ? C.levels : C.panels[j - 1].levels;
-      const int c0 = j == 0 ? 0 : C.panels[j - 1].c0;
-      const int pw = j == 0 ? C.panel0_w : C.panels[j - 1].pw;
-      T* down = j + 1 < np ? (T*)C.panels[j].levels[0].rhs.ptr : nullptr;
-      for (size_t l = 0; l < LV.size(); ++l) {
-        TsqrLevel& L = LV[l];
-        const bool top = l + 1 == LV.size();
-        T* rn = !top ? (T*)LV[l + 1].rhs.ptr : (np > 1 ? (T*)C.cs.ptr + c0 : nullptr);
-        LAUNCH(ctx, tsqr_apply_qt_kernel<T><<<(unsigned)L.tiles, kTileThreads, 0, st>>>(
-                        (const T*)L.X.ptr, L.ld, L.M, pw, C.tile_rows, (const T*)L.tau.ptr, (T*)L.rhs.ptr, rn, down,
-                        L.down0));
+    const int64_t head = reduced_head(ctx), tail = C.levels[0].M - head - C.red_rows;   // damping rows and padding
+    if (head > 0) QRKIT_CUDA_TRY(ctx, cudaMemsetAsync(C.levels[0].rhs.ptr, 0, (size_t)head * sizeof(T), st));
+    if (tail > 0) QRKIT_CUDA_TRY(ctx, cudaMemsetAsync(rhs0 + C.red_rows, 0, (size_t)tail * sizeof(T), st));
+    bool done = false;
+    if constexpr (sizeof(T) == sizeof(float)) {
+      // Q^T of every panel's levels: a level's top rows go up (the last level's into c_S), the
+      // others into the next panel's first level
+      const int np = 1 + (int)C.panels.size();
+      for (int j = 0; j < np && np > 1; ++j) {
+        std::vector<TsqrLevel>& LV = j == 0 ? C.levels : C.panels[j - 1].levels;
+        float* down = j + 1 < np ? (float*)C.panels[j].levels[0].rhs.ptr : nullptr;
+        for (size_t l = 0; l < LV.size(); ++l) {
+          TsqrLevel& L = LV[l];
+          float* rn = l + 1 < LV.size() ? (float*)LV[l + 1].rhs.ptr : (float*)C.cs.ptr + j * kPanelCols;
+          qrkit_status rc = tsqr_panel_qt(ctx, (const float*)L.X.ptr, L.ld, L.M, (const float*)L.tau.ptr,
+                                          (const float*)L.rhs.ptr, rn, down, L.down0, L.tiles);
+          if (rc != QRKIT_OK) return rc;
+        }
+        done = true;
       }
+    }
+    for (size_t l = 0; l < C.levels.size() && !done; ++l) {
+      TsqrLevel& L = C.levels[l];
+      T* rn = l + 1 < C.levels.size() ? (T*)C.levels[l + 1].rhs.ptr : nullptr;
+      LAUNCH(ctx, tsqr_apply_qt_kernel<T><<<(unsigned)L.tiles, kTileThreads, 0, st>>>(
+                      (const T*)L.X.ptr, L.ld, L.M, s, C.tile_rows, (const T*)L.tau.ptr, (T*)L.rhs.ptr, rn));
     }
   }
   if (V.coupled == QRKIT_COUPLED_WINDOW && qt_only)
@@ -1607,22 +1620,24 @@ qrkit_status composed_layout(qrkit_ctx* ctx, size_t elem) {
     if (s > 64 && !panels)
       return fail(ctx, QRKIT_EUNSUPPORTED,
                   "dense shared block: s <= 64, or (float) s a multiple of 32 up to 512");
-    const int64_t M0 = C.red_rows + (C.damp ? s : 0);
+    int64_t M0 = C.red_rows + (C.damp ? s : 0);
     if (M0 < s) return fail(ctx, QRKIT_EINVAL, "reduced shared block has fewer rows than columns");
     if (elem == sizeof(float) &&
         (rc = ensure(ctx, C.dref, dense_refine_bytes(P.rows, P.cols, s), "refinement sums")) != QRKIT_OK)
       return rc;
     C.tile_rows = 256;
+    const int tr = panels ? kPanelRows : C.tile_rows;
+    if (panels) M0 = (M0 + 3) & ~int64_t(3);   // zero rows: every row count below is then a multiple of 4
     // the TSQR levels of a panel of pw columns over M rows, w columns wide (panel + trailing);
     // each level's leading dimension is padded to 16 bytes, and the rows that leave a panel
     // (all but its R rows) are laid out level by level, tile by tile, for the next panel
-    auto build_levels = [&](std::vector<TsqrLevel>& LV, int64_t M, int pw, int w, bool need_T) -> qrkit_status {
+    auto build_levels = [&](std::vector<TsqrLevel>& LV, int64_t M, int pw, int w) -> qrkit_status {
       std::vector<int64_t> Ms;
       while (true) {
         Ms.push_back(M);
-        const int64_t tiles = (M + C.tile_rows - 1) / C.tile_rows;
+        const int64_t tiles = (M + tr - 1) / tr;
         if (tiles <= 1) break;
-        const int64_t last = M - (tiles - 1) * C.tile_rows;
+        const int64_t last = M - (tiles - 1) * tr;
         M = (tiles - 1) * pw + std::min<int64_t>(last, pw);
       }
       if (LV.size() != Ms.size()) {
@@ -1635,21 +1650,20 @@ qrkit_status composed_layout(qrkit_ctx* ctx, size_t elem) {
         TsqrLevel& L = LV[l];
         L.M = Ms[l];
         L.ld = (L.M + 3) & ~int64_t(3);
-        L.tiles = (L.M + C.tile_rows - 1) / C.tile_rows;
+        L.tiles = (L.M + tr - 1) / tr;
         L.down0 = down;
         down += L.M - (l + 1 < Ms.size() ? Ms[l + 1] : (int64_t)pw);
         if ((rc2 = ensure(ctx, L.X, (size_t)L.ld * w * elem, "reduced block")) != QRKIT_OK) return rc2;
-        if ((rc2 = ensure(ctx, L.tau, (size_t)L.tiles * pw * elem, "reduced tau")) != QRKIT_OK) return rc2;
         if ((rc2 = ensure(ctx, L.rhs, (size_t)L.ld * elem, "reduced rhs")) != QRKIT_OK) return rc2;
-        if (need_T && (rc2 = ensure(ctx, L.T, (size_t)L.tiles * pw * 32 * elem, "reduced T")) != QRKIT_OK)
+        if ((rc2 = ensure(ctx, L.tau, (size_t)L.tiles * pw * (panels ? pw : 1) * elem, "reduced tau")) != QRKIT_OK)
           return rc2;
+        if (panels && (rc2 = ensure(ctx, L.T, (size_t)L.tiles * pw * pw * elem, "reduced T")) != QRKIT_OK) return rc2;
       }
       return QRKIT_OK;
     };
-    C.panel0_w = panels ? kPanelCols : s;
-    if ((rc = build_levels(C.levels, M0, C.panel0_w, s, panels)) != QRKIT_OK) return rc;
+    if ((rc = build_levels(C.levels, M0, panels ? kPanelCols : s, s)) != QRKIT_OK) return rc;
     if (panels) {
-      const int np = (s + kPanelCols - 1) / kPanelCols;
+      const int np = s / kPanelCols;
       if ((int)C.panels.size() != np - 1) {
         for (auto& Pn : C.panels) release_levels(Pn.levels);
         C.panels.assign(np - 1, TsqrPanel());
@@ -1657,9 +1671,7 @@ qrkit_status composed_layout(qrkit_ctx* ctx, size_t elem) {
       for (int j = 1; j < np; ++j) {
         TsqrPanel& Pn = C.panels[j - 1];
         Pn.c0 = j * kPanelCols;
-        Pn.pw = std::min(kPanelCols, s - Pn.c0);
-        Pn.w = s - Pn.c0;
-        if ((rc = build_levels(Pn.levels, M0 - Pn.c0, Pn.pw, Pn.w, j + 1 < np)) != QRKIT_OK) return rc;
+        if ((rc = build_levels(Pn.levels, M0 - Pn.c0, kPanelCols, s - Pn.c0)) != QRKIT_OK) return rc;
       }
       if ((rc = ensure(ctx, C.Rs, (size_t)s * s * elem, "R_S")) != QRKIT_OK) return rc;
       if ((rc = ensure(ctx, C.cs, (size_t)s * elem, "R_S rhs")) != QRKIT_OK) return rc;

@@ -161,15 +161,14 @@ struct TsqrLevel {
   int64_t ld = 0;     // its leading dimension: M rounded up to a multiple of 4 (16-byte columns)
   int64_t tiles = 0;
   int64_t down0 = 0;  // column panels: first row of this level's retired rows in the next panel
-  DevBuf X, tau, rhs;
-  DevBuf T;           // column panels: the tiles' compact-WY T factors (32 x 32 per 32 columns)
+  DevBuf X, tau, rhs; // tau: per column of every tile; column panels: G with tau on its diagonal
+  DevBuf T;           // column panels: the tiles' compact-WY T factors (32 x 32)
 };
 
-// One column panel of a dense reduced block wider than one tile: columns [c0, c0 + pw) are
-// factored by TSQR over the rows the earlier panels left, and the panel's Q^T is applied to
-// the w - pw columns after it.
+// One column panel of a dense reduced block: columns [c0, c0 + 32) are factored by TSQR over the
+// rows the earlier panels left, and the panel's Q^T is applied to the columns after it.
 struct TsqrPanel {
-  int c0 = 0, pw = 0, w = 0;
+  int c0 = 0;
   std::vector<TsqrLevel> levels;
 };
 
@@ -194,8 +193,7 @@ struct Composed {
   DevBuf nrm_D, nrm_L, nrm_W, nrm_y, nrm_As, nrm_rs, nrm_seg;
   DevBuf d_aug_off_d, d_aug_off_u, d_red_off_d, d_red_off_u;
   std::vector<TsqrLevel> levels;   // TSQR levels of the first (or only) column panel
-  std::vector<TsqrPanel> panels;   // s > 128: the column panels after the first
-  int panel0_w = 0;                // columns of the first panel's factor (s, or 128 with panels)
+  std::vector<TsqrPanel> panels;   // the column panels after the first (float, s a multiple of 32 from 64)
   DevBuf Rs, cs;                   // with panels: R_S (s x s, column-major) and its rhs
   DevBuf dref;                     // float dense S: residual pairs and column partials of a refinement step
   DevBuf dense_ws;                 // qrkit_dense_lstsq: the copied matrix and rhs
@@ -318,19 +316,22 @@ qrkit_status reduced_row_sort(qrkit_ctx* ctx, const RowSortTables& t, int64_t ns
                               const int64_t* Xstart, const void* Xw, int w, int* hist, int64_t* spos,
                               int64_t* order, int64_t* Xstart_s, void* Xw_s);
 qrkit_status window_start_copy(qrkit_ctx* ctx, const int32_t* in);
-// One TSQR level of a 32-column panel (float, 256-row tiles, columns in registers): reflectors
-// and R in place, tau per column, each tile's 32 x 32 T (Tout, optional), the R rows to Xn.
-qrkit_status tsqr_panel_tile(qrkit_ctx* ctx, float* X, int64_t ld, int64_t M, float* taus, float* Xn, int64_t ldn,
-                             int64_t tiles, float* Tout);
-// Column-panel TSQR (float): the Q^T of every 256-row tile of a factored panel
-// (reflectors in X's first pw columns, T factors from tsqr_panel_tile) applied to the n trailing
-// columns X[:, pw .. pw + n); the tile's top pw rows go to `up` (row tile * pw), the rest to
-// `down` (row down0 + tile * (256 - pw)).  ld, ldu and ldd are multiples of 4.
-qrkit_status tsqr_panel_apply(qrkit_ctx* ctx, const float* X, int64_t ld, int64_t M, int pw, const float* T,
-                              int n, float* up, int64_t ldu, float* down, int64_t ldd, int64_t down0,
-                              int64_t tiles);
+// Column-panel TSQR (float; tsqr_tc.cu), one level of a 32-column panel in tiles of kPanelRows rows;
+// every pointer 16-byte aligned, every ld, row count and row offset a multiple of 4.
+// tsqr_panel_tile: reflectors and R in place, each tile's 32 x 32 T and G = Y^T Y (strict upper part,
+// tau on the diagonal), its R rows to Xn.
+// tsqr_panel_apply: the tiles' Q^T (reflectors in X's first 32 columns) applied to the n trailing
+// columns X[:, 32 .. 32 + n): a tile's top 32 rows go to `up` (row 32 tile), the rest to `down` (row
+// down0 + tile (kPanelRows - 32)).  tsqr_panel_qt: the same for a right-hand side.
 constexpr int kPanelCols = 32;    // column panel width of a (float) dense reduced block wider than that
+constexpr int kPanelRows = 1024;  // rows of a column panel's TSQR tile
 constexpr int kMaxDenseS = 512;   // widest dense reduced block (float, column panels)
+qrkit_status tsqr_panel_tile(qrkit_ctx* ctx, float* X, int64_t ld, int64_t M, float* Xn, int64_t ldn, int64_t tiles,
+                             float* Tout, float* Gout);
+qrkit_status tsqr_panel_apply(qrkit_ctx* ctx, const float* X, int64_t ld, int64_t M, const float* T, int n, float* up,
+                              int64_t ldu, float* down, int64_t ldd, int64_t down0, int64_t tiles);
+qrkit_status tsqr_panel_qt(qrkit_ctx* ctx, const float* X, int64_t ld, int64_t M, const float* G, const float* rhs,
+                           float* rhs_next, float* rhs_down, int64_t down0, int64_t tiles);
 // Solves with a dense S (dense_solve.cu): x = R_S^{-1} c; dp = R_S^{-1} R_S^{-T} g, also added to x;
 // R_i x_i = rhs_i - R12_i x_S by a warp per block; and, for float plans, a refinement step's
 // h_B = R_i^{-T} g_B and g_S - R12^T h_B with g = J^T (b - J p) - lambda D^2 p (ws: dense_refine_bytes).

@@ -1,21 +1,23 @@
-// Column-panel TSQR of the dense reduced shared block (float, s a multiple of 32, 256-row tiles).
-// The reduced block is factored by panels of 32 columns (Sec. 2, compact WY): each panel is a
-// TSQR whose tiles are factored by tsqr_panel_tile_kernel (Householder QR with the columns in
-// registers, then the panel's T), and after every TSQR level tsqr_panel_apply_kernel applies the
-// tiles' Q^T = I - Y T^T Y^T to the later columns:
-//   1. W = Y^T C for the trailing columns C, then Z = T^T W (CUDA cores);
-//   2. C -= Y Z on the tensor cores: tcgen05.mma kind::tf32 with the 3xTF32 split
-//      (Y = Y_hi + Y_lo, Z = Z_hi + Z_lo, Y Z ~ Y_hi Z_hi + Y_hi Z_lo + Y_lo Z_hi), FP32
-//      accumulation in TMEM, M = 128 rows per half tile, K = 32, N = trailing columns; the
-//      product is read back with tcgen05.ld and subtracted in shared memory.
-// Operands are staged in shared memory in the canonical K-major no-swizzle layout (8-row x
-// 16-byte core matrices) and described by tcgen05 shared-memory descriptors.  Tiles arrive by
-// bulk copies (TMA).  The outputs are those of any Householder TSQR (V below / R on and above
-// the diagonal, tau per column, the tile's R rows to the next TSQR level), so Q^T b and the
-// solves apply it reflector by reflector.
+// Column-panel TSQR of the dense reduced shared block (float, s a multiple of 32).
+//
+// The reduced block is factored by panels of 32 columns (Sec. 2, compact WY): each panel is a TSQR
+// over tiles of kPanelRows = 1024 rows.  tsqr_panel_tile_kernel factors a tile (Householder QR with
+// the columns in registers, and the tile's compact-WY T); tsqr_panel_apply_kernel applies the tiles'
+// Q^T = I - Y T^T Y^T to the later columns; tsqr_panel_qt_kernel does the same for a right-hand side.
+//
+// Tiles of 1024 rows leave 32 R rows of 1024 for the next level, so 400,000 rows need three levels
+// (391, 13 and 1 tiles) where tiles of 256 rows needed five, and a reflector's reductions and
+// barriers are paid once per 1024 rows.  100,000 blocks 4 x 2, factor + solve with one refinement
+// step, against 256-row tiles with tcgen05 updates: s = 512 37.4 -> 13.0 ms (panel tiles 9.07 -> 2.63,
+// updates 21.6 -> 6.34, Q^T b 3.25 -> 0.49), s = 128 5.58 -> 2.30 ms.
+//
+// Level matrices are column-major with a leading dimension, a row count and row offsets that are
+// multiples of 4 (the first level is padded with zero rows), so every access is a 16-byte one.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
+
+#include <algorithm>
 
 #include "device_util.cuh"
 #include "internal.h"
@@ -23,37 +25,34 @@
 namespace qrkit {
 namespace {
 
-constexpr int kRows = 256;      // tile rows (two MMA halves of 128)
-constexpr int kNb = 32;         // panel width = MMA K
-constexpr int kThr = 512;       // threads of the panel update (16 warps)
-constexpr uint32_t kWaitLimit = 1u << 26;
+constexpr int kTR = kPanelRows;   // tile rows
+constexpr int kNb = kPanelCols;   // panel width
+static_assert(kTR == 1024 && kNb == 32, "the kernels' thread layouts");
 
-__device__ __forceinline__ uint32_t su32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ float to_tf32(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return __uint_as_float(r);
+// Two floats at a time (fma.rn.f32x2 and mul.rn.f32x2): half the instructions of the scalar forms.
+using f2 = unsigned long long;
+__device__ __forceinline__ f2 pack2(float x, float y) {
+  f2 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+  return d;
 }
-
-// Byte offset of (row, k) in a K-major, no-swizzle operand with K = 32: 8-row x 16-byte core
-// matrices, adjacent in K at 128 B (LBO), 8-row groups at 1024 B (SBO).
-__device__ __forceinline__ uint32_t koff(int row, int k) {
-  return (uint32_t)((row >> 3) * 1024 + (k >> 2) * 128 + (row & 7) * 16 + (k & 3) * 4);
+__device__ __forceinline__ void unpack2(f2 d, float& x, float& y) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(d));
 }
-
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
-  uint64_t d = (uint64_t)((addr >> 4) & 0x3FFF);
-  d |= (uint64_t)(128 >> 4) << 16;    // leading byte offset: next core matrix in K
-  d |= (uint64_t)(1024 >> 4) << 32;   // stride byte offset: next 8-row group
-  d |= (uint64_t)1 << 46;             // descriptor version
-  return d;                           // base offset 0, no swizzle
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+  f2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
 }
-
-__device__ __forceinline__ uint32_t idesc_tf32(int m, int n) {
-  // D f32 (bits 4-5 = 1), A and B tf32 (= 2 at bits 7-9, 10-12), both K-major, N >> 3 at
-  // bits 17-22, M >> 4 at bits 24-28
-  return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+  f2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ float sum2(f2 d) {
+  float x, y;
+  unpack2(d, x, y);
+  return x + y;
 }
 
 __device__ __forceinline__ float warp_sum(float v) {
@@ -78,111 +77,70 @@ __device__ __forceinline__ float transpose_reduce(float (&v)[32], int lane) {
   return v[0];
 }
 
-__device__ __forceinline__ void tc_record(int* status, int code) {
-  if (status) atomicCAS(status, 0, code);
-}
-
-// Rows [r0, r0 + r) of `cols` columns of a column-major matrix (ld a multiple of 4, 16-byte
-// aligned base) into shared memory at a column stride of kRows, by bulk copies (TMA) on one
-// mbarrier; issued by one thread.  Each copy takes the rows rounded up to a multiple of 4 (inside
-// the padded column), so the caller zeroes rows r .. kRows - 1 after the wait.
-__device__ __forceinline__ uint32_t column_bytes(int r) { return (uint32_t)((r + 3) & ~3) * 4u; }
-__device__ __forceinline__ void stage_columns(float* dst, const float* src, int64_t ld, int64_t r0, int r,
-                                              int cols, uint64_t* bar) {
-  const uint32_t cb = column_bytes(r);
-  for (int c = 0; c < cols; ++c) dev::bulk_g2s(dst + (size_t)c * kRows, src + (int64_t)c * ld + r0, cb, bar);
-}
-
-// Bounded wait for the mbarrier's phase `parity`; false if the limit ran out.
-__device__ __forceinline__ bool wait_phase(uint64_t* bar, uint32_t parity) {
-  for (uint32_t it = 0; it < kWaitLimit; ++it)
-    if (dev::mbar_try_wait(bar, parity)) return true;
-  return false;
-}
-
-// ---- Column-panel TSQR: the QR of one 256-row tile of a 32-column panel ----
+// ---- the QR of one tile (up to 1024 x 32) of a panel ----
 //
-// Householder QR (Sec. 2) of a 256 x 32 tile with its columns in registers: column j lives on
-// warp j % 16, row i = lane + 32 u (u < 8) of it on the lane.  At step k the reflector v_k of
-// column k goes through shared memory (two alternating slots); every warp applies it to its
-// columns after k (a dot product, then an axpy, in registers) and takes the products
-// G[c][k] = v_c^T v_k of its columns c before k, its two reductions interleaved; the warp that
-// holds column k + 1 forms the next reflector right after updating it.  Then the compact-WY T
-// (T[k][k] = tau_k, column k of the strict upper part = -tau_k T[:, :k] G[:k, k]) for the panel
-// update.  Outputs as any TSQR tile: reflectors below / R on and above the diagonal in place,
-// tau per column, T, the R rows to the next level.
-constexpr int kPT = 512;        // threads of a panel tile (16 warps, two columns each)
-constexpr int kPad = kNb + 1;   // row stride of G and T in shared memory (conflict-free rows)
+// 16 warps; column j lives in the registers of warp j % 16, rows 128 u + 4 lane + q (u < NU, q < 4)
+// on the lane.  At step k the reflector v_k goes through shared memory (two alternating slots);
+// every warp takes v_k against its two columns: those after k are updated, those before k give
+// G[c][k] = v_c^T v_k (v_k is zero above row k, so the R entries above a reflector drop out).  The
+// warp that holds column k + 1 forms the next reflector right after updating it, and one other warp
+// adds column k - 1 of T (T[k][k] = tau_k, the strict upper part -tau_k T[:, :k] G[:k, k]).  Bound by
+// the chain of a step (update, reduction, next reflector, barrier).  NU = 2, 4 or 8: the smallest
+// that covers the level's tiles, so that a short top level does not walk 1024 rows.
+constexpr int kPT = 512;
+constexpr int kPad = kNb + 1;   // row stride of G and T in shared memory (conflict-free columns)
 
-size_t panel_tile_smem() {
-  return (size_t)kRows * kNb * 4 + 2 * (size_t)kRows * 4 + 2 * (size_t)kNb * kPad * 4;
-}
-
+template <int NU>
 __global__ void __launch_bounds__(kPT, 1)
-tsqr_panel_tile_kernel(float* X, int64_t ld, int64_t M, float* taus, float* Xn, int64_t ldn, float* Tout,
-                       int* status) {
-  extern __shared__ __align__(1024) unsigned char smem_raw[];
-  float* A = reinterpret_cast<float*>(smem_raw);   // 256 x 32, column-major
-  float* V = A + kRows * kNb;                      // two reflector slots of 256
-  float* Gs = V + 2 * kRows;                       // 32 x 33: G[m][k] at m * kPad + k
-  float* Tm = Gs + kNb * kPad;                     // 32 x 33: T[l][k] at l * kPad + k
-  __shared__ float tslot[2];
-  __shared__ float tau_s[kNb];
-  __shared__ __align__(8) uint64_t mbar_ld;
-
+tsqr_panel_tile_kernel(float* X, int64_t ld, int64_t M, float* Xn, int64_t ldn, float* Tout, float* Gout) {
+  __shared__ __align__(16) float V[2][128 * NU];
+  __shared__ float Gs[kNb * kPad], Tm[kNb * kPad];
+  __shared__ float tslot[2], tau_s[kNb];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t r0 = (int64_t)blockIdx.x * kRows;
-  const int r = (int)(M - r0 < (int64_t)kRows ? M - r0 : (int64_t)kRows);
+  const int64_t r0 = (int64_t)blockIdx.x * kTR;
+  const int r = (int)(M - r0 < (int64_t)kTR ? M - r0 : (int64_t)kTR);   // a multiple of 4
   const int kmax = r < kNb ? r : kNb;
-  const bool bulk = (ld & 3) == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+  const int c0 = warp, c1 = warp + 16;
+  float* x0 = X + (int64_t)c0 * ld + r0 + 4 * lane;
+  float* x1 = X + (int64_t)c1 * ld + r0 + 4 * lane;
 
-  if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&mbar_ld)), "r"(1));
-    asm volatile("fence.mbarrier_init.release.cluster;");
-    if (bulk) {
-      dev::mbar_expect_tx(&mbar_ld, column_bytes(r) * (uint32_t)kNb);
-      stage_columns(A, X, ld, r0, r, kNb, &mbar_ld);
-    }
-  }
-  if (!bulk)
-    for (int e = tid; e < kRows * kNb; e += kPT) {
-      const int c = e / kRows, i = e % kRows;
-      A[e] = i < r ? X[(int64_t)c * ld + r0 + i] : 0.f;
-    }
-  __syncthreads();
-  if (bulk) {
-    const bool ok = wait_phase(&mbar_ld, 0u);
-    if (__syncthreads_or(!ok)) {
-      // the copies may still be in flight: one more bounded wait before the CTA exits
-      if (tid == 0) tc_record(status, QRKIT_ETIMEOUT);
-      wait_phase(&mbar_ld, 0u);
-      return;
-    }
-    for (int e = tid; e < (kRows - r) * kNb; e += kPT) {   // rows past the tile's end
-      const int c = e / (kRows - r), i = r + e % (kRows - r);
-      A[c * kRows + i] = 0.f;
-    }
-    __syncthreads();
-  }
-  // the warp's two columns in registers
-  float a0[kRows / 32], a1[kRows / 32];
+  f2 a0[2 * NU], a1[2 * NU];
 #pragma unroll
-  for (int u = 0; u < kRows / 32; ++u) {
-    a0[u] = A[warp * kRows + lane + 32 * u];
-    a1[u] = A[(warp + 16) * kRows + lane + 32 * u];
+  for (int u = 0; u < NU; ++u) {
+    float4 p = make_float4(0.f, 0.f, 0.f, 0.f), q = p;
+    if (128 * u + 4 * lane < r) {
+      p = *reinterpret_cast<const float4*>(x0 + 128 * u);
+      q = *reinterpret_cast<const float4*>(x1 + 128 * u);
+    }
+    a0[2 * u] = pack2(p.x, p.y);
+    a0[2 * u + 1] = pack2(p.z, p.w);
+    a1[2 * u] = pack2(q.x, q.y);
+    a1[2 * u + 1] = pack2(q.z, q.w);
   }
+  for (int e = tid; e < kNb * kPad; e += kPT) Gs[e] = Tm[e] = 0.f;
+  if (tid < kNb) tau_s[tid] = 0.f;
+
   // the reflector of column k from its register column a (its owner warp): the column below k
   // scaled to v (v_k = 1, stored implicitly), beta on the diagonal, v written to slot `slot`
-  auto form = [&](int k, float (&a)[kRows / 32], int slot) {
-    float sq = 0.f, ak = 0.f;
+  auto form = [&](int k, f2 (&a)[2 * NU], int slot) {
+    float h[4];   // rows 4 lane .. 4 lane + 3: the only ones that can lie on or above row k
+    unpack2(a[0], h[0], h[1]);
+    unpack2(a[1], h[2], h[3]);
+    f2 s2 = 0ull, s3 = 0ull;
 #pragma unroll
-    for (int u = 0; u < kRows / 32; ++u) {
-      const int i = lane + 32 * u;
-      if (i > k) sq += a[u] * a[u];
-      if (u == (k >> 5)) ak = a[u];
+    for (int u = 1; u < NU; ++u) {
+      s2 = fma2(a[2 * u], a[2 * u], s2);
+      s3 = fma2(a[2 * u + 1], a[2 * u + 1], s3);
+    }
+    float sq = sum2(s2) + sum2(s3), ak = 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = 4 * lane + q;
+      if (i > k) sq += h[q] * h[q];
+      if (i == k) ak = h[q];
     }
     sq = warp_sum(sq);
-    const float alpha = __shfl_sync(0xffffffffu, ak, k & 31);
+    const float alpha = __shfl_sync(0xffffffffu, ak, k >> 2);
     const float norm = sqrtf(alpha * alpha + sq);
     float beta = 0.f, t = 0.f, scale = 0.f;
     if (norm != 0.f) {
@@ -190,322 +148,441 @@ tsqr_panel_tile_kernel(float* X, int64_t ld, int64_t M, float* taus, float* Xn, 
       t = (beta - alpha) / beta;
       scale = 1.f / (alpha - beta);
     }
+    float v[4];
 #pragma unroll
-    for (int u = 0; u < kRows / 32; ++u) {
-      const int i = lane + 32 * u;
-      if (i > k) a[u] *= scale;
-      else if (i == k) a[u] = beta;
-      V[slot * kRows + i] = i > k ? a[u] : (i == k ? 1.f : 0.f);
+    for (int q = 0; q < 4; ++q) {
+      const int i = 4 * lane + q;
+      if (i > k) h[q] *= scale;
+      else if (i == k) h[q] = beta;
+      v[q] = i > k ? h[q] : (i == k ? 1.f : 0.f);
+    }
+    a[0] = pack2(h[0], h[1]);
+    a[1] = pack2(h[2], h[3]);
+    float* dst = V[slot] + 4 * lane;
+    *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+    const f2 sc = pack2(scale, scale);
+#pragma unroll
+    for (int u = 1; u < NU; ++u) {
+      a[2 * u] = mul2(a[2 * u], sc);
+      a[2 * u + 1] = mul2(a[2 * u + 1], sc);
+      *reinterpret_cast<ulonglong2*>(dst + 128 * u) = make_ulonglong2(a[2 * u], a[2 * u + 1]);
     }
     if (lane == 0) {
       tslot[slot] = t;
       tau_s[k] = t;
-      taus[(int64_t)blockIdx.x * kNb + k] = t;
     }
   };
-  for (int e = tid; e < kNb * kPad; e += kPT) Gs[e] = 0.f;
-  if (warp == 0 && kmax > 0) form(0, a0, 0);
-  const int c0 = warp, c1 = warp + 16;   // the warp's columns (a0, a1)
+  // column k of T by one warp (lane l holds row l).  The sum runs over all 32 m: T[l][m] is still
+  // zero for m >= k and below the diagonal, and G[m][k] for m >= k.
+  auto t_column = [&](int k) {
+    const float tk = tau_s[k];
+    float q[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int m = 0; m < kNb; ++m) q[m & 3] += Tm[lane * kPad + m] * Gs[m * kPad + k];
+    const float v = -((q[0] + q[1]) + (q[2] + q[3])) * tk;
+    __syncwarp();
+    if (lane < k) Tm[lane * kPad + k] = v;
+    if (lane == k) Tm[k * kPad + k] = tk;
+  };
+
+  __syncthreads();
+  if (warp == 0) form(0, a0, 0);
   for (int k = 0; k < kmax; ++k) {
-    __syncthreads();   // reflector k in slot k & 1; column k + 1 not yet updated
+    __syncthreads();   // reflector k is in slot k & 1, G[:k - 1][k - 1] and T[:, :k - 1] are complete
     const int slot = k & 1;
     const float t = tslot[slot];
-    // v_k against each own column: the column itself if it is after k (to update it: a -= t
-    // (v^T a) v), its reflector y_c (1 at row c, v_c below, 0 above) if it is before k (G[c][k])
-    float v[kRows / 32], p0 = 0.f, p1 = 0.f;
+    f2 v[2 * NU];
 #pragma unroll
-    for (int u = 0; u < kRows / 32; ++u) {
-      const int i = lane + 32 * u;
-      v[u] = V[slot * kRows + i];
-      const float y0 = c0 > k ? a0[u] : (i > c0 ? a0[u] : (i == c0 ? 1.f : 0.f));
-      const float y1 = c1 > k ? a1[u] : (i > c1 ? a1[u] : (i == c1 ? 1.f : 0.f));
-      p0 += v[u] * y0;
-      p1 += v[u] * y1;
+    for (int u = 0; u < NU; ++u) {
+      const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(V[slot] + 128 * u + 4 * lane);
+      v[2 * u] = w.x;
+      v[2 * u + 1] = w.y;
     }
+    f2 d0 = 0ull, e0 = 0ull, d1 = 0ull, e1 = 0ull;
+#pragma unroll
+    for (int u = 0; u < NU; ++u) {
+      d0 = fma2(v[2 * u], a0[2 * u], d0);
+      d1 = fma2(v[2 * u], a1[2 * u], d1);
+      e0 = fma2(v[2 * u + 1], a0[2 * u + 1], e0);
+      e1 = fma2(v[2 * u + 1], a1[2 * u + 1], e1);
+    }
+    float p0 = sum2(d0) + sum2(e0), p1 = sum2(d1) + sum2(e1);
 #pragma unroll
     for (int d = 16; d >= 1; d >>= 1) {
       p0 += __shfl_xor_sync(0xffffffffu, p0, d);
       p1 += __shfl_xor_sync(0xffffffffu, p1, d);
     }
     if (c0 > k) {
-      const float w = p0 * t;
+      const float w = -(p0 * t);
+      const f2 w2 = pack2(w, w);
 #pragma unroll
-      for (int u = 0; u < kRows / 32; ++u) a0[u] -= w * v[u];
+      for (int u = 0; u < 2 * NU; ++u) a0[u] = fma2(w2, v[u], a0[u]);
     } else if (c0 < k && lane == 0) {
       Gs[c0 * kPad + k] = p0;
     }
     if (c1 > k) {
-      const float w = p1 * t;
+      const float w = -(p1 * t);
+      const f2 w2 = pack2(w, w);
 #pragma unroll
-      for (int u = 0; u < kRows / 32; ++u) a1[u] -= w * v[u];
+      for (int u = 0; u < 2 * NU; ++u) a1[u] = fma2(w2, v[u], a1[u]);
     } else if (c1 < k && lane == 0) {
       Gs[c1 * kPad + k] = p1;
     }
     if (k + 1 < kmax && ((k + 1) & 15) == warp) {
       if (k + 1 < 16) form(k + 1, a0, slot ^ 1);
       else form(k + 1, a1, slot ^ 1);
+    } else if (k > 0 && ((k + 9) & 15) == warp) {
+      t_column(k - 1);
     }
   }
+  // V below / R on and above the diagonal in place; the R rows (zeros below) to the next level
 #pragma unroll
-  for (int u = 0; u < kRows / 32; ++u) {
-    A[warp * kRows + lane + 32 * u] = a0[u];
-    A[(warp + 16) * kRows + lane + 32 * u] = a1[u];
-  }
-  for (int e = tid; e < kNb * kPad; e += kPT) Tm[e] = 0.f;
-  __syncthreads();
-  // T, column by column on warp 0 (lane l holds row l).  The sum runs over all 32 m: T[l][m]
-  // is still zero for m >= k and below the diagonal, and G[m][k] for m >= k.
-  if (warp == 0) {
-    for (int k = 0; k < kNb; ++k) {
-      const float tk = k < kmax ? tau_s[k] : 0.f;
-      float q[4] = {0.f, 0.f, 0.f, 0.f};
+  for (int u = 0; u < NU; ++u)
+    if (128 * u + 4 * lane < r) {
+      *reinterpret_cast<ulonglong2*>(x0 + 128 * u) = make_ulonglong2(a0[2 * u], a0[2 * u + 1]);
+      *reinterpret_cast<ulonglong2*>(x1 + 128 * u) = make_ulonglong2(a1[2 * u], a1[2 * u + 1]);
+    }
+  if (4 * lane < kmax) {
+    const int64_t n0 = (int64_t)blockIdx.x * kNb + 4 * lane;
 #pragma unroll
-      for (int m = 0; m < kNb; ++m) q[m & 3] += Tm[lane * kPad + m] * Gs[m * kPad + k];
-      const float v = -((q[0] + q[1]) + (q[2] + q[3])) * tk;
-      __syncwarp();
-      if (lane < k) Tm[lane * kPad + k] = v;
-      if (lane == k) Tm[k * kPad + k] = tk;
-      __syncwarp();
+    for (int cc = 0; cc < 2; ++cc) {
+      const int c = cc ? c1 : c0;
+      float h[4];
+      unpack2(cc ? a1[0] : a0[0], h[0], h[1]);
+      unpack2(cc ? a1[1] : a0[1], h[2], h[3]);
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (4 * lane + q > c) h[q] = 0.f;
+      *reinterpret_cast<float4*>(Xn + (int64_t)c * ldn + n0) = make_float4(h[0], h[1], h[2], h[3]);
     }
   }
   __syncthreads();
-  if (Tout)
-    for (int e = tid; e < kNb * kNb; e += kPT)
-      Tout[(int64_t)blockIdx.x * (kNb * kNb) + e] = Tm[(e / kNb) * kPad + e % kNb];
-  for (int e = tid; e < r * kNb; e += kPT) {
-    const int c = e / r, i = e % r;
-    X[(int64_t)c * ld + r0 + i] = A[c * kRows + i];
-  }
-  if (Xn) {
-    const int64_t n0 = (int64_t)blockIdx.x * kNb;
-    for (int e = tid; e < kmax * kNb; e += kPT) {
-      const int c = e / kmax, i = e % kmax;
-      Xn[(int64_t)c * ldn + n0 + i] = (c >= i) ? A[c * kRows + i] : 0.f;
-    }
+  if (warp == 0) t_column(kmax - 1);
+  __syncthreads();
+  for (int e = tid; e < kNb * kNb; e += kPT) {
+    const int m = e / kNb, k = e % kNb;
+    Tout[(int64_t)blockIdx.x * (kNb * kNb) + e] = Tm[m * kPad + k];
+    Gout[(int64_t)blockIdx.x * (kNb * kNb) + e] = m == k ? tau_s[k] : Gs[m * kPad + k];
   }
 }
 
-// ---- Column-panel TSQR: a factored panel's tile reflectors applied to the columns after it ----
+// ---- a factored panel's tile reflectors applied to the columns after it ----
 //
-// One CTA takes one 256-row tile of a TSQR level and kCw of the trailing columns C (staged by
-// bulk copies).  For each group of 32 reflectors of the tile's panel (Y, with the panel tile's
-// T), Q_group^T C = C - Y (T^T (Y^T C)): W = Y^T C and Z = T^T W on the CUDA cores, C -= Y Z on
-// the tensor cores (kind::tf32, 3xTF32, FP32 accumulation in TMEM).  The
-// transformed tile's top rows (R rows of the panel) go up to the next level, the others down to
-// the next panel.  Y arrives column by column in the space of its low operand half and is kept
-// row-major (rows padded to kYr floats), so that a lane reads four reflectors of its row in one
-// 16-byte load.
-constexpr int kCw = 64;   // trailing columns per CTA
-constexpr int kYr = 36;   // row stride of the row-major Y: 16-byte rows, conflict-free quarter warps
+// One CTA takes a tile and a range of the trailing columns C; its two teams of 8 warps take 16
+// columns at a time in turn, so that one team's loads and barriers overlap the other's arithmetic.
+// A warp holds 128 rows x 16 columns of C in registers, in the fragment layout of
+// mma.m16n8k8 (tf32, the columns of C as its rows), which serves both products:
+//   W^T = C^T Y      C as the A operand (a permutation of the rows within a group of 16, the same
+//                    in both operands, makes a thread's four consecutive rows two k pairs);
+//   C^T -= Z^T Y^T   the same registers as the accumulator layout, Z = T^T W.
+// The warps' partial W are added through shared memory.  Products are 3xTF32 (x = hi + lo, hi hi +
+// hi lo + lo hi) with FP32 accumulation; W is accumulated on the tensor cores over 16 rows at a time
+// and then added in FP32, so a sum over 1024 rows is rounded like one of FP32 multiply-adds (a
+// 256-row sum by chunks of 16: 1.1e-7 against 3.3e-7 for a chain of fmaf), and the correction is
+// subtracted in FP32.  At K = 32 the update does 16 flop per byte of C, so it is bound by memory
+// and by the 286 TFLOP/s that mma.sync reaches here about equally; C crosses the chip once and
+// never goes through shared memory, which tcgen05 operands in hi and lo halves would need twice.
+constexpr int kAT = 512;        // threads: two teams of 8 warps
+constexpr int kGC = 16;         // columns per group
+constexpr int kPW = 40;         // row stride of the partial W and of Z (conflict-free)
 
 size_t panel_apply_smem() {
-  return (size_t)kRows * kCw * 4 + (size_t)kRows * kYr * 4 + 2 * (size_t)kRows * kNb * 4 +
-         2 * (size_t)kCw * kNb * 4 + (size_t)kNb * kNb * 4 + (size_t)kNb * kCw * 4;
+  return (size_t)kNb * kTR * 4 + (size_t)kNb * kNb * 4 + 2 * 8 * (size_t)kGC * kPW * 4 + 2 * 2 * (size_t)kGC * kPW * 4;
 }
 
-__global__ void __launch_bounds__(kThr, 1)
-tsqr_panel_apply_kernel(const float* X, int64_t ld, int64_t M, int pw, const float* Tin, int n, float* up,
-                        int64_t ldu, float* down, int64_t ldd, int64_t down0, int* status) {
-  extern __shared__ __align__(1024) unsigned char smem_raw[];
-  float* Cs = reinterpret_cast<float*>(smem_raw);                          // 256 x kCw, column-major
-  float* Yr = Cs + kRows * kCw;                                            // 256 x 32, row-major (kYr)
-  unsigned char* Yhi = reinterpret_cast<unsigned char*>(Yr + kRows * kYr);  // 256 x 32 operand
-  unsigned char* Ylo = Yhi + kRows * kNb * 4;
-  float* Yf = reinterpret_cast<float*>(Ylo);   // Y as copied (256 x 32, column-major), until Yr is formed
-  unsigned char* Zhi = Ylo + kRows * kNb * 4;                              // kCw x 32 operand
-  unsigned char* Zlo = Zhi + kCw * kNb * 4;
-  float* Tm = reinterpret_cast<float*>(Zlo + kCw * kNb * 4);               // 32 x 32 (row l, col k)
-  float* W = Tm + kNb * kNb;                                               // 32 x kCw, row-major
-  __shared__ uint32_t tmem_slot;
-  __shared__ __align__(8) uint64_t mbar_ld, mbar_mma;
+// Shared-memory position of row i of reflector l: bits 3 and 4 of the row flipped by l, which keeps
+// both products' reads (16-byte over rows, 8-byte over reflectors) free of bank conflicts.
+__device__ __forceinline__ int ypos(int l, int i) { return l * kTR + (i ^ (((l & 1) << 4) | ((l & 2) << 2))); }
 
+struct Split {
+  uint32_t h, l;
+};
+__device__ __forceinline__ Split split_tf32(float x) {
+  Split s;
+  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(s.h) : "f"(x));
+  const float d = x - __uint_as_float(s.h);
+  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(s.l) : "f"(d));
+  return s;
+}
+__device__ __forceinline__ void mma_tf32(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                         uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void team_sync(int team) {
+  asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "r"(kAT / 2) : "memory");
+}
+
+__global__ void __launch_bounds__(kAT, 1)
+tsqr_panel_apply_kernel(const float* X, int64_t ld, int64_t M, const float* Tin, int n, int chunk, float* up,
+                        int64_t ldu, float* down, int64_t ldd, int64_t down0) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float* Y = reinterpret_cast<float*>(smem_raw);   // 32 reflectors x 1024 rows, ypos()
+  float* Tm = Y + kNb * kTR;                       // 32 x 32: T[l][i] at l * 32 + i
+  float* Pt = Tm + kNb * kNb;                      // partial W per team and warp: [col][reflector]
+  float* Zs = Pt + 2 * 8 * kGC * kPW;              // W and Z per team: [col][reflector]
+
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int team = tid >> 8, tt = tid & 255, warp = tt >> 5;
+  const int kq = lane & 3, nq = lane >> 2;
+  const int64_t tile = blockIdx.x;
+  const int64_t r0 = tile * kTR;
+  const int r = (int)(M - r0 < (int64_t)kTR ? M - r0 : (int64_t)kTR);   // a multiple of 4
+  const int kmax = r < kNb ? r : kNb;
+  const int j0 = (int)blockIdx.y * chunk;
+  const int nc = n - j0 < chunk ? n - j0 : chunk;   // a multiple of 32
+
+  // Y: the stored reflectors, zero past the tile's end
+  for (int e = tid; e < kNb * (kTR / 4); e += kAT) {
+    const int l = e / (kTR / 4), i = 4 * (e % (kTR / 4));
+    float* dst = Y + ypos(l, i);
+    if (i < r) dev::cp_async16(dst, X + (int64_t)l * ld + r0 + i);
+    else *reinterpret_cast<float4*>(dst) = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  dev::cp_async_commit();
+  for (int e = tid; e < kNb * kNb; e += kAT) Tm[e] = Tin[tile * (kNb * kNb) + e];
+  dev::cp_async_wait_all();
+  __syncthreads();
+  // 1 on the diagonal, 0 above it (where R is stored) and for reflectors a short tile lacks
+  for (int e = tid; e < kNb * kNb; e += kAT) {
+    const int l = e / kNb, i = e % kNb;
+    if (i <= l || l >= kmax) Y[ypos(l, i)] = (i == l && l < kmax) ? 1.f : 0.f;
+  }
+  __syncthreads();
+
+  float* part = Pt + (team * 8 + warp) * (kGC * kPW);
+  float* Ws = Zs + team * 2 * (kGC * kPW);
+  float* Zt = Ws + kGC * kPW;
+  const int wr = 128 * warp;                       // the warp's first row
+  for (int g = team; g < nc / kGC; g += 2) {
+    const int jc = j0 + g * kGC;
+    const float* Cg = X + (int64_t)(kNb + jc + nq) * ld + r0;
+    float4 ca[8], cb[8];                           // columns nq and nq + 8, rows wr + 16 G + 4 kq ..
+#pragma unroll
+    for (int G = 0; G < 8; ++G) {
+      const int i = wr + 16 * G + 4 * kq;
+      ca[G] = cb[G] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (i < r) {
+        ca[G] = *reinterpret_cast<const float4*>(Cg + i);
+        cb[G] = *reinterpret_cast<const float4*>(Cg + 8 * ld + i);
+      }
+    }
+    // W^T = C^T Y over the warp's rows
+    float w[4][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) w[j][q] = 0.f;
+    if (wr < r) {
+#pragma unroll
+      for (int G = 0; G < 8; ++G) {
+        const Split ax = split_tf32(ca[G].x), ay = split_tf32(ca[G].y), az = split_tf32(ca[G].z),
+                    aw = split_tf32(ca[G].w);
+        const Split bx = split_tf32(cb[G].x), by = split_tf32(cb[G].y), bz = split_tf32(cb[G].z),
+                    bw = split_tf32(cb[G].w);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float4 yv = *reinterpret_cast<const float4*>(Y + ypos(8 * j + nq, wr + 16 * G + 4 * kq));
+          const Split yx = split_tf32(yv.x), yy = split_tf32(yv.y), yz = split_tf32(yv.z), yw = split_tf32(yv.w);
+          float d[4] = {0.f, 0.f, 0.f, 0.f};
+          mma_tf32(d, ax.l, bx.l, az.l, bz.l, yx.h, yz.h);
+          mma_tf32(d, ay.l, by.l, aw.l, bw.l, yy.h, yw.h);
+          mma_tf32(d, ax.h, bx.h, az.h, bz.h, yx.l, yz.l);
+          mma_tf32(d, ay.h, by.h, aw.h, bw.h, yy.l, yw.l);
+          mma_tf32(d, ax.h, bx.h, az.h, bz.h, yx.h, yz.h);
+          mma_tf32(d, ay.h, by.h, aw.h, bw.h, yy.h, yw.h);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) w[j][q] += d[q];
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      *reinterpret_cast<float2*>(part + nq * kPW + 8 * j + 2 * kq) = make_float2(w[j][0], w[j][1]);
+      *reinterpret_cast<float2*>(part + (nq + 8) * kPW + 8 * j + 2 * kq) = make_float2(w[j][2], w[j][3]);
+    }
+    team_sync(team);
+    {
+      // 16 threads per column (half a warp): W, then Z = T^T W (entry i from rows l <= i)
+      const int col = tt >> 4, i2 = 2 * (tt & 15);
+      const float* src = Pt + team * 8 * (kGC * kPW) + col * kPW + i2;
+      float2 s = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const float2 v = *reinterpret_cast<const float2*>(src + q * (kGC * kPW));
+        s.x += v.x;
+        s.y += v.y;
+      }
+      *reinterpret_cast<float2*>(Ws + col * kPW + i2) = s;
+      __syncwarp();
+      float z0 = 0.f, z1 = 0.f;
+#pragma unroll
+      for (int l = 0; l < kNb; l += 4) {
+        const float4 wv = *reinterpret_cast<const float4*>(Ws + col * kPW + l);
+        const float2 t0 = *reinterpret_cast<const float2*>(Tm + l * kNb + i2);
+        const float2 t1 = *reinterpret_cast<const float2*>(Tm + (l + 1) * kNb + i2);
+        const float2 t2 = *reinterpret_cast<const float2*>(Tm + (l + 2) * kNb + i2);
+        const float2 t3 = *reinterpret_cast<const float2*>(Tm + (l + 3) * kNb + i2);
+        z0 += t0.x * wv.x + t1.x * wv.y + t2.x * wv.z + t3.x * wv.w;
+        z1 += t0.y * wv.x + t1.y * wv.y + t2.y * wv.z + t3.y * wv.w;
+      }
+      *reinterpret_cast<float2*>(Zt + col * kPW + i2) = make_float2(-z0, -z1);
+    }
+    team_sync(team);
+    if (wr < r) {
+      Split z[4][4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        z[j][0] = split_tf32(Zt[nq * kPW + 8 * j + kq]);
+        z[j][1] = split_tf32(Zt[(nq + 8) * kPW + 8 * j + kq]);
+        z[j][2] = split_tf32(Zt[nq * kPW + 8 * j + kq + 4]);
+        z[j][3] = split_tf32(Zt[(nq + 8) * kPW + 8 * j + kq + 4]);
+      }
+#pragma unroll
+      for (int G = 0; G < 8; ++G) {
+        const int i = wr + 16 * G;
+        float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float2 u = *reinterpret_cast<const float2*>(Y + ypos(8 * j + kq, i + 2 * nq));
+          const float2 v = *reinterpret_cast<const float2*>(Y + ypos(8 * j + kq + 4, i + 2 * nq));
+          const Split ux = split_tf32(u.x), uy = split_tf32(u.y), vx = split_tf32(v.x), vy = split_tf32(v.y);
+          mma_tf32(d0, z[j][0].l, z[j][1].l, z[j][2].l, z[j][3].l, ux.h, vx.h);
+          mma_tf32(d1, z[j][0].l, z[j][1].l, z[j][2].l, z[j][3].l, uy.h, vy.h);
+          mma_tf32(d0, z[j][0].h, z[j][1].h, z[j][2].h, z[j][3].h, ux.l, vx.l);
+          mma_tf32(d1, z[j][0].h, z[j][1].h, z[j][2].h, z[j][3].h, uy.l, vy.l);
+          mma_tf32(d0, z[j][0].h, z[j][1].h, z[j][2].h, z[j][3].h, ux.h, vx.h);
+          mma_tf32(d1, z[j][0].h, z[j][1].h, z[j][2].h, z[j][3].h, uy.h, vy.h);
+        }
+        // rows i + 4 kq, + 1, + 2, + 3 of column nq, then of column nq + 8
+        ca[G].x += d0[0]; ca[G].z += d0[1]; cb[G].x += d0[2]; cb[G].z += d0[3];
+        ca[G].y += d1[0]; ca[G].w += d1[1]; cb[G].y += d1[2]; cb[G].w += d1[3];
+        // the tile's top kmax rows up (the next level, or R_S), the others down (the next panel)
+        const int row = i + 4 * kq;
+        if (row < r) {
+          float* dst;
+          int64_t ldd_;
+          if (row < kNb) {
+            dst = up + (int64_t)(jc + nq) * ldu + tile * kNb + row;
+            ldd_ = ldu;
+          } else {
+            dst = down + (int64_t)(jc + nq) * ldd + down0 + tile * (kTR - kNb) + (row - kNb);
+            ldd_ = ldd;
+          }
+          *reinterpret_cast<float4*>(dst) = ca[G];
+          *reinterpret_cast<float4*>(dst + 8 * ldd_) = cb[G];
+        }
+      }
+    }
+  }
+}
+
+// ---- the tiles' Q^T applied to a right-hand side: y -= Y z, z = T^T (Y^T y) ----
+//
+// One CTA per tile, thread t owns rows 4 t .. 4 t + 3 and keeps its 32 x 4 reflector entries in
+// registers between the two products, so the reflectors are read once, all loads in flight.  z comes
+// from G and tau, z_k = tau_k (w_k - sum_{j<k} G[j][k] z_j) with the sum in the order in which row k
+// then subtracts Y[k][j] z_j: a column that is zero but for its damping row has a reflector that
+// swaps the pivot row out (tau = 1, G[j][k] = Y[k][j]), and row k of the result is then exactly 0,
+// as when the reflectors are applied one by one.
+constexpr int kQT = kTR / 4;
+
+__global__ void __launch_bounds__(kQT, 1)
+tsqr_panel_qt_kernel(const float* X, int64_t ld, int64_t M, const float* Gin, const float* rhs, float* rhs_next,
+                     float* rhs_down, int64_t down0) {
+  __shared__ float ws[kQT / 32][kNb];
+  __shared__ float zs[kNb];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t tile = blockIdx.x;
-  const int64_t r0 = tile * kRows;
-  const int r = (int)(M - r0 < (int64_t)kRows ? M - r0 : (int64_t)kRows);
-  const int kmax = r < pw ? r : pw;
-  const int j0 = blockIdx.y * kCw;
-  const int nc = n - j0 < kCw ? n - j0 : kCw;   // a multiple of 32
-  const float* Cg = X + (int64_t)(pw + j0) * ld;
-
+  const int64_t r0 = tile * kTR;
+  const int r = (int)(M - r0 < (int64_t)kTR ? M - r0 : (int64_t)kTR);   // a multiple of 4
+  const int kmax = r < kNb ? r : kNb;
+  const int i = 4 * tid;
+  const bool have = i < r;
+  float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 v[kNb];
+#pragma unroll
+  for (int c = 0; c < kNb; ++c) {
+    v[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (have && c < kmax) v[c] = *reinterpret_cast<const float4*>(X + (int64_t)c * ld + r0 + i);
+  }
+  if (have) y = *reinterpret_cast<const float4*>(rhs + r0 + i);
+  if (i < kNb) {
+#pragma unroll
+    for (int c = 0; c < kNb; ++c) {
+      const float one = c < kmax ? 1.f : 0.f;
+      v[c].x = i > c ? v[c].x : (i == c ? one : 0.f);
+      v[c].y = i + 1 > c ? v[c].y : (i + 1 == c ? one : 0.f);
+      v[c].z = i + 2 > c ? v[c].z : (i + 2 == c ? one : 0.f);
+      v[c].w = i + 3 > c ? v[c].w : (i + 3 == c ? one : 0.f);
+    }
+  }
+  float p[kNb];
+#pragma unroll
+  for (int c = 0; c < kNb; ++c) p[c] = v[c].x * y.x + v[c].y * y.y + v[c].z * y.z + v[c].w * y.w;
+  ws[warp][lane] = transpose_reduce(p, lane);
+  __syncthreads();
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tmem_slot)),
-                 "r"(2 * kCw));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    float w = 0.f;
+#pragma unroll
+    for (int q = 0; q < kQT / 32; ++q) w += ws[q][lane];
+    const float* G = Gin + tile * (kNb * kNb);
+    float gc[kNb];   // column `lane` of G above the diagonal
+#pragma unroll
+    for (int j = 0; j < kNb; ++j) gc[j] = j < lane ? G[j * kNb + lane] : 0.f;
+    const float tau = G[lane * kNb + lane];
+    float z = 0.f;
+#pragma unroll
+    for (int j = 0; j < kNb; ++j) {
+      if (lane == j) z = tau * w;
+      const float zj = __shfl_sync(0xffffffffu, z, j);
+      if (j < lane) w = __fmaf_rn(-gc[j], zj, w);
+    }
+    zs[lane] = z;
   }
-  if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&mbar_ld)), "r"(1));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&mbar_mma)), "r"(1));
-    asm volatile("fence.mbarrier_init.release.cluster;");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;");
-  const uint32_t tmem = tmem_slot;
-  uint32_t ph_ld = 0, ph_mma = 0;
-  int pending = 0;   // 1: a bulk load, 2: the MMAs still outstanding after a timeout
-
-  for (int p0 = 0; p0 < kmax; p0 += kNb) {
-    const int nk = kmax - p0 < kNb ? kmax - p0 : kNb;
-    // (a) Y of this group of reflectors (and, the first time, the tile's trailing columns)
-    dev::fence_proxy_async();
-    __syncthreads();   // every earlier read of Yf and Cs is done
-    if (tid == 0) {
-      dev::mbar_expect_tx(&mbar_ld, column_bytes(r) * (uint32_t)(nk + (p0 == 0 ? nc : 0)));
-      stage_columns(Yf, X + (int64_t)p0 * ld, ld, r0, r, nk, &mbar_ld);
-      if (p0 == 0) stage_columns(Cs, Cg, ld, r0, r, nc, &mbar_ld);
-    }
-    for (int e = tid; e < kNb * kNb; e += kThr) Tm[e] = Tin[(tile * (pw / kNb) + p0 / kNb) * (kNb * kNb) + e];
-    const bool ok = wait_phase(&mbar_ld, ph_ld);
-    ph_ld ^= 1u;
-    if (__syncthreads_or(!ok)) {
-      pending = 1;
-      break;
-    }
-    // Y[i][l]: 1 at i = p0 + l, the stored v below, 0 above, past the tile and for l >= nk
-    for (int e = tid; e < kRows * kNb; e += kThr) {
-      const int l = e / kRows, i = e % kRows, d = p0 + l;
-      Yr[i * kYr + l] = (l >= nk || i < d || i >= r) ? 0.f : (i == d ? 1.f : Yf[e]);
-    }
-    if (p0 == 0)
-      for (int e = tid; e < (kRows - r) * nc; e += kThr) {
-        const int c = e / (kRows - r), i = r + e % (kRows - r);
-        Cs[c * kRows + i] = 0.f;
-      }
-    __syncthreads();
-    // (b) W = Y^T C (32 x nc): a warp per pair of columns, lanes over rows p0.., each row's 32
-    // reflector values in eight 16-byte loads; the 32 sums of a column reduced together
-    for (int j = 2 * warp; j < nc; j += 2 * (kThr / 32)) {
-      float acc0[32], acc1[32];
+  if (!have) return;
 #pragma unroll
-      for (int l = 0; l < 32; ++l) acc0[l] = acc1[l] = 0.f;
-      const float* x0 = Cs + j * kRows;
-      const float* x1 = x0 + kRows;
-      for (int i = p0 + lane; i < kRows; i += 32) {
-        const float c0 = x0[i], c1 = x1[i];
-        const float4* yrow = reinterpret_cast<const float4*>(Yr + i * kYr);
-#pragma unroll
-        for (int q = 0; q < kNb / 4; ++q) {
-          const float4 y = yrow[q];
-          acc0[4 * q] += y.x * c0;
-          acc0[4 * q + 1] += y.y * c0;
-          acc0[4 * q + 2] += y.z * c0;
-          acc0[4 * q + 3] += y.w * c0;
-          acc1[4 * q] += y.x * c1;
-          acc1[4 * q + 1] += y.y * c1;
-          acc1[4 * q + 2] += y.z * c1;
-          acc1[4 * q + 3] += y.w * c1;
-        }
-      }
-      W[lane * kCw + j] = transpose_reduce(acc0, lane);
-      W[lane * kCw + j + 1] = transpose_reduce(acc1, lane);
-    }
-    __syncthreads();
-    // (c) Z = T^T W in place (row i of Z from rows l <= i of W)
-    for (int j = tid; j < nc; j += kThr)
-      for (int i = kNb - 1; i >= 0; --i) {
-        float z = 0.f;
-        for (int l = 0; l <= i; ++l) z += Tm[l * kNb + i] * W[l * kCw + j];
-        W[i * kCw + j] = z;
-      }
-    __syncthreads();
-    // (d) operands: Z (nc x 32, K-major) and Y (256 x 32), each split into TF32 hi + lo
-    for (int e = tid; e < kNb * nc; e += kThr) {
-      const int i = e / nc, j = e % nc;
-      const float v = W[i * kCw + j], h = to_tf32(v);
-      *reinterpret_cast<float*>(Zhi + koff(j, i)) = h;
-      *reinterpret_cast<float*>(Zlo + koff(j, i)) = to_tf32(v - h);
-    }
-    for (int e = tid; e < kRows * kNb; e += kThr) {
-      const int l = e / kRows, i = e % kRows;
-      const float v = Yr[i * kYr + l], h = to_tf32(v);
-      const uint32_t o = (uint32_t)(i >> 7) * (128 * kNb * 4) + koff(i & 127, l);
-      *reinterpret_cast<float*>(Yhi + o) = h;
-      *reinterpret_cast<float*>(Ylo + o) = to_tf32(v - h);
-    }
-    asm volatile("fence.proxy.async.shared::cta;");
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    // (e) D_h = Y_h Z for the two 128-row halves (3 products each: hi hi, hi lo, lo hi)
-    if (tid == 0) {
-      const uint32_t id = idesc_tf32(128, nc);
-      for (int h = 0; h < 2; ++h) {
-        const uint32_t yo = (uint32_t)h * (128 * kNb * 4);
-        int first = 1;
-        for (int ks = 0; ks < kNb / 8; ++ks) {
-          const uint32_t ko = (uint32_t)ks * 256;
-          for (int sp = 0; sp < 3; ++sp) {
-            const unsigned char* ya = sp == 2 ? Ylo : Yhi;
-            const unsigned char* zb = sp == 1 ? Zlo : Zhi;
-            const uint64_t ad = smem_desc(su32(ya) + yo + ko), bd = smem_desc(su32(zb) + ko);
-            const uint32_t acc = first ? 0u : 1u;
-            asm volatile(
-                "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}" ::"r"(tmem + (uint32_t)(h * kCw)),
-                "l"(ad), "l"(bd), "r"(id), "r"(acc));
-            first = 0;
-          }
-        }
-      }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-          su32(&mbar_mma)));
-    }
-    const bool mma_ok = wait_phase(&mbar_mma, ph_mma);
-    ph_mma ^= 1u;
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    if (__syncthreads_or(!mma_ok)) {
-      pending = 2;
-      break;
-    }
-    // (f) C -= D: warp w reads TMEM lanes 32 (w % 4) .. of half (w / 4) % 2, 8-column groups
-    // (w / 8), (w / 8) + 2, ...
-    {
-      const int qd = warp & 3, h = (warp >> 2) & 1, part = warp >> 3;
-      const int row = h * 128 + qd * 32 + lane;
-      for (int c0 = part * 8; c0 < nc; c0 += 8 * (kThr / 256)) {
-        uint32_t v[8];
-        const uint32_t ta = tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)(h * kCw + c0);
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-                       "=r"(v[7])
-                     : "r"(ta));
-        asm volatile("tcgen05.wait::ld.sync.aligned;");
-#pragma unroll
-        for (int j = 0; j < 8; ++j) Cs[(c0 + j) * kRows + row] -= __uint_as_float(v[j]);
-      }
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
+  for (int c = 0; c < kNb; ++c) {
+    const float z = -zs[c];
+    y.x = __fmaf_rn(v[c].x, z, y.x);
+    y.y = __fmaf_rn(v[c].y, z, y.y);
+    y.z = __fmaf_rn(v[c].z, z, y.z);
+    y.w = __fmaf_rn(v[c].w, z, y.w);
   }
-  if (pending) {
-    if (tid == 0) tc_record(status, QRKIT_ETIMEOUT);
-    // what timed out may still be running: wait once more (bounded) before TMEM and shared
-    // memory are given up
-    if (pending == 1) wait_phase(&mbar_ld, ph_ld ^ 1u);
-    else wait_phase(&mbar_mma, ph_mma ^ 1u);
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;");
-  __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * kCw));
-  if (pending) return;
-  // the tile's top kmax rows up (the next level, or R_S), the others down (the next panel)
-  for (int e = tid; e < r * nc; e += kThr) {
-    const int c = e / r, i = e % r;
-    const float v = Cs[c * kRows + i];
-    if (i < kmax) up[(int64_t)(j0 + c) * ldu + tile * pw + i] = v;
-    else down[(int64_t)(j0 + c) * ldd + down0 + tile * (kRows - pw) + (i - kmax)] = v;
-  }
+  if (i < kNb) *reinterpret_cast<float4*>(rhs_next + tile * kNb + i) = y;
+  else if (rhs_down) *reinterpret_cast<float4*>(rhs_down + down0 + tile * (kTR - kNb) + (i - kNb)) = y;
 }
 
 }  // namespace
 
-qrkit_status tsqr_panel_apply(qrkit_ctx* ctx, const float* X, int64_t ld, int64_t M, int pw, const float* T,
-                              int n, float* up, int64_t ldu, float* down, int64_t ldd, int64_t down0,
-                              int64_t tiles) {
+// Alignment that every level matrix of a panel has by construction (composed_layout).
+static bool panel_aligned(const void* p, int64_t ld, int64_t M) {
+  return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && (ld & 3) == 0 && (M & 3) == 0;
+}
+
+qrkit_status tsqr_panel_tile(qrkit_ctx* ctx, float* X, int64_t ld, int64_t M, float* Xn, int64_t ldn, int64_t tiles,
+                             float* Tout, float* Gout) {
+  if (!panel_aligned(X, ld, M) || !panel_aligned(Xn, ldn, 0))
+    return fail(ctx, QRKIT_EINVAL, "column-panel TSQR: unaligned level matrix");
+  const unsigned g = (unsigned)tiles;
+  if (M <= 256)
+    tsqr_panel_tile_kernel<2><<<g, kPT, 0, ctx->stream>>>(X, ld, M, Xn, ldn, Tout, Gout);
+  else if (M <= 512)
+    tsqr_panel_tile_kernel<4><<<g, kPT, 0, ctx->stream>>>(X, ld, M, Xn, ldn, Tout, Gout);
+  else
+    tsqr_panel_tile_kernel<8><<<g, kPT, 0, ctx->stream>>>(X, ld, M, Xn, ldn, Tout, Gout);
+  ctx->launches += 1;
+  QRKIT_CUDA_TRY(ctx, cudaGetLastError());
+  return QRKIT_OK;
+}
+
+qrkit_status tsqr_panel_apply(qrkit_ctx* ctx, const float* X, int64_t ld, int64_t M, const float* T, int n, float* up,
+                              int64_t ldu, float* down, int64_t ldd, int64_t down0, int64_t tiles) {
   if (n <= 0 || tiles <= 0) return QRKIT_OK;
-  if ((ld & 3) != 0 || (reinterpret_cast<uintptr_t>(X) & 15) != 0 || pw % kNb != 0 || n % kNb != 0 ||
-      pw > kRows / 2)
+  if (!panel_aligned(X, ld, M) || !panel_aligned(up, ldu, 0) || !panel_aligned(down, ldd, down0) || n % kNb != 0)
     return fail(ctx, QRKIT_EINVAL, "column-panel TSQR: unaligned level matrix or panel shape");
   const size_t smem = panel_apply_smem();
   if (smem > ctx->max_smem_optin)
@@ -515,25 +592,23 @@ qrkit_status tsqr_panel_apply(qrkit_ctx* ctx, const float* X, int64_t ld, int64_
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     ctx->smem_attr[15] = smem;
   }
-  const dim3 grid((unsigned)tiles, (unsigned)((n + kCw - 1) / kCw));
-  tsqr_panel_apply_kernel<<<grid, kThr, smem, ctx->stream>>>(X, ld, M, pw, T, n, up, ldu, down, ldd, down0,
-                                                             ctx->d_status);
+  // column ranges: as few as give every SM about four CTAs (a CTA stages the tile's reflectors once)
+  const int64_t want = std::max<int64_t>(1, (4 * (int64_t)ctx->num_sms + tiles - 1) / tiles);
+  const int parts = (int)std::min<int64_t>(want, n / kNb);
+  const int chunk = (n / kNb + parts - 1) / parts * kNb;
+  const dim3 grid((unsigned)tiles, (unsigned)((n + chunk - 1) / chunk));
+  tsqr_panel_apply_kernel<<<grid, kAT, smem, ctx->stream>>>(X, ld, M, T, n, chunk, up, ldu, down, ldd, down0);
   ctx->launches += 1;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());
   return QRKIT_OK;
 }
 
-qrkit_status tsqr_panel_tile(qrkit_ctx* ctx, float* X, int64_t ld, int64_t M, float* taus, float* Xn, int64_t ldn,
-                             int64_t tiles, float* Tout) {
-  const size_t smem = panel_tile_smem();
-  if (smem > ctx->max_smem_optin)
-    return fail(ctx, QRKIT_EUNSUPPORTED, "not enough shared memory for the panel tile kernel");
-  if (ctx->smem_attr[13] < smem) {
-    QRKIT_CUDA_TRY(ctx, cudaFuncSetAttribute(tsqr_panel_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem));
-    ctx->smem_attr[13] = smem;
-  }
-  tsqr_panel_tile_kernel<<<(unsigned)tiles, kPT, smem, ctx->stream>>>(X, ld, M, taus, Xn, ldn, Tout, ctx->d_status);
+qrkit_status tsqr_panel_qt(qrkit_ctx* ctx, const float* X, int64_t ld, int64_t M, const float* G, const float* rhs,
+                           float* rhs_next, float* rhs_down, int64_t down0, int64_t tiles) {
+  if (!panel_aligned(X, ld, M) || !panel_aligned(rhs, 0, 0) || !panel_aligned(rhs_next, 0, 0) ||
+      !panel_aligned(rhs_down, 0, down0))
+    return fail(ctx, QRKIT_EINVAL, "column-panel TSQR: unaligned right-hand side");
+  tsqr_panel_qt_kernel<<<(unsigned)tiles, kQT, 0, ctx->stream>>>(X, ld, M, G, rhs, rhs_next, rhs_down, down0);
   ctx->launches += 1;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());
   return QRKIT_OK;
