@@ -294,19 +294,22 @@ size_t panel_apply_smem() {
 // both products' reads (16-byte over rows, 8-byte over reflectors) free of bank conflicts.
 __device__ __forceinline__ int ypos(int l, int i) { return l * kTR + (i ^ (((l & 1) << 4) | ((l & 2) << 2))); }
 
+// x = h + l for 3xTF32: h rounded to TF32, l = x - h exactly.  l has at most 12 bits, of which the tensor
+// core reads the top 11: an error of at most one unit of x's last place, the same as rounding l.
+// The rounding is an add and a mask, which issue at twice the rate of cvt.rna.tf32 here; a NaN whose
+// mantissa the add overflows still arrives through l.
 struct Split {
   uint32_t h, l;
 };
 __device__ __forceinline__ Split split_tf32(float x) {
   Split s;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(s.h) : "f"(x));
-  const float d = x - __uint_as_float(s.h);
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(s.l) : "f"(d));
+  s.h = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
+  s.l = __float_as_uint(x - __uint_as_float(s.h));
   return s;
 }
 __device__ __forceinline__ void mma_tf32(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
                                          uint32_t b1) {
-  asm volatile(
+  asm(
       "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
@@ -359,6 +362,13 @@ tsqr_panel_apply_kernel(const float* X, int64_t ld, int64_t M, const float* Tin,
   for (int g = team; g < nc / kGC; g += 2) {
     const int jc = j0 + g * kGC;
     const float* Cg = X + (int64_t)(kNb + jc + nq) * ld + r0;
+    if (g + 2 < nc / kGC)   // the team's next columns on their way into L2
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int i = 32 * (tt & 31);
+        if (i < r)
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(X + (int64_t)(kNb + jc + 2 * kGC + 2 * warp + q) * ld + r0 + i));
+      }
     float4 ca[8], cb[8];                           // columns nq and nq + 8, rows wr + 16 G + 4 kq ..
 #pragma unroll
     for (int G = 0; G < 8; ++G) {
@@ -592,10 +602,19 @@ qrkit_status tsqr_panel_apply(qrkit_ctx* ctx, const float* X, int64_t ld, int64_
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     ctx->smem_attr[15] = smem;
   }
-  // column ranges: as few as give every SM about four CTAs (a CTA stages the tile's reflectors once)
-  const int64_t want = std::max<int64_t>(1, (4 * (int64_t)ctx->num_sms + tiles - 1) / tiles);
-  const int parts = (int)std::min<int64_t>(want, n / kNb);
-  const int chunk = (n / kNb + parts - 1) / parts * kNb;
+  // Column ranges: one CTA per SM at a time, so the split that takes the least by waves x (columns of a
+  // range + 16, the cost of staging a tile's reflectors in columns).
+  int chunk = n;
+  int64_t best = INT64_MAX;
+  for (int parts = 1; parts <= n / kNb; ++parts) {
+    const int ch = (n / kNb + parts - 1) / parts * kNb;
+    const int64_t ctas = tiles * ((n + ch - 1) / ch);
+    const int64_t cost = (ctas + ctx->num_sms - 1) / ctx->num_sms * (ch + 16);
+    if (cost < best) {
+      best = cost;
+      chunk = ch;
+    }
+  }
   const dim3 grid((unsigned)tiles, (unsigned)((n + chunk - 1) / chunk));
   tsqr_panel_apply_kernel<<<grid, kAT, smem, ctx->stream>>>(X, ld, M, T, n, chunk, up, ldu, down, ldd, down0);
   ctx->launches += 1;
