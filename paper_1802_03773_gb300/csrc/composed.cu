@@ -28,7 +28,20 @@ __device__ __forceinline__ void record(int* status, int code) {
   if (status) atomicCAS(status, 0, code);
 }
 
-// ---- column norms D = diag(J^T J)^(1/2) (Sec. 5.2), accumulated in double ----
+// Compensated float accumulation (Dot2, Ogita-Rump-Oishi): (sh + sl) += a x with the product's
+// rounding error from an FMA and the sum's from TwoSum (Knuth).
+__device__ __forceinline__ void dot2_acc(float& sh, float& sl, float a, float x) {
+  const float p = __fmul_rn(a, x);
+  const float pe = __fmaf_rn(a, x, -p);
+  float t, e;
+  dev::two_sum(sh, p, t, e);
+  sh = t;
+  sl = __fadd_rn(sl, __fadd_rn(e, pe));
+}
+
+// ---- column norms D = diag(J^T J)^(1/2) (Sec. 5.2): sums in double, those of a float dense S as
+// float pairs per thread first (FP64 runs at 1/73 of the FP32 rate: 811 us in FP64 for an S of
+// 819 MB) ----
 template <typename T>
 __global__ void colnorm_blocks_kernel(ComposedView<T> V, double* sq) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -61,9 +74,17 @@ __global__ void __launch_bounds__(kNormThreads) colnorm_dense_part_kernel(Compos
   for (int64_t col = blockIdx.y; col < V.s; col += gridDim.y) {
     const T* c = V.S + col * V.rows;
     double s = 0;
-    for (int64_t r = r0 + threadIdx.x; r < r1; r += kNormThreads) {
-      const double x = (double)c[r];
-      s += x * x;
+    if constexpr (sizeof(T) == sizeof(float)) {
+      // at most 32 squares per thread as a float pair (Dot2)
+      float sh = 0.f, sl = 0.f;
+#pragma unroll 8
+      for (int64_t r = r0 + threadIdx.x; r < r1; r += kNormThreads) dot2_acc(sh, sl, c[r], c[r]);
+      s = (double)sh + (double)sl;
+    } else {
+      for (int64_t r = r0 + threadIdx.x; r < r1; r += kNormThreads) {
+        const double x = (double)c[r];
+        s += x * x;
+      }
     }
     for (int d = 16; d >= 1; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
     if (lane == 0) ws[wid] = s;
@@ -109,7 +130,7 @@ __global__ void finalize_norms_kernel(const double* sq, double* D, int64_t N) {
   D[j] = d == 0.0 ? 1.0 : d;   // zero column norm -> 1 (MINPACK convention)
 }
 
-// ---- per-block factor (Sec. 4.1) with Q_i^T applied to the coupled columns (Sec. 4.2) ----
+// ---- per-block factor (Sec. 4.1) with Q_i^T applied to the coupled columns of windows (Sec. 4.2) ----
 // One thread per block; the augmented block B_i = [J_i; lambda^(1/2) D_i] (na x m) is held
 // column-major in local arrays.  Outputs: factor Fa (na x m, V below / R on and above the
 // diagonal), tau, R12 rows (m x w) and the reduced rows (na - m rows).
@@ -185,7 +206,7 @@ __device__ __forceinline__ void block_factor_small(const ComposedView<T>& V, con
 #pragma unroll
   for (int k = 0; k < MM; ++k)
     if (k < m) O.tau[V.col_off[i] + k] = tau[k];
-  if (V.coupled == QRKIT_COUPLED_NONE) return;
+  if (V.coupled != QRKIT_COUPLED_WINDOW) return;   // a dense S: dense_block.cu
   const int64_t red0 = O.red_off[i];
   if constexpr (sizeof(T) == 4 && NA == 3 && MM == 1) {
     // the 2 x 1 point blocks of curve fits with windows of 8 (damped): the window, R12 and
@@ -234,10 +255,7 @@ __device__ __forceinline__ void block_factor_small(const ComposedView<T>& V, con
 #pragma unroll
       for (int r = 0; r < NA; ++r) {
         T v = T(0);
-        if (c < cw && r < n) {
-          if (V.coupled == QRKIT_COUPLED_DENSE) v = V.S[(int64_t)(c0 + c) * V.rows + V.row_off[i] + r];
-          else v = V.S[V.row_off[i] * V.w + (int64_t)(c0 + c) * n + r];
-        }
+        if (c < cw && r < n) v = V.S[V.row_off[i] * V.w + (int64_t)(c0 + c) * n + r];
         C[c][r] = v;
       }
 #pragma unroll
@@ -266,12 +284,8 @@ __device__ __forceinline__ void block_factor_small(const ComposedView<T>& V, con
             O.R12[(V.col_off[i] + r) * (int64_t)V.w + c0 + c] = C[c][r];
           } else if (r < na) {
             const int64_t row = red0 + (r - m);
-            if (V.coupled == QRKIT_COUPLED_DENSE) {
-              O.X0[(int64_t)(c0 + c) * O.ld0 + row] = C[c][r];
-            } else {
-              O.Xw[row * V.w + c0 + c] = C[c][r];
-              if (c0 + c == 0) O.Xstart[row] = V.start[i];
-            }
+            O.Xw[row * V.w + c0 + c] = C[c][r];
+            if (c0 + c == 0) O.Xstart[row] = V.start[i];
           }
         }
       }
@@ -335,18 +349,13 @@ __global__ void block_factor_kernel(ComposedView<T> V, FactorOut<T> O) {
   for (int e = 0; e < na * m; ++e) F[e] = B[e];
   for (int k = 0; k < m; ++k) O.tau[V.col_off[i] + k] = tau[k];
   // coupled columns, kChunk at a time
-  if (V.coupled == QRKIT_COUPLED_NONE) return;
+  if (V.coupled != QRKIT_COUPLED_WINDOW) return;   // a dense S: dense_block.cu
   const int64_t red0 = O.red_off[i];
   for (int c0 = 0; c0 < V.w; c0 += kChunk) {
     const int cw = min(kChunk, V.w - c0);
     T C[kMaxRows * kChunk];
     for (int c = 0; c < cw; ++c) {
-      for (int r = 0; r < n; ++r) {
-        T v;
-        if (V.coupled == QRKIT_COUPLED_DENSE) v = V.S[(int64_t)(c0 + c) * V.rows + V.row_off[i] + r];
-        else v = V.S[V.row_off[i] * V.w + (int64_t)(c0 + c) * n + r];
-        C[c * na + r] = v;
-      }
+      for (int r = 0; r < n; ++r) C[c * na + r] = V.S[V.row_off[i] * V.w + (int64_t)(c0 + c) * n + r];
       for (int r = n; r < na; ++r) C[c * na + r] = 0;
     }
     for (int k = 0; k < m; ++k) {
@@ -364,12 +373,8 @@ __global__ void block_factor_kernel(ComposedView<T> V, FactorOut<T> O) {
       for (int r = 0; r < m; ++r) O.R12[(V.col_off[i] + r) * (int64_t)V.w + c0 + c] = C[c * na + r];
       for (int r = m; r < na; ++r) {
         const int64_t row = red0 + (r - m);
-        if (V.coupled == QRKIT_COUPLED_DENSE) {
-          O.X0[(int64_t)(c0 + c) * O.ld0 + row] = C[c * na + r];
-        } else {
-          O.Xw[row * V.w + c0 + c] = C[c * na + r];
-          if (c0 + c == 0) O.Xstart[row] = V.start[i];
-        }
+        O.Xw[row * V.w + c0 + c] = C[c * na + r];
+        if (c0 + c == 0) O.Xstart[row] = V.start[i];
       }
     }
   }
@@ -658,17 +663,6 @@ __device__ __forceinline__ void resid_g_block(ComposedView<T> V, const T* b, con
       if (acc != 0.0 && st + t < V.s) atomicAdd(&gS[st + t - goff], acc);
     }
   }
-}
-
-// Compensated float accumulation (Dot2, Ogita-Rump-Oishi): (sh + sl) += a x with the product's
-// rounding error from an FMA and the sum's from TwoSum (Knuth).
-__device__ __forceinline__ void dot2_acc(float& sh, float& sl, float a, float x) {
-  const float p = __fmul_rn(a, x);
-  const float pe = __fmaf_rn(a, x, -p);
-  float t, e;
-  dev::two_sum(sh, p, t, e);
-  sh = t;
-  sl = __fadd_rn(sl, __fadd_rn(e, pe));
 }
 
 // resid_g_small for float data: the residual b - J p - S p_S and the sums J^T r, S^T r in
@@ -1241,6 +1235,7 @@ static qrkit_status factor_typed(qrkit_ctx* ctx, const void* J, const void* S, c
     LAUNCH(ctx, (block_factor_small_kernel<T, 6, 2><<<blocks_for(P.K, 128), 128, 0, st>>>(V, O)));
   else
     LAUNCH(ctx, block_factor_kernel<T><<<blocks_for(P.K, 64), 64, 0, st>>>(V, O));
+  if (V.coupled == QRKIT_COUPLED_DENSE && (rc = dense_apply_blocks<T>(ctx, V, O)) != QRKIT_OK) return rc;
   if (V.coupled == QRKIT_COUPLED_WINDOW) {
     // P_r of the reduced block: its rows sorted by leading column per segment (Sec. 4.3)
     rc = reduced_row_sort(ctx, C.sort, (int64_t)P.seg_cols.size(), C.sort_hist_entries,

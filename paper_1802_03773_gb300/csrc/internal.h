@@ -332,6 +332,10 @@ qrkit_status tsqr_panel_apply(qrkit_ctx* ctx, const float* X, int64_t ld, int64_
                               int64_t ldu, float* down, int64_t ldd, int64_t down0, int64_t tiles);
 qrkit_status tsqr_panel_qt(qrkit_ctx* ctx, const float* X, int64_t ld, int64_t M, const float* G, const float* rhs,
                            float* rhs_next, float* rhs_down, int64_t down0, int64_t tiles);
+// Q_i^T of the factored blocks applied to a dense S (dense_block.cu): top rows to R12, the others to
+// the reduced block's first level.
+template <typename T>
+qrkit_status dense_apply_blocks(qrkit_ctx* ctx, const ComposedView<T>& V, const FactorOut<T>& O);
 // Solves with a dense S (dense_solve.cu): x = R_S^{-1} c; dp = R_S^{-1} R_S^{-T} g, also added to x;
 // R_i x_i = rhs_i - R12_i x_S by a warp per block; and, for float plans, a refinement step's
 // h_B = R_i^{-T} g_B and g_S - R12^T h_B with g = J^T (b - J p) - lambda D^2 p (ws: dense_refine_bytes).
