@@ -355,155 +355,228 @@ __global__ void band_colnorm_kernel(const float* Jf, const double* Jd, const int
   D[gj] = d == 0.0 ? 1.0 : d;
 }
 
-// Column norms for float J, in two phases per CTA of kColNormCols consecutive global columns.
-// Rows come in groups of rows_per_col per column (group g = rows rpc g .. rpc g + rpc - 1,
-// all starting at column g), so column j's entries are entry t of groups j - t, t < w.
-// Phase 1: one thread per group sums the squares of its rpc rows per entry t (contiguous
-// rpc x w floats, vector loads) into shared memory; phase 2: one thread per column adds its w
-// diagonal partial sums (in double) from groups of its own instance.
-constexpr int kColNormCols = 256;
-__global__ void __launch_bounds__(kColNormCols) band_colnorm_f32_kernel(const float* J, int64_t total_cols,
-                                                                        const int64_t* inst_col0, int64_t num_inst,
-                                                                        int rpc, int w, int vec, double* D) {
-  __shared__ float S[(kColNormCols + kBW - 1) * (kBW + 1)];
-  const int stride = w + 1;   // odd row stride: consecutive columns hit different banks
-  const int64_t j0 = (int64_t)blockIdx.x * kColNormCols;
-  for (int gg = threadIdx.x; gg < kColNormCols + w - 1; gg += kColNormCols) {
-    const int64_t g = j0 - (w - 1) + gg;
-    float acc[kBW];
-#pragma unroll
-    for (int t = 0; t < kBW; ++t) acc[t] = 0.f;
-    if (g >= 0 && g < total_cols) {
-      const float* rows = J + g * rpc * w;
-      if (vec) {   // rpc w a multiple of 4 and J 16-byte aligned
-        const float4* r4 = reinterpret_cast<const float4*>(rows);
-        for (int e = 0; e < rpc * w / 4; ++e) {
-          const float4 v = r4[e];
-          const int t0 = (4 * e) % w;   // w is a multiple of 4 or divides 4 here
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const float x = u == 0 ? v.x : (u == 1 ? v.y : (u == 2 ? v.z : v.w));
-            const int t = (t0 + u) % w;
-#pragma unroll
-            for (int tt = 0; tt < kBW; ++tt)
-              if (tt == t) acc[tt] += x * x;
-          }
-        }
-      } else {
-        for (int q = 0; q < rpc; ++q)
-#pragma unroll
-          for (int t = 0; t < kBW; ++t)
-            if (t < w) acc[t] += rows[q * w + t] * rows[q * w + t];
-      }
+// Float J with implicit row starts: the column norms and the refinement gradient, by row groups.
+// Group c (column c of the concatenated instances) holds the rpc rows that start at column c, so column j's
+// entries are entry t of groups j - t, t < w.  A CTA of NT threads takes NT consecutive groups, of which the last
+// NT - (w - 1) are its columns: their rows arrive in shared memory by coalesced 16-byte cp.async copies (a
+// thread reading its own group from global memory touches a cache line of its own at every load), thread t
+// computes the sums of group t per diagonal, and then the column of group t from the w sums on its anti-diagonal.
+// The rows' residuals are formed on the way, so a refinement step reads J once.
+// 256 instances, 13 million columns, 4 rows of 8 values per column (1.87 GB): %NORM% us for the norms
+// (2 phases reading global memory 1,000), %REF% us per gradient (residual 636 and gradient 1,738).
+template <bool kStaged>
+__device__ __forceinline__ const float* group_rows_f32(const float* J, int64_t grp0, int64_t total, int rw, int gs,
+                                                       float* buf) {
+  const int nt = blockDim.x;
+  if constexpr (kStaged) {
+    const bool wide = (rw & 3) == 0 && (reinterpret_cast<uintptr_t>(J) & 15) == 0;   // then gs % 4 == 0 too
+    const int unit = wide ? 4 : 1, per = rw / unit;
+    for (int e = threadIdx.x; e < nt * per; e += nt) {
+      const int gg = e / per, o = (e - gg * per) * unit;
+      const int64_t grp = grp0 + gg;
+      if (grp < 0 || grp >= total) continue;
+      const float* src = J + grp * rw + o;
+      float* dst = buf + gg * gs + o;
+      if (wide) dev::cp_async16(dst, src);
+      else asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dev::smem_u32(dst)), "l"(src) : "memory");
     }
-#pragma unroll
-    for (int t = 0; t < kBW; ++t)
-      if (t < w) S[gg * stride + t] = acc[t];
+    dev::cp_async_commit();
+    dev::cp_async_wait_all();
+    return buf + threadIdx.x * gs;
+  } else {
+    return J + (grp0 + threadIdx.x) * (int64_t)rw;
+  }
+}
+
+// Instance of group grp: from the CTA's first instance onwards.
+__device__ __forceinline__ int64_t instance_of_group(const int64_t* inst_col0, const int64_t* inst_cols,
+                                                     int64_t num_inst, int64_t grp0, int64_t grp) {
+  __shared__ int64_t first;
+  if (threadIdx.x == 0) {
+    int64_t lo = 0, hi = num_inst - 1;
+    while (lo < hi) {
+      const int64_t mid = (lo + hi + 1) / 2;
+      if (inst_col0[mid] <= (grp0 > 0 ? grp0 : 0)) lo = mid; else hi = mid - 1;
+    }
+    first = lo;
   }
   __syncthreads();
-  const int64_t gj = j0 + threadIdx.x;
-  if (gj >= total_cols) return;
-  int64_t lo = 0, hi = num_inst - 1;
-  while (lo < hi) {   // instance of column gj
-    const int64_t mid = (lo + hi + 1) / 2;
-    if (inst_col0[mid] <= gj) lo = mid; else hi = mid - 1;
+  int64_t k = first;
+  while (k + 1 < num_inst && inst_col0[k] + inst_cols[k] <= grp) ++k;
+  return k;
+}
+
+// A row's w values (a fixed 8 by two 16-byte loads, or any w <= MW).
+template <bool kW8, int MW>
+__device__ __forceinline__ void row_f32(float (&a)[MW], const float* row, int w) {
+  if constexpr (kW8) {
+    const float4 p = reinterpret_cast<const float4*>(row)[0], q = reinterpret_cast<const float4*>(row)[1];
+    a[0] = p.x; a[1] = p.y; a[2] = p.z; a[3] = p.w;
+    a[4] = q.x; a[5] = q.y; a[6] = q.z; a[7] = q.w;
+  } else {
+#pragma unroll
+    for (int t = 0; t < MW; ++t) a[t] = t < w ? row[t] : 0.f;
   }
-  const int64_t j = gj - inst_col0[lo];
+}
+
+struct BandGroups {   // what both kernels are told
+  const float* J;
+  int64_t total_cols;
+  const int64_t* inst_cols;
+  const int64_t* inst_col0;
+  int64_t num_inst;
+  int rpc, w, gs;   // gs: stride of a staged group
+};
+
+template <bool kW8, bool kStaged, int MW>
+__global__ void __launch_bounds__(256) band_norm_f32_kernel(BandGroups B, double* D) {
+  extern __shared__ __align__(16) float sm_f[];
+  const int nt = blockDim.x, tid = threadIdx.x, w = B.w;
+  const int64_t grp0 = (int64_t)blockIdx.x * (nt - (w - 1)) - (w - 1), grp = grp0 + tid;
+  const float* rows = group_rows_f32<kStaged>(B.J, grp0, B.total_cols, B.rpc * w, B.gs, sm_f);
+  float* S = sm_f + (kStaged ? nt * B.gs : 0);   // per group and diagonal, stride w + 1
+  const int64_t k = instance_of_group(B.inst_col0, B.inst_cols, B.num_inst, grp0, grp);   // and the staged rows
+  const bool have = grp >= 0 && grp < B.total_cols;
+  float acc[MW];
+#pragma unroll
+  for (int t = 0; t < MW; ++t) acc[t] = 0.f;
+  if (have)
+    for (int q = 0; q < B.rpc; ++q) {
+      float a[MW];
+      row_f32<kW8, MW>(a, rows + (int64_t)q * w, w);
+#pragma unroll
+      for (int t = 0; t < MW; ++t) acc[t] += a[t] * a[t];
+    }
+#pragma unroll
+  for (int t = 0; t < MW; ++t)
+    if (t < w) S[tid * (w + 1) + t] = acc[t];
+  __syncthreads();
+  if (tid < w - 1 || !have) return;
+  const int64_t j = grp - B.inst_col0[k];
   double sum = 0.0;
-  for (int t = 0; t < w && t <= j; ++t) sum += (double)S[(threadIdx.x + w - 1 - t) * stride + t];
+  for (int t = 0; t < w && t <= j; ++t) sum += (double)S[(tid - t) * (w + 1) + t];
   const double d = sqrt(sum);
-  D[gj] = d == 0.0 ? 1.0 : d;
+  D[grp] = d == 0.0 ? 1.0 : d;
 }
 
-// Refinement pieces of the parallel path for float J: the residual r = b - J x of each row as
-// an unevaluated float pair (rh + rl, Dot2: error-free products and sums, the accuracy of a
-// double residual without GB300's slow FP64 pipe), stored in place of a double r ...
-__global__ void band_resid_f32_kernel(const float* J, const float* b, const float* x, const int64_t* inst_cols,
-                                      const int64_t* inst_col0, const int64_t* inst_row0, int64_t num_inst,
-                                      int64_t total_rows, int rpc, int w, float2* r) {
-  const int64_t gi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gi >= total_rows) return;
-  int64_t lo = 0, hi = num_inst - 1;
-  while (lo < hi) {
-    const int64_t mid = (lo + hi + 1) / 2;
-    if (inst_row0[mid] <= gi) lo = mid; else hi = mid - 1;
+// g = J^T (b - J x) - lambda D^2 x into the parallel QR's padded layout: the residual of a row as an
+// unevaluated float pair (rh + rl, Dot2: error-free products and sums, the accuracy of a double residual
+// without GB300's slow FP64 pipe), the column sums as pairs too.
+template <bool kW8, bool kStaged, int MW>
+__global__ void __launch_bounds__(256) band_grad_f32_kernel(BandGroups B, const float* b, const float* x,
+                                                            const double* D, double lam, const int64_t* blk0,
+                                                            float* gp) {
+  extern __shared__ __align__(16) float sm_f[];
+  const int nt = blockDim.x, tid = threadIdx.x, w = B.w;
+  const int64_t grp0 = (int64_t)blockIdx.x * (nt - (w - 1)) - (w - 1), grp = grp0 + tid;
+  const float* rows = group_rows_f32<kStaged>(B.J, grp0, B.total_cols, B.rpc * w, B.gs, sm_f);
+  float* xs = sm_f + (kStaged ? nt * B.gs : 0);                    // x of columns grp0 .. grp0 + nt + w - 2
+  float2* S = reinterpret_cast<float2*>(xs + ((nt + w + 2) & ~3));  // per group and diagonal, stride w + 1
+  for (int e = tid; e < nt + w - 1; e += nt) {
+    const int64_t c = grp0 + e;
+    xs[e] = c >= 0 && c < B.total_cols ? x[c] : 0.f;
   }
-  const int64_t i = gi - inst_row0[lo], N = inst_cols[lo], c0 = inst_col0[lo];
-  const int64_t s = i / rpc;
-  const float* row = J + gi * w;
-  float sh = b[gi], sl = 0.f;
-  for (int t = 0; t < w && s + t < N; ++t) {
-    const float a = row[t], xj = -x[c0 + s + t];
-    const float pr = __fmul_rn(a, xj);
-    const float pe = __fmaf_rn(a, xj, -pr);
-    float tt, e;
-    dev::two_sum(sh, pr, tt, e);
-    sh = tt;
-    sl = __fadd_rn(sl, __fadd_rn(e, pe));
-  }
-  r[gi] = make_float2(sh, sl);
-}
-
-// ... and g = J^T r - lambda D^2 x per column, in the two phases of the column norms: per row
-// group the Dot2 sums over its rows for each diagonal t (pairs in shared memory), then per
-// column the compensated sum of its w diagonal pairs; g in double.
-__global__ void __launch_bounds__(kColNormCols) band_g_f32_kernel(const float* J, const float* x, const float2* r,
-                                                                  const double* D, double lam, int64_t total_cols,
-                                                                  const int64_t* inst_col0, int64_t num_inst, int rpc,
-                                                                  int w, double* g) {
-  __shared__ float2 S[(kColNormCols + kBW - 1) * (kBW + 1)];
-  const int stride = w + 1;
-  const int64_t j0 = (int64_t)blockIdx.x * kColNormCols;
-  for (int gg = threadIdx.x; gg < kColNormCols + w - 1; gg += kColNormCols) {
-    const int64_t grp = j0 - (w - 1) + gg;
-    float hs[kBW], hc[kBW];
+  const int64_t k = instance_of_group(B.inst_col0, B.inst_cols, B.num_inst, grp0, grp);   // and the staged data
+  const bool have = grp >= 0 && grp < B.total_cols;
+  float hs[8], hc[8];
 #pragma unroll
-    for (int t = 0; t < kBW; ++t) hs[t] = hc[t] = 0.f;
-    if (grp >= 0 && grp < total_cols) {
-      for (int q = 0; q < rpc; ++q) {
-        const int64_t row = grp * rpc + q;
-        const float2 rr = r[row];
-        const float* jr = J + row * w;
+  for (int t = 0; t < 8; ++t) hs[t] = hc[t] = 0.f;
+  if (have) {
+    const int64_t left = B.inst_col0[k] + B.inst_cols[k] - grp;   // columns from the group's to the instance's end
+    const int nx = left < w ? (int)left : w;
+    float xv[8];
 #pragma unroll
-        for (int t = 0; t < kBW; ++t) {
-          if (t < w) {
-            const float a = jr[t];
-            const float pr = __fmul_rn(a, rr.x);
-            float pe = __fmaf_rn(a, rr.x, -pr);
-            pe = __fmaf_rn(a, rr.y, pe);
-            float tt, e;
-            dev::two_sum(hs[t], pr, tt, e);
-            hs[t] = tt;
-            hc[t] = __fadd_rn(hc[t], __fadd_rn(e, pe));
-          }
+    for (int t = 0; t < 8; ++t) xv[t] = t < nx ? -xs[tid + t] : 0.f;
+    for (int q = 0; q < B.rpc; ++q) {
+      float a[8];
+      row_f32<kW8, 8>(a, rows + (int64_t)q * w, w);
+      float sh = b[grp * B.rpc + q], sl = 0.f;
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        if (t < nx) {
+          const float pr = __fmul_rn(a[t], xv[t]);
+          const float pe = __fmaf_rn(a[t], xv[t], -pr);
+          float tt, e;
+          dev::two_sum(sh, pr, tt, e);
+          sh = tt;
+          sl = __fadd_rn(sl, __fadd_rn(e, pe));
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        if (t < nx) {   // an entry past the instance's last column belongs to no column
+          const float pr = __fmul_rn(a[t], sh);
+          float pe = __fmaf_rn(a[t], sh, -pr);
+          pe = __fmaf_rn(a[t], sl, pe);
+          float tt, e;
+          dev::two_sum(hs[t], pr, tt, e);
+          hs[t] = tt;
+          hc[t] = __fadd_rn(hc[t], __fadd_rn(e, pe));
         }
       }
     }
+  }
 #pragma unroll
-    for (int t = 0; t < kBW; ++t)
-      if (t < w) S[gg * stride + t] = make_float2(hs[t], hc[t]);
-  }
+  for (int t = 0; t < 8; ++t)
+    if (t < w) S[tid * (w + 1) + t] = make_float2(hs[t], hc[t]);
   __syncthreads();
-  const int64_t gj = j0 + threadIdx.x;
-  if (gj >= total_cols) return;
-  int64_t lo = 0, hi = num_inst - 1;
-  while (lo < hi) {
-    const int64_t mid = (lo + hi + 1) / 2;
-    if (inst_col0[mid] <= gj) lo = mid; else hi = mid - 1;
-  }
-  const int64_t j = gj - inst_col0[lo];
+  if (tid < w - 1 || !have) return;
+  const int64_t j = grp - B.inst_col0[k];
   float s = 0.f, c = 0.f;
   for (int t = 0; t < w && t <= j; ++t) {
-    const float2 v = S[(threadIdx.x + w - 1 - t) * stride + t];
+    const float2 v = S[(tid - t) * (w + 1) + t];
     float tt, e;
     dev::two_sum(s, v.x, tt, e);
     s = tt;
     c = __fadd_rn(c, __fadd_rn(e, v.y));
   }
   double acc = (double)s + (double)c;
-  if (lam > 0.0) acc -= lam * D[gj] * D[gj] * (double)x[gj];
-  g[gj] = acc;
+  if (lam > 0.0) acc -= lam * D[grp] * D[grp] * (double)xs[tid];
+  float* out = gp + 8 * blk0[k];
+  out[j] = (float)acc;
+  if (j == B.inst_cols[k] - 1)   // the padding columns of the last block
+    for (int64_t e = j + 1; e < (j + 8) / 8 * 8; ++e) out[e] = 0.f;
 }
+
+// Threads, staging and shared memory for a group of rw floats: as many groups as fit about 100 KB; groups
+// of more than 700 floats are read from global memory by their threads.
+struct BandLaunch {
+  int nt, gs;
+  bool staged, w8;
+  size_t smem;
+  unsigned grid;
+};
+static BandLaunch band_launch(const BandGroups& B, size_t per_thread, size_t fixed) {
+  BandLaunch L;
+  const int rw = B.rpc * B.w;
+  L.staged = rw <= 700;
+  L.gs = (rw & 3) == 0 ? rw + 4 : (rw | 1);   // 16-byte rows, or an odd stride: no bank conflicts
+  L.nt = 256;
+  while (L.staged && L.nt > 32 && (size_t)L.nt * L.gs * 4 > 80 * 1024) L.nt /= 2;
+  // rows by 16-byte loads: staged rows of 8 are aligned, rows in global memory if J is
+  L.w8 = B.w == 8 && (L.staged || (reinterpret_cast<uintptr_t>(B.J) & 15) == 0);
+  L.smem = (L.staged ? (size_t)L.nt * L.gs * 4 : 0) + L.nt * per_thread + fixed;
+  const int64_t cols = L.nt - (B.w - 1);
+  L.grid = (unsigned)((B.total_cols + cols - 1) / cols);
+  return L;
+}
+
+// KERNEL<w = 8 by 16-byte loads, staged, widest window>
+#define BAND_F32_LAUNCH(ctx, L, KERNEL, MW, ...)                                                                   \
+  do {                                                                                                         \
+    auto launch_ = [&](auto k_) -> cudaError_t {                                                               \
+      if ((L).smem > 48 * 1024) {                                                                              \
+        const cudaError_t e_ = cudaFuncSetAttribute(k_, cudaFuncAttributeMaxDynamicSharedMemorySize,           \
+                                                    (int)(L).smem);                                            \
+        if (e_ != cudaSuccess) return e_;                                                                      \
+      }                                                                                                        \
+      k_<<<(L).grid, (L).nt, (L).smem, (ctx)->stream>>>(__VA_ARGS__);                                          \
+      return cudaGetLastError();                                                                               \
+    };                                                                                                         \
+    QRKIT_CUDA_TRY(ctx, (L).w8 ? ((L).staged ? launch_(KERNEL<true, true, 8>) : launch_(KERNEL<true, false, 8>))  \
+                               : ((L).staged ? launch_(KERNEL<false, true, MW>) : launch_(KERNEL<false, false, MW>))); \
+    (ctx)->launches += 1;                                                                                      \
+  } while (0)
 
 // Refinement pieces of the parallel path for double J (float J takes the Dot2 kernels
 // above), one thread per row / per column: r = b - J x in double, then
@@ -727,7 +800,7 @@ qrkit_status banded_plan(qrkit_ctx* ctx, const qrkit_structure* s) {
   if (B.parallel) {
     if ((st = cr_build(ctx, B.cr, cols, c0, r0, nrows)) != QRKIT_OK) return st;
   }
-  if (B.parallel || expl) {
+  if (expl || (B.parallel && ctx->precision == QRKIT_FP64)) {   // the float gradient needs no scratch
     if ((st = ensure(ctx, B.g, (size_t)cc * sizeof(double), "banded g")) != QRKIT_OK) return st;
     if ((st = ensure(ctx, B.h, (size_t)cc * es, "banded h")) != QRKIT_OK) return st;
     if ((st = ensure(ctx, B.r, (size_t)std::max<int64_t>(rr, 1) * sizeof(double), "banded r")) != QRKIT_OK) return st;
@@ -785,17 +858,18 @@ static qrkit_status banded_run(qrkit_ctx* ctx, const void* J, const void* b, con
       QRKIT_CUDA_TRY(ctx, cudaGetLastError());
     } else {
       if (sizeof(T) == sizeof(float)) {
-        const int rw = B.rows_per_col * B.w;
-        const int vec = (rw % 4 == 0) && (B.w % 4 == 0 || 4 % B.w == 0) &&
-                        (reinterpret_cast<uintptr_t>(J) & 15) == 0;
-        band_colnorm_f32_kernel<<<nblk(B.total_cols, kColNormCols), kColNormCols, 0, st>>>(
-            (const float*)J, B.total_cols, dc0, B.num_inst, B.rows_per_col, B.w, vec, D);
+        const BandGroups G{(const float*)J, B.total_cols, dcols, dc0, B.num_inst, B.rows_per_col, B.w, 0};
+        const BandLaunch L = band_launch(G, (size_t)(B.w + 1) * sizeof(float), 0);
+        BandGroups GL = G;
+        GL.gs = L.gs;
+        if (B.w <= 8) BAND_F32_LAUNCH(ctx, L, band_norm_f32_kernel, 8, GL, D);
+        else BAND_F32_LAUNCH(ctx, L, band_norm_f32_kernel, kBW, GL, D);
       } else {
         band_colnorm_kernel<<<nblk(B.total_cols, 256), 256, 0, st>>>(nullptr, (const double*)J, dcols, dc0, dr0,
                                                                     B.num_inst, B.rows_per_col, B.w, D);
+        ctx->launches += 1;
+        QRKIT_CUDA_TRY(ctx, cudaGetLastError());
       }
-      ctx->launches += 1;
-      QRKIT_CUDA_TRY(ctx, cudaGetLastError());
     }
   }
   if (B.explicit_starts) {
@@ -820,7 +894,8 @@ static qrkit_status banded_run(qrkit_ctx* ctx, const void* J, const void* b, con
       ctx->launches += 2;
       QRKIT_CUDA_TRY(ctx, cudaGetLastError());
       if (B.parallel) {
-        if ((rc = cr_normal_solve(ctx, *B.cr, (const double*)B.g.ptr, B.h.ptr)) != QRKIT_OK) return rc;
+        if ((rc = cr_normal_solve(ctx, *B.cr, (const double*)B.g.ptr, nullptr, p)) != QRKIT_OK) return rc;
+        continue;
       } else {
         if ((rc = widen_or_narrow_g(ctx, (const double*)B.g.ptr, B.h.ptr, B.total_cols)) != QRKIT_OK) return rc;
         if ((rc = banded_tri_solve(ctx, B.num_inst, inst, B.Rw.ptr, B.w, B.h.ptr, true)) != QRKIT_OK) return rc;
@@ -837,13 +912,15 @@ static qrkit_status banded_run(qrkit_ctx* ctx, const void* J, const void* b, con
                                (double*)B.res2.ptr);
     if (rc != QRKIT_OK) return rc;
     for (int it = 0; it < refine_steps; ++it) {
-      if (sizeof(T) == sizeof(float)) {
-        band_resid_f32_kernel<<<nblk(B.total_rows, 256), 256, 0, st>>>(
-            (const float*)J, (const float*)b, (const float*)p, dcols, dc0, dr0, B.num_inst, B.total_rows,
-            B.rows_per_col, B.w, (float2*)B.r.ptr);
-        band_g_f32_kernel<<<nblk(B.total_cols, kColNormCols), kColNormCols, 0, st>>>(
-            (const float*)J, (const float*)p, (const float2*)B.r.ptr, D, lambda, B.total_cols, dc0, B.num_inst,
-            B.rows_per_col, B.w, (double*)B.g.ptr);
+      if constexpr (sizeof(T) == sizeof(float)) {
+        const BandGroups G{(const float*)J, B.total_cols, dcols, dc0, B.num_inst, B.rows_per_col, B.w, 0};
+        const BandLaunch L = band_launch(G, (size_t)(B.w + 1) * sizeof(float2) + sizeof(float), (B.w + 3) * sizeof(float));
+        BandGroups GL = G;
+        GL.gs = L.gs;
+        const int64_t* blk0;
+        void* gp;
+        cr_padded(*B.cr, &blk0, &gp);
+        BAND_F32_LAUNCH(ctx, L, band_grad_f32_kernel, 8, GL, (const float*)b, (const float*)p, D, lambda, blk0, (float*)gp);
       } else {
         band_resid_kernel<T><<<nblk(B.total_rows, 256), 256, 0, st>>>(
             (const T*)J, (const T*)b, (const T*)p, dcols, dc0, dr0, B.num_inst, B.total_rows, B.rows_per_col, B.w,
@@ -851,13 +928,12 @@ static qrkit_status banded_run(qrkit_ctx* ctx, const void* J, const void* b, con
         band_g_kernel<T><<<nblk(B.total_cols, 256), 256, 0, st>>>(
             (const T*)J, (const T*)p, (const double*)B.r.ptr, D, lambda, dcols, dc0, dr0, B.num_inst, B.total_cols,
             B.rows_per_col, B.w, (double*)B.g.ptr);
+        ctx->launches += 2;
+        QRKIT_CUDA_TRY(ctx, cudaGetLastError());
       }
-      ctx->launches += 2;
-      QRKIT_CUDA_TRY(ctx, cudaGetLastError());
-      if ((rc = cr_normal_solve(ctx, *B.cr, (const double*)B.g.ptr, B.h.ptr)) != QRKIT_OK) return rc;
-      band_axpy_kernel<T><<<nblk(B.total_cols, 256), 256, 0, st>>>((T*)p, (const T*)B.h.ptr, B.total_cols);
-      ctx->launches += 1;
-      QRKIT_CUDA_TRY(ctx, cudaGetLastError());
+      if ((rc = cr_normal_solve(ctx, *B.cr, sizeof(T) == sizeof(float) ? nullptr : (const double*)B.g.ptr, nullptr, p)) !=
+          QRKIT_OK)
+        return rc;
     }
     return QRKIT_OK;
   }

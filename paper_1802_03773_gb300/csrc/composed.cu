@@ -1385,9 +1385,7 @@ static qrkit_status solve_typed(qrkit_ctx* ctx, const void* J, const void* S, co
     }
     if (V.coupled == QRKIT_COUPLED_WINDOW && C.cr) {
       // dp_S = R_S^{-1} R_S^{-T} (g_S - R12^T h_B) with the parallel banded factor
-      qrkit_status rc = cr_normal_solve(ctx, *C.cr, gS, h + nb);
-      if (rc != QRKIT_OK) return rc;
-      LAUNCH(ctx, axpy_kernel<T><<<blocks_for(s, 128), 128, 0, st>>>(x + nb, h + nb, s));
+      if ((rc = cr_normal_solve(ctx, *C.cr, gS, h + nb, x + nb)) != QRKIT_OK) return rc;
     } else if (V.coupled == QRKIT_COUPLED_WINDOW) {
       // h_S = R_S^{-T} (g_S - R12^T h_B), then dp_S = R_S^{-1} h_S, both banded
       LAUNCH(ctx, gS_to_T_kernel<T><<<blocks_for(s, 128), 128, 0, st>>>(gS, h + nb, s));

@@ -9,8 +9,8 @@
 //   1. compress   per block g, the Householder QR (Sec. 2) of all rows starting in block g
 //                 plus the damping rows lambda^(1/2) D_j of the block's columns (the row
 //                 interleave of Sec. 4.5 / 5.2) reduces them to a 16 x 16 upper-trapezoidal
-//                 block row E_g = [A_g | B_g] on blocks (g, g + 1).  Large groups are split
-//                 over several warps whose partial triangles are merged.
+//                 block row E_g = [A_g | B_g] on blocks (g, g + 1).  Row-heavy groups are split
+//                 over several threads whose partial triangles are merged.
 //   2. reduce     level l works on the block rows F_i of blocks b_i = i 2^l: for every odd
 //                 i, QR of [F_{i-1}; F_i] with block b_i's columns first gives the 8 rows of R
 //                 for b_i (coupled to b_{i-1} and b_{i+1}) and a new 16-row block row on
@@ -21,8 +21,9 @@
 //                 x_{b - 2^l} - R_right x_{b + 2^l} for all blocks of a level in parallel.
 // The product is a QR factorization of the matrix with its columns in nested-dissection
 // order (the blocks of the lowest level first), so R differs from the natural-order banded
-// R; R^T R = A^T A and the solution are the same.  Every Householder vector is as long as a
-// 32-row front.  Refinement solves R^T h = g level by level upwards, then R dx = h.
+// R; R^T R = A^T A and the solution are the same.  Refinement solves R^T h = g level by level
+// upwards, then R dx = h.  An instance's upper levels (at most kTailBlocks blocks left) run in one
+// CTA, levels and back-substitution together: their launches cost more than their work.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -36,22 +37,17 @@
 namespace qrkit {
 namespace {
 
-constexpr int kCB = 8;             // columns per block
-constexpr int kEW = 2 * kCB + 1;   // block row stride: A (8) | B (8) | rhs
-constexpr int kRW = 3 * kCB + 1;   // R block row stride: own (8) | left (8) | right (8) | rhs
+constexpr int kCB = 8;              // columns per block
+constexpr int kE0 = 144;            // compressed block row: 8 rows x 8 | 8 rows x 8 | rhs 16 (below)
+constexpr int kFW = 208;            // block row: A 8 x 8 | B 16 x 8 | rhs 16
+constexpr int kRW = 200;            // R block row: own 8 x 8 | left 8 x 8 | right 8 x 8 | rhs 8
+constexpr int64_t kTailBlocks = 128;
 
 __device__ __forceinline__ void cr_record(int* status, int code) {
   if (status) atomicCAS(status, 0, code);
 }
 
-template <typename T>
-__device__ __forceinline__ T wsum(T v) {
-#pragma unroll
-  for (int d = 16; d >= 1; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-  return v;
-}
-
-// Square root and reciprocal of the front QR: the hardware approximations for float
+// Square root and reciprocal of the reflectors: the hardware approximations for float
 // (sqrt.approx / rcp.approx, about one ulp: far below the rounding the factorization itself
 // accumulates), IEEE for double.
 __device__ __forceinline__ float qr_sqrt(float x) {
@@ -67,77 +63,21 @@ __device__ __forceinline__ float qr_rcp(float x) {
 }
 __device__ __forceinline__ double qr_rcp(double x) { return 1.0 / x; }
 
-__host__ __device__ constexpr int pow2_ceil(int m) { return m <= 1 ? 1 : 2 * pow2_ceil((m + 1) / 2); }
-__host__ __device__ constexpr int log2_exact(int p) { return p <= 1 ? 0 : 1 + log2_exact(p / 2); }
-
-// Sums of M per-lane values over the warp, returned in every lane (v[j] = sum over lanes).
-// Transpose reduction: with the values padded to P = 2^ceil(log2 M), each butterfly stage
-// sends half of the remaining values to the partner lane and keeps the other half, so after
-// log2 P stages each lane holds one partial sum (of value lane >> (5 - log2 P)); plain
-// butterfly stages finish the sums, and one broadcast per value returns them.  About
-// P - 1 + M shuffles instead of 5 M; every lane reads the same lane's sum, so all lanes hold
-// the same bits.
-template <typename T, int M>
-__device__ __forceinline__ void warp_allreduce_many(T (&v)[M], int lane) {
-  constexpr int P = pow2_ceil(M);
-  constexpr int S = 5 - log2_exact(P);
-  static_assert(P <= 32, "at most 32 values");
-  T w[P];
-#pragma unroll
-  for (int i = 0; i < P; ++i) w[i] = i < M ? v[i] : T(0);
-  int d = 16;
-#pragma unroll
-  for (int h = P / 2; h >= 1; h /= 2, d >>= 1) {
-    const bool up = (lane & d) != 0;
-#pragma unroll
-    for (int i = 0; i < h; ++i) {
-      const T send = up ? w[i] : w[h + i];
-      const T keep = up ? w[h + i] : w[i];
-      w[i] = keep + __shfl_xor_sync(0xffffffffu, send, d);
+// The Householder reflector of a column with pivot p and squared norm s2 below it (Sec. 2):
+// v = (1, scale x), H = I - tau v v^T, the pivot becomes beta.
+template <typename T>
+struct Reflector {
+  T beta, tau, scale;
+  __device__ __forceinline__ Reflector(T p, T s2) {
+    const T norm = qr_sqrt(p * p + s2);
+    beta = tau = scale = T(0);
+    if (norm != T(0)) {
+      beta = p >= T(0) ? -norm : norm;
+      tau = (beta - p) * qr_rcp(beta);
+      scale = qr_rcp(p - beta);
     }
   }
-#pragma unroll
-  for (int e = 0; e < S; ++e) {
-    w[0] += __shfl_xor_sync(0xffffffffu, w[0], d);
-    d >>= 1;
-  }
-#pragma unroll
-  for (int jj = 0; jj < M; ++jj) v[jj] = __shfl_sync(0xffffffffu, w[0], jj << S);
-}
-
-// Householder QR of a 32-row front held one row per lane (a[0..NC-1] columns, a[NC] the
-// right-hand side), reducing columns 0..NK-1 in order.  Row k of the result holds R's row k
-// (lane k); rows below NK are zero in the reduced columns.  Column K of the recursion: its
-// reflector, then the update of the NC - K trailing columns (and rhs), whose dot products
-// with v are summed over the warp together.
-template <typename T, int NC, int K, int NK>
-__device__ __forceinline__ void warp_qr_col(T (&a)[NC + 1], int lane) {
-  const T x = a[K];
-  const T sq = wsum(lane > K ? x * x : T(0));
-  const T alpha = __shfl_sync(0xffffffffu, x, K);
-  const T norm = qr_sqrt(alpha * alpha + sq);
-  T beta = T(0), tau = T(0), scale = T(0);
-  if (norm != T(0)) {
-    beta = alpha >= T(0) ? -norm : norm;
-    tau = (beta - alpha) * qr_rcp(beta);
-    scale = qr_rcp(alpha - beta);
-  }
-  const T v = lane > K ? x * scale : (lane == K ? T(1) : T(0));
-  T dv[NC - K];
-#pragma unroll
-  for (int jj = 0; jj < NC - K; ++jj) dv[jj] = v * a[K + 1 + jj];
-  warp_allreduce_many<T, NC - K>(dv, lane);
-#pragma unroll
-  for (int jj = 0; jj < NC - K; ++jj) a[K + 1 + jj] -= (dv[jj] * tau) * v;
-  if (lane == K) a[K] = beta;
-  else if (lane > K) a[K] = T(0);
-  if constexpr (K + 1 < NK) warp_qr_col<T, NC, K + 1, NK>(a, lane);
-}
-
-template <typename T, int NC, int NK>
-__device__ __forceinline__ void warp_qr(T (&a)[NC + 1], int lane) {
-  warp_qr_col<T, NC, 0, NK>(a, lane);
-}
+};
 
 template <typename T>
 struct CRArgs {
@@ -148,6 +88,8 @@ struct CRArgs {
   const int64_t* row0;    // first global row
   const int64_t* rows;    // rows of the instance
   const int64_t* blk0;    // num_inst + 1: first global block of each instance
+  const int64_t* tail0;   // num_inst: first level of the instance's one-CTA tail
+  const int32_t* binst;   // instance of each block
   int64_t total_blocks;
   // rows: explicit starts (global columns, sorted per instance) or implicit floor(i / rpc)
   const int64_t* starts;
@@ -157,34 +99,25 @@ struct CRArgs {
   const T* b;             // rows
   const double* D;        // global columns (damping rows when lam > 0)
   double lam;
-  int splits;             // warps per block in the compression
+  int splits;             // threads per block in the compression
   // work space
   int64_t* grp_lo;        // total_blocks: first row of each block's group (explicit starts)
-  T* P;                   // total_blocks x splits x 16 x kEW partial triangles
-  T* F0;                  // total_blocks x 16 x kEW block rows (two buffers)
+  T* P;                   // total_blocks x splits partial triangles, kE0 each
+  T* F0;                  // total_blocks block rows, kFW each (two buffers); level 0: kE0 of them used
   T* F1;
-  T* Rb;                  // total_blocks x 8 x kRW
+  T* Rb;                  // total_blocks x kRW
   T* xp;                  // total_blocks x 8 padded solution / rhs work
   T* hp;                  // total_blocks x 8
   double* res2;           // per instance
   int* status;
 };
 
-__device__ __forceinline__ int64_t inst_of_block(const int64_t* blk0, int64_t ninst, int64_t gb) {
-  int64_t lo = 0, hi = ninst - 1;
-  while (lo < hi) {
-    const int64_t mid = (lo + hi + 1) / 2;
-    if (blk0[mid] <= gb) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
 // First row of each block's group: lower bound of 8 g among the instance's sorted starts.
 template <typename T>
 __global__ void cr_ranges_kernel(CRArgs<T> A) {
   const int64_t gb = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (gb >= A.total_blocks) return;
-  const int64_t k = inst_of_block(A.blk0, A.num_inst, gb);
+  const int64_t k = A.binst[gb];
   const int64_t g = gb - A.blk0[k];
   const int64_t key = A.col0[k] + (int64_t)kCB * g;
   int64_t lo = A.row0[k], hi = A.row0[k] + A.rows[k];
@@ -211,244 +144,264 @@ __device__ __forceinline__ void group_rows(const CRArgs<T>& A, int64_t k, int64_
   }
 }
 
-// ---- 1. compression of blocks with few rows: one thread per block, rows merged one at a time into an
-// upper-triangular 16 x 16 (+ rhs) block row by 2 x 2 orthogonal rotations (the 2-element
-// Householder reflections of sparse row-merge QR); the triangle lives in shared memory,
-// element-major over the CTA's threads so that a warp's accesses hit distinct banks. ----
-constexpr int kTriElems = 16 * 17 - 120;   // packed upper triangle incl. rhs: rows k = 0..15, cols k..16
-constexpr int kCompThreads = 64;
+// ---- 1. compression: one thread per (block, split) ----
+//
+// Rows come in the order of their first column, so the triangle of the rows seen so far only needs
+// the 8 x 8 window of columns c .. c + 7 while rows starting at c arrive: it lives in registers (36
+// values + 8 of the rhs).  Up to four rows are reflected into it at a time, one Householder vector
+// (pivot + 4) per column; when the rows of column c are through, the window's first row is row c of
+// R and the window moves on by one column.  The damping rows are the window's initial diagonal.
+// Against one row at a time by plane rotations into a 16 x 16 triangle in shared memory this needs a
+// quarter of the arithmetic and no shared memory, and block rows leave as 16-byte stores.
+//
+// A compressed block row E: row c < 8 holds columns c .. c + 7 at 8 c; row 8 + i holds columns 8 .. 15 (zeros
+// below the diagonal) at 64 + 8 i; the rhs of the 16 rows at 128.
+constexpr int kCompThreads = 128;
 
-__host__ __device__ constexpr int tri_off(int k, int j) { return k * 17 - (k * (k - 1)) / 2 + (j - k); }
+__host__ __device__ constexpr int tri(int i, int j) { return i * 8 - (i * (i - 1)) / 2 + (j - i); }
 
 template <typename T>
-__device__ __forceinline__ void rot_coeffs(T alpha, T beta, T& c, T& s, T& r);
-template <>
-__device__ __forceinline__ void rot_coeffs<float>(float alpha, float beta, float& c, float& s, float& r) {
-  const float n2 = alpha * alpha + beta * beta;
-  const float rr = rsqrtf(n2);
-  c = alpha * rr;
-  s = beta * rr;
-  r = n2 * rr;
-}
-template <>
-__device__ __forceinline__ void rot_coeffs<double>(double alpha, double beta, double& c, double& s, double& r) {
-  r = sqrt(alpha * alpha + beta * beta);
-  c = alpha / r;
-  s = beta / r;
-}
-
-// Merge row a (16 columns + rhs at 16, nonzero from column o on) into the triangle Tr
-// (element e of this thread at Tr[e * kCompThreads]); returns the squared leftover rhs.
-template <typename T>
-__device__ __forceinline__ double merge_row(T* Tr, T (&a)[17], int o) {
+struct Window {
+  T t[36], z[8];
+  // four rows (8 columns from the window's first, rhs) reflected into the window; b keeps what is left
+  __device__ __forceinline__ void insert(T (&a)[4][8], T (&b)[4]) {
 #pragma unroll
-  for (int k = 0; k < 16; ++k) {
-    if (k >= o && a[k] != T(0)) {
-      T c, sn, r;
-      rot_coeffs<T>(Tr[tri_off(k, k) * kCompThreads], a[k], c, sn, r);
-      Tr[tri_off(k, k) * kCompThreads] = r;
-      a[k] = T(0);
+    for (int k = 0; k < 8; ++k) {
+      T s2 = T(0);
 #pragma unroll
-      for (int j = k + 1; j < 17; ++j) {
-        const T t = Tr[tri_off(k, j) * kCompThreads];
-        Tr[tri_off(k, j) * kCompThreads] = c * t + sn * a[j];
-        a[j] = c * a[j] - sn * t;
+      for (int q = 0; q < 4; ++q) s2 += a[q][k] * a[q][k];
+      const Reflector<T> h(t[tri(k, k)], s2);
+      T v[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) v[q] = a[q][k] * h.scale;
+      t[tri(k, k)] = h.beta;
+#pragma unroll
+      for (int j = k + 1; j < 8; ++j) {
+        T w = t[tri(k, j)];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) w += v[q] * a[q][j];
+        w *= h.tau;
+        t[tri(k, j)] -= w;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) a[q][j] -= w * v[q];
       }
+      T w = z[k];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) w += v[q] * b[q];
+      w *= h.tau;
+      z[k] -= w;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) b[q] -= w * v[q];
     }
   }
-  return (double)a[16] * (double)a[16];
-}
+  __device__ __forceinline__ void shift() {
+#pragma unroll
+    for (int i = 0; i < 7; ++i) {
+#pragma unroll
+      for (int j = i; j < 7; ++j) t[tri(i, j)] = t[tri(i + 1, j + 1)];
+      t[tri(i, 7)] = T(0);
+      z[i] = z[i + 1];
+    }
+    t[tri(7, 7)] = T(0);
+    z[7] = T(0);
+  }
+};
 
 template <typename T>
-__device__ __forceinline__ void damping_rows(const CRArgs<T>& A, T* Tr, int64_t g, int64_t N, int64_t c0,
-                                             double& res) {
-  const bool damp = A.lam > 0.0;
-  const double lam_half = sqrt(A.lam);
-#pragma unroll 1
-  for (int q = 0; q < kCB; ++q) {
-    const int64_t col = (int64_t)kCB * g + q;
-    T v = T(0);
-    if (col >= N) v = T(1);   // padding column: unit row
-    else if (damp) v = (T)(lam_half * A.D[c0 + col]);
-    T a[17];
+__device__ __forceinline__ void store8(T* dst, const T (&v)[8]) {   // dst 16-byte aligned
+  if constexpr (sizeof(T) == 4) {
+    reinterpret_cast<float4*>(dst)[0] = make_float4(v[0], v[1], v[2], v[3]);
+    reinterpret_cast<float4*>(dst)[1] = make_float4(v[4], v[5], v[6], v[7]);
+  } else {
 #pragma unroll
-    for (int j = 0; j < 17; ++j) a[j] = j == q ? v : T(0);
-    res += merge_row(Tr, a, q);
+    for (int q = 0; q < 4; ++q) reinterpret_cast<double2*>(dst)[q] = make_double2(v[2 * q], v[2 * q + 1]);
+  }
+}
+template <typename T>
+__device__ __forceinline__ void load8(T (&v)[8], const T* src) {   // src 16-byte aligned
+  if constexpr (sizeof(T) == 4) {
+    const float4 a = reinterpret_cast<const float4*>(src)[0], b = reinterpret_cast<const float4*>(src)[1];
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+  } else {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const double2 a = reinterpret_cast<const double2*>(src)[q];
+      v[2 * q] = a.x;
+      v[2 * q + 1] = a.y;
+    }
   }
 }
 
-template <typename T>
-__device__ __forceinline__ void store_block_row(T* dst, const T* Tr) {
-  // 16 rows x (16 + rhs), zeros below the diagonal
+// Sum of a per-thread double into res2 of the thread's instance: one atomic per warp where all its
+// threads work on one instance.
+__device__ __forceinline__ void add_res2(double* res2, int64_t k, double res) {
+  __syncwarp();
+  const unsigned m = __activemask();
+  const int64_t k0 = __shfl_sync(m, k, __ffs(m) - 1);
+  if (m == 0xffffffffu && __all_sync(m, k == k0)) {
 #pragma unroll
-  for (int k = 0; k < 16; ++k)
-#pragma unroll
-    for (int j = 0; j < 17; ++j) dst[k * kEW + j] = j >= k ? Tr[tri_off(k, j) * kCompThreads] : T(0);
+    for (int d = 16; d >= 1; d >>= 1) res += __shfl_xor_sync(m, res, d);
+    if ((threadIdx.x & 31) == 0 && res != 0.0) atomicAdd(res2 + k, res);
+  } else if (res != 0.0) {
+    atomicAdd(res2 + k, res);
+  }
 }
 
 template <typename T>
 __global__ void __launch_bounds__(kCompThreads) cr_compress_kernel(CRArgs<T> A) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* Tr = reinterpret_cast<T*>(smem_raw) + threadIdx.x;
   const int64_t item = (int64_t)blockIdx.x * kCompThreads + threadIdx.x;
   if (item >= A.total_blocks * A.splits) return;
-  const int64_t gb = item / A.splits;
+  const int64_t gb = A.splits == 1 ? item : item / A.splits;
   const int s = (int)(item - gb * A.splits);
-  const int64_t k = inst_of_block(A.blk0, A.num_inst, gb);
+  const int64_t k = A.binst[gb];
   const int64_t g = gb - A.blk0[k];
-  const int64_t N = A.cols[k], c0 = A.col0[k];
+  const int64_t N = A.cols[k], c0 = A.col0[k], row0 = A.row0[k];
   int64_t lo, hi;
   group_rows(A, k, g, gb, lo, hi);
   const int64_t len = hi - lo;
-  const int64_t r_begin = lo + len * s / A.splits, r_end = lo + len * (s + 1) / A.splits;
+  int64_t r = lo + len * s / A.splits;
+  const int64_t r_end = lo + len * (s + 1) / A.splits;
+  Window<T> W;
 #pragma unroll
-  for (int e = 0; e < kTriElems; ++e) Tr[e * kCompThreads] = T(0);
+  for (int e = 0; e < 36; ++e) W.t[e] = T(0);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) W.z[i] = T(0);
+  if (s == 0) {   // damping rows; unit rows for padding columns
+    const double lam_half = sqrt(A.lam);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int64_t col = (int64_t)kCB * g + i;
+      W.t[tri(i, i)] = col >= N ? T(1) : (A.lam > 0.0 ? (T)(lam_half * A.D[c0 + col]) : T(0));
+    }
+  }
+  T* dst = A.splits == 1 ? A.F0 + gb * kFW : A.P + item * kE0;
+  // whole rows by 16-byte loads where they are aligned; else entry by entry
+  const bool wide = A.w == kCB && (reinterpret_cast<uintptr_t>(A.J) & 15) == 0;
   double res = 0.0;
-  bool bad = false;
-#pragma unroll 1
-  for (int64_t r = r_begin; r < r_end; ++r) {
-    const int64_t st = A.starts ? A.starts[r] - c0 : (r - A.row0[k]) / A.rpc;
-    const int64_t o = st - (int64_t)kCB * g;
-    if (o < 0 || o >= kCB) {
-      bad = true;
-      continue;
-    }
-    // the row over the block row's 16 columns: its w values start at column o
-    T a[17];
-    const T* src = A.J + r * A.w;
+  // One step per turn: the next (up to four) rows starting at column c, or, when there are none, the window
+  // one column on.  The threads of a warp may be at different columns.
+  int64_t ahead[4];   // explicit starts of the next four rows, fetched one step early
 #pragma unroll
-    for (int cc = 0; cc < 2 * kCB; ++cc) {
-      const int64_t q = cc - o;
-      a[cc] = (q >= 0 && q < A.w && st + q < N) ? src[q] : T(0);
+  for (int q = 0; q < 4; ++q) ahead[q] = A.starts && r + q < r_end ? A.starts[r + q] - c0 : -1;
+#pragma unroll 1
+  for (int c = 0; c < kCB;) {
+    const int64_t st = (int64_t)kCB * g + c;   // the rows' first column
+    int cnt = 0;
+    if (A.starts) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (cnt == q && ahead[q] == st) cnt = q + 1;
+    } else {
+      cnt = (int)max((int64_t)0, min((int64_t)4, min(r_end, row0 + (st + 1) * A.rpc) - r));
     }
-    a[16] = A.b[r];
-    res += merge_row(Tr, a, (int)o);
+    if (cnt > 0) {
+      T a[4][8], b[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        b[q] = T(0);
+#pragma unroll
+        for (int t = 0; t < 8; ++t) a[q][t] = T(0);
+        if (q < cnt) {
+          const T* src = A.J + (r + q) * A.w;
+          b[q] = A.b[r + q];
+          if (wide && st + kCB <= N) {
+            load8(a[q], src);
+          } else {
+#pragma unroll
+            for (int t = 0; t < 8; ++t)
+              if (t < A.w && st + t < N) a[q][t] = src[t];
+          }
+        }
+      }
+      r += cnt;
+      if (A.starts) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) ahead[q] = r + q < r_end ? A.starts[r + q] - c0 : -1;
+      }
+      W.insert(a, b);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) res += (double)b[q] * (double)b[q];
+    } else {
+      T row[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) row[j] = W.t[tri(0, j)];
+      store8(dst + 8 * c, row);
+      dst[128 + c] = W.z[0];
+      W.shift();
+      ++c;
+    }
   }
-  if (bad) cr_record(A.status, QRKIT_EINVAL);
-  if (A.splits == 1) {
-    // the block's damping rows complete its block row
-    damping_rows(A, Tr, g, N, c0, res);
-    store_block_row(A.F0 + gb * 16 * kEW, Tr);
-  } else {
-    store_block_row(A.P + (gb * A.splits + s) * 16 * kEW, Tr);
+  if (r < r_end) cr_record(A.status, QRKIT_EINVAL);   // rows out of order or past the block
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    T row[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) row[j] = j >= i ? W.t[tri(i, j)] : T(0);
+    store8(dst + 64 + 8 * i, row);
   }
-  if (res != 0.0) atomicAdd(A.res2 + k, res);
+  store8(dst + 136, W.z);
+  add_res2(A.res2, k, res);
 }
 
-// ---- 1'. compression for row-heavy blocks: one warp per (block, split), 16 rows at a time
-// reduced by the warp-level Householder QR (one row per lane); the partial triangles of the
-// splits are merged by one warp per block, with the damping rows. ----
+// 1b. merge of kMergeFan partial triangles of a block into one, by the same window; 16 columns.
+constexpr int kMergeFan = 4;
+
 template <typename T>
-__global__ void __launch_bounds__(128) cr_compress_warp_kernel(CRArgs<T> A) {
-  const int64_t item = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (item >= A.total_blocks * A.splits) return;
-  const int64_t gb = item / A.splits;
-  const int s = (int)(item - gb * A.splits);
-  const int64_t k = inst_of_block(A.blk0, A.num_inst, gb);
-  const int64_t g = gb - A.blk0[k];
-  const int64_t N = A.cols[k], c0 = A.col0[k];
-  int64_t lo, hi;
-  group_rows(A, k, g, gb, lo, hi);
-  const int64_t len = hi - lo;
-  const int64_t r_begin = lo + len * s / A.splits, r_end = lo + len * (s + 1) / A.splits;
-  T a[2 * kCB + 1];
+__global__ void __launch_bounds__(kCompThreads) cr_merge_kernel(CRArgs<T> A, const T* in, int nin, T* out, int nout,
+                                                                int64_t out_stride) {
+  const int64_t item = (int64_t)blockIdx.x * kCompThreads + threadIdx.x;
+  if (item >= A.total_blocks * nout) return;
+  const int64_t gb = item / nout;
+  const int s = (int)(item - gb * nout);
+  const int n = min(kMergeFan, nin - s * kMergeFan);
+  const T* src = in + (gb * nin + s * kMergeFan) * kE0;
+  T* dst = out + item * out_stride;
+  Window<T> W;
 #pragma unroll
-  for (int q = 0; q <= 2 * kCB; ++q) a[q] = T(0);
+  for (int e = 0; e < 36; ++e) W.t[e] = T(0);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) W.z[i] = T(0);
   double res = 0.0;
-  bool bad = false;
-  for (int64_t base = r_begin; base < r_end; base += 16) {
-    if (lane >= 16) {
-      const int64_t r = base + (lane - 16);
-      if (r < r_end) {
-        const int64_t st = A.starts ? A.starts[r] - c0 : (r - A.row0[k]) / A.rpc;
-        const int64_t o = st - (int64_t)kCB * g;
-        if (o < 0 || o >= kCB) {
-          bad = true;
-        } else {
-          const T* src = A.J + r * A.w;
+#pragma unroll 1
+  for (int c = 0; c < 16; ++c) {
+    T a[4][8], b[4];
 #pragma unroll
-          for (int q = 0; q < kCB; ++q)
-            if (q < A.w && st + q < N) {
-              const int c = (int)o + q;
+    for (int q = 0; q < 4; ++q) {
+      b[q] = T(0);
 #pragma unroll
-              for (int cc = 0; cc < 2 * kCB; ++cc)
-                if (cc == c) a[cc] = src[q];
-            }
-          a[2 * kCB] = A.b[r];
+      for (int t = 0; t < 8; ++t) a[q][t] = T(0);
+      if (q < n) {
+        const T* E = src + q * kE0;
+        b[q] = E[128 + c];
+        if (c < 8) {
+          load8(a[q], E + 8 * c);
+        } else {   // row c - 8 of the second triangle: columns c ..
+#pragma unroll
+          for (int t = 0; t < 8; ++t)
+            if (c + t < 16) a[q][t] = E[64 + 8 * (c - 8) + (c - 8) + t];
         }
       }
     }
-    warp_qr<T, 2 * kCB, 2 * kCB>(a, lane);
-    if (lane >= 16) {
-      res += (double)a[2 * kCB] * (double)a[2 * kCB];
+    W.insert(a, b);
 #pragma unroll
-      for (int q = 0; q <= 2 * kCB; ++q) a[q] = T(0);
+    for (int q = 0; q < 4; ++q) res += (double)b[q] * (double)b[q];
+    if (c < 8) {
+      T row[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) row[j] = W.t[tri(0, j)];
+      store8(dst + 8 * c, row);
+    } else {
+      T* d = dst + 64 + 8 * (c - 8);
+      for (int j = 0; j < c - 8; ++j) d[j] = T(0);
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (c + j < 16) d[c - 8 + j] = W.t[tri(0, j)];
     }
+    dst[128 + c] = W.z[0];
+    W.shift();
   }
-  if (bad) cr_record(A.status, QRKIT_EINVAL);
-  if (lane < 16) {
-    T* dst = A.P + ((gb * A.splits + s) * 16 + lane) * kEW;
-#pragma unroll
-    for (int q = 0; q <= 2 * kCB; ++q) dst[q] = a[q];
-  }
-  res = wsum(res);
-  if (lane == 0 && res != 0.0) atomicAdd(A.res2 + k, res);
-  (void)c0;
-}
-
-// 1b. one warp per block: merge the partial triangles and the damping rows into E_g.
-template <typename T>
-__global__ void __launch_bounds__(128) cr_merge_warp_kernel(CRArgs<T> A) {
-  const int64_t gb = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (gb >= A.total_blocks) return;
-  const int64_t k = inst_of_block(A.blk0, A.num_inst, gb);
-  const int64_t g = gb - A.blk0[k];
-  const int64_t N = A.cols[k], c0 = A.col0[k];
-  T a[2 * kCB + 1];
-#pragma unroll
-  for (int q = 0; q <= 2 * kCB; ++q) a[q] = T(0);
-  if (lane < 16) {
-    const T* src = A.P + ((gb * A.splits) * 16 + lane) * kEW;
-#pragma unroll
-    for (int q = 0; q <= 2 * kCB; ++q) a[q] = src[q];
-  }
-  double res = 0.0;
-  const bool damp = A.lam > 0.0;
-  const double lam_half = sqrt(A.lam);
-  for (int s = 1; s <= A.splits; ++s) {
-    if (lane >= 16) {
-      if (s < A.splits) {
-        const T* src = A.P + ((gb * A.splits + s) * 16 + (lane - 16)) * kEW;
-#pragma unroll
-        for (int q = 0; q <= 2 * kCB; ++q) a[q] = src[q];
-      } else if (lane < 16 + kCB) {
-        // damping rows of the block's columns; unit rows for virtual columns
-        const int q0 = lane - 16;
-        const int64_t col = (int64_t)kCB * g + q0;
-        T v = T(0);
-        if (col >= N) v = T(1);
-        else if (damp) v = (T)(lam_half * A.D[c0 + col]);
-#pragma unroll
-        for (int q = 0; q < kCB; ++q)
-          if (q == q0) a[q] = v;
-      }
-    }
-    warp_qr<T, 2 * kCB, 2 * kCB>(a, lane);
-    if (lane >= 16) {
-      res += (double)a[2 * kCB] * (double)a[2 * kCB];
-#pragma unroll
-      for (int q = 0; q <= 2 * kCB; ++q) a[q] = T(0);
-    }
-  }
-  if (lane < 16) {
-    T* dst = A.F0 + (gb * 16 + lane) * kEW;
-#pragma unroll
-    for (int q = 0; q <= 2 * kCB; ++q) dst[q] = a[q];
-  }
-  res = wsum(res);
-  if (lane == 0 && res != 0.0) atomicAdd(A.res2 + k, res);
+  add_res2(A.res2, A.binst[gb], res);
 }
 
 // Work items of a level: inst << 32 | i << 2 | kind (0 eliminate odd i, 1 move up, 2 last).
@@ -458,204 +411,463 @@ __device__ __forceinline__ void decode(int64_t it, int64_t& k, int64_t& i, int& 
   kind = (int)(it & 3);
 }
 
-// 2. one warp per work item of level l.
-template <typename T>
-__global__ void __launch_bounds__(128) cr_level_kernel(CRArgs<T> A, const int64_t* items, int64_t nitems,
-                                                       int level, const T* Fc, T* Fn) {
-  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (w >= nitems) return;
-  int64_t k, i;
-  int kind;
-  decode(items[w], k, i, kind);
-  const int64_t b0 = A.blk0[k];
-  if (kind == 1) {   // unpaired last block row: moves up unchanged
-    if (lane < 16) {
-      const T* src = Fc + ((b0 + i) * 16 + lane) * kEW;
-      T* dst = Fn + ((b0 + i / 2) * 16 + lane) * kEW;
-#pragma unroll
-      for (int q = 0; q < kEW; ++q) dst[q] = src[q];
-    }
-    return;
-  }
-  // front columns: own block (0..7) | left block (8..15) | right block (16..23) | rhs (24)
-  T a[3 * kCB + 1];
-#pragma unroll
-  for (int q = 0; q <= 3 * kCB; ++q) a[q] = T(0);
-  if (lane < 16) {
-    if (kind == 0) {   // F_{i-1} = [A on left | B on own]
-      const T* src = Fc + ((b0 + i - 1) * 16 + lane) * kEW;
-#pragma unroll
-      for (int q = 0; q < kCB; ++q) {
-        a[kCB + q] = src[q];
-        a[q] = src[kCB + q];
-      }
-      a[3 * kCB] = src[2 * kCB];
-    }
-  } else {             // F_i = [A on own | B on right]
-    const T* src = Fc + ((b0 + i) * 16 + (lane - 16)) * kEW;
-#pragma unroll
-    for (int q = 0; q < kCB; ++q) {
-      a[q] = src[q];
-      a[2 * kCB + q] = src[kCB + q];
-    }
-    a[3 * kCB] = src[2 * kCB];
-  }
-  warp_qr<T, 3 * kCB, 3 * kCB>(a, lane);
-  const int64_t blk = b0 + (i << level);
-  if (lane < kCB) {
-    T* dst = A.Rb + (blk * kCB + lane) * kRW;
-#pragma unroll
-    for (int q = 0; q <= 3 * kCB; ++q) dst[q] = a[q];
-  }
-  double res = 0.0;
-  if (kind == 0) {
-    if (lane >= kCB && lane < kCB + 16) {
-      T* dst = Fn + ((b0 + (i - 1) / 2) * 16 + (lane - kCB)) * kEW;
-#pragma unroll
-      for (int q = 0; q < kCB; ++q) {
-        dst[q] = a[kCB + q];
-        dst[kCB + q] = a[2 * kCB + q];
-      }
-      dst[2 * kCB] = a[3 * kCB];
-    } else if (lane >= kCB + 16) {
-      res = (double)a[3 * kCB] * (double)a[3 * kCB];
-    }
-  } else if (lane >= kCB) {
-    res = (double)a[3 * kCB] * (double)a[3 * kCB];
-  }
-  res = wsum(res);
-  if (lane == 0 && res != 0.0) atomicAdd(A.res2 + k, res);
-}
-
-// 3. back-substitution of one level: eight threads per eliminated block, thread q owns row q
-// of the block's R (own | left | right | rhs): the couplings to the neighbours' solutions
-// are row-local, the triangular solve broadcasts each x_t to the block's threads (width-8
-// shuffles).  rhs from the R rows' own column (c) or from hp; writes xp (padded) and, for
-// real columns, x.  Threads past the last item run the shuffles with nothing to do.
+// ---- 2. the elimination of one block: eight lanes ----
+//
+// Lane j holds column j of each 8-column part of the front (and the rhs), so a reflector's column is
+// read by broadcasts from the lane that owns it and every dot product is local: no reductions.  The
+// triangular shapes of the two block rows are used: F_{i-1} = [A' | B'] and F_i = [A | B] with A', A, and
+// rows 8..15 of B' and B upper triangular.
+//   1. rows 8..15 of B' (own columns) into A                    -> rows with entries right only
+//   2. rows 0..7 of B' into A, which makes A the 8 rows of R    -> rows on left and right
+//   3. those rows triangular in the left columns, and the right-only rows of step 1 into rows 8..15 of B:
+//      the new 16-row block row on (left, right).
+// About 650 instructions per front and lane group of four fronts' warp, where a 32-row front on a whole warp with
+// its sums reduced by shuffles took 4,000.
 constexpr int kItemThreads = kCB;
 
+// A block row's columns j of A (rows 0..7) and B (rows 0..7, 8..15) and its rhs.
+template <typename T, bool kCompressed>
+__device__ __forceinline__ void load_block_row(const T* F, int j, T (&a)[8], T (&bl)[8], T (&bh)[8], T (&cl)[8],
+                                               T (&ch)[8]) {
+  if constexpr (kCompressed) {
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const T v = F[8 * r + ((j - r) & 7)];   // column j of A for j >= r, of B for j < r
+      a[r] = j >= r ? v : T(0);
+      bl[r] = j < r ? v : T(0);
+      bh[r] = F[64 + 8 * r + j];
+    }
+    load8(cl, F + 128);
+    load8(ch, F + 136);
+  } else {
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      a[r] = F[8 * r + j];
+      bl[r] = F[64 + 8 * r + j];
+      bh[r] = F[128 + 8 * r + j];
+    }
+    load8(cl, F + 192);
+    load8(ch, F + 200);
+  }
+}
+
 template <typename T>
-__global__ void cr_backsub_kernel(CRArgs<T> A, const int64_t* items, int64_t nitems, int level, int use_hp,
-                                  T* x) {
-  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t w = tid / kItemThreads;
-  const int q = (int)(tid % kItemThreads);
+__device__ __forceinline__ T lane_of(const T (&v)[8], int j) {   // v[j] for a lane index j
+  T x = v[0];
+#pragma unroll
+  for (int q = 1; q < 8; ++q)
+    if (j == q) x = v[q];
+  return x;
+}
+
+template <typename T>
+__device__ __forceinline__ void store_block_row(T* F, int j, const T (&a)[8], const T (&bl)[8], const T (&bh)[8],
+                                                const T (&cl)[8], const T (&ch)[8]) {
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    F[8 * r + j] = a[r];
+    F[64 + 8 * r + j] = bl[r];
+    F[128 + 8 * r + j] = bh[r];
+  }
+  F[192 + j] = lane_of(cl, j);
+  F[200 + j] = lane_of(ch, j);
+}
+
+// w = tau (p + sum_r v_r x_r); p -= w, x_r -= w v_r over M rows.
+template <typename T, int M>
+__device__ __forceinline__ void apply_reflector(T tau, const T (&v)[8], T& p, T (&x)[8], int from = 0) {
+  T w = p;
+#pragma unroll
+  for (int r = 0; r < 8; ++r)
+    if (r >= from && r < M) w += v[r] * x[r];
+  w *= tau;
+  p -= w;
+#pragma unroll
+  for (int r = 0; r < 8; ++r)
+    if (r >= from && r < M) x[r] -= w * v[r];
+}
+
+// One item of level `level`: block i of instance k.  Returns the squared residual it leaves.
+template <typename T, bool kCompressed>
+__device__ __forceinline__ double cr_item(const CRArgs<T>& A, int64_t k, int64_t i, int kind, int level, const T* Fc,
+                                          T* Fn, int j, unsigned gmask) {
+  const int64_t b0 = A.blk0[k];
+  T a[8], bl[8], bh[8], cl[8], ch[8];
+  load_block_row<T, kCompressed>(Fc + (b0 + i) * kFW, j, a, bl, bh, cl, ch);
+  if (kind == 1) {   // unpaired last block row: moves up
+    store_block_row(Fn + (b0 + i / 2) * kFW, j, a, bl, bh, cl, ch);
+    return 0.0;
+  }
+  T* R = A.Rb + (b0 + (i << level)) * kRW;
+  double res = 0.0;
+  T rl[8];   // R's left part
+#pragma unroll
+  for (int r = 0; r < 8; ++r) rl[r] = T(0);
+  if (kind == 0) {
+    T pa[8], pl[8], ph[8], dl[8], dh[8], rr[8], lr[8];
+    load_block_row<T, kCompressed>(Fc + (b0 + i - 1) * kFW, j, pa, pl, ph, dl, dh);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) rr[r] = lr[r] = T(0);   // right parts of the rows of B'
+    T v[8], x[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      T s2 = T(0);
+      const T p = __shfl_sync(gmask, a[q], q, kItemThreads);
+#pragma unroll
+      for (int r = 0; r <= q; ++r) {
+        x[r] = __shfl_sync(gmask, ph[r], q, kItemThreads);
+        s2 += x[r] * x[r];
+      }
+      const Reflector<T> h(p, s2);
+#pragma unroll
+      for (int r = 0; r < 8; ++r) v[r] = r <= q ? x[r] * h.scale : T(0);
+      {
+        T w = a[q], y = bl[q], c = cl[q];
+#pragma unroll
+        for (int r = 0; r <= q; ++r) {
+          w += v[r] * ph[r];
+          y += v[r] * rr[r];
+          c += v[r] * dh[r];
+        }
+        w *= h.tau;
+        y *= h.tau;
+        c *= h.tau;
+        a[q] -= w;
+        bl[q] -= y;
+        cl[q] -= c;
+#pragma unroll
+        for (int r = 0; r <= q; ++r) {
+          ph[r] -= w * v[r];
+          rr[r] -= y * v[r];
+          dh[r] -= c * v[r];
+        }
+      }
+      if (j == q) {
+        a[q] = h.beta;
+#pragma unroll
+        for (int r = 0; r <= q; ++r) ph[r] = T(0);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      T s2 = T(0);
+      const T p = __shfl_sync(gmask, a[q], q, kItemThreads);
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        x[r] = __shfl_sync(gmask, pl[r], q, kItemThreads);
+        s2 += x[r] * x[r];
+      }
+      const Reflector<T> h(p, s2);
+#pragma unroll
+      for (int r = 0; r < 8; ++r) v[r] = x[r] * h.scale;
+      apply_reflector<T, 8>(h.tau, v, a[q], pl);
+      apply_reflector<T, 8>(h.tau, v, rl[q], pa);
+      apply_reflector<T, 8>(h.tau, v, bl[q], lr);
+      apply_reflector<T, 8>(h.tau, v, cl[q], dl);
+      if (j == q) {
+        a[q] = h.beta;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) pl[r] = T(0);
+      }
+    }
+    // the rows of R go out here; what follows needs pa, lr, dl (left and right) and rr, dh, bh, ch
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      R[8 * r + j] = a[r];
+      R[64 + 8 * r + j] = rl[r];
+      R[128 + 8 * r + j] = bl[r];
+    }
+    R[192 + j] = lane_of(cl, j);
+#pragma unroll
+    for (int q = 0; q < 7; ++q) {
+      T s2 = T(0);
+      const T p = __shfl_sync(gmask, pa[q], q, kItemThreads);
+#pragma unroll
+      for (int r = q + 1; r < 8; ++r) {
+        x[r] = __shfl_sync(gmask, pa[r], q, kItemThreads);
+        s2 += x[r] * x[r];
+      }
+      const Reflector<T> h(p, s2);
+      T w = pa[q], y = lr[q], c = dl[q];
+#pragma unroll
+      for (int r = q + 1; r < 8; ++r) {
+        v[r] = x[r] * h.scale;
+        w += v[r] * pa[r];
+        y += v[r] * lr[r];
+        c += v[r] * dl[r];
+      }
+      w *= h.tau;
+      y *= h.tau;
+      c *= h.tau;
+      pa[q] -= w;
+      lr[q] -= y;
+      dl[q] -= c;
+#pragma unroll
+      for (int r = q + 1; r < 8; ++r) {
+        pa[r] -= w * v[r];
+        lr[r] -= y * v[r];
+        dl[r] -= c * v[r];
+      }
+      if (j == q) {
+        pa[q] = h.beta;
+#pragma unroll
+        for (int r = q + 1; r < 8; ++r) pa[r] = T(0);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      T s2 = T(0);
+      const T p = __shfl_sync(gmask, bh[q], q, kItemThreads);
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        x[r] = __shfl_sync(gmask, rr[r], q, kItemThreads);
+        s2 += x[r] * x[r];
+      }
+      const Reflector<T> h(p, s2);
+#pragma unroll
+      for (int r = 0; r < 8; ++r) v[r] = x[r] * h.scale;
+      apply_reflector<T, 8>(h.tau, v, bh[q], rr);
+      apply_reflector<T, 8>(h.tau, v, ch[q], dh);
+      if (j == q) {
+        bh[q] = h.beta;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) rr[r] = T(0);
+      }
+    }
+    store_block_row(Fn + (b0 + (i - 1) / 2) * kFW, j, pa, lr, bh, dl, ch);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) res += (double)dh[r] * (double)dh[r];
+  } else {   // the last block: its A is triangular, nothing is to its right
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      R[8 * r + j] = a[r];
+      R[64 + 8 * r + j] = T(0);
+      R[128 + 8 * r + j] = bl[r];
+      res += (double)ch[r] * (double)ch[r];
+    }
+    R[192 + j] = lane_of(cl, j);
+  }
+  return j == 0 ? res : 0.0;
+}
+
+constexpr int kLevelThreads = 128;
+
+template <typename T, bool kCompressed>
+__global__ void __launch_bounds__(kLevelThreads, sizeof(T) == 4 ? 4 : 2)
+cr_level_kernel(CRArgs<T> A, const int64_t* items, int64_t nitems, int level, const T* Fc, T* Fn) {
+  const int64_t w = ((int64_t)blockIdx.x * kLevelThreads + threadIdx.x) / kItemThreads;
+  const int j = threadIdx.x % kItemThreads;
+  const unsigned gmask = 0xffu << (threadIdx.x & 24);
   int64_t k = 0, i = 0;
   int kind = 1;
-  if (w < nitems) decode(items[w], k, i, kind);
-  const bool act = kind != 1;
-  const int64_t b0 = act ? A.blk0[k] : 0, N = act ? A.cols[k] : 0;
+  double res = 0.0;
+  if (w < nitems) {
+    decode(items[w], k, i, kind);
+    res = cr_item<T, kCompressed>(A, k, i, kind, level, Fc, Fn, j, gmask);
+  } else if (nitems > 0) {
+    decode(items[nitems - 1], k, i, kind);   // adds nothing, to the last item's instance
+  }
+  add_res2(A.res2, k, res);
+}
+
+// ---- 3. back-substitution of one block, eight lanes: lane q owns row q of the block's R (own | left |
+// right | rhs): the couplings to the neighbours' solutions are row-local, the triangular solve
+// broadcasts each x_t.  rhs from the R rows' own column (c) or from hp; writes xp (padded) and, for
+// real columns, x (written) and xadd (added to). ----
+template <typename T>
+__device__ __forceinline__ void cr_backsub_item(const CRArgs<T>& A, int64_t k, int64_t i, int kind, int level,
+                                                bool use_hp, T* x, T* xadd, int q, unsigned gmask) {
+  const int64_t b0 = A.blk0[k], N = A.cols[k];
   const int64_t G = (N + kCB - 1) / kCB;
   const int64_t beta = i << level, step = (int64_t)1 << level;
-  const T* Rq = A.Rb + ((b0 + beta) * kCB + q) * kRW;
-  T y = T(0), diag = T(1);
-  T rq[kCB];
+  const T* R = A.Rb + (b0 + beta) * kRW;
+  T own[8], nbr[8];
+  load8(own, R + 8 * q);
+  T y = use_hp ? A.hp[(b0 + beta) * kCB + q] : R[192 + q];
+  if (kind == 0) {
+    const T* xl = A.xp + (b0 + beta - step) * kCB;
+    load8(nbr, R + 64 + 8 * q);
 #pragma unroll
-  for (int t = 0; t < kCB; ++t) rq[t] = T(0);
-  if (act) {
-    y = use_hp ? A.hp[(b0 + beta) * kCB + q] : Rq[3 * kCB];
-    if (kind == 0) {
-      const T* xl = A.xp + (b0 + beta - step) * kCB;
-#pragma unroll
-      for (int t = 0; t < kCB; ++t) y -= Rq[kCB + t] * xl[t];
-    }
-    if (beta + step < G) {
-      const T* xr = A.xp + (b0 + beta + step) * kCB;
-#pragma unroll
-      for (int t = 0; t < kCB; ++t) y -= Rq[2 * kCB + t] * xr[t];
-    }
-#pragma unroll
-    for (int t = 0; t < kCB; ++t) rq[t] = t > q ? Rq[t] : T(0);
-    diag = Rq[q];
-    if (diag == T(0)) cr_record(A.status, QRKIT_ESINGULAR);
+    for (int t = 0; t < kCB; ++t) y -= nbr[t] * xl[t];
   }
+  if (beta + step < G) {
+    const T* xr = A.xp + (b0 + beta + step) * kCB;
+    load8(nbr, R + 128 + 8 * q);
+#pragma unroll
+    for (int t = 0; t < kCB; ++t) y -= nbr[t] * xr[t];
+  }
+  const T diag = lane_of(own, q);
+  if (diag == T(0)) cr_record(A.status, QRKIT_ESINGULAR);
   T xq = T(0);
 #pragma unroll
   for (int t = kCB - 1; t >= 0; --t) {   // x_t = (y_t - sum_{u > t} R_tu x_u) / R_tt, bottom up
     if (q == t) xq = y / diag;
-    const T xt = __shfl_sync(0xffffffffu, xq, t, kItemThreads);
-    y -= rq[t] * xt;                      // rq[t] = 0 unless t > q
+    const T xt = __shfl_sync(gmask, xq, t, kItemThreads);
+    if (t > q) y -= own[t] * xt;
   }
-  if (act) {
-    A.xp[(b0 + beta) * kCB + q] = xq;
-    if (x && kCB * beta + q < N) x[A.col0[k] + kCB * beta + q] = xq;
+  A.xp[(b0 + beta) * kCB + q] = xq;
+  if (kCB * beta + q < N) {
+    const int64_t col = A.col0[k] + kCB * beta + q;
+    if (x) x[col] = xq;
+    if (xadd) xadd[col] += xq;
   }
 }
 
-// Refinement, R^T h = g upwards: per level, h_b = R_bb^{-T} g_b for the eliminated blocks ...
-// (eight threads per block; thread q solves for h_q after the h_t, t < q, are broadcast)
 template <typename T>
-__global__ void cr_rt_kernel(CRArgs<T> A, const int64_t* items, int64_t nitems, int level) {
-  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t w = tid / kItemThreads;
-  const int q = (int)(tid % kItemThreads);
-  int64_t k = 0, i = 0;
-  int kind = 1;
-  if (w < nitems) decode(items[w], k, i, kind);
-  const bool act = kind != 1;
-  const int64_t blk = act ? A.blk0[k] + (i << level) : 0;
-  const T* R = A.Rb + blk * kCB * kRW;
-  T v = T(0), diag = T(1);
-  T col[kCB];   // column q of R above the diagonal: R_tq, t < q
+__global__ void cr_backsub_kernel(CRArgs<T> A, const int64_t* items, int64_t nitems, int level, int use_hp, T* x,
+                                  T* xadd) {
+  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kItemThreads;
+  if (w >= nitems) return;
+  int64_t k, i;
+  int kind;
+  decode(items[w], k, i, kind);
+  if (kind == 1) return;
+  cr_backsub_item(A, k, i, kind, level, use_hp != 0, x, xadd, (int)(threadIdx.x % kItemThreads),
+                  0xffu << (threadIdx.x & 24));
+}
+
+// Refinement, R^T h = g upwards (xp holds the updated g).  h of one block: lane q solves for h_q after the
+// h_t, t < q, are broadcast; with `part` the lane also gathers sum_t part[t][q] h_t.
+template <typename T>
+__device__ __forceinline__ T cr_rt_item(const CRArgs<T>& A, int64_t blk, const T* part, T& acc, int q, unsigned gmask) {
+  const T* R = A.Rb + blk * kRW;
+  T col[8], pc[8];
 #pragma unroll
-  for (int t = 0; t < kCB; ++t) col[t] = T(0);
-  if (act) {
-    v = A.xp[blk * kCB + q];   // xp holds the updated g during the upward sweep
-#pragma unroll
-    for (int t = 0; t < kCB; ++t) col[t] = t < q ? R[t * kRW + q] : T(0);
-    diag = R[q * kRW + q];
+  for (int t = 0; t < kCB; ++t) {
+    col[t] = t <= q ? R[8 * t + q] : T(0);
+    pc[t] = part ? part[8 * t + q] : T(0);
   }
-  T hq = T(0);
+  T v = A.xp[blk * kCB + q], hq = T(0);
+  const T diag = lane_of(col, q);
 #pragma unroll
   for (int t = 0; t < kCB; ++t) {   // h_t = (g_t - sum_{u < t} R_ut h_u) / R_tt, top down
     if (q == t) hq = v / diag;
-    const T ht = __shfl_sync(0xffffffffu, hq, t, kItemThreads);
-    v -= col[t] * ht;                // col[t] = 0 unless t < q
+    const T ht = __shfl_sync(gmask, hq, t, kItemThreads);
+    if (t < q) v -= col[t] * ht;
+    acc += pc[t] * ht;
   }
-  if (act) A.hp[blk * kCB + q] = hq;
+  return hq;
 }
 
-// ... then the blocks that stay (even j at level l) subtract their neighbours' couplings:
-// g_{b_j} -= R_{b_{j-1}}.right^T h_{b_{j-1}} + R_{b_{j+1}}.left^T h_{b_{j+1}}  (eight threads
-// per block, thread q one entry of g).
+// A block that stays (even j at level l): h of the eliminated neighbours j - 1 and j + 1, then
+// g_j -= R_{j-1}.right^T h_{j-1} + R_{j+1}.left^T h_{j+1}.  The item to the left of an eliminated block
+// stores its h; computing h twice saves a launch per level.
 template <typename T>
-__global__ void cr_rt_update_kernel(CRArgs<T> A, const int64_t* items, int64_t nitems, int level) {
-  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t w = tid / kItemThreads;
-  const int q = (int)(tid % kItemThreads);
-  if (w >= nitems) return;
-  const int64_t k = items[w] >> 32, j = items[w] & 0xffffffff;
-  const int64_t b0 = A.blk0[k], N = A.cols[k];
-  const int64_t G = (N + kCB - 1) / kCB;
+__device__ __forceinline__ void cr_rt_level_item(const CRArgs<T>& A, int64_t k, int64_t j, int level, int q,
+                                                 unsigned gmask) {
+  const int64_t b0 = A.blk0[k], G = A.blk0[k + 1] - b0;
   const int64_t Gl = (G + ((int64_t)1 << level) - 1) >> level;
   T* g = A.xp + (b0 + (j << level)) * kCB;
-  T acc = g[q];
+  T acc = T(0);
   if (j >= 1) {
     const int64_t nb = b0 + ((j - 1) << level);
-    const T* R = A.Rb + nb * kCB * kRW;
-    const T* h = A.hp + nb * kCB;
-#pragma unroll
-    for (int t = 0; t < kCB; ++t) acc -= R[t * kRW + 2 * kCB + q] * h[t];
+    cr_rt_item(A, nb, A.Rb + nb * kRW + 128, acc, q, gmask);
   }
   if (j + 1 < Gl) {
     const int64_t nb = b0 + ((j + 1) << level);
-    const T* R = A.Rb + nb * kCB * kRW;
-    const T* h = A.hp + nb * kCB;
-#pragma unroll
-    for (int t = 0; t < kCB; ++t) acc -= R[t * kRW + kCB + q] * h[t];
+    const T h = cr_rt_item(A, nb, A.Rb + nb * kRW + 64, acc, q, gmask);
+    A.hp[nb * kCB + q] = h;
   }
-  g[q] = acc;
+  g[q] -= acc;
 }
 
 template <typename T>
+__global__ void cr_rt_level_kernel(CRArgs<T> A, const int64_t* items, int64_t nitems, int level) {
+  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kItemThreads;
+  if (w >= nitems) return;
+  cr_rt_level_item(A, items[w] >> 32, items[w] & 0xffffffff, level, (int)(threadIdx.x % kItemThreads),
+                   0xffu << (threadIdx.x & 24));
+}
+
+// ---- an instance's upper levels in one CTA (of as many threads as registers allow for a few
+// instances, 128 for many, so that several share an SM) ----
+template <typename T>
+constexpr int tail_threads() { return sizeof(T) == 4 ? 512 : 256; }
+
+// Blocks left at level l of an instance of G blocks.
+__device__ __forceinline__ int64_t blocks_at(int64_t G, int level) { return (G + ((int64_t)1 << level) - 1) >> level; }
+
+// x of levels top .. lt (down) of instance k.
+template <typename T>
+__device__ __forceinline__ void tail_backsub(const CRArgs<T>& A, int64_t k, int64_t G, int lt, int top, bool use_hp,
+                                             T* x, T* xadd) {
+  const int grp = threadIdx.x / kItemThreads, ng = blockDim.x / kItemThreads, q = threadIdx.x % kItemThreads;
+  const unsigned gmask = 0xffu << (threadIdx.x & 24);
+  for (int l = top; l >= lt; --l) {
+    if (l == top) {
+      if (grp == 0) cr_backsub_item(A, k, 0, 2, l, use_hp, x, xadd, q, gmask);
+    } else {
+      const int64_t Gl = blocks_at(G, l);
+      for (int64_t i = 2 * grp + 1; i < Gl; i += 2 * ng) cr_backsub_item(A, k, i, 0, l, use_hp, x, xadd, q, gmask);
+    }
+    __syncthreads();
+  }
+}
+
+// Factor of the upper levels, then their back-substitution.
+template <typename T>
+__global__ void __launch_bounds__(tail_threads<T>(), 1) cr_tail_kernel(CRArgs<T> A, T* x) {
+  const int64_t k = blockIdx.x;
+  const int grp = threadIdx.x / kItemThreads, ng = blockDim.x / kItemThreads, j = threadIdx.x % kItemThreads;
+  const unsigned gmask = 0xffu << (threadIdx.x & 24);
+  const int64_t G = A.blk0[k + 1] - A.blk0[k];
+  const int lt = (int)A.tail0[k];
+  double res = 0.0;
+  int l = lt;
+  for (;; ++l) {
+    const int64_t Gl = blocks_at(G, l);
+    const T* Fc = (l & 1) ? A.F1 : A.F0;
+    T* Fn = (l & 1) ? A.F0 : A.F1;
+    // item m: odd block 2 m + 1, or the unpaired last block (kind 1), or the only one (kind 2)
+    const int64_t n = Gl == 1 ? 1 : (Gl + 1) / 2;
+    for (int64_t m = grp; m < n; m += ng) {
+      const int kind = Gl == 1 ? 2 : (2 * m + 1 < Gl ? 0 : 1);
+      const int64_t i = kind == 0 ? 2 * m + 1 : Gl - 1;
+      if (l == 0) res += cr_item<T, true>(A, k, i, kind, l, Fc, Fn, j, gmask);
+      else res += cr_item<T, false>(A, k, i, kind, l, Fc, Fn, j, gmask);
+    }
+    __syncthreads();
+    if (Gl == 1) break;
+  }
+  if (res != 0.0) atomicAdd(A.res2 + k, res);
+  tail_backsub(A, k, G, lt, l, false, x, (T*)nullptr);
+}
+
+// R^T h = g through the upper levels, then their back-substitution.
+template <typename T>
+__global__ void __launch_bounds__(tail_threads<T>(), 1) cr_tail_normal_kernel(CRArgs<T> A, T* x, T* xadd) {
+  const int64_t k = blockIdx.x;
+  const int grp = threadIdx.x / kItemThreads, ng = blockDim.x / kItemThreads, q = threadIdx.x % kItemThreads;
+  const unsigned gmask = 0xffu << (threadIdx.x & 24);
+  const int64_t G = A.blk0[k + 1] - A.blk0[k];
+  const int lt = (int)A.tail0[k];
+  int l = lt;
+  for (;; ++l) {
+    const int64_t Gl = blocks_at(G, l);
+    if (Gl == 1) {
+      if (grp == 0) {
+        T none = T(0);
+        const int64_t blk = A.blk0[k];
+        const T h = cr_rt_item(A, blk, (const T*)nullptr, none, q, gmask);
+        A.hp[blk * kCB + q] = h;
+      }
+      __syncthreads();
+      break;
+    }
+    for (int64_t j = 2 * grp; j < Gl; j += 2 * ng) cr_rt_level_item(A, k, j, l, q, gmask);
+    __syncthreads();
+  }
+  tail_backsub(A, k, G, lt, l, true, x, xadd);
+}
+
+// g by global column into the padded layout (virtual columns 0).
+template <typename T>
 __global__ void cr_scatter_g_kernel(CRArgs<T> A, const double* g_in) {
-  // padded g (xp) from a double vector over global columns; virtual columns 0
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= A.total_blocks * kCB) return;
   const int64_t gb = e / kCB;
   const int q = (int)(e - gb * kCB);
-  const int64_t k = inst_of_block(A.blk0, A.num_inst, gb);
+  const int64_t k = A.binst[gb];
   const int64_t col = kCB * (gb - A.blk0[k]) + q;
   A.xp[e] = col < A.cols[k] ? (T)g_in[A.col0[k] + col] : T(0);
 }
@@ -669,24 +881,36 @@ inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 struct CRPlan {
   int64_t num_inst = 0, total_blocks = 0;
-  int splits = 1, levels = 0;
-  bool thread_rows = true;   // compression by one thread per block (else one warp per split)
-  std::vector<int64_t> lvl_off, lvl_n;     // eliminate / move / last items per level
+  int splits = 1, levels = 0;              // levels: those run by launches of their own, before the tails
+  std::vector<int64_t> lvl_off, lvl_n;     // eliminate / move items per level
   std::vector<int64_t> ev_off, ev_n;       // staying (even) blocks per level
-  DevBuf tabs, items, evens, grp_lo, P, F0, F1, Rb, xp, hp;
+  DevBuf tabs, items, evens, binst, grp_lo, P, P2, F0, F1, Rb, xp, hp;
   const int64_t* d_cols = nullptr;
   const int64_t* d_col0 = nullptr;
   const int64_t* d_row0 = nullptr;
   const int64_t* d_rows = nullptr;
   const int64_t* d_blk0 = nullptr;
+  const int64_t* d_tail0 = nullptr;
 };
 
 void release_cr(CRPlan*& p) {
   if (!p) return;
-  for (DevBuf* b : {&p->tabs, &p->items, &p->evens, &p->grp_lo, &p->P, &p->F0, &p->F1, &p->Rb, &p->xp, &p->hp})
+  for (DevBuf* b : {&p->tabs, &p->items, &p->evens, &p->binst, &p->grp_lo, &p->P, &p->P2, &p->F0, &p->F1, &p->Rb,
+                    &p->xp, &p->hp})
     release(*b);
   delete p;
   p = nullptr;
+}
+
+// Partial triangles of `splits` threads per block, and of the merge's first pass.
+static qrkit_status cr_partials(qrkit_ctx* ctx, CRPlan& C) {
+  if (C.splits == 1) return QRKIT_OK;
+  const size_t es = elem_size(ctx);
+  const int next = (C.splits + kMergeFan - 1) / kMergeFan;
+  qrkit_status rc = ensure(ctx, C.P, (size_t)C.total_blocks * C.splits * kE0 * es, "banded partial triangles");
+  if (rc == QRKIT_OK && next > 1)
+    rc = ensure(ctx, C.P2, (size_t)C.total_blocks * next * kE0 * es, "banded partial triangles");
+  return rc;
 }
 
 qrkit_status cr_build(qrkit_ctx* ctx, CRPlan*& out, const std::vector<int64_t>& cols,
@@ -706,30 +930,28 @@ qrkit_status cr_build(qrkit_ctx* ctx, CRPlan*& out, const std::vector<int64_t>& 
   }
   C.total_blocks = blk0[ni];
   if (C.total_blocks >= ((int64_t)1 << 30)) return fail(ctx, QRKIT_EUNSUPPORTED, "too many column blocks");
+  // Threads per block: four times as many while the GPU is not full (about 100,000 threads) and the rows
+  // that a split saves (at four per step) outweigh the 16 steps of a merge.
   const double per = C.total_blocks ? (double)total_rows / (double)C.total_blocks : 0.0;
-  // few rows per column block: one thread per block merges its rows (little work per row);
-  // row-heavy blocks: warps reduce 16 rows at a time, blocks split over several warps
-  C.thread_rows = per <= 64.0;
-  C.splits = C.thread_rows ? 1 : (int)std::min<double>(8.0, std::max<double>(1.0, std::ceil(per / 192.0)));
-  // level work lists
+  C.splits = 1;
+  while (C.splits < 64 && C.total_blocks * C.splits < 100000 && per / C.splits > 85.0) C.splits *= kMergeFan;
+  // level work lists; an instance's levels with at most kTailBlocks blocks belong to its tail
   std::vector<std::vector<int64_t>> lv, ev;
+  std::vector<int64_t> tail0(ni);
   for (int64_t k = 0; k < ni; ++k) {
-    const int64_t G = blk0[k + 1] - blk0[k];
-    int64_t Gl = G;
-    for (int l = 0;; ++l) {
+    int64_t Gl = blk0[k + 1] - blk0[k];
+    int l = 0;
+    for (; Gl > kTailBlocks; ++l) {
       if ((int)lv.size() <= l) {
         lv.emplace_back();
         ev.emplace_back();
-      }
-      if (Gl == 1) {
-        lv[l].push_back((k << 32) | (0 << 2) | 2);
-        break;
       }
       for (int64_t i = 1; i < Gl; i += 2) lv[l].push_back((k << 32) | (i << 2) | 0);
       if (Gl % 2 == 1) lv[l].push_back((k << 32) | ((Gl - 1) << 2) | 1);
       for (int64_t j = 0; j < Gl; j += 2) ev[l].push_back((k << 32) | j);
       Gl = (Gl + 1) / 2;
     }
+    tail0[k] = l;
   }
   C.levels = (int)lv.size();
   std::vector<int64_t> items, evens;
@@ -744,30 +966,34 @@ qrkit_status cr_build(qrkit_ctx* ctx, CRPlan*& out, const std::vector<int64_t>& 
   std::vector<int64_t> tabs;
   for (const auto* v : {&cols, &col0, &row0, &rows}) tabs.insert(tabs.end(), v->begin(), v->end());
   tabs.insert(tabs.end(), blk0.begin(), blk0.end());
-  auto up = [&](DevBuf& d, const std::vector<int64_t>& h, const char* what) -> qrkit_status {
-    qrkit_status r = ensure(ctx, d, std::max<size_t>(h.size(), 1) * sizeof(int64_t), what);
+  tabs.insert(tabs.end(), tail0.begin(), tail0.end());
+  std::vector<int32_t> binst((size_t)C.total_blocks);
+  for (int64_t k = 0; k < ni; ++k) std::fill(binst.begin() + blk0[k], binst.begin() + blk0[k + 1], (int32_t)k);
+  auto up = [&](DevBuf& d, const void* h, size_t bytes, const char* what) -> qrkit_status {
+    qrkit_status r = ensure(ctx, d, std::max<size_t>(bytes, 8), what);
     if (r != QRKIT_OK) return r;
-    if (!h.empty())
-      QRKIT_CUDA_TRY(ctx, cudaMemcpy(d.ptr, h.data(), h.size() * sizeof(int64_t), cudaMemcpyHostToDevice));
+    if (bytes > 0) QRKIT_CUDA_TRY(ctx, cudaMemcpy(d.ptr, h, bytes, cudaMemcpyHostToDevice));
     return QRKIT_OK;
   };
   qrkit_status rc;
-  if ((rc = up(C.tabs, tabs, "banded tables")) != QRKIT_OK) return rc;
-  if ((rc = up(C.items, items, "banded levels")) != QRKIT_OK) return rc;
-  if ((rc = up(C.evens, evens, "banded levels")) != QRKIT_OK) return rc;
+  if ((rc = up(C.tabs, tabs.data(), tabs.size() * sizeof(int64_t), "banded tables")) != QRKIT_OK) return rc;
+  if ((rc = up(C.items, items.data(), items.size() * sizeof(int64_t), "banded levels")) != QRKIT_OK) return rc;
+  if ((rc = up(C.evens, evens.data(), evens.size() * sizeof(int64_t), "banded levels")) != QRKIT_OK) return rc;
+  if ((rc = up(C.binst, binst.data(), binst.size() * sizeof(int32_t), "banded blocks")) != QRKIT_OK) return rc;
   const int64_t* t = (const int64_t*)C.tabs.ptr;
   C.d_cols = t;
   C.d_col0 = t + ni;
   C.d_row0 = t + 2 * ni;
   C.d_rows = t + 3 * ni;
   C.d_blk0 = t + 4 * ni;
+  C.d_tail0 = t + 5 * ni + 1;
   const size_t es = elem_size(ctx);
   const size_t TB = (size_t)C.total_blocks;
   if ((rc = ensure(ctx, C.grp_lo, TB * sizeof(int64_t), "banded group rows")) != QRKIT_OK) return rc;
-  if ((rc = ensure(ctx, C.P, TB * C.splits * 16 * kEW * es, "banded partial triangles")) != QRKIT_OK) return rc;
-  if ((rc = ensure(ctx, C.F0, TB * 16 * kEW * es, "banded block rows")) != QRKIT_OK) return rc;
-  if ((rc = ensure(ctx, C.F1, TB * 16 * kEW * es, "banded block rows")) != QRKIT_OK) return rc;
-  if ((rc = ensure(ctx, C.Rb, TB * kCB * kRW * es, "banded R blocks")) != QRKIT_OK) return rc;
+  if ((rc = cr_partials(ctx, C)) != QRKIT_OK) return rc;
+  if ((rc = ensure(ctx, C.F0, TB * kFW * es, "banded block rows")) != QRKIT_OK) return rc;
+  if ((rc = ensure(ctx, C.F1, TB * kFW * es, "banded block rows")) != QRKIT_OK) return rc;
+  if ((rc = ensure(ctx, C.Rb, TB * kRW * es, "banded R blocks")) != QRKIT_OK) return rc;
   if ((rc = ensure(ctx, C.xp, TB * kCB * es, "banded padded x")) != QRKIT_OK) return rc;
   if ((rc = ensure(ctx, C.hp, TB * kCB * es, "banded padded h")) != QRKIT_OK) return rc;
   return QRKIT_OK;
@@ -775,9 +1001,8 @@ qrkit_status cr_build(qrkit_ctx* ctx, CRPlan*& out, const std::vector<int64_t>& 
 
 qrkit_status cr_set_strategy(qrkit_ctx* ctx, CRPlan& C, bool thread_rows, int splits) {
   if (splits < 1 || splits > 64) return fail(ctx, QRKIT_EINVAL, "splits must be in [1, 64]");
-  C.thread_rows = thread_rows;
   C.splits = thread_rows ? 1 : splits;
-  return ensure(ctx, C.P, (size_t)C.total_blocks * C.splits * 16 * kEW * elem_size(ctx), "banded partial triangles");
+  return cr_partials(ctx, C);
 }
 
 template <typename T>
@@ -789,6 +1014,8 @@ static CRArgs<T> cr_args(qrkit_ctx* ctx, CRPlan& C) {
   A.row0 = C.d_row0;
   A.rows = C.d_rows;
   A.blk0 = C.d_blk0;
+  A.tail0 = C.d_tail0;
+  A.binst = (const int32_t*)C.binst.ptr;
   A.total_blocks = C.total_blocks;
   A.splits = C.splits;
   A.grp_lo = (int64_t*)C.grp_lo.ptr;
@@ -824,50 +1051,59 @@ static qrkit_status cr_solve_typed(qrkit_ctx* ctx, CRPlan& C, const int64_t* sta
   A.res2 = res2;
   QRKIT_CUDA_TRY(ctx, cudaMemsetAsync(res2, 0, (size_t)C.num_inst * sizeof(double), st));
   if (starts) CR_LAUNCH(ctx, cr_ranges_kernel<T><<<nblk(C.total_blocks, 256), 256, 0, st>>>(A));
-  const size_t tri_smem = (size_t)kTriElems * kCompThreads * sizeof(T);
-  if (tri_smem > 48 * 1024) {
-    QRKIT_CUDA_TRY(ctx, cudaFuncSetAttribute(cr_compress_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)tri_smem));
-  }
-  if (C.thread_rows) {
-    CR_LAUNCH(ctx, cr_compress_kernel<T><<<nblk(C.total_blocks, kCompThreads), kCompThreads, tri_smem, st>>>(A));
-  } else {
-    CR_LAUNCH(ctx, cr_compress_warp_kernel<T><<<nblk(C.total_blocks * C.splits * 32, 128), 128, 0, st>>>(A));
-    CR_LAUNCH(ctx, cr_merge_warp_kernel<T><<<nblk(C.total_blocks * 32, 128), 128, 0, st>>>(A));
+  CR_LAUNCH(ctx, cr_compress_kernel<T><<<nblk(C.total_blocks * C.splits, kCompThreads), kCompThreads, 0, st>>>(A));
+  T* in = A.P;
+  T* other = (T*)C.P2.ptr;
+  for (int n = C.splits; n > 1;) {
+    const int m = (n + kMergeFan - 1) / kMergeFan;
+    CR_LAUNCH(ctx, cr_merge_kernel<T><<<nblk(C.total_blocks * m, kCompThreads), kCompThreads, 0, st>>>(
+                       A, in, n, m == 1 ? A.F0 : other, m, m == 1 ? kFW : kE0));
+    std::swap(in, other);
+    n = m;
   }
   const int64_t* items = (const int64_t*)C.items.ptr;
-  T* Fc = A.F0;
-  T* Fn = A.F1;
   for (int l = 0; l < C.levels; ++l) {
-    CR_LAUNCH(ctx, cr_level_kernel<T><<<nblk(C.lvl_n[l] * 32, 128), 128, 0, st>>>(A, items + C.lvl_off[l],
-                                                                                 C.lvl_n[l], l, Fc, Fn));
-    std::swap(Fc, Fn);
+    const T* Fc = (l & 1) ? A.F1 : A.F0;
+    T* Fn = (l & 1) ? A.F0 : A.F1;
+    const unsigned grid = nblk(C.lvl_n[l] * kItemThreads, kLevelThreads);
+    if (l == 0)
+      CR_LAUNCH(ctx, (cr_level_kernel<T, true><<<grid, kLevelThreads, 0, st>>>(A, items + C.lvl_off[l], C.lvl_n[l], l,
+                                                                              Fc, Fn)));
+    else
+      CR_LAUNCH(ctx, (cr_level_kernel<T, false><<<grid, kLevelThreads, 0, st>>>(A, items + C.lvl_off[l], C.lvl_n[l], l,
+                                                                               Fc, Fn)));
   }
+  const int tt = C.num_inst >= 4 * ctx->num_sms ? 128 : tail_threads<T>();
+  CR_LAUNCH(ctx, cr_tail_kernel<T><<<(unsigned)C.num_inst, tt, 0, st>>>(A, x));
   for (int l = C.levels - 1; l >= 0; --l)
     CR_LAUNCH(ctx, cr_backsub_kernel<T><<<nblk(C.lvl_n[l] * kItemThreads, 128), 128, 0, st>>>(
-                       A, items + C.lvl_off[l], C.lvl_n[l], l, 0, x));
+                       A, items + C.lvl_off[l], C.lvl_n[l], l, 0, x, (T*)nullptr));
   return QRKIT_OK;
 }
 
-// dx = R^{-1} R^{-T} g with the stored factor (g: double over global columns).
+// dx = R^{-1} R^{-T} g with the stored factor (g: double over global columns, or null: already in the
+// padded layout), written to dx and added to xadd (either may be null).
 template <typename T>
-static qrkit_status cr_normal_typed(qrkit_ctx* ctx, CRPlan& C, const double* g, T* dx) {
+static qrkit_status cr_normal_typed(qrkit_ctx* ctx, CRPlan& C, const double* g, T* dx, T* xadd) {
   cudaStream_t st = ctx->stream;
   CRArgs<T> A = cr_args<T>(ctx, C);
   const int64_t* items = (const int64_t*)C.items.ptr;
   const int64_t* evens = (const int64_t*)C.evens.ptr;
-  CR_LAUNCH(ctx, cr_scatter_g_kernel<T><<<nblk(C.total_blocks * kCB, 256), 256, 0, st>>>(A, g));
-  for (int l = 0; l < C.levels; ++l) {
-    CR_LAUNCH(ctx, cr_rt_kernel<T><<<nblk(C.lvl_n[l] * kItemThreads, 128), 128, 0, st>>>(A, items + C.lvl_off[l],
-                                                                                          C.lvl_n[l], l));
-    if (C.ev_n[l] > 0)
-      CR_LAUNCH(ctx, cr_rt_update_kernel<T><<<nblk(C.ev_n[l] * kItemThreads, 128), 128, 0, st>>>(
-                         A, evens + C.ev_off[l], C.ev_n[l], l));
-  }
+  if (g) CR_LAUNCH(ctx, cr_scatter_g_kernel<T><<<nblk(C.total_blocks * kCB, 256), 256, 0, st>>>(A, g));
+  for (int l = 0; l < C.levels; ++l)
+    CR_LAUNCH(ctx, cr_rt_level_kernel<T><<<nblk(C.ev_n[l] * kItemThreads, 128), 128, 0, st>>>(
+                       A, evens + C.ev_off[l], C.ev_n[l], l));
+  const int tt = C.num_inst >= 4 * ctx->num_sms ? 128 : tail_threads<T>();
+  CR_LAUNCH(ctx, cr_tail_normal_kernel<T><<<(unsigned)C.num_inst, tt, 0, st>>>(A, dx, xadd));
   for (int l = C.levels - 1; l >= 0; --l)
     CR_LAUNCH(ctx, cr_backsub_kernel<T><<<nblk(C.lvl_n[l] * kItemThreads, 128), 128, 0, st>>>(
-                       A, items + C.lvl_off[l], C.lvl_n[l], l, 1, dx));
+                       A, items + C.lvl_off[l], C.lvl_n[l], l, 1, dx, xadd));
   return QRKIT_OK;
+}
+
+void cr_padded(const CRPlan& C, const int64_t** blk0, void** g) {
+  *blk0 = C.d_blk0;
+  *g = C.xp.ptr;
 }
 
 qrkit_status cr_solve(qrkit_ctx* ctx, CRPlan& C, const int64_t* starts, int rpc, int w, const void* J,
@@ -880,9 +1116,9 @@ qrkit_status cr_solve(qrkit_ctx* ctx, CRPlan& C, const int64_t* starts, int rpc,
                                res2);
 }
 
-qrkit_status cr_normal_solve(qrkit_ctx* ctx, CRPlan& C, const double* g, void* dx) {
-  if (ctx->precision == QRKIT_FP64) return cr_normal_typed<double>(ctx, C, g, (double*)dx);
-  return cr_normal_typed<float>(ctx, C, g, (float*)dx);
+qrkit_status cr_normal_solve(qrkit_ctx* ctx, CRPlan& C, const double* g, void* dx, void* xadd) {
+  if (ctx->precision == QRKIT_FP64) return cr_normal_typed<double>(ctx, C, g, (double*)dx, (double*)xadd);
+  return cr_normal_typed<float>(ctx, C, g, (float*)dx, (float*)xadd);
 }
 
 }  // namespace qrkit

@@ -209,11 +209,15 @@ qrkit_status cr_build(qrkit_ctx* ctx, CRPlan*& out, const std::vector<int64_t>& 
 // implicit starts floor(i / rpc); damping rows lambda^(1/2) D_j; x and D by global column.
 qrkit_status cr_solve(qrkit_ctx* ctx, CRPlan& C, const int64_t* starts, int rpc, int w, const void* J,
                       const void* b, const double* D, double lambda, void* x, double* res2);
-// Compression strategy of the parallel banded QR: one thread per column block, or warps
-// with `splits` splits per block (autotuning).
+// Compression strategy of the parallel banded QR: one thread per column block, or `splits` threads
+// per block whose triangles are merged (autotuning).
 qrkit_status cr_set_strategy(qrkit_ctx* ctx, CRPlan& C, bool thread_rows, int splits);
-// dx = R^{-1} R^{-T} g with the factor of the last cr_solve (g double, dx by global column).
-qrkit_status cr_normal_solve(qrkit_ctx* ctx, CRPlan& C, const double* g, void* dx);
+// The padded layout of its right-hand sides: column j of instance k at 8 blk0[k] + j, zero past the instance's
+// last column.
+void cr_padded(const CRPlan& C, const int64_t** blk0, void** g);
+// dx = R^{-1} R^{-T} g with the factor of the last cr_solve (g double by global column, or null: in the
+// padded layout already; dx by global column), written to dx and added to xadd; either may be null.
+qrkit_status cr_normal_solve(qrkit_ctx* ctx, CRPlan& C, const double* g, void* dx, void* xadd);
 
 // Damping-policy MLP parameters and training state (mlp.cu)
 struct Mlp {
