@@ -429,7 +429,7 @@ struct BandGroups {   // what both kernels are told
 };
 
 template <bool kW8, bool kStaged, int MW>
-__global__ void __launch_bounds__(256) band_norm_f32_kernel(BandGroups B, double* D) {
+__global__ void __launch_bounds__(256) band_norm_f32_kernel(BandGroups B, double* D, float2* D2) {
   extern __shared__ __align__(16) float sm_f[];
   const int nt = blockDim.x, tid = threadIdx.x, w = B.w;
   const int64_t grp0 = (int64_t)blockIdx.x * (nt - (w - 1)) - (w - 1), grp = grp0 + tid;
@@ -453,10 +453,37 @@ __global__ void __launch_bounds__(256) band_norm_f32_kernel(BandGroups B, double
   __syncthreads();
   if (tid < w - 1 || !have) return;
   const int64_t j = grp - B.inst_col0[k];
-  double sum = 0.0;
-  for (int t = 0; t < w && t <= j; ++t) sum += (double)S[(tid - t) * (w + 1) + t];
-  const double d = sqrt(sum);
-  D[grp] = d == 0.0 ? 1.0 : d;
+  float h = 0.f, l = 0.f;   // the sum, and then its root, as float pairs
+  for (int t = 0; t < w && t <= j; ++t) {
+    float tt, e;
+    dev::two_sum(h, S[(tid - t) * (w + 1) + t], tt, e);
+    h = tt;
+    l = __fadd_rn(l, e);
+  }
+  const float s = h + l;
+  l = (h - s) + l;
+  float r = 1.f, c = 0.f;
+  if (s > 0.f) {
+    r = sqrtf(s);
+    c = (__fmaf_rn(-r, r, s) + l) / (2.f * r);   // one Newton step for the root of s + l
+  } else if (s == 0.f) {
+    D2[grp] = make_float2(1.f, 0.f);   // zero norm -> 1
+    D[grp] = 1.0;
+    return;
+  } else {
+    r = s;   // NaN
+  }
+  D2[grp] = make_float2(s, l);
+  D[grp] = (double)r + (double)c;
+}
+
+// D and D^2 (a float pair) of a given float D.
+__global__ void band_given_d_kernel(const float* in, double* D, float2* D2, int64_t n) {
+  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= n) return;
+  const float d = in[j], p = __fmul_rn(d, d);
+  D[j] = (double)d;
+  D2[j] = make_float2(p, __fmaf_rn(d, d, -p));
 }
 
 // g = J^T (b - J x) - lambda D^2 x into the parallel QR's padded layout: the residual of a row as an
@@ -464,8 +491,8 @@ __global__ void __launch_bounds__(256) band_norm_f32_kernel(BandGroups B, double
 // without GB300's slow FP64 pipe), the column sums as pairs too.
 template <bool kW8, bool kStaged, int MW>
 __global__ void __launch_bounds__(256) band_grad_f32_kernel(BandGroups B, const float* b, const float* x,
-                                                            const double* D, double lam, const int64_t* blk0,
-                                                            float* gp) {
+                                                            const float2* D2, float lam_h, float lam_l,
+                                                            const int64_t* blk0, float* gp) {
   extern __shared__ __align__(16) float sm_f[];
   const int nt = blockDim.x, tid = threadIdx.x, w = B.w;
   const int64_t grp0 = (int64_t)blockIdx.x * (nt - (w - 1)) - (w - 1), grp = grp0 + tid;
@@ -530,10 +557,21 @@ __global__ void __launch_bounds__(256) band_grad_f32_kernel(BandGroups B, const 
     s = tt;
     c = __fadd_rn(c, __fadd_rn(e, v.y));
   }
-  double acc = (double)s + (double)c;
-  if (lam > 0.0) acc -= lam * D[grp] * D[grp] * (double)xs[tid];
+  if (lam_h > 0.f) {   // - lambda D^2 x, all factors but x pairs
+    const float2 d2 = D2[grp];
+    float p = __fmul_rn(lam_h, d2.x);
+    float pe = __fmaf_rn(lam_h, d2.x, -p);
+    pe = __fmaf_rn(lam_h, d2.y, __fmaf_rn(lam_l, d2.x, pe));
+    const float xj = -xs[tid];
+    const float q = __fmul_rn(p, xj);
+    const float qe = __fmaf_rn(pe, xj, __fmaf_rn(p, xj, -q));
+    float tt, e;
+    dev::two_sum(s, q, tt, e);
+    s = tt;
+    c = __fadd_rn(c, __fadd_rn(e, qe));
+  }
   float* out = gp + 8 * blk0[k];
-  out[j] = (float)acc;
+  out[j] = s + c;
   if (j == B.inst_cols[k] - 1)   // the padding columns of the last block
     for (int64_t e = j + 1; e < (j + 8) / 8 * 8; ++e) out[e] = 0.f;
 }
@@ -796,6 +834,7 @@ qrkit_status banded_plan(qrkit_ctx* ctx, const qrkit_structure* s) {
   if ((st = ensure(ctx, B.Rw, (size_t)cc * B.w * es, "banded R")) != QRKIT_OK) return st;
   if ((st = ensure(ctx, B.c, (size_t)cc * es, "banded c")) != QRKIT_OK) return st;
   if ((st = ensure(ctx, B.D, (size_t)cc * sizeof(double), "banded D")) != QRKIT_OK) return st;
+  if (es == sizeof(float) && (st = ensure(ctx, B.D2, (size_t)cc * sizeof(float2), "banded D")) != QRKIT_OK) return st;
   if ((st = ensure(ctx, B.res2, (size_t)B.num_inst * sizeof(double), "banded residual")) != QRKIT_OK) return st;
   if (B.parallel) {
     if ((st = cr_build(ctx, B.cr, cols, c0, r0, nrows)) != QRKIT_OK) return st;
@@ -847,8 +886,10 @@ static qrkit_status banded_run(qrkit_ctx* ctx, const void* J, const void* b, con
         QRKIT_CUDA_TRY(ctx, cudaMemcpyAsync(D, Dext, (size_t)B.total_cols * sizeof(double),
                                             cudaMemcpyDeviceToDevice, st));
       } else {
-        qrkit_status rc = widen_to_double(ctx, (const float*)Dext, D, B.total_cols);
-        if (rc != QRKIT_OK) return rc;
+        band_given_d_kernel<<<nblk(B.total_cols, 256), 256, 0, st>>>((const float*)Dext, D, (float2*)B.D2.ptr,
+                                                                    B.total_cols);
+        ctx->launches += 1;
+        QRKIT_CUDA_TRY(ctx, cudaGetLastError());
       }
     } else if (B.explicit_starts) {
       band_colnorm_explicit_kernel<T><<<nblk(B.total_cols, 256), 256, 0, st>>>(
@@ -862,8 +903,8 @@ static qrkit_status banded_run(qrkit_ctx* ctx, const void* J, const void* b, con
         const BandLaunch L = band_launch(G, (size_t)(B.w + 1) * sizeof(float), 0);
         BandGroups GL = G;
         GL.gs = L.gs;
-        if (B.w <= 8) BAND_F32_LAUNCH(ctx, L, band_norm_f32_kernel, 8, GL, D);
-        else BAND_F32_LAUNCH(ctx, L, band_norm_f32_kernel, kBW, GL, D);
+        if (B.w <= 8) BAND_F32_LAUNCH(ctx, L, band_norm_f32_kernel, 8, GL, D, (float2*)B.D2.ptr);
+        else BAND_F32_LAUNCH(ctx, L, band_norm_f32_kernel, kBW, GL, D, (float2*)B.D2.ptr);
       } else {
         band_colnorm_kernel<<<nblk(B.total_cols, 256), 256, 0, st>>>(nullptr, (const double*)J, dcols, dc0, dr0,
                                                                     B.num_inst, B.rows_per_col, B.w, D);
@@ -920,7 +961,8 @@ static qrkit_status banded_run(qrkit_ctx* ctx, const void* J, const void* b, con
         const int64_t* blk0;
         void* gp;
         cr_padded(*B.cr, &blk0, &gp);
-        BAND_F32_LAUNCH(ctx, L, band_grad_f32_kernel, 8, GL, (const float*)b, (const float*)p, D, lambda, blk0, (float*)gp);
+        BAND_F32_LAUNCH(ctx, L, band_grad_f32_kernel, 8, GL, (const float*)b, (const float*)p, (const float2*)B.D2.ptr,
+                        (float)lambda, (float)(lambda - (double)(float)lambda), blk0, (float*)gp);
       } else {
         band_resid_kernel<T><<<nblk(B.total_rows, 256), 256, 0, st>>>(
             (const T*)J, (const T*)b, (const T*)p, dcols, dc0, dr0, B.num_inst, B.total_rows, B.rows_per_col, B.w,
@@ -1063,7 +1105,7 @@ qrkit_status banded_get_factor(qrkit_ctx* ctx, void* Rw_out, void* c_out, double
 void release_band(Band& B) {
   release(B.d_cols); release(B.d_col0); release(B.d_row0); release(B.Rw); release(B.c);
   release(B.d_inst); release(B.d_rows); release(B.d_start);
-  release(B.D); release(B.res2); release(B.g); release(B.h); release(B.r);
+  release(B.D); release(B.D2); release(B.res2); release(B.g); release(B.h); release(B.r);
   release_cr(B.cr);
   B = Band();
 }

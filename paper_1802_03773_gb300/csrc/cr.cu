@@ -32,6 +32,7 @@
 #include <string>
 #include <vector>
 
+#include "device_util.cuh"
 #include "internal.h"
 
 namespace qrkit {
@@ -233,20 +234,47 @@ __device__ __forceinline__ void load8(T (&v)[8], const T* src) {   // src 16-byt
   }
 }
 
-// Sum of a per-thread double into res2 of the thread's instance: one atomic per warp where all its
-// threads work on one instance.
-__device__ __forceinline__ void add_res2(double* res2, int64_t k, double res) {
-  __syncwarp();
-  const unsigned m = __activemask();
-  const int64_t k0 = __shfl_sync(m, k, __ffs(m) - 1);
-  if (m == 0xffffffffu && __all_sync(m, k == k0)) {
-#pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) res += __shfl_xor_sync(m, res, d);
-    if ((threadIdx.x & 31) == 0 && res != 0.0) atomicAdd(res2 + k, res);
-  } else if (res != 0.0) {
-    atomicAdd(res2 + k, res);
+// A thread's squared residual: a float pair (Dot2) for float, a double for double.  (A warp's FP64 instruction
+// occupies the SM's FP64 unit for 16 cycles here: summing every square in double took a quarter of the
+// compression's and of the fronts' time.)
+template <typename T>
+struct ResidualSum {
+  T h = T(0), l = T(0);
+  __device__ __forceinline__ void square(T x) {
+    if constexpr (sizeof(T) == 4) {
+      const T p = __fmul_rn(x, x), pe = __fmaf_rn(x, x, -p);
+      add(p, pe);
+    } else {
+      h += x * x;
+    }
   }
-}
+  __device__ __forceinline__ void add(T ph, T pl) {
+    if constexpr (sizeof(T) == 4) {
+      T t, e;
+      dev::two_sum(h, ph, t, e);
+      h = t;
+      l = __fadd_rn(l, __fadd_rn(e, pl));
+    } else {
+      h += ph;
+    }
+  }
+  // into res2 of the thread's instance: one atomic per warp where all its threads work on one instance
+  __device__ __forceinline__ void flush(double* res2, int64_t k) {
+    __syncwarp();
+    const unsigned m = __activemask();
+    const int64_t k0 = __shfl_sync(m, k, __ffs(m) - 1);
+    if (m == 0xffffffffu && __all_sync(m, k == k0)) {
+#pragma unroll
+      for (int d = 16; d >= 1; d >>= 1) {
+        const T ph = __shfl_xor_sync(m, h, d), pl = __shfl_xor_sync(m, l, d);
+        add(ph, pl);
+      }
+      if ((threadIdx.x & 31) == 0 && h != T(0)) atomicAdd(res2 + k, (double)h + (double)l);
+    } else if (h != T(0)) {
+      atomicAdd(res2 + k, (double)h + (double)l);
+    }
+  }
+};
 
 template <typename T>
 __global__ void __launch_bounds__(kCompThreads) cr_compress_kernel(CRArgs<T> A) {
@@ -278,7 +306,7 @@ __global__ void __launch_bounds__(kCompThreads) cr_compress_kernel(CRArgs<T> A) 
   T* dst = A.splits == 1 ? A.F0 + gb * kFW : A.P + item * kE0;
   // whole rows by 16-byte loads where they are aligned; else entry by entry
   const bool wide = A.w == kCB && (reinterpret_cast<uintptr_t>(A.J) & 15) == 0;
-  double res = 0.0;
+  ResidualSum<T> res;
   // One step per turn: the next (up to four) rows starting at column c, or, when there are none, the window
   // one column on.  The threads of a warp may be at different columns.
   int64_t ahead[4];   // explicit starts of the next four rows, fetched one step early
@@ -321,7 +349,7 @@ __global__ void __launch_bounds__(kCompThreads) cr_compress_kernel(CRArgs<T> A) 
       }
       W.insert(a, b);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) res += (double)b[q] * (double)b[q];
+      for (int q = 0; q < 4; ++q) res.square(b[q]);
     } else {
       T row[8];
 #pragma unroll
@@ -341,7 +369,7 @@ __global__ void __launch_bounds__(kCompThreads) cr_compress_kernel(CRArgs<T> A) 
     store8(dst + 64 + 8 * i, row);
   }
   store8(dst + 136, W.z);
-  add_res2(A.res2, k, res);
+  res.flush(A.res2, k);
 }
 
 // 1b. merge of kMergeFan partial triangles of a block into one, by the same window; 16 columns.
@@ -362,7 +390,7 @@ __global__ void __launch_bounds__(kCompThreads) cr_merge_kernel(CRArgs<T> A, con
   for (int e = 0; e < 36; ++e) W.t[e] = T(0);
 #pragma unroll
   for (int i = 0; i < 8; ++i) W.z[i] = T(0);
-  double res = 0.0;
+  ResidualSum<T> res;
 #pragma unroll 1
   for (int c = 0; c < 16; ++c) {
     T a[4][8], b[4];
@@ -385,7 +413,7 @@ __global__ void __launch_bounds__(kCompThreads) cr_merge_kernel(CRArgs<T> A, con
     }
     W.insert(a, b);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) res += (double)b[q] * (double)b[q];
+    for (int q = 0; q < 4; ++q) res.square(b[q]);
     if (c < 8) {
       T row[8];
 #pragma unroll
@@ -401,7 +429,7 @@ __global__ void __launch_bounds__(kCompThreads) cr_merge_kernel(CRArgs<T> A, con
     dst[128 + c] = W.z[0];
     W.shift();
   }
-  add_res2(A.res2, A.binst[gb], res);
+  res.flush(A.res2, A.binst[gb]);
 }
 
 // Work items of a level: inst << 32 | i << 2 | kind (0 eliminate odd i, 1 move up, 2 last).
@@ -487,19 +515,18 @@ __device__ __forceinline__ void apply_reflector(T tau, const T (&v)[8], T& p, T 
     if (r >= from && r < M) x[r] -= w * v[r];
 }
 
-// One item of level `level`: block i of instance k.  Returns the squared residual it leaves.
+// One item of level `level`: block i of instance k.  The lanes add their share of the residual it leaves to res.
 template <typename T, bool kCompressed>
-__device__ __forceinline__ double cr_item(const CRArgs<T>& A, int64_t k, int64_t i, int kind, int level, const T* Fc,
-                                          T* Fn, int j, unsigned gmask) {
+__device__ __forceinline__ void cr_item(const CRArgs<T>& A, int64_t k, int64_t i, int kind, int level, const T* Fc,
+                                        T* Fn, int j, unsigned gmask, ResidualSum<T>& res) {
   const int64_t b0 = A.blk0[k];
   T a[8], bl[8], bh[8], cl[8], ch[8];
   load_block_row<T, kCompressed>(Fc + (b0 + i) * kFW, j, a, bl, bh, cl, ch);
   if (kind == 1) {   // unpaired last block row: moves up
     store_block_row(Fn + (b0 + i / 2) * kFW, j, a, bl, bh, cl, ch);
-    return 0.0;
+    return;
   }
   T* R = A.Rb + (b0 + (i << level)) * kRW;
-  double res = 0.0;
   T rl[8];   // R's left part
 #pragma unroll
   for (int r = 0; r < 8; ++r) rl[r] = T(0);
@@ -635,19 +662,17 @@ __device__ __forceinline__ double cr_item(const CRArgs<T>& A, int64_t k, int64_t
       }
     }
     store_block_row(Fn + (b0 + (i - 1) / 2) * kFW, j, pa, lr, bh, dl, ch);
-#pragma unroll
-    for (int r = 0; r < 8; ++r) res += (double)dh[r] * (double)dh[r];
+    res.square(lane_of(dh, j));
   } else {   // the last block: its A is triangular, nothing is to its right
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
       R[8 * r + j] = a[r];
       R[64 + 8 * r + j] = T(0);
       R[128 + 8 * r + j] = bl[r];
-      res += (double)ch[r] * (double)ch[r];
     }
     R[192 + j] = lane_of(cl, j);
+    res.square(lane_of(ch, j));
   }
-  return j == 0 ? res : 0.0;
 }
 
 constexpr int kLevelThreads = 128;
@@ -660,14 +685,14 @@ cr_level_kernel(CRArgs<T> A, const int64_t* items, int64_t nitems, int level, co
   const unsigned gmask = 0xffu << (threadIdx.x & 24);
   int64_t k = 0, i = 0;
   int kind = 1;
-  double res = 0.0;
+  ResidualSum<T> res;
   if (w < nitems) {
     decode(items[w], k, i, kind);
-    res = cr_item<T, kCompressed>(A, k, i, kind, level, Fc, Fn, j, gmask);
+    cr_item<T, kCompressed>(A, k, i, kind, level, Fc, Fn, j, gmask, res);
   } else if (nitems > 0) {
     decode(items[nitems - 1], k, i, kind);   // adds nothing, to the last item's instance
   }
-  add_res2(A.res2, k, res);
+  res.flush(A.res2, k);
 }
 
 // ---- 3. back-substitution of one block, eight lanes: lane q owns row q of the block's R (own | left |
@@ -812,7 +837,7 @@ __global__ void __launch_bounds__(tail_threads<T>(), 1) cr_tail_kernel(CRArgs<T>
   const unsigned gmask = 0xffu << (threadIdx.x & 24);
   const int64_t G = A.blk0[k + 1] - A.blk0[k];
   const int lt = (int)A.tail0[k];
-  double res = 0.0;
+  ResidualSum<T> res;
   int l = lt;
   for (;; ++l) {
     const int64_t Gl = blocks_at(G, l);
@@ -823,13 +848,13 @@ __global__ void __launch_bounds__(tail_threads<T>(), 1) cr_tail_kernel(CRArgs<T>
     for (int64_t m = grp; m < n; m += ng) {
       const int kind = Gl == 1 ? 2 : (2 * m + 1 < Gl ? 0 : 1);
       const int64_t i = kind == 0 ? 2 * m + 1 : Gl - 1;
-      if (l == 0) res += cr_item<T, true>(A, k, i, kind, l, Fc, Fn, j, gmask);
-      else res += cr_item<T, false>(A, k, i, kind, l, Fc, Fn, j, gmask);
+      if (l == 0) cr_item<T, true>(A, k, i, kind, l, Fc, Fn, j, gmask, res);
+      else cr_item<T, false>(A, k, i, kind, l, Fc, Fn, j, gmask, res);
     }
     __syncthreads();
     if (Gl == 1) break;
   }
-  if (res != 0.0) atomicAdd(A.res2 + k, res);
+  res.flush(A.res2, k);
   tail_backsub(A, k, G, lt, l, false, x, (T*)nullptr);
 }
 
