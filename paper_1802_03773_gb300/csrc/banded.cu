@@ -371,14 +371,23 @@ __device__ __forceinline__ const float* group_rows_f32(const float* J, int64_t g
   if constexpr (kStaged) {
     const bool wide = (rw & 3) == 0 && (reinterpret_cast<uintptr_t>(J) & 15) == 0;   // then gs % 4 == 0 too
     const int unit = wide ? 4 : 1, per = rw / unit;
-    for (int e = threadIdx.x; e < nt * per; e += nt) {
-      const int gg = e / per, o = (e - gg * per) * unit;
-      const int64_t grp = grp0 + gg;
-      if (grp < 0 || grp >= total) continue;
-      const float* src = J + grp * rw + o;
-      float* dst = buf + gg * gs + o;
-      if (wide) dev::cp_async16(dst, src);
-      else asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dev::smem_u32(dst)), "l"(src) : "memory");
+    int gg = threadIdx.x / per, o = (threadIdx.x - gg * per) * unit;   // of the thread's next copy
+    const int dg = nt / per, dq = (nt - dg * per) * unit;
+    const float* src0 = J + grp0 * rw;
+    const int lo = grp0 < 0 ? (int)-grp0 : 0, hi = (int)(total - grp0 < nt ? total - grp0 : nt);
+    for (int e = 0; e < per; ++e) {
+      if (gg >= lo && gg < hi) {
+        const float* src = src0 + gg * rw + o;
+        float* dst = buf + gg * gs + o;
+        if (wide) dev::cp_async16(dst, src);
+        else asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dev::smem_u32(dst)), "l"(src) : "memory");
+      }
+      gg += dg;
+      o += dq;
+      if (o >= rw) {
+        o -= rw;
+        ++gg;
+      }
     }
     dev::cp_async_commit();
     dev::cp_async_wait_all();

@@ -100,11 +100,17 @@ struct CRArgs {
   const T* b;             // rows
   const double* D;        // global columns (damping rows when lam > 0)
   double lam;
-  int splits;             // threads per block in the compression
+  // compression: num_items threads; item_blk: block of each (null: one per block), blk_item0: first item of a block
+  int64_t num_items;
+  const int32_t* item_blk;
+  const int32_t* blk_item0;
   // work space
   int64_t* grp_lo;        // total_blocks: first row of each block's group (explicit starts)
-  T* P;                   // total_blocks x splits partial triangles, kE0 each
-  T* F0;                  // total_blocks block rows, kFW each (two buffers); level 0: kE0 of them used
+  T* P;                   // num_items partial triangles, e0_at()
+  T* E0;                  // total_blocks compressed block rows (level 0), e0_at().  A buffer of their own: the rows of
+                          // different instances share lines, and an instance's tail may still read its own
+                          // when another's upper levels write block rows.
+  T* F0;                  // total_blocks block rows, kFW each (two buffers; level l reads F1 when l is odd)
   T* F1;
   T* Rb;                  // total_blocks x kRW
   T* xp;                  // total_blocks x 8 padded solution / rhs work
@@ -156,8 +162,18 @@ __device__ __forceinline__ void group_rows(const CRArgs<T>& A, int64_t k, int64_
 // quarter of the arithmetic and no shared memory, and block rows leave as 16-byte stores.
 //
 // A compressed block row E: row c < 8 holds columns c .. c + 7 at 8 c; row 8 + i holds columns 8 .. 15 (zeros
-// below the diagonal) at 64 + 8 i; the rhs of the 16 rows at 128.
+// below the diagonal) at 64 + 8 i; the rhs of the 16 rows at 128.  Block rows are stored 32 at a time,
+// their 16-byte pieces interleaved: a warp's threads, a block row each, store whole lines, and the lane
+// groups that read adjacent block rows share them.  (A thread per block row storing 576 bytes of its own
+// kept the L1 at 86 % with lines touched.)
 constexpr int kCompThreads = 128;
+
+// Position of element e of compressed block row `it`.
+template <typename T>
+__host__ __device__ __forceinline__ int64_t e0_at(int64_t it, int e) {
+  constexpr int E = 16 / (int)sizeof(T), P = kE0 / E;
+  return (((it >> 5) * P + e / E) * 32 + (it & 31)) * E + e % E;
+}
 
 __host__ __device__ constexpr int tri(int i, int j) { return i * 8 - (i * (i - 1)) / 2 + (j - i); }
 
@@ -234,6 +250,35 @@ __device__ __forceinline__ void load8(T (&v)[8], const T* src) {   // src 16-byt
   }
 }
 
+// Eight consecutive elements of a compressed block row, from a multiple of 8 on.
+template <typename T>
+__device__ __forceinline__ void store_e0(T* base, int64_t it, int e, const T (&v)[8]) {
+  if constexpr (sizeof(T) == 4) {
+    *reinterpret_cast<float4*>(base + e0_at<T>(it, e)) = make_float4(v[0], v[1], v[2], v[3]);
+    *reinterpret_cast<float4*>(base + e0_at<T>(it, e + 4)) = make_float4(v[4], v[5], v[6], v[7]);
+  } else {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      *reinterpret_cast<double2*>(base + e0_at<T>(it, e + 2 * q)) = make_double2(v[2 * q], v[2 * q + 1]);
+  }
+}
+template <typename T>
+__device__ __forceinline__ void load_e0(T (&v)[8], const T* base, int64_t it, int e) {
+  if constexpr (sizeof(T) == 4) {
+    const float4 a = *reinterpret_cast<const float4*>(base + e0_at<T>(it, e));
+    const float4 b = *reinterpret_cast<const float4*>(base + e0_at<T>(it, e + 4));
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+  } else {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const double2 a = *reinterpret_cast<const double2*>(base + e0_at<T>(it, e + 2 * q));
+      v[2 * q] = a.x;
+      v[2 * q + 1] = a.y;
+    }
+  }
+}
+
 // A thread's squared residual: a float pair (Dot2) for float, a double for double.  (A warp's FP64 instruction
 // occupies the SM's FP64 unit for 16 cycles here: summing every square in double took a quarter of the
 // compression's and of the fronts' time.)
@@ -276,20 +321,29 @@ struct ResidualSum {
   }
 };
 
+// Rows of 8 aligned values (kStaged) arrive through shared memory: the lanes of a warp fetch each thread's next
+// four rows together (8 or 16 lanes a thread, whole lines, where a thread's own 16-byte loads touch a line of
+// their own each), one step ahead.  Other rows are read by their thread, entry by entry.
 template <typename T>
-__global__ void __launch_bounds__(kCompThreads) cr_compress_kernel(CRArgs<T> A) {
+constexpr int stage_stride() { return 4 * kCB * (int)sizeof(T) + 16; }   // bytes of a thread's four rows, padded
+
+template <typename T, bool kStaged>
+__global__ void __launch_bounds__(kCompThreads, sizeof(T) == 4 ? 4 : 2) cr_compress_kernel(CRArgs<T> A) {
+  extern __shared__ __align__(16) unsigned char stage[];   // two buffers of kCompThreads x stage_stride
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t item = (int64_t)blockIdx.x * kCompThreads + threadIdx.x;
-  if (item >= A.total_blocks * A.splits) return;
-  const int64_t gb = A.splits == 1 ? item : item / A.splits;
-  const int s = (int)(item - gb * A.splits);
+  const bool have = item < A.num_items;   // threads past the end only help with the copies
+  const int64_t gb = !have ? 0 : (A.item_blk ? A.item_blk[item] : item);
+  const int s = have && A.item_blk ? (int)(item - A.blk_item0[gb]) : 0;
+  const int splits = A.item_blk ? A.blk_item0[gb + 1] - A.blk_item0[gb] : 1;
   const int64_t k = A.binst[gb];
   const int64_t g = gb - A.blk0[k];
   const int64_t N = A.cols[k], c0 = A.col0[k], row0 = A.row0[k];
   int64_t lo, hi;
   group_rows(A, k, g, gb, lo, hi);
-  const int64_t len = hi - lo;
-  int64_t r = lo + len * s / A.splits;
-  const int64_t r_end = lo + len * (s + 1) / A.splits;
+  const int64_t len = have ? hi - lo : 0;
+  int64_t r = lo + len * s / splits;
+  const int64_t r_end = lo + len * (s + 1) / splits;
   Window<T> W;
 #pragma unroll
   for (int e = 0; e < 36; ++e) W.t[e] = T(0);
@@ -303,46 +357,87 @@ __global__ void __launch_bounds__(kCompThreads) cr_compress_kernel(CRArgs<T> A) 
       W.t[tri(i, i)] = col >= N ? T(1) : (A.lam > 0.0 ? (T)(lam_half * A.D[c0 + col]) : T(0));
     }
   }
-  T* dst = A.splits == 1 ? A.F0 + gb * kFW : A.P + item * kE0;
-  // whole rows by 16-byte loads where they are aligned; else entry by entry
-  const bool wide = A.w == kCB && (reinterpret_cast<uintptr_t>(A.J) & 15) == 0;
+  T* dst = splits == 1 ? A.E0 : A.P;
+  const int64_t at = splits == 1 ? gb : item;
+  constexpr int kLanes = 2 * (int)sizeof(T);   // 16-byte pieces of four rows
+  auto fetch = [&](int buf) {   // the warp's threads' rows r .. r + 3 (those before r_end) into buffer buf
+    unsigned char* base = stage + (buf * kCompThreads + warp * 32) * stage_stride<T>();
+    const int avail = (int)max((int64_t)0, min((int64_t)4, r_end - r));
+#pragma unroll
+    for (int i = 0; i < kLanes; ++i) {
+      const int q = i * (32 / kLanes) + lane / kLanes;   // the thread whose rows these are
+      const int64_t rq = __shfl_sync(0xffffffffu, r, q);
+      const int nq = __shfl_sync(0xffffffffu, avail, q);
+      const int o = (lane % kLanes) * 16;
+      if (o < nq * kCB * (int)sizeof(T))
+        dev::cp_async16(base + q * stage_stride<T>() + o, reinterpret_cast<const unsigned char*>(A.J + rq * kCB) + o);
+    }
+    dev::cp_async_commit();
+  };
+  int buf = 0;
+  if constexpr (kStaged) fetch(0);
   ResidualSum<T> res;
   // One step per turn: the next (up to four) rows starting at column c, or, when there are none, the window
   // one column on.  The threads of a warp may be at different columns.
   int64_t ahead[4];   // explicit starts of the next four rows, fetched one step early
 #pragma unroll
   for (int q = 0; q < 4; ++q) ahead[q] = A.starts && r + q < r_end ? A.starts[r + q] - c0 : -1;
+  int c = have ? 0 : kCB;
 #pragma unroll 1
-  for (int c = 0; c < kCB;) {
+  while (__any_sync(0xffffffffu, c < kCB)) {
     const int64_t st = (int64_t)kCB * g + c;   // the rows' first column
     int cnt = 0;
-    if (A.starts) {
+    if (c < kCB) {
+      if (A.starts) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (cnt == q && ahead[q] == st) cnt = q + 1;
-    } else {
-      cnt = (int)max((int64_t)0, min((int64_t)4, min(r_end, row0 + (st + 1) * A.rpc) - r));
+        for (int q = 0; q < 4; ++q)
+          if (cnt == q && ahead[q] == st) cnt = q + 1;
+      } else {
+        cnt = (int)max((int64_t)0, min((int64_t)4, min(r_end, row0 + (st + 1) * A.rpc) - r));
+      }
     }
+    T a[4][8], b[4];
     if (cnt > 0) {
-      T a[4][8], b[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        b[q] = T(0);
+      for (int q = 0; q < 4; ++q) b[q] = q < cnt ? A.b[r + q] : T(0);
+    }
+    if constexpr (kStaged) {
+      dev::cp_async_wait_all();
+      __syncwarp();
+      const T* mine = reinterpret_cast<const T*>(stage + (buf * kCompThreads + threadIdx.x) * stage_stride<T>());
+      if (cnt > 0) {
+        const int nt = (int)min((int64_t)kCB, N - st);   // entries past the last column are ignored
 #pragma unroll
-        for (int t = 0; t < 8; ++t) a[q][t] = T(0);
-        if (q < cnt) {
-          const T* src = A.J + (r + q) * A.w;
-          b[q] = A.b[r + q];
-          if (wide && st + kCB <= N) {
-            load8(a[q], src);
-          } else {
+        for (int q = 0; q < 4; ++q) {
 #pragma unroll
-            for (int t = 0; t < 8; ++t)
-              if (t < A.w && st + t < N) a[q][t] = src[t];
+          for (int t = 0; t < 8; ++t) a[q][t] = T(0);
+          if (q < cnt) {
+            load8(a[q], mine + kCB * q);
+            if (nt < kCB) {
+#pragma unroll
+              for (int t = 0; t < 8; ++t)
+                if (t >= nt) a[q][t] = T(0);
+            }
           }
         }
       }
-      r += cnt;
+    } else if (cnt > 0) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+#pragma unroll
+        for (int t = 0; t < 8; ++t) a[q][t] = q < cnt && t < A.w && st + t < N ? A.J[(r + q) * A.w + t] : T(0);
+      }
+    }
+    r += cnt;
+    if constexpr (kStaged) {
+      // a turn of shifts only leaves every buffer as it is; otherwise all threads fetch, those that did
+      // not move the same rows again
+      if (__any_sync(0xffffffffu, cnt > 0)) {
+        buf ^= 1;
+        fetch(buf);
+      }
+    }
+    if (cnt > 0) {
       if (A.starts) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) ahead[q] = r + q < r_end ? A.starts[r + q] - c0 : -1;
@@ -350,41 +445,48 @@ __global__ void __launch_bounds__(kCompThreads) cr_compress_kernel(CRArgs<T> A) 
       W.insert(a, b);
 #pragma unroll
       for (int q = 0; q < 4; ++q) res.square(b[q]);
-    } else {
+    } else if (c < kCB) {
       T row[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) row[j] = W.t[tri(0, j)];
-      store8(dst + 8 * c, row);
-      dst[128 + c] = W.z[0];
+      store_e0(dst, at, 8 * c, row);
+      dst[e0_at<T>(at, 128 + c)] = W.z[0];
       W.shift();
       ++c;
     }
   }
-  if (r < r_end) cr_record(A.status, QRKIT_EINVAL);   // rows out of order or past the block
+  if constexpr (kStaged) dev::cp_async_wait_all();
+  if (have) {
+    if (r < r_end) cr_record(A.status, QRKIT_EINVAL);   // rows out of order or past the block
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    T row[8];
+    for (int i = 0; i < 8; ++i) {
+      T row[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) row[j] = j >= i ? W.t[tri(i, j)] : T(0);
-    store8(dst + 64 + 8 * i, row);
+      for (int j = 0; j < 8; ++j) row[j] = j >= i ? W.t[tri(i, j)] : T(0);
+      store_e0(dst, at, 64 + 8 * i, row);
+    }
+    store_e0(dst, at, 136, W.z);
   }
-  store8(dst + 136, W.z);
   res.flush(A.res2, k);
 }
 
-// 1b. merge of kMergeFan partial triangles of a block into one, by the same window; 16 columns.
+// 1b. merge of up to kMergeFan partial triangles of a block into one, by the same window; 16 columns.
 constexpr int kMergeFan = 4;
 
+struct MergeItem {
+  int32_t blk, first, n;   // block; its partials first .. first + n - 1 of the input
+  int32_t out;             // partial of the output, or -1: the block's compressed row
+};
+
 template <typename T>
-__global__ void __launch_bounds__(kCompThreads) cr_merge_kernel(CRArgs<T> A, const T* in, int nin, T* out, int nout,
-                                                                int64_t out_stride) {
-  const int64_t item = (int64_t)blockIdx.x * kCompThreads + threadIdx.x;
-  if (item >= A.total_blocks * nout) return;
-  const int64_t gb = item / nout;
-  const int s = (int)(item - gb * nout);
-  const int n = min(kMergeFan, nin - s * kMergeFan);
-  const T* src = in + (gb * nin + s * kMergeFan) * kE0;
-  T* dst = out + item * out_stride;
+__global__ void __launch_bounds__(kCompThreads) cr_merge_kernel(CRArgs<T> A, const MergeItem* items, int64_t nitems,
+                                                                const T* in, T* part) {
+  const int64_t w = (int64_t)blockIdx.x * kCompThreads + threadIdx.x;
+  if (w >= nitems) return;
+  const MergeItem M = items[w];
+  const int n = M.n;
+  const int64_t first = M.first, gb = M.blk, item = M.out < 0 ? gb : M.out;
+  T* out = M.out < 0 ? A.E0 : part;
   Window<T> W;
 #pragma unroll
   for (int e = 0; e < 36; ++e) W.t[e] = T(0);
@@ -400,14 +502,13 @@ __global__ void __launch_bounds__(kCompThreads) cr_merge_kernel(CRArgs<T> A, con
 #pragma unroll
       for (int t = 0; t < 8; ++t) a[q][t] = T(0);
       if (q < n) {
-        const T* E = src + q * kE0;
-        b[q] = E[128 + c];
+        b[q] = in[e0_at<T>(first + q, 128 + c)];
         if (c < 8) {
-          load8(a[q], E + 8 * c);
+          load_e0(a[q], in, first + q, 8 * c);
         } else {   // row c - 8 of the second triangle: columns c ..
 #pragma unroll
           for (int t = 0; t < 8; ++t)
-            if (c + t < 16) a[q][t] = E[64 + 8 * (c - 8) + (c - 8) + t];
+            if (c + t < 16) a[q][t] = in[e0_at<T>(first + q, 64 + 9 * (c - 8) + t)];
         }
       }
     }
@@ -418,15 +519,15 @@ __global__ void __launch_bounds__(kCompThreads) cr_merge_kernel(CRArgs<T> A, con
       T row[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) row[j] = W.t[tri(0, j)];
-      store8(dst + 8 * c, row);
+      store_e0(out, item, 8 * c, row);
     } else {
-      T* d = dst + 64 + 8 * (c - 8);
-      for (int j = 0; j < c - 8; ++j) d[j] = T(0);
+      const int d = 64 + 8 * (c - 8);
+      for (int j = 0; j < c - 8; ++j) out[e0_at<T>(item, d + j)] = T(0);
 #pragma unroll
       for (int j = 0; j < 8; ++j)
-        if (c + j < 16) d[c - 8 + j] = W.t[tri(0, j)];
+        if (c + j < 16) out[e0_at<T>(item, d + c - 8 + j)] = W.t[tri(0, j)];
     }
-    dst[128 + c] = W.z[0];
+    out[e0_at<T>(item, 128 + c)] = W.z[0];
     W.shift();
   }
   res.flush(A.res2, A.binst[gb]);
@@ -453,21 +554,22 @@ __device__ __forceinline__ void decode(int64_t it, int64_t& k, int64_t& i, int& 
 // its sums reduced by shuffles took 4,000.
 constexpr int kItemThreads = kCB;
 
-// A block row's columns j of A (rows 0..7) and B (rows 0..7, 8..15) and its rhs.
+// Columns j of A (rows 0..7) and B (rows 0..7, 8..15) of block row `it`, and its rhs.
 template <typename T, bool kCompressed>
-__device__ __forceinline__ void load_block_row(const T* F, int j, T (&a)[8], T (&bl)[8], T (&bh)[8], T (&cl)[8],
-                                               T (&ch)[8]) {
+__device__ __forceinline__ void load_block_row(const T* base, int64_t it, int j, T (&a)[8], T (&bl)[8], T (&bh)[8],
+                                               T (&cl)[8], T (&ch)[8]) {
   if constexpr (kCompressed) {
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
-      const T v = F[8 * r + ((j - r) & 7)];   // column j of A for j >= r, of B for j < r
+      const T v = base[e0_at<T>(it, 8 * r + ((j - r) & 7))];   // column j of A for j >= r, of B for j < r
       a[r] = j >= r ? v : T(0);
       bl[r] = j < r ? v : T(0);
-      bh[r] = F[64 + 8 * r + j];
+      bh[r] = base[e0_at<T>(it, 64 + 8 * r + j)];
     }
-    load8(cl, F + 128);
-    load8(ch, F + 136);
+    load_e0(cl, base, it, 128);
+    load_e0(ch, base, it, 136);
   } else {
+    const T* F = base + it * kFW;
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
       a[r] = F[8 * r + j];
@@ -521,7 +623,7 @@ __device__ __forceinline__ void cr_item(const CRArgs<T>& A, int64_t k, int64_t i
                                         T* Fn, int j, unsigned gmask, ResidualSum<T>& res) {
   const int64_t b0 = A.blk0[k];
   T a[8], bl[8], bh[8], cl[8], ch[8];
-  load_block_row<T, kCompressed>(Fc + (b0 + i) * kFW, j, a, bl, bh, cl, ch);
+  load_block_row<T, kCompressed>(Fc, b0 + i, j, a, bl, bh, cl, ch);
   if (kind == 1) {   // unpaired last block row: moves up
     store_block_row(Fn + (b0 + i / 2) * kFW, j, a, bl, bh, cl, ch);
     return;
@@ -532,7 +634,7 @@ __device__ __forceinline__ void cr_item(const CRArgs<T>& A, int64_t k, int64_t i
   for (int r = 0; r < 8; ++r) rl[r] = T(0);
   if (kind == 0) {
     T pa[8], pl[8], ph[8], dl[8], dh[8], rr[8], lr[8];
-    load_block_row<T, kCompressed>(Fc + (b0 + i - 1) * kFW, j, pa, pl, ph, dl, dh);
+    load_block_row<T, kCompressed>(Fc, b0 + i - 1, j, pa, pl, ph, dl, dh);
 #pragma unroll
     for (int r = 0; r < 8; ++r) rr[r] = lr[r] = T(0);   // right parts of the rows of B'
     T v[8], x[8];
@@ -841,7 +943,7 @@ __global__ void __launch_bounds__(tail_threads<T>(), 1) cr_tail_kernel(CRArgs<T>
   int l = lt;
   for (;; ++l) {
     const int64_t Gl = blocks_at(G, l);
-    const T* Fc = (l & 1) ? A.F1 : A.F0;
+    const T* Fc = l == 0 ? A.E0 : ((l & 1) ? A.F1 : A.F0);
     T* Fn = (l & 1) ? A.F0 : A.F1;
     // item m: odd block 2 m + 1, or the unpaired last block (kind 1), or the only one (kind 2)
     const int64_t n = Gl == 1 ? 1 : (Gl + 1) / 2;
@@ -906,10 +1008,13 @@ inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 struct CRPlan {
   int64_t num_inst = 0, total_blocks = 0;
-  int splits = 1, levels = 0;              // levels: those run by launches of their own, before the tails
+  int levels = 0;                          // those run by launches of their own, before the tails
+  int64_t num_items = 0;                   // threads of the compression
+  std::vector<int64_t> h_blk0, h_rows;     // kept for the compression's strategy
+  std::vector<int64_t> mg_off, mg_n;       // merge items per pass
   std::vector<int64_t> lvl_off, lvl_n;     // eliminate / move items per level
   std::vector<int64_t> ev_off, ev_n;       // staying (even) blocks per level
-  DevBuf tabs, items, evens, binst, grp_lo, P, P2, F0, F1, Rb, xp, hp;
+  DevBuf tabs, items, evens, binst, item_blk, blk_item0, merges, grp_lo, P, P2, E0, F0, F1, Rb, xp, hp;
   const int64_t* d_cols = nullptr;
   const int64_t* d_col0 = nullptr;
   const int64_t* d_row0 = nullptr;
@@ -920,21 +1025,69 @@ struct CRPlan {
 
 void release_cr(CRPlan*& p) {
   if (!p) return;
-  for (DevBuf* b : {&p->tabs, &p->items, &p->evens, &p->binst, &p->grp_lo, &p->P, &p->P2, &p->F0, &p->F1, &p->Rb,
+  for (DevBuf* b : {&p->tabs, &p->items, &p->evens, &p->binst, &p->item_blk, &p->blk_item0, &p->merges, &p->grp_lo, &p->P, &p->P2, &p->E0, &p->F0, &p->F1, &p->Rb,
                     &p->xp, &p->hp})
     release(*b);
   delete p;
   p = nullptr;
 }
 
-// Partial triangles of `splits` threads per block, and of the merge's first pass.
-static qrkit_status cr_partials(qrkit_ctx* ctx, CRPlan& C) {
-  if (C.splits == 1) return QRKIT_OK;
+static qrkit_status upload(qrkit_ctx* ctx, DevBuf& d, const void* h, size_t bytes, const char* what) {
+  qrkit_status r = ensure(ctx, d, std::max<size_t>(bytes, 8), what);
+  if (r != QRKIT_OK) return r;
+  if (bytes > 0) QRKIT_CUDA_TRY(ctx, cudaMemcpy(d.ptr, h, bytes, cudaMemcpyHostToDevice));
+  return QRKIT_OK;
+}
+
+// The compression's threads: splits[k] per block of instance k, and the merges of their triangles.
+static qrkit_status cr_split(qrkit_ctx* ctx, CRPlan& C, const std::vector<int>& splits) {
+  C.num_items = 0;
+  C.mg_off.clear();
+  C.mg_n.clear();
+  for (int64_t k = 0; k < C.num_inst; ++k) C.num_items += (C.h_blk0[k + 1] - C.h_blk0[k]) * splits[k];
+  if (C.num_items >= ((int64_t)1 << 31)) return fail(ctx, QRKIT_EUNSUPPORTED, "too many column blocks");
+  if (C.num_items == C.total_blocks) return QRKIT_OK;   // one thread per block
+  std::vector<int32_t> item_blk((size_t)C.num_items), item0((size_t)C.total_blocks + 1);
+  std::vector<int32_t> first((size_t)C.total_blocks), n((size_t)C.total_blocks);   // a block's partials at this pass
+  int64_t it = 0;
+  for (int64_t k = 0; k < C.num_inst; ++k)
+    for (int64_t gb = C.h_blk0[k]; gb < C.h_blk0[k + 1]; ++gb) {
+      item0[gb] = first[gb] = (int32_t)it;
+      n[gb] = splits[k];
+      for (int q = 0; q < splits[k]; ++q) item_blk[it++] = (int32_t)gb;
+    }
+  item0[C.total_blocks] = (int32_t)it;
+  std::vector<MergeItem> mg;
+  int64_t parts2 = 0;
+  for (bool more = true; more;) {
+    more = false;
+    C.mg_off.push_back((int64_t)mg.size());
+    int64_t out = 0;
+    for (int64_t gb = 0; gb < C.total_blocks; ++gb) {
+      if (n[gb] <= 1) continue;
+      const int m = (n[gb] + kMergeFan - 1) / kMergeFan;
+      for (int q = 0; q < m; ++q)
+        mg.push_back({(int32_t)gb, first[gb] + q * kMergeFan, std::min(kMergeFan, n[gb] - q * kMergeFan),
+                      m == 1 ? -1 : (int32_t)(out + q)});
+      first[gb] = (int32_t)out;
+      n[gb] = m;
+      if (m > 1) {
+        out += m;
+        more = true;
+      }
+    }
+    parts2 = std::max(parts2, out);
+    C.mg_n.push_back((int64_t)mg.size() - C.mg_off.back());
+  }
   const size_t es = elem_size(ctx);
-  const int next = (C.splits + kMergeFan - 1) / kMergeFan;
-  qrkit_status rc = ensure(ctx, C.P, (size_t)C.total_blocks * C.splits * kE0 * es, "banded partial triangles");
-  if (rc == QRKIT_OK && next > 1)
-    rc = ensure(ctx, C.P2, (size_t)C.total_blocks * next * kE0 * es, "banded partial triangles");
+  qrkit_status rc;
+  if ((rc = upload(ctx, C.item_blk, item_blk.data(), item_blk.size() * 4, "banded splits")) != QRKIT_OK) return rc;
+  if ((rc = upload(ctx, C.blk_item0, item0.data(), item0.size() * 4, "banded splits")) != QRKIT_OK) return rc;
+  if ((rc = upload(ctx, C.merges, mg.data(), mg.size() * sizeof(MergeItem), "banded merges")) != QRKIT_OK) return rc;
+  if ((rc = ensure(ctx, C.P, ((size_t)C.num_items + 31) / 32 * 32 * kE0 * es, "banded partial triangles")) != QRKIT_OK)
+    return rc;
+  if (parts2 > 0)
+    rc = ensure(ctx, C.P2, ((size_t)parts2 + 31) / 32 * 32 * kE0 * es, "banded partial triangles");
   return rc;
 }
 
@@ -955,11 +1108,8 @@ qrkit_status cr_build(qrkit_ctx* ctx, CRPlan*& out, const std::vector<int64_t>& 
   }
   C.total_blocks = blk0[ni];
   if (C.total_blocks >= ((int64_t)1 << 30)) return fail(ctx, QRKIT_EUNSUPPORTED, "too many column blocks");
-  // Threads per block: four times as many while the GPU is not full (about 100,000 threads) and the rows
-  // that a split saves (at four per step) outweigh the 16 steps of a merge.
-  const double per = C.total_blocks ? (double)total_rows / (double)C.total_blocks : 0.0;
-  C.splits = 1;
-  while (C.splits < 64 && C.total_blocks * C.splits < 100000 && per / C.splits > 85.0) C.splits *= kMergeFan;
+  C.h_blk0 = blk0;
+  C.h_rows = rows;
   // level work lists; an instance's levels with at most kTailBlocks blocks belong to its tail
   std::vector<std::vector<int64_t>> lv, ev;
   std::vector<int64_t> tail0(ni);
@@ -994,17 +1144,11 @@ qrkit_status cr_build(qrkit_ctx* ctx, CRPlan*& out, const std::vector<int64_t>& 
   tabs.insert(tabs.end(), tail0.begin(), tail0.end());
   std::vector<int32_t> binst((size_t)C.total_blocks);
   for (int64_t k = 0; k < ni; ++k) std::fill(binst.begin() + blk0[k], binst.begin() + blk0[k + 1], (int32_t)k);
-  auto up = [&](DevBuf& d, const void* h, size_t bytes, const char* what) -> qrkit_status {
-    qrkit_status r = ensure(ctx, d, std::max<size_t>(bytes, 8), what);
-    if (r != QRKIT_OK) return r;
-    if (bytes > 0) QRKIT_CUDA_TRY(ctx, cudaMemcpy(d.ptr, h, bytes, cudaMemcpyHostToDevice));
-    return QRKIT_OK;
-  };
   qrkit_status rc;
-  if ((rc = up(C.tabs, tabs.data(), tabs.size() * sizeof(int64_t), "banded tables")) != QRKIT_OK) return rc;
-  if ((rc = up(C.items, items.data(), items.size() * sizeof(int64_t), "banded levels")) != QRKIT_OK) return rc;
-  if ((rc = up(C.evens, evens.data(), evens.size() * sizeof(int64_t), "banded levels")) != QRKIT_OK) return rc;
-  if ((rc = up(C.binst, binst.data(), binst.size() * sizeof(int32_t), "banded blocks")) != QRKIT_OK) return rc;
+  if ((rc = upload(ctx, C.tabs, tabs.data(), tabs.size() * sizeof(int64_t), "banded tables")) != QRKIT_OK) return rc;
+  if ((rc = upload(ctx, C.items, items.data(), items.size() * sizeof(int64_t), "banded levels")) != QRKIT_OK) return rc;
+  if ((rc = upload(ctx, C.evens, evens.data(), evens.size() * sizeof(int64_t), "banded levels")) != QRKIT_OK) return rc;
+  if ((rc = upload(ctx, C.binst, binst.data(), binst.size() * sizeof(int32_t), "banded blocks")) != QRKIT_OK) return rc;
   const int64_t* t = (const int64_t*)C.tabs.ptr;
   C.d_cols = t;
   C.d_col0 = t + ni;
@@ -1015,7 +1159,19 @@ qrkit_status cr_build(qrkit_ctx* ctx, CRPlan*& out, const std::vector<int64_t>& 
   const size_t es = elem_size(ctx);
   const size_t TB = (size_t)C.total_blocks;
   if ((rc = ensure(ctx, C.grp_lo, TB * sizeof(int64_t), "banded group rows")) != QRKIT_OK) return rc;
-  if ((rc = cr_partials(ctx, C)) != QRKIT_OK) return rc;
+  // Threads per block of an instance: about 120,000 in all where that leaves each at least 64 rows (16 steps of
+  // four, what a merge pass takes), at most 64 per block.  A batch's instances differ in rows per block
+  // (curve fits: 60 to 10,000), and the longest thread bounds the kernel.
+  {
+    const double target = std::max(64.0, (double)total_rows / 120000.0);
+    std::vector<int> splits(ni);
+    for (int64_t k = 0; k < ni; ++k) {
+      const double per = (double)rows[k] / (double)(blk0[k + 1] - blk0[k]);
+      splits[k] = (int)std::min(64.0, std::max(1.0, std::floor(per / target + 0.5)));
+    }
+    if ((rc = cr_split(ctx, C, splits)) != QRKIT_OK) return rc;
+  }
+  if ((rc = ensure(ctx, C.E0, (TB + 31) / 32 * 32 * kE0 * es, "banded block rows")) != QRKIT_OK) return rc;
   if ((rc = ensure(ctx, C.F0, TB * kFW * es, "banded block rows")) != QRKIT_OK) return rc;
   if ((rc = ensure(ctx, C.F1, TB * kFW * es, "banded block rows")) != QRKIT_OK) return rc;
   if ((rc = ensure(ctx, C.Rb, TB * kRW * es, "banded R blocks")) != QRKIT_OK) return rc;
@@ -1026,8 +1182,7 @@ qrkit_status cr_build(qrkit_ctx* ctx, CRPlan*& out, const std::vector<int64_t>& 
 
 qrkit_status cr_set_strategy(qrkit_ctx* ctx, CRPlan& C, bool thread_rows, int splits) {
   if (splits < 1 || splits > 64) return fail(ctx, QRKIT_EINVAL, "splits must be in [1, 64]");
-  C.splits = thread_rows ? 1 : splits;
-  return cr_partials(ctx, C);
+  return cr_split(ctx, C, std::vector<int>((size_t)C.num_inst, thread_rows ? 1 : splits));
 }
 
 template <typename T>
@@ -1042,9 +1197,13 @@ static CRArgs<T> cr_args(qrkit_ctx* ctx, CRPlan& C) {
   A.tail0 = C.d_tail0;
   A.binst = (const int32_t*)C.binst.ptr;
   A.total_blocks = C.total_blocks;
-  A.splits = C.splits;
+  A.num_items = C.num_items;
+  const bool split = C.num_items != C.total_blocks;
+  A.item_blk = split ? (const int32_t*)C.item_blk.ptr : nullptr;
+  A.blk_item0 = split ? (const int32_t*)C.blk_item0.ptr : nullptr;
   A.grp_lo = (int64_t*)C.grp_lo.ptr;
   A.P = (T*)C.P.ptr;
+  A.E0 = (T*)C.E0.ptr;
   A.F0 = (T*)C.F0.ptr;
   A.F1 = (T*)C.F1.ptr;
   A.Rb = (T*)C.Rb.ptr;
@@ -1076,19 +1235,26 @@ static qrkit_status cr_solve_typed(qrkit_ctx* ctx, CRPlan& C, const int64_t* sta
   A.res2 = res2;
   QRKIT_CUDA_TRY(ctx, cudaMemsetAsync(res2, 0, (size_t)C.num_inst * sizeof(double), st));
   if (starts) CR_LAUNCH(ctx, cr_ranges_kernel<T><<<nblk(C.total_blocks, 256), 256, 0, st>>>(A));
-  CR_LAUNCH(ctx, cr_compress_kernel<T><<<nblk(C.total_blocks * C.splits, kCompThreads), kCompThreads, 0, st>>>(A));
+  const unsigned cgrid = nblk(C.num_items, kCompThreads);
+  if (w == kCB && (reinterpret_cast<uintptr_t>(J) & 15) == 0) {
+    const size_t smem = 2 * (size_t)kCompThreads * stage_stride<T>();
+    auto kc = cr_compress_kernel<T, true>;
+    if (smem > 48 * 1024)
+      QRKIT_CUDA_TRY(ctx, cudaFuncSetAttribute(kc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CR_LAUNCH(ctx, kc<<<cgrid, kCompThreads, smem, st>>>(A));
+  } else {
+    CR_LAUNCH(ctx, (cr_compress_kernel<T, false><<<cgrid, kCompThreads, 0, st>>>(A)));
+  }
   T* in = A.P;
   T* other = (T*)C.P2.ptr;
-  for (int n = C.splits; n > 1;) {
-    const int m = (n + kMergeFan - 1) / kMergeFan;
-    CR_LAUNCH(ctx, cr_merge_kernel<T><<<nblk(C.total_blocks * m, kCompThreads), kCompThreads, 0, st>>>(
-                       A, in, n, m == 1 ? A.F0 : other, m, m == 1 ? kFW : kE0));
+  for (size_t q = 0; q < C.mg_n.size(); ++q) {
+    CR_LAUNCH(ctx, cr_merge_kernel<T><<<nblk(C.mg_n[q], kCompThreads), kCompThreads, 0, st>>>(
+                       A, (const MergeItem*)C.merges.ptr + C.mg_off[q], C.mg_n[q], in, other));
     std::swap(in, other);
-    n = m;
   }
   const int64_t* items = (const int64_t*)C.items.ptr;
   for (int l = 0; l < C.levels; ++l) {
-    const T* Fc = (l & 1) ? A.F1 : A.F0;
+    const T* Fc = l == 0 ? A.E0 : ((l & 1) ? A.F1 : A.F0);
     T* Fn = (l & 1) ? A.F0 : A.F1;
     const unsigned grid = nblk(C.lvl_n[l] * kItemThreads, kLevelThreads);
     if (l == 0)

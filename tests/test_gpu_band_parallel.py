@@ -55,3 +55,12 @@ def test_split_compression_matches_oracle(splits):
     x, _, r2 = oracle_solutions(inst, 1e-2)
     np.testing.assert_allclose(p, x, rtol=1e-11, atol=1e-11 * np.abs(x).max())
     np.testing.assert_allclose(res2, r2, rtol=1e-9)
+
+
+def test_many_instances_of_mixed_depth():
+    """Instances whose compressed block rows share lines with instances that are levels ahead of them."""
+    g = np.random.default_rng(4)
+    cols = list(g.integers(1, 40, size=300)) + [1100, 2100, 5, 1030] + list(g.integers(200, 900, size=40))
+    p, _, inst = solve(cols, 4, 8, "fp32_refined", 1e-3)
+    x, _, _ = oracle_solutions(inst, 1e-3)
+    assert_close(p, x, 1e-6)
