@@ -929,7 +929,7 @@ static qrkit_status banded_run(qrkit_ctx* ctx, const void* J, const void* b, con
     const int64_t* inst = (const int64_t*)B.d_inst.ptr;
     qrkit_status rc;
     if (B.parallel) {
-      rc = cr_solve(ctx, *B.cr, gs, 1, B.w, J, b, D, lambda, p, (double*)B.res2.ptr);
+      rc = cr_solve(ctx, *B.cr, gs, nullptr, 1, B.w, J, b, D, lambda, p, (double*)B.res2.ptr);
     } else {
       rc = banded_explicit_solve(ctx, B.num_inst, inst, J, gs, b, B.w, D, lambda, B.Rw.ptr, B.c.ptr, p,
                                  (double*)B.res2.ptr);
@@ -958,7 +958,7 @@ static qrkit_status banded_run(qrkit_ctx* ctx, const void* J, const void* b, con
     return QRKIT_OK;
   }
   if (B.parallel) {
-    qrkit_status rc = cr_solve(ctx, *B.cr, nullptr, B.rows_per_col, B.w, J, b, D, lambda, p,
+    qrkit_status rc = cr_solve(ctx, *B.cr, nullptr, nullptr, B.rows_per_col, B.w, J, b, D, lambda, p,
                                (double*)B.res2.ptr);
     if (rc != QRKIT_OK) return rc;
     for (int it = 0; it < refine_steps; ++it) {

@@ -207,7 +207,7 @@ __device__ __forceinline__ void block_factor_small(const ComposedView<T>& V, con
   for (int k = 0; k < MM; ++k)
     if (k < m) O.tau[V.col_off[i] + k] = tau[k];
   if (V.coupled != QRKIT_COUPLED_WINDOW) return;   // a dense S: dense_block.cu
-  const int64_t red0 = O.red_off[i];
+  const int64_t red0 = O.bpos ? (int64_t)O.bpos[i] * O.q : O.red_off[i];
   if constexpr (sizeof(T) == 4 && NA == 3 && MM == 1) {
     // the 2 x 1 point blocks of curve fits with windows of 8 (damped): the window, R12 and
     // the two reduced rows are moved by 16-byte loads and stores (all 32-byte aligned)
@@ -242,8 +242,7 @@ __device__ __forceinline__ void block_factor_small(const ComposedView<T>& V, con
       dx[1] = make_float4(x1[4], x1[5], x1[6], x1[7]);
       dx[2] = make_float4(x2[0], x2[1], x2[2], x2[3]);
       dx[3] = make_float4(x2[4], x2[5], x2[6], x2[7]);
-      O.Xstart[red0] = V.start[i];
-      O.Xstart[red0 + 1] = V.start[i];
+      if (O.Xstart) O.Xstart[red0] = O.Xstart[red0 + 1] = V.start[i];
       return;
     }
   }
@@ -285,7 +284,7 @@ __device__ __forceinline__ void block_factor_small(const ComposedView<T>& V, con
           } else if (r < na) {
             const int64_t row = red0 + (r - m);
             O.Xw[row * V.w + c0 + c] = C[c][r];
-            if (c0 + c == 0) O.Xstart[row] = V.start[i];
+            if (c0 + c == 0 && O.Xstart) O.Xstart[row] = V.start[i];
           }
         }
       }
@@ -350,7 +349,7 @@ __global__ void block_factor_kernel(ComposedView<T> V, FactorOut<T> O) {
   for (int k = 0; k < m; ++k) O.tau[V.col_off[i] + k] = tau[k];
   // coupled columns, kChunk at a time
   if (V.coupled != QRKIT_COUPLED_WINDOW) return;   // a dense S: dense_block.cu
-  const int64_t red0 = O.red_off[i];
+  const int64_t red0 = O.bpos ? (int64_t)O.bpos[i] * O.q : O.red_off[i];
   for (int c0 = 0; c0 < V.w; c0 += kChunk) {
     const int cw = min(kChunk, V.w - c0);
     T C[kMaxRows * kChunk];
@@ -374,7 +373,7 @@ __global__ void block_factor_kernel(ComposedView<T> V, FactorOut<T> O) {
       for (int r = m; r < na; ++r) {
         const int64_t row = red0 + (r - m);
         O.Xw[row * V.w + c0 + c] = C[c * na + r];
-        if (c0 + c == 0) O.Xstart[row] = V.start[i];
+        if (c0 + c == 0 && O.Xstart) O.Xstart[row] = V.start[i];
       }
     }
   }
@@ -515,6 +514,7 @@ __global__ void block_apply_qt_kernel(ComposedView<T> V, FactorOut<T> O, const T
 #pragma unroll
     for (int r = 0; r < NA; ++r) y[r] = r < n ? b[V.row_off[i] + r] : T(0);
     const T* F = O.Fa + O.aug_off[i];
+    const int64_t red0 = O.bpos ? (int64_t)O.bpos[i] * O.q : O.red_off[i];
 #pragma unroll
     for (int k = 0; k < MM; ++k) {
       if (k < m) {
@@ -532,7 +532,7 @@ __global__ void block_apply_qt_kernel(ComposedView<T> V, FactorOut<T> O, const T
 #pragma unroll
     for (int r = 0; r < NA; ++r) {
       if (r < m) O.ctop[V.col_off[i] + r] = y[r];
-      else if (rhs0 && r < na) rhs0[O.red_off[i] + (r - m)] = y[r];
+      else if (rhs0 && r < na) rhs0[red0 + (r - m)] = y[r];
     }
     return;
   }
@@ -551,8 +551,9 @@ __global__ void block_apply_qt_kernel(ComposedView<T> V, FactorOut<T> O, const T
     for (int r = k + 1; r < na; ++r) y[r] -= w * x[r];
   }
   for (int r = 0; r < m; ++r) O.ctop[V.col_off[i] + r] = y[r];
+  const int64_t red0 = O.bpos ? (int64_t)O.bpos[i] * O.q : O.red_off[i];
   if (rhs0)
-    for (int r = m; r < na; ++r) rhs0[O.red_off[i] + (r - m)] = y[r];
+    for (int r = m; r < na; ++r) rhs0[red0 + (r - m)] = y[r];
 }
 
 // Per-block R_i x_i = rhs_i - R12_i x_S; rhs from ctop (T) or from a double vector.  NA > 0:
@@ -1099,8 +1100,10 @@ static FactorOut<T> fout(qrkit_ctx* ctx) {
   O.red_off = (const int64_t*)(C.damp ? C.d_red_off_d.ptr : C.d_red_off_u.ptr);
   O.X0 = C.levels.empty() ? nullptr : (T*)C.levels[0].X.ptr + reduced_head(ctx);
   O.ld0 = C.levels.empty() ? 0 : C.levels[0].ld;
-  O.Xw = (T*)C.Xw.ptr;
-  O.Xstart = (int64_t*)C.Xstart.ptr;
+  O.Xw = (T*)(C.bins ? C.Xw_s.ptr : C.Xw.ptr);
+  O.Xstart = C.bins ? nullptr : (int64_t*)C.Xstart.ptr;
+  O.bpos = C.bins ? (const int32_t*)C.bpos.ptr : nullptr;
+  O.q = C.bins ? (int)(C.red_rows / ctx->plan.K) : 0;
   O.status = ctx->d_status;
   return O;
 }
@@ -1139,9 +1142,29 @@ static qrkit_status launch_block_backsub(qrkit_ctx* ctx, const ComposedView<T>& 
   return QRKIT_OK;
 }
 
-// D = column norms of J (Sec. 5.2), zero -> 1, in double; C.sq is the scratch.
 template <typename T>
-static qrkit_status norms_typed(qrkit_ctx* ctx, const ComposedView<T>& V, double* D) {
+static WindowSums<T> window_sums(qrkit_ctx* ctx, const ComposedView<T>& V, double* out) {
+  const Composed& C = ctx->comp;
+  WindowSums<T> A{};
+  A.K = V.K;
+  A.n = ctx->plan.max_n;
+  A.m = ctx->plan.max_m;
+  A.w = V.w;
+  A.s = V.s;
+  A.bord = (const int32_t*)C.bord.ptr;
+  A.start = V.start;
+  A.S = V.S;
+  A.R12 = (const T*)C.R12.ptr;
+  A.r = (const T*)C.wres.ptr;
+  A.h = (const T*)C.h.ptr;
+  A.out = out;
+  return A;
+}
+
+// D = column norms of J (Sec. 5.2), zero -> 1, in double; C.sq is the scratch.  sorted: the plan's blocks have
+// been sorted by their window starts.
+template <typename T>
+static qrkit_status norms_typed(qrkit_ctx* ctx, const ComposedView<T>& V, double* D, bool sorted) {
   Plan& P = ctx->plan;
   Composed& C = ctx->comp;
   cudaStream_t st = ctx->stream;
@@ -1159,8 +1182,12 @@ static qrkit_status norms_typed(qrkit_ctx* ctx, const ComposedView<T>& V, double
     const dim3 grid((unsigned)nchunk, (unsigned)std::min<int64_t>(V.s, 65535));
     LAUNCH(ctx, colnorm_dense_part_kernel<T><<<grid, kNormThreads, 0, st>>>(V, sq + N, nchunk));
     LAUNCH(ctx, colnorm_dense_sum_kernel<<<blocks_for(V.s, 128), 128, 0, st>>>(sq + N, nchunk, V.s, sq + V.nb));
-  } else if (V.coupled == QRKIT_COUPLED_WINDOW)
+  } else if (V.coupled == QRKIT_COUPLED_WINDOW && sorted) {
+    const WindowSums<T> A = window_sums<T>(ctx, V, sq + V.nb);
+    if ((rc = window_square_sums<T>(ctx, A)) != QRKIT_OK) return rc;
+  } else if (V.coupled == QRKIT_COUPLED_WINDOW) {
     LAUNCH(ctx, colnorm_window_kernel<T><<<blocks_for(P.K, 128), 128, 0, st>>>(V, sq));
+  }
   LAUNCH(ctx, finalize_norms_kernel<<<blocks_for(N, 256), 256, 0, st>>>(sq, D, N));
   return QRKIT_OK;
 }
@@ -1201,7 +1228,7 @@ static qrkit_status factor_panels(qrkit_ctx* ctx, int s) {
 
 template <typename T>
 static qrkit_status factor_typed(qrkit_ctx* ctx, const void* J, const void* S, const void* Dext,
-                                 double lambda, bool dext_double = false) {
+                                 double lambda, bool dext_double = false, bool sorted = false) {
   Plan& P = ctx->plan;
   Composed& C = ctx->comp;
   cudaStream_t st = ctx->stream;
@@ -1214,6 +1241,7 @@ static qrkit_status factor_typed(qrkit_ctx* ctx, const void* J, const void* S, c
   C.lam_half = sqrt(lambda);
   if ((rc = composed_layout(ctx, sizeof(T))) != QRKIT_OK) return rc;
   ComposedView<T> V = view<T>(ctx, J, S);
+  if (!sorted && (rc = composed_sort_blocks(ctx, &sorted)) != QRKIT_OK) return rc;
   // D: caller's (copied to double) or column norms of J
   if (Dext) {
     if (sizeof(T) == sizeof(double) || dext_double) {
@@ -1223,7 +1251,7 @@ static qrkit_status factor_typed(qrkit_ctx* ctx, const void* J, const void* S, c
       rc = widen_to_double(ctx, (const float*)Dext, (double*)C.D.ptr, N);
       if (rc != QRKIT_OK) return rc;
     }
-  } else if ((rc = norms_typed<T>(ctx, V, (double*)C.D.ptr)) != QRKIT_OK) {
+  } else if ((rc = norms_typed<T>(ctx, V, (double*)C.D.ptr, sorted)) != QRKIT_OK) {
     return rc;
   }
   FactorOut<T> O = fout<T>(ctx);
@@ -1236,7 +1264,7 @@ static qrkit_status factor_typed(qrkit_ctx* ctx, const void* J, const void* S, c
   else
     LAUNCH(ctx, block_factor_kernel<T><<<blocks_for(P.K, 64), 64, 0, st>>>(V, O));
   if (V.coupled == QRKIT_COUPLED_DENSE && (rc = dense_apply_blocks<T>(ctx, V, O)) != QRKIT_OK) return rc;
-  if (V.coupled == QRKIT_COUPLED_WINDOW) {
+  if (V.coupled == QRKIT_COUPLED_WINDOW && !C.bins) {
     // P_r of the reduced block: its rows sorted by leading column per segment (Sec. 4.3)
     rc = reduced_row_sort(ctx, C.sort, (int64_t)P.seg_cols.size(), C.sort_hist_entries,
                           (const int64_t*)C.Xstart.ptr, C.Xw.ptr, V.w, (int*)C.hist.ptr,
@@ -1282,7 +1310,7 @@ static qrkit_status solve_typed(qrkit_ctx* ctx, const void* J, const void* S, co
   T* x = (T*)p;
   // Q^T [b; 0]
   T* rhs0 = (V.coupled == QRKIT_COUPLED_DENSE) ? (T*)C.levels[0].rhs.ptr + reduced_head(ctx)
-             : (V.coupled == QRKIT_COUPLED_WINDOW ? (T*)C.rhs_red.ptr : nullptr);
+             : (V.coupled == QRKIT_COUPLED_WINDOW ? (T*)(C.bins ? C.rhs_s.ptr : C.rhs_red.ptr) : nullptr);
   LAUNCH_SHAPED(ctx, small_class(P, O.damp), block_apply_qt_kernel, blocks_for(P.K, 64), 64, 0, st, V, O, (const T*)b,
                 rhs0);
   if (V.coupled == QRKIT_COUPLED_DENSE) {
@@ -1336,10 +1364,12 @@ static qrkit_status solve_typed(qrkit_ctx* ctx, const void* J, const void* S, co
   } else if (V.coupled == QRKIT_COUPLED_WINDOW) {
     // reduced banded block of every segment (Sec. 4.4), rows in P_r order, the shared
     // columns' damping rows interleaved
-    qrkit_status rc = reduced_rhs_sort(ctx, (const int64_t*)C.spos.ptr, C.rhs_red.ptr, C.rhs_s.ptr, C.red_rows);
+    qrkit_status rc = QRKIT_OK;
+    if (!C.bins) rc = reduced_rhs_sort(ctx, (const int64_t*)C.spos.ptr, C.rhs_red.ptr, C.rhs_s.ptr, C.red_rows);
     if (rc != QRKIT_OK) return rc;
     if (C.cr)
-      rc = cr_solve(ctx, *C.cr, (const int64_t*)C.Xstart_s.ptr, 1, V.w, C.Xw_s.ptr, C.rhs_s.ptr, O.D + nb,
+      rc = cr_solve(ctx, *C.cr, C.bins ? nullptr : (const int64_t*)C.Xstart_s.ptr,
+                    C.bins ? (const int32_t*)C.colptr.ptr : nullptr, C.bins ? O.q : 1, V.w, C.Xw_s.ptr, C.rhs_s.ptr, O.D + nb,
                     C.damp ? C.lam : 0.0, x + nb, (double*)C.res2.ptr);
     else
       rc = banded_explicit_solve(ctx, (int64_t)P.seg_cols.size(), (const int64_t*)C.seg_inst.ptr, C.Xw_s.ptr,
@@ -1364,6 +1394,15 @@ static qrkit_status solve_typed(qrkit_ctx* ctx, const void* J, const void* S, co
         if ((rc = dense_refine_gradient(ctx, V, O, (const float*)b, x, C.lam, C.dref.ptr, h, gS)) != QRKIT_OK) return rc;
         have_g = true;
       }
+    }
+    if (C.bins) {
+      QRKIT_CUDA_TRY(ctx, cudaMemsetAsync(gS, 0, (size_t)s * sizeof(double), st));
+      WindowSums<T> A = window_sums<T>(ctx, V, gS);
+      if ((rc = window_refine_gradient<T>(ctx, V, O, (const T*)b, x, C.lam, A)) != QRKIT_OK) return rc;
+      LAUNCH(ctx, gS_damping_kernel<<<blocks_for(s, 128), 128, 0, st>>>(
+                      gS, sizeof(T) == 4 ? (const float*)x : nullptr, sizeof(T) == 8 ? (const double*)x : nullptr, O.D,
+                      nb, s, C.lam));
+      have_g = true;
     }
     if (!have_g) {
       if (s > 0) QRKIT_CUDA_TRY(ctx, cudaMemsetAsync(gS, 0, (size_t)s * sizeof(double), st));
@@ -1420,13 +1459,28 @@ template ComposedView<float> composed_view<float>(qrkit_ctx*, const void*, const
 template ComposedView<double> composed_view<double>(qrkit_ctx*, const void*, const void*);
 
 qrkit_status composed_column_norms(qrkit_ctx* ctx, const void* J, const void* S, double* D) {
-  if (ctx->precision == QRKIT_FP64) return norms_typed<double>(ctx, view<double>(ctx, J, S), D);
-  return norms_typed<float>(ctx, view<float>(ctx, J, S), D);
+  if (ctx->precision == QRKIT_FP64) return norms_typed<double>(ctx, view<double>(ctx, J, S), D, false);
+  return norms_typed<float>(ctx, view<float>(ctx, J, S), D, false);
 }
 
-qrkit_status composed_factor_scaled(qrkit_ctx* ctx, const void* J, const void* S, const double* E) {
-  if (ctx->precision == QRKIT_FP64) return factor_typed<double>(ctx, J, S, E, 1.0, true);
-  return factor_typed<float>(ctx, J, S, E, 1.0, true);
+qrkit_status composed_factor_scaled(qrkit_ctx* ctx, const void* J, const void* S, const double* E, bool sorted) {
+  if (ctx->precision == QRKIT_FP64) return factor_typed<double>(ctx, J, S, E, 1.0, true, sorted);
+  return factor_typed<float>(ctx, J, S, E, 1.0, true, sorted);
+}
+
+qrkit_status composed_sort_blocks(qrkit_ctx* ctx, bool* done) {
+  Composed& C = ctx->comp;
+  *done = C.bins;
+  if (!C.bins) return QRKIT_OK;
+  return block_sort(ctx, C.bsort, (const int32_t*)ctx->plan.d_start.ptr, (int*)C.hist.ptr, C.bsort_hist,
+                    (int32_t*)C.colptr.ptr, (int32_t*)C.bpos.ptr, (int32_t*)C.bord.ptr);
+}
+
+qrkit_status composed_window_sums(qrkit_ctx* ctx, const void* S, double* sq) {
+  QRKIT_CUDA_TRY(ctx, cudaMemsetAsync(sq, 0, (size_t)ctx->plan.s.shared_cols * sizeof(double), ctx->stream));
+  if (ctx->precision == QRKIT_FP64)
+    return window_square_sums<double>(ctx, window_sums<double>(ctx, view<double>(ctx, nullptr, S), sq));
+  return window_square_sums<float>(ctx, window_sums<float>(ctx, view<float>(ctx, nullptr, S), sq));
 }
 
 qrkit_status composed_solve(qrkit_ctx* ctx, const void* J, const void* S, const void* b, void* p,
@@ -1471,6 +1525,7 @@ void release_composed(Composed& C) {
   release(C.res2); release(C.meta); release(C.dense_ws);
   release(C.sort_tab); release(C.hist); release(C.spos); release(C.order); release(C.Xw_s);
   release(C.Xstart_s); release(C.rhs_s); release(C.seg_inst);
+  release(C.bs_tab); release(C.bs_colseg); release(C.colptr); release(C.bpos); release(C.bord); release(C.wres);
   release_cr(C.cr);
   release(C.nrm_D); release(C.nrm_L); release(C.nrm_W); release(C.nrm_y); release(C.nrm_As);
   release(C.nrm_rs); release(C.nrm_seg);
@@ -1535,17 +1590,26 @@ qrkit_status composed_layout(qrkit_ctx* ctx, size_t elem) {
     // the reduced rows form a banded matrix (rows sorted by window start); its QR runs with
     // the right-hand side in qrkit_solve (the banded solver does not keep Q)
     const int64_t Mr = C.red_rows > 0 ? C.red_rows : 1;
-    if ((rc = ensure(ctx, C.Xw, (size_t)Mr * w * elem, "reduced rows")) != QRKIT_OK) return rc;
-    if ((rc = ensure(ctx, C.Xstart, (size_t)Mr * sizeof(int64_t), "reduced row starts")) != QRKIT_OK) return rc;
-    if ((rc = ensure(ctx, C.rhs_red, (size_t)Mr * elem, "reduced rhs")) != QRKIT_OK) return rc;
+    const int64_t nseg = (int64_t)P.seg_cols.size();
+    // blocks of one shape and a parallel banded QR of the segments: the blocks are sorted
+    C.bins = P.uniform && w <= 8 && C.red_rows > 0 && P.K < ((int64_t)1 << 31) && (int64_t)s < ((int64_t)1 << 31);
+    if (!C.bins) {
+      if ((rc = ensure(ctx, C.Xw, (size_t)Mr * w * elem, "reduced rows")) != QRKIT_OK) return rc;
+      if ((rc = ensure(ctx, C.Xstart, (size_t)Mr * sizeof(int64_t), "reduced row starts")) != QRKIT_OK) return rc;
+      if ((rc = ensure(ctx, C.rhs_red, (size_t)Mr * elem, "reduced rhs")) != QRKIT_OK) return rc;
+      if ((rc = ensure(ctx, C.spos, (size_t)Mr * sizeof(int64_t), "reduced row order")) != QRKIT_OK) return rc;
+      if ((rc = ensure(ctx, C.order, (size_t)Mr * sizeof(int64_t), "reduced row order")) != QRKIT_OK) return rc;
+      if ((rc = ensure(ctx, C.Xstart_s, (size_t)Mr * sizeof(int64_t), "sorted row starts")) != QRKIT_OK) return rc;
+    } else {
+      if ((rc = ensure(ctx, C.colptr, (size_t)(s + 1) * sizeof(int32_t), "block sort")) != QRKIT_OK) return rc;
+      if ((rc = ensure(ctx, C.bpos, (size_t)P.K * sizeof(int32_t), "block sort")) != QRKIT_OK) return rc;
+      if ((rc = ensure(ctx, C.bord, (size_t)P.K * sizeof(int32_t), "block sort")) != QRKIT_OK) return rc;
+      if ((rc = ensure(ctx, C.wres, (size_t)2 * P.rows * elem, "refinement residual")) != QRKIT_OK) return rc;
+    }
     if ((rc = ensure(ctx, C.RwS, (size_t)s * w * elem, "reduced R")) != QRKIT_OK) return rc;
     if ((rc = ensure(ctx, C.cS, (size_t)s * elem, "reduced c")) != QRKIT_OK) return rc;
-    const int64_t nseg = (int64_t)P.seg_cols.size();
     if ((rc = ensure(ctx, C.res2, sizeof(double) * nseg, "reduced residual")) != QRKIT_OK) return rc;
-    if ((rc = ensure(ctx, C.spos, (size_t)Mr * sizeof(int64_t), "reduced row order")) != QRKIT_OK) return rc;
-    if ((rc = ensure(ctx, C.order, (size_t)Mr * sizeof(int64_t), "reduced row order")) != QRKIT_OK) return rc;
     if ((rc = ensure(ctx, C.Xw_s, (size_t)Mr * w * elem, "sorted reduced rows")) != QRKIT_OK) return rc;
-    if ((rc = ensure(ctx, C.Xstart_s, (size_t)Mr * sizeof(int64_t), "sorted row starts")) != QRKIT_OK) return rc;
     if ((rc = ensure(ctx, C.rhs_s, (size_t)Mr * elem, "sorted reduced rhs")) != QRKIT_OK) return rc;
     if (C.sort_damp != (C.damp ? 1 : 0)) {
       // chunk tables of the device row sort and the segments' banded instances (host, once
@@ -1582,27 +1646,66 @@ qrkit_status composed_layout(qrkit_ctx* ctx, size_t elem) {
       std::vector<int64_t> tab;
       for (auto* v : {&c_row0, &c_rows, &c_hoff, &c_col0, &c_cols, &c_out0}) tab.insert(tab.end(), v->begin(), v->end());
       tab.insert(tab.end(), seg_chunk0.begin(), seg_chunk0.end());
-      if ((rc = upload_i64(ctx, C.sort_tab, tab, "row sort tables")) != QRKIT_OK) return rc;
+      if (!C.bins && (rc = upload_i64(ctx, C.sort_tab, tab, "row sort tables")) != QRKIT_OK) return rc;
       if ((rc = upload_i64(ctx, C.seg_inst, inst, "segment instances")) != QRKIT_OK) return rc;
       if (w <= 8) {
         std::vector<int64_t> ic(inst.begin(), inst.begin() + nseg), i0(inst.begin() + nseg, inst.begin() + 2 * nseg),
             r0v(inst.begin() + 2 * nseg, inst.begin() + 3 * nseg), rv(inst.begin() + 3 * nseg, inst.end());
         if ((rc = cr_build(ctx, C.cr, ic, i0, r0v, rv)) != QRKIT_OK) return rc;
       }
-      // histograms, then one bin total per shared column (the scan's second pass)
-      if ((rc = ensure(ctx, C.hist, (size_t)std::max<int64_t>(hoff + P.s.shared_cols, 1) * sizeof(int),
-                       "row sort histograms")) != QRKIT_OK)
-        return rc;
-      const int64_t* t = (const int64_t*)C.sort_tab.ptr;
-      C.sort.num_chunks = nc;
-      C.sort.chunk_row0 = t;
-      C.sort.chunk_rows = t + nc;
-      C.sort.chunk_hoff = t + 2 * nc;
-      C.sort.chunk_col0 = t + 3 * nc;
-      C.sort.chunk_cols = t + 4 * nc;
-      C.sort.chunk_out0 = t + 5 * nc;
-      C.sort.seg_chunk0 = t + 6 * nc;
-      C.sort_hist_entries = hoff;
+      if (C.bins && !C.bs_tab.ptr) {
+        // block sort: chunks of at least 256 blocks, and of an eighth of the segment's columns, which bounds the
+        // histograms by 8 counters per block
+        std::vector<int64_t> blk0, cseg, chunk0(nseg + 1), hoff(nseg + 1, 0);
+        std::vector<int32_t> col_seg((size_t)s);
+        for (int64_t k = 0; k < nseg; ++k) {
+          const int64_t per = std::max<int64_t>(256, P.seg_cols[k] / 8);
+          chunk0[k] = (int64_t)blk0.size();
+          for (int64_t q = P.seg_blk0[k]; q < P.seg_blk0[k + 1]; q += per) {
+            blk0.push_back(q);
+            cseg.push_back(k);
+          }
+          hoff[k + 1] = hoff[k] + ((int64_t)blk0.size() - chunk0[k]) * P.seg_cols[k];
+          std::fill(col_seg.begin() + P.seg_col0[k], col_seg.begin() + P.seg_col0[k] + P.seg_cols[k], (int32_t)k);
+        }
+        chunk0[nseg] = (int64_t)blk0.size();
+        const int64_t nch = (int64_t)blk0.size();
+        blk0.push_back(P.K);
+        std::vector<int64_t> tab;
+        for (auto* v : {&blk0, &cseg, &P.seg_blk0, &P.seg_col0, &chunk0, &hoff}) tab.insert(tab.end(), v->begin(), v->end());
+        if ((rc = upload_i64(ctx, C.bs_tab, tab, "block sort tables")) != QRKIT_OK) return rc;
+        if ((rc = ensure(ctx, C.bs_colseg, col_seg.size() * sizeof(int32_t), "block sort tables")) != QRKIT_OK) return rc;
+        QRKIT_CUDA_TRY(ctx, cudaMemcpy(C.bs_colseg.ptr, col_seg.data(), col_seg.size() * sizeof(int32_t),
+                                       cudaMemcpyHostToDevice));
+        C.bsort_hist = hoff[nseg];
+        if ((rc = ensure(ctx, C.hist, (size_t)std::max<int64_t>(C.bsort_hist, 1) * sizeof(int), "block sort")) != QRKIT_OK)
+          return rc;
+        const int64_t* t = (const int64_t*)C.bs_tab.ptr;
+        C.bsort.num_chunks = nch;
+        C.bsort.chunk_blk0 = t;
+        C.bsort.chunk_seg = t + (nch + 1);
+        C.bsort.seg_blk0 = t + (2 * nch + 1);
+        C.bsort.seg_col0 = C.bsort.seg_blk0 + (nseg + 1);
+        C.bsort.seg_chunk0 = C.bsort.seg_col0 + (nseg + 1);
+        C.bsort.seg_hoff = C.bsort.seg_chunk0 + (nseg + 1);
+        C.bsort.col_seg = (const int32_t*)C.bs_colseg.ptr;
+      }
+      if (!C.bins) {
+        // histograms, then one bin total per shared column (the scan's second pass)
+        if ((rc = ensure(ctx, C.hist, (size_t)std::max<int64_t>(hoff + P.s.shared_cols, 1) * sizeof(int),
+                         "row sort histograms")) != QRKIT_OK)
+          return rc;
+        const int64_t* t = (const int64_t*)C.sort_tab.ptr;
+        C.sort.num_chunks = nc;
+        C.sort.chunk_row0 = t;
+        C.sort.chunk_rows = t + nc;
+        C.sort.chunk_hoff = t + 2 * nc;
+        C.sort.chunk_col0 = t + 3 * nc;
+        C.sort.chunk_cols = t + 4 * nc;
+        C.sort.chunk_out0 = t + 5 * nc;
+        C.sort.seg_chunk0 = t + 6 * nc;
+        C.sort_hist_entries = hoff;
+      }
       C.sort_damp = C.damp ? 1 : 0;
     }
   }

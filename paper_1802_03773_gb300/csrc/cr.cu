@@ -93,7 +93,9 @@ struct CRArgs {
   const int32_t* binst;   // instance of each block
   int64_t total_blocks;
   // rows: explicit starts (global columns, sorted per instance) or implicit floor(i / rpc)
+  // or colptr: the rows that start at global column j are rpc colptr[j] .. rpc colptr[j + 1] - 1
   const int64_t* starts;
+  const int32_t* colptr;
   int rpc;
   int w;
   const T* J;             // rows x w
@@ -143,6 +145,10 @@ __device__ __forceinline__ void group_rows(const CRArgs<T>& A, int64_t k, int64_
   if (A.starts) {
     lo = A.grp_lo[gb];
     hi = g + 1 < nb ? A.grp_lo[gb + 1] : end;
+  } else if (A.colptr) {
+    const int64_t j0 = A.col0[k] + kCB * g, j1 = A.col0[k] + min((int64_t)kCB * (g + 1), A.cols[k]);
+    lo = (int64_t)A.colptr[j0] * A.rpc;
+    hi = (int64_t)A.colptr[j1] * A.rpc;
   } else {
     const int64_t r0 = A.row0[k] + (int64_t)A.rpc * kCB * g;
     lo = r0 < end ? r0 : end;
@@ -383,6 +389,12 @@ __global__ void __launch_bounds__(kCompThreads, sizeof(T) == 4 ? 4 : 2) cr_compr
 #pragma unroll
   for (int q = 0; q < 4; ++q) ahead[q] = A.starts && r + q < r_end ? A.starts[r + q] - c0 : -1;
   int c = have ? 0 : kCB;
+  // first row that starts past column `col` of the instance (implicit starts)
+  auto rows_end = [&](int64_t col) -> int64_t {
+    const int64_t e = A.colptr ? (col < N ? (int64_t)A.colptr[c0 + col + 1] * A.rpc : r_end) : row0 + (col + 1) * A.rpc;
+    return min(r_end, e);
+  };
+  int64_t c_end = A.starts ? r_end : rows_end((int64_t)kCB * g);   // of column c
 #pragma unroll 1
   while (__any_sync(0xffffffffu, c < kCB)) {
     const int64_t st = (int64_t)kCB * g + c;   // the rows' first column
@@ -393,7 +405,7 @@ __global__ void __launch_bounds__(kCompThreads, sizeof(T) == 4 ? 4 : 2) cr_compr
         for (int q = 0; q < 4; ++q)
           if (cnt == q && ahead[q] == st) cnt = q + 1;
       } else {
-        cnt = (int)max((int64_t)0, min((int64_t)4, min(r_end, row0 + (st + 1) * A.rpc) - r));
+        cnt = (int)max((int64_t)0, min((int64_t)4, c_end - r));
       }
     }
     T a[4][8], b[4];
@@ -453,6 +465,7 @@ __global__ void __launch_bounds__(kCompThreads, sizeof(T) == 4 ? 4 : 2) cr_compr
       dst[e0_at<T>(at, 128 + c)] = W.z[0];
       W.shift();
       ++c;
+      if (!A.starts) c_end = rows_end((int64_t)kCB * g + c);
     }
   }
   if constexpr (kStaged) dev::cp_async_wait_all();
@@ -1221,11 +1234,12 @@ static CRArgs<T> cr_args(qrkit_ctx* ctx, CRPlan& C) {
   } while (0)
 
 template <typename T>
-static qrkit_status cr_solve_typed(qrkit_ctx* ctx, CRPlan& C, const int64_t* starts, int rpc, int w,
+static qrkit_status cr_solve_typed(qrkit_ctx* ctx, CRPlan& C, const int64_t* starts, const int32_t* colptr, int rpc, int w,
                                    const T* J, const T* b, const double* D, double lambda, T* x, double* res2) {
   cudaStream_t st = ctx->stream;
   CRArgs<T> A = cr_args<T>(ctx, C);
   A.starts = starts;
+  A.colptr = colptr;
   A.rpc = rpc;
   A.w = w;
   A.J = J;
@@ -1297,13 +1311,13 @@ void cr_padded(const CRPlan& C, const int64_t** blk0, void** g) {
   *g = C.xp.ptr;
 }
 
-qrkit_status cr_solve(qrkit_ctx* ctx, CRPlan& C, const int64_t* starts, int rpc, int w, const void* J,
-                      const void* b, const double* D, double lambda, void* x, double* res2) {
+qrkit_status cr_solve(qrkit_ctx* ctx, CRPlan& C, const int64_t* starts, const int32_t* colptr, int rpc, int w,
+                      const void* J, const void* b, const double* D, double lambda, void* x, double* res2) {
   if (w < 1 || w > kCB) return fail(ctx, QRKIT_EUNSUPPORTED, "the parallel banded QR needs w <= 8");
   if (ctx->precision == QRKIT_FP64)
-    return cr_solve_typed<double>(ctx, C, starts, rpc, w, (const double*)J, (const double*)b, D, lambda,
+    return cr_solve_typed<double>(ctx, C, starts, colptr, rpc, w, (const double*)J, (const double*)b, D, lambda,
                                   (double*)x, res2);
-  return cr_solve_typed<float>(ctx, C, starts, rpc, w, (const float*)J, (const float*)b, D, lambda, (float*)x,
+  return cr_solve_typed<float>(ctx, C, starts, colptr, rpc, w, (const float*)J, (const float*)b, D, lambda, (float*)x,
                                res2);
 }
 

@@ -133,6 +133,7 @@ static qrkit_status plan_blocks(qrkit_ctx* ctx, const qrkit_structure* s) {
     if (n < m && P.first_wide < 0) P.first_wide = i;
     if (n + m > 16 && P.first_tall_aug < 0) P.first_tall_aug = i;
   }
+  P.uniform = P.rows == P.K * P.max_n && P.cols == P.K * P.max_m;
   P.val_off.assign(P.K + 1, 0);
   P.row_off.assign(P.K + 1, 0);
   P.col_off.assign(P.K + 1, 0);
@@ -529,6 +530,8 @@ qrkit_status qrkit_get_row_order(qrkit_ctx* ctx, int64_t* order) {
     return fail(ctx, QRKIT_ESTATE, "qrkit_get_row_order needs a windowed block plan");
   if (!ctx->comp_factored) return fail(ctx, QRKIT_ESTATE, "qrkit_get_row_order before qrkit_factor");
   if (!order) return fail(ctx, QRKIT_EINVAL, "order is required");
+  if (ctx->comp.bins)
+    return block_row_order(ctx, (const int32_t*)ctx->comp.bord.ptr, (int)(ctx->comp.red_rows / P.K), order);
   if (ctx->comp.red_rows > 0)
     QRKIT_CUDA_TRY(ctx, cudaMemcpyAsync(order, ctx->comp.order.ptr, (size_t)ctx->comp.red_rows * sizeof(int64_t),
                                         cudaMemcpyDeviceToDevice, ctx->stream));

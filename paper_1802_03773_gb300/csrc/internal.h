@@ -63,6 +63,7 @@ struct Plan {
   int64_t cols = 0;       // sum m_i (block columns)
   int64_t values = 0;     // sum n_i m_i
   int max_n = 0, max_m = 0;
+  bool uniform = false;   // every block max_n x max_m
   int64_t first_wide = -1;      // first block with n_i < m_i (needs damping rows), or -1
   int64_t first_tall_aug = -1;  // first block with n_i + m_i > 16 (no room for damping rows)
   // host copies
@@ -126,7 +127,9 @@ struct FactorOut {
   T* X0;
   int64_t ld0;
   T* Xw;            // windowed reduced rows (rows x w, row-major)
-  int64_t* Xstart;  // their first column
+  int64_t* Xstart;  // their first column (null with bpos)
+  const int32_t* bpos;   // blocks of one shape: sorted position of each block, q reduced rows each, in P_r order
+  int q;
   int* status;
 };
 
@@ -143,6 +146,32 @@ struct RowSortTables {
   const int64_t* chunk_cols;   // shared columns of that segment
   const int64_t* chunk_out0;   // first sorted position of that segment
   const int64_t* seg_chunk0;   // nseg + 1: first chunk of each segment
+};
+
+// Chunk and segment tables of the block sort (plans whose blocks all have one shape).
+struct BlockSortTables {
+  int64_t num_chunks;
+  const int64_t* chunk_blk0;   // num_chunks + 1 (chunks do not cross segments)
+  const int64_t* chunk_seg;
+  const int64_t* seg_blk0;     // nseg + 1: first block, first shared column, first chunk, histogram offset
+  const int64_t* seg_col0;
+  const int64_t* seg_chunk0;
+  const int64_t* seg_hoff;
+  const int32_t* col_seg;      // segment of each shared column
+};
+
+// Sums over the blocks' windows by shared column (window_sums.cu): blocks n x m of one shape, sorted.
+template <typename T>
+struct WindowSums {
+  int64_t K;
+  int n, m, w, s;
+  const int32_t* bord;    // block at each sorted position
+  const int32_t* start;
+  const T* S;
+  const T* R12;           // gradient: R12, the residual pairs (2 per row) and h_B
+  const T* r;
+  const T* h;
+  double* out;            // s sums, added to
 };
 
 // Device state of a batch of banded instances (Sec. 4.4).
@@ -188,6 +217,11 @@ struct Composed {
   int64_t sort_hist_entries = 0;
   RowSortTables sort{};
   DevBuf sort_tab, hist, spos, order, Xw_s, Xstart_s, rhs_s;
+  // blocks of one shape: sorted before the factorization, which then writes the reduced rows in P_r order
+  bool bins = false;
+  BlockSortTables bsort{};
+  int64_t bsort_hist = 0;
+  DevBuf bs_tab, bs_colseg, colptr, bpos, bord, wres;   // colptr: s + 1 first sorted blocks; wres: residual pairs
   DevBuf seg_inst;                 // 4 x nseg: cols, col0, row0, rows of the segments' banded solves
   CRPlan* cr = nullptr;            // parallel banded QR of the segments (window <= 8)
   // normal-equations (Cholesky) comparison path
@@ -208,8 +242,10 @@ qrkit_status cr_build(qrkit_ctx* ctx, CRPlan*& out, const std::vector<int64_t>& 
                       const std::vector<int64_t>& rows);
 // QR + solve of every instance: rows with explicit sorted starts (global columns) or
 // implicit starts floor(i / rpc); damping rows lambda^(1/2) D_j; x and D by global column.
-qrkit_status cr_solve(qrkit_ctx* ctx, CRPlan& C, const int64_t* starts, int rpc, int w, const void* J,
-                      const void* b, const double* D, double lambda, void* x, double* res2);
+// With colptr instead (s + 1 entries over the global columns), the rows that start at column j are
+// rpc colptr[j] .. rpc colptr[j + 1] - 1.
+qrkit_status cr_solve(qrkit_ctx* ctx, CRPlan& C, const int64_t* starts, const int32_t* colptr, int rpc, int w,
+                      const void* J, const void* b, const double* D, double lambda, void* x, double* res2);
 // Compression strategy of the parallel banded QR: one thread per column block, or `splits` threads
 // per block whose triangles are merged (autotuning).
 qrkit_status cr_set_strategy(qrkit_ctx* ctx, CRPlan& C, bool thread_rows, int splits);
@@ -290,8 +326,9 @@ qrkit_status composed_layout(qrkit_ctx* ctx, size_t elem);
 qrkit_status widen_to_double(qrkit_ctx* ctx, const float* in, double* out, int64_t n);
 qrkit_status composed_factor(qrkit_ctx* ctx, const void* J, const void* S, const void* D, double lambda);
 // Composed factor with the damping diagonal given directly as E = lambda^(1/2) D (double,
-// N entries) and lambda = 1: per-column damping, e.g. one lambda per independent problem.
-qrkit_status composed_factor_scaled(qrkit_ctx* ctx, const void* J, const void* S, const double* E);
+// N entries) and lambda = 1: per-column damping, e.g. one lambda per independent problem; sorted:
+// composed_sort_blocks has been called for these starts.
+qrkit_status composed_factor_scaled(qrkit_ctx* ctx, const void* J, const void* S, const double* E, bool sorted);
 // D = column norms of the block structure's J (zero -> 1), N doubles.
 qrkit_status composed_column_norms(qrkit_ctx* ctx, const void* J, const void* S, double* D);
 template <typename T> ComposedView<T> composed_view(qrkit_ctx* ctx, const void* J, const void* S);
@@ -321,6 +358,22 @@ qrkit_status reduced_row_sort(qrkit_ctx* ctx, const RowSortTables& t, int64_t ns
                               const int64_t* Xstart, const void* Xw, int w, int* hist, int64_t* spos,
                               int64_t* order, int64_t* Xstart_s, void* Xw_s);
 qrkit_status window_start_copy(qrkit_ctx* ctx, const int32_t* in);
+// Stable sort of the blocks by (segment, start): bpos, its inverse bord, and colptr[j] = first sorted block that
+// starts at shared column j or later.  block_row_order: the reduced rows' order, q per block.
+qrkit_status block_sort(qrkit_ctx* ctx, const BlockSortTables& t, const int32_t* start, int* hist, int64_t hist_entries,
+                        int32_t* colptr, int32_t* bpos, int32_t* bord);
+qrkit_status block_row_order(qrkit_ctx* ctx, const int32_t* bord, int q, int64_t* order);
+// out[j] += sum of the squares of S's column j; and a refinement step's h_B = R_i^{-T} g_B (to A.h, the residual
+// pairs to A.r) with out[j] += (S^T r - R12^T h_B)_j.
+template <typename T>
+qrkit_status window_square_sums(qrkit_ctx* ctx, const WindowSums<T>& A);
+template <typename T>
+qrkit_status window_refine_gradient(qrkit_ctx* ctx, const ComposedView<T>& V, const FactorOut<T>& O, const T* b,
+                                    const T* p, double lam, const WindowSums<T>& A);
+// The block sort of a windowed plan whose blocks have one shape, for the starts now in the plan, and the squared
+// column sums of its S (s doubles, written); false in *done if the plan has no block sort.
+qrkit_status composed_sort_blocks(qrkit_ctx* ctx, bool* done);
+qrkit_status composed_window_sums(qrkit_ctx* ctx, const void* S, double* sq);
 // Column-panel TSQR (float; tsqr_tc.cu), one level of a 32-column panel in tiles of kPanelRows rows;
 // every pointer 16-byte aligned, every ld, row count and row offset a multiple of 4.
 // tsqr_panel_tile: reflectors and R in place, each tile's 32 x 32 T and G = Y^T Y (strict upper part,

@@ -419,7 +419,7 @@ qrkit_status lm_iteration(qrkit_ctx* ctx, double* x, int refine_steps, double ft
   LM_LAUNCH(ctx, lm_damp_kernel<<<nblk(t.N, 256), 256, 0, st>>>(t, d2, S, E));
   qrkit_status rc = window_start_copy(ctx, (const int32_t*)L.start.ptr);
   if (rc != QRKIT_OK) return rc;
-  if ((rc = composed_factor_scaled(ctx, J, Sv, E)) != QRKIT_OK) return rc;
+  if ((rc = composed_factor_scaled(ctx, J, Sv, E, false)) != QRKIT_OK) return rc;
   if ((rc = composed_solve(ctx, J, Sv, b, p, refine_steps)) != QRKIT_OK) return rc;
   double* xn = (double*)L.xnew.ptr;
   LM_LAUNCH(ctx, lm_xnew_kernel<T><<<nblk(t.N, 256), 256, 0, st>>>(t.N, x, p, xn));

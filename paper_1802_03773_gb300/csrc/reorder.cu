@@ -14,6 +14,14 @@
 //           writes the sorted rows (values, starts) and both directions of the permutation.
 // A start outside its segment is recorded as QRKIT_EINVAL and clamped into the segment so
 // that every index stays in bounds.
+//
+// Plans whose blocks all have one shape sort the blocks instead of their rows, before the factorization:
+// every block leaves the same number q of reduced rows, all with its start, so the rows' order is the
+// blocks' order q rows at a time, and the factorization and Q^T b write their rows in place.  The same
+// counting sort, with one warp per bin for the prefixes over the chunks (bin-major histograms, so that they
+// are contiguous) and chunks short enough that a scatter warp takes a few dozen steps.  200,000 blocks and
+// 4,096 columns: 50 us against 355 us for the 400,000 rows; 10.5 million blocks in 1,024 segments:
+// 434 us against 1.31 ms.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -177,6 +185,121 @@ __global__ void rsort_rhs_kernel(const int64_t* spos, const T* rhs, T* rhs_s, in
   if (r < rows) rhs_s[spos[r]] = rhs[r];
 }
 
+// ---- blocks of one shape ----
+__global__ void __launch_bounds__(256) bsort_count_kernel(BlockSortTables t, const int32_t* start, int* hist,
+                                                          int* status) {
+  const int64_t c = blockIdx.x;
+  const int64_t k = t.chunk_seg[c], b0 = t.chunk_blk0[c], b1 = t.chunk_blk0[c + 1];
+  const int64_t col0 = t.seg_col0[k], cols = t.seg_col0[k + 1] - col0, nch = t.seg_chunk0[k + 1] - t.seg_chunk0[k];
+  int* h = hist + t.seg_hoff[k] + (c - t.seg_chunk0[k]);
+  for (int64_t i = b0 + threadIdx.x; i < b1; i += 256) atomicAdd(h + clamp_key(start[i], col0, cols, status) * nch, 1);
+}
+
+// Bin of shared column j: its chunk counts to exclusive prefixes in place, the total to colptr[j].
+__global__ void __launch_bounds__(256) bsort_prefix_kernel(BlockSortTables t, int64_t s, int* hist, int32_t* colptr) {
+  const int64_t j = ((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (j >= s) return;
+  const int64_t k = t.col_seg[j], nch = t.seg_chunk0[k + 1] - t.seg_chunk0[k];
+  int* h = hist + t.seg_hoff[k] + (j - t.seg_col0[k]) * nch;
+  int carry = 0;
+  for (int64_t c0 = 0; c0 < nch; c0 += 32) {
+    const int v = c0 + lane < nch ? h[c0 + lane] : 0;
+    int incl = v;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += u;
+    }
+    if (c0 + lane < nch) h[c0 + lane] = carry + incl - v;
+    carry += __shfl_sync(0xffffffffu, incl, 31);
+  }
+  if (lane == 0) colptr[j] = carry;
+}
+
+// Per segment (one CTA): bin totals to first sorted blocks, in place; colptr[s] = all blocks.
+__global__ void __launch_bounds__(kScanThreads) bsort_scan_kernel(BlockSortTables t, int64_t s, int64_t K,
+                                                                  int32_t* colptr) {
+  __shared__ int warp_tot[kScanThreads / 32];
+  __shared__ int carry_s;
+  const int64_t k = blockIdx.x;
+  const int64_t cols = t.seg_col0[k + 1] - t.seg_col0[k];
+  int32_t* tt = colptr + t.seg_col0[k];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (threadIdx.x == 0) {
+    carry_s = (int)t.seg_blk0[k];
+    if (k == 0) colptr[s] = (int32_t)K;
+  }
+  __syncthreads();
+  for (int64_t b0 = 0; b0 < cols; b0 += blockDim.x) {
+    const int64_t b = b0 + threadIdx.x;
+    const int v0 = b < cols ? tt[b] : 0;
+    int incl = v0;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += v;
+    }
+    if (lane == 31) warp_tot[wid] = incl;
+    __syncthreads();
+    if (wid == 0) {
+      int v = lane < (int)(blockDim.x >> 5) ? warp_tot[lane] : 0;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, v, d);
+        if (lane >= d) v += u;
+      }
+      warp_tot[lane] = v;   // inclusive over warps
+    }
+    __syncthreads();
+    const int carry = carry_s;
+    if (b < cols) tt[b] = carry + (wid ? warp_tot[wid - 1] : 0) + incl - v0;
+    __syncthreads();
+    if (threadIdx.x == 0) carry_s = carry + warp_tot[(blockDim.x >> 5) - 1];
+    __syncthreads();
+  }
+}
+
+// One warp per chunk, its blocks in order: bpos[i] = sorted position of block i, bord its inverse.
+__global__ void __launch_bounds__(128) bsort_scatter_kernel(BlockSortTables t, const int32_t* start, int* hist,
+                                                            const int32_t* colptr, int32_t* bpos, int32_t* bord) {
+  const int64_t c = ((int64_t)blockIdx.x * 128 + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (c >= t.num_chunks) return;
+  const int64_t k = t.chunk_seg[c], b0 = t.chunk_blk0[c], b1 = t.chunk_blk0[c + 1];
+  const int64_t col0 = t.seg_col0[k], cols = t.seg_col0[k + 1] - col0, nch = t.seg_chunk0[k + 1] - t.seg_chunk0[k];
+  int* h = hist + t.seg_hoff[k] + (c - t.seg_chunk0[k]);
+  int64_t next = b0 + lane < b1 ? clamp_key(start[b0 + lane], col0, cols, nullptr) : -1;
+  for (int64_t i0 = b0; i0 < b1; i0 += 32) {
+    const int64_t i = i0 + lane, key = next;
+    next = i + 32 < b1 ? clamp_key(start[i + 32], col0, cols, nullptr) : -1;
+    const bool active = i < b1;
+    const unsigned amask = __ballot_sync(0xffffffffu, active);
+    if (active) {
+      const unsigned peers = __match_any_sync(amask, (unsigned long long)key);
+      const int leader = __ffs(peers) - 1;
+      const int rank = __popc(peers & ((1u << lane) - 1u));
+      int base = 0;
+      if (lane == leader) {
+        base = h[key * nch];
+        h[key * nch] = base + __popc(peers);
+        base += colptr[col0 + key];
+      }
+      base = __shfl_sync(amask, base, leader);
+      bpos[i] = base + rank;
+      bord[base + rank] = (int32_t)i;
+    }
+    __syncwarp();
+  }
+}
+
+// The order of the reduced rows from that of the blocks, q rows each.
+__global__ void rows_of_blocks_kernel(const int32_t* bord, int64_t K, int q, int64_t* order) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= K * q) return;
+  order[e] = (int64_t)bord[e / q] * q + e % q;
+}
+
 // Copy of caller-given window starts into the plan, each checked against its segment
 // (block i belongs to segment k with seg_blk0[k] <= i < seg_blk0[k + 1]); a start outside
 // is recorded as QRKIT_EINVAL and clamped.
@@ -240,6 +363,30 @@ qrkit_status reduced_row_sort(qrkit_ctx* ctx, const RowSortTables& t, int64_t ns
   else
     rsort_scatter_kernel<float><<<nblk(t.num_chunks * 32, 128), 128, 0, st>>>(
         t, Xstart, (const float*)Xw, w, hist, spos, order, Xstart_s, (float*)Xw_s);
+  ctx->launches += 1;
+  QRKIT_CUDA_TRY(ctx, cudaGetLastError());
+  return QRKIT_OK;
+}
+
+qrkit_status block_sort(qrkit_ctx* ctx, const BlockSortTables& t, const int32_t* start, int* hist, int64_t hist_entries,
+                        int32_t* colptr, int32_t* bpos, int32_t* bord) {
+  Plan& P = ctx->plan;
+  cudaStream_t st = ctx->stream;
+  const int64_t s = P.s.shared_cols, nseg = (int64_t)P.seg_cols.size();
+  QRKIT_CUDA_TRY(ctx, cudaMemsetAsync(hist, 0, (size_t)hist_entries * sizeof(int), st));
+  bsort_count_kernel<<<(unsigned)t.num_chunks, 256, 0, st>>>(t, start, hist, ctx->d_status);
+  bsort_prefix_kernel<<<nblk(s * 32, 256), 256, 0, st>>>(t, s, hist, colptr);
+  bsort_scan_kernel<<<(unsigned)nseg, nseg >= 2 * ctx->num_sms ? 128 : kScanThreads, 0, st>>>(t, s, P.K, colptr);
+  bsort_scatter_kernel<<<nblk(t.num_chunks * 32, 128), 128, 0, st>>>(t, start, hist, colptr, bpos, bord);
+  ctx->launches += 4;
+  QRKIT_CUDA_TRY(ctx, cudaGetLastError());
+  return QRKIT_OK;
+}
+
+qrkit_status block_row_order(qrkit_ctx* ctx, const int32_t* bord, int q, int64_t* order) {
+  const int64_t K = ctx->plan.K;
+  if (K * q == 0) return QRKIT_OK;
+  rows_of_blocks_kernel<<<nblk(K * q, 256), 256, 0, ctx->stream>>>(bord, K, q, order);
   ctx->launches += 1;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());
   return QRKIT_OK;
