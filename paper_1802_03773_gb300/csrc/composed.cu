@@ -1499,6 +1499,11 @@ qrkit_status composed_apply_qt(qrkit_ctx* ctx, const void* b, void* qtb) {
 
 namespace qrkit {
 
+__global__ void multiples_kernel(int64_t* out, int64_t n, int64_t step) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i < n) out[i] = i * step;
+}
+
 static qrkit_status upload_i64(qrkit_ctx* ctx, DevBuf& buf, const std::vector<int64_t>& v, const char* what) {
   qrkit_status rc = ensure(ctx, buf, v.size() * sizeof(int64_t), what);
   if (rc != QRKIT_OK) return rc;
@@ -1549,7 +1554,20 @@ qrkit_status composed_layout(qrkit_ctx* ctx, size_t elem) {
   Plan& P = ctx->plan;
   Composed& C = ctx->comp;
   qrkit_status rc;
-  if (!C.d_aug_off_d.ptr) {
+  if (!C.d_aug_off_d.ptr && P.uniform) {
+    // blocks of one shape: the offsets are multiples, written on the device
+    const int64_t n = P.max_n, m = P.max_m, K = P.K;
+    const int64_t step[4] = {(n + m) * m, n * m, n, n - m};
+    DevBuf* buf[4] = {&C.d_aug_off_d, &C.d_aug_off_u, &C.d_red_off_d, &C.d_red_off_u};
+    for (int q = 0; q < 4; ++q) {
+      if ((rc = ensure(ctx, *buf[q], (size_t)(K + 1) * sizeof(int64_t), "block offsets")) != QRKIT_OK) return rc;
+      multiples_kernel<<<blocks_for(K + 1, 256), 256, 0, ctx->stream>>>((int64_t*)buf[q]->ptr, K + 1, step[q]);
+      ctx->launches += 1;
+      QRKIT_CUDA_TRY(ctx, cudaGetLastError());
+    }
+    C.aug_values_d = K * step[0]; C.aug_values_u = K * step[1];
+    C.red_rows_d = K * step[2]; C.red_rows_u = K * step[3];
+  } else if (!C.d_aug_off_d.ptr) {
     std::vector<int64_t> ad(P.K + 1), au(P.K + 1), rd(P.K + 1), ru(P.K + 1);
     ad[0] = au[0] = rd[0] = ru[0] = 0;
     for (int64_t i = 0; i < P.K; ++i) {

@@ -29,13 +29,13 @@
 #include <string>
 #include <vector>
 
+#include "device_util.cuh"
 #include "internal.h"
 #include "mlp_policy.cuh"
 
 namespace qrkit {
 
 constexpr int kTilePts = 256;   // points per reduction tile (tiles never cross problems)
-constexpr int kEvalSumCols = 2048;   // problems up to this many columns: S column sums per tile in shared memory
 
 struct LMTables {
   int64_t B = 0, NP = 0, s = 0, N = 0, num_tiles = 0;
@@ -52,11 +52,10 @@ struct LM {
   std::vector<int64_t> h_p0, h_c0, h_tile_p0, h_prob_tile0;
   DevBuf tabs, tile_prob, col_prob;
   const double* data = nullptr;        // caller's points (device)
-  DevBuf J, S, b, p, start, d2, E, xnew, tile_cost, tile_new, tile_pred, state, ndone;
+  DevBuf J, S, b, p, start, d2, E, coef, tile_cost, tile_new, tile_pred, state, ndone;
   DevBuf hist, feat;                   // per problem: step history (12) and policy features (16)
   bool policy = false;                 // damping from the MLP after accepted steps
   bool prepared = false;
-  int sum_cols = 0;                    // columns of the widest problem when it fits a tile's shared sums
   cudaGraphExec_t graph = nullptr;
   int graph_refine = -1;
   int64_t graph_launches = 0;          // kernels in one captured iteration
@@ -68,7 +67,7 @@ void release_lm(LM*& lm) {
   if (!lm) return;
   if (lm->graph) cudaGraphExecDestroy(lm->graph);
   for (DevBuf* b : {&lm->tabs, &lm->tile_prob, &lm->col_prob, &lm->J, &lm->S, &lm->b, &lm->p, &lm->start,
-                    &lm->d2, &lm->E, &lm->xnew, &lm->tile_cost, &lm->tile_new, &lm->tile_pred, &lm->state,
+                    &lm->d2, &lm->E, &lm->coef, &lm->tile_cost, &lm->tile_new, &lm->tile_pred, &lm->state,
                     &lm->ndone, &lm->hist, &lm->feat})
     release(*b);
   delete lm;
@@ -77,137 +76,143 @@ void release_lm(LM*& lm) {
 
 namespace {
 
-// Uniform cubic B-spline basis and its derivative at u in [0, 1] (extrapolated outside),
-// in Horner form with multiplications only (double division is slow on this part):
-//   6 B_0 = (1-u)^3, 6 B_1 = (3u - 6) u^2 + 4, 6 B_2 = ((-3u + 3) u + 3) u + 1, 6 B_3 = u^3,
-//   B_0' = -(1-u)^2 / 2, B_1' = (3u/2 - 2) u, B_2' = (-3u/2 + 1) u + 1/2, B_3' = u^2 / 2.
-__device__ __forceinline__ void bspline(double u, double B[4], double dB[4]) {
-  const double sixth = 1.0 / 6.0;
-  const double v = 1.0 - u, u2 = u * u;
-  B[0] = v * v * v * sixth;
-  B[1] = fma(fma(3.0, u, -6.0), u2, 4.0) * sixth;
-  B[2] = fma(fma(fma(-3.0, u, 3.0), u, 3.0), u, 1.0) * sixth;
-  B[3] = u2 * u * sixth;
-  dB[0] = -0.5 * v * v;
-  dB[1] = fma(1.5, u, -2.0) * u;
-  dB[2] = fma(fma(-1.5, u, 1.0), u, 0.5);
-  dB[3] = 0.5 * u2;
+// The curve on a segment as a cubic in u = t - seg, from its four control points P0 .. P3:
+//   c(u) = a0 + u (a1 + u (a2 + u a3)), c'(u) = a1 + u (2 a2 + 3 a3 u),
+//   a0 = (P0 + 4 P1 + P2) / 6, a1 = (P2 - P0) / 2, a2 = (P0 - 2 P1 + P2) / 2, a3 = (P3 - P0 + 3 (P1 - P2)) / 6.
+// One thread per segment and coordinate once per evaluation, so that a point costs 10 FP64 multiply-adds instead of
+// the basis, its derivative and 16 products: the model kernels are bound by the FP64 unit, which a warp's
+// instruction holds for 16 cycles here.  kCoef values per segment: a0 a1 a2 a3 2a2 3a3 for x, then for y.
+constexpr int kCoef = 12;
+
+template <typename T>
+__global__ void cf_coef_kernel(LMTables t, const double* x, const T* p, double* coef) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // shared column: control point e / 2, coordinate e % 2
+  if (e + 6 >= t.s) return;
+  // a segment that starts in the last three control points of a problem mixes two problems' and is never used
+  const int64_t j = t.NP + e;
+  double P[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) P[q] = x[j + 2 * q] + (p ? (double)p[j + 2 * q] : 0.0);
+  double* c = coef + (e / 2) * kCoef + (e & 1) * (kCoef / 2);
+  const double a2 = 0.5 * (P[0] + P[2]) - P[1], a3 = (P[3] - P[0] + 3.0 * (P[1] - P[2])) * (1.0 / 6.0);
+  c[0] = (P[0] + 4.0 * P[1] + P[2]) * (1.0 / 6.0);
+  c[1] = 0.5 * (P[2] - P[0]);
+  c[2] = a2;
+  c[3] = a3;
+  c[4] = 2.0 * a2;
+  c[5] = 3.0 * a3;
 }
 
-// The basis alone (the trial cost needs no derivative).
+// The basis functions at u: 6 B_0 = (1-u)^3, 6 B_3 = u^3, B_1 = (u/2 - 1) u^2 + 2/3, and B_2 the rest of
+// their sum 1.
 __device__ __forceinline__ void bspline_values(double u, double B[4]) {
   const double sixth = 1.0 / 6.0;
   const double v = 1.0 - u, u2 = u * u;
   B[0] = v * v * v * sixth;
-  B[1] = fma(fma(3.0, u, -6.0), u2, 4.0) * sixth;
-  B[2] = fma(fma(fma(-3.0, u, 3.0), u, 3.0), u, 1.0) * sixth;
+  B[1] = fma(fma(0.5, u, -1.0), u2, 4.0 * sixth);
   B[3] = u2 * u * sixth;
+  B[2] = (1.0 - B[1]) - (B[0] + B[3]);
 }
 
-__device__ __forceinline__ int64_t segment_of(double t, int64_t Kc) {
-  const double hi = (double)(Kc - 4);
+// Segment of parameter t and u = t - segment.
+__device__ __forceinline__ int segment_of(double t, int64_t Kc, double& u) {
+  const double hi = (double)(int)(Kc - 4);
   double f = floor(t);
   if (!(f >= 0.0)) f = 0.0;   // also NaN
   if (f > hi) f = hi;
-  return (int64_t)f;
+  u = t - f;
+  return (int)f;
 }
 
-__device__ __forceinline__ double block_sum(double v, double* red) {
-#pragma unroll
-  for (int d = 16; d >= 1; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) red[wid] = v;
+// Sum over the CTA of kTilePts threads, in thread 0: through shared memory, so that the FP64 additions are those of
+// one warp.
+__device__ __forceinline__ double tile_sum(double v, double* buf) {
+  buf[threadIdx.x] = v;
   __syncthreads();
   double s = 0.0;
-  if (threadIdx.x == 0)
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-  return s;   // valid in thread 0
+  if (threadIdx.x < 32) {
+#pragma unroll
+    for (int q = 0; q < kTilePts / 32; ++q) s += buf[threadIdx.x + 32 * q];
+#pragma unroll
+    for (int d = 16; d >= 1; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+  }
+  return s;
 }
 
-// Residual, Jacobian blocks, windows, b = -f, squared column norms and the cost per tile.
-// A tile lies in one problem: when the problem's columns fit (sum_cols > 0), the squared
-// column sums of S are gathered in shared memory and leave the tile with one global atomic per
-// column touched, instead of eight per point.
+// Residual, Jacobian blocks, windows, b = -f and the cost per tile.
 template <typename T>
 __global__ void __launch_bounds__(kTilePts)
-cf_eval_kernel(LMTables t, const double* x, const double* data, T* J, T* S, T* b, int32_t* start,
-               double* d2, double* tile_cost, int sum_cols) {
-  __shared__ double red[kTilePts / 32];
-  extern __shared__ double scol[];
+cf_eval_kernel(LMTables t, const double* x, const double* data, const double* coef, T* J, T* S, T* b, int32_t* start,
+               double* tile_cost) {
+  __shared__ double red[kTilePts];
   const int64_t tile = blockIdx.x;
   const int64_t i = t.tile_p0[tile] + threadIdx.x;
-  const int kt = t.tile_prob[tile];
-  const int ncol = (int)(t.c0[kt + 1] - t.c0[kt]);
-  const bool tile_sum = ncol <= sum_cols;
-  if (tile_sum) {
-    for (int c = threadIdx.x; c < ncol; c += blockDim.x) scol[c] = 0.0;
-    __syncthreads();
-  }
   double fsq = 0.0;
   if (i < t.tile_p0[tile + 1]) {
-    const int k = kt;
-    const int64_t Kc = (t.c0[k + 1] - t.c0[k]) / 2;
-    const double ti = x[i];
-    const int64_t seg = segment_of(ti, Kc);
-    double Bv[4], dB[4];
-    bspline(ti - (double)seg, Bv, dB);
-    const double* P = x + t.NP + t.c0[k] + 2 * seg;
-    double cx = 0, cy = 0, dx = 0, dy = 0;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      cx += Bv[q] * P[2 * q];
-      cy += Bv[q] * P[2 * q + 1];
-      dx += dB[q] * P[2 * q];
-      dy += dB[q] * P[2 * q + 1];
-    }
-    const double fx = cx - data[2 * i], fy = cy - data[2 * i + 1];
-    fsq = fx * fx + fy * fy;
-    const T jx = (T)dx, jy = (T)dy;
-    J[2 * i] = jx;
-    J[2 * i + 1] = jy;
+    const int k = t.tile_prob[tile];
+    const int64_t c0 = t.c0[k], Kc = (t.c0[k + 1] - c0) / 2;
+    double u;
+    const int seg = segment_of(x[i], Kc, u);
+    const double2* c = reinterpret_cast<const double2*>(coef + (c0 / 2 + seg) * kCoef);
+    const double2 x01 = c[0], x23 = c[1], xd = c[2], y01 = c[3], y23 = c[4], yd = c[5];
+    const double fx = fma(fma(fma(x23.y, u, x23.x), u, x01.y), u, x01.x) - data[2 * i];
+    const double fy = fma(fma(fma(y23.y, u, y23.x), u, y01.y), u, y01.x) - data[2 * i + 1];
+    fsq = fma(fx, fx, fy * fy);
+    J[2 * i] = (T)fma(fma(xd.y, u, xd.x), u, x01.y);
+    J[2 * i + 1] = (T)fma(fma(yd.y, u, yd.x), u, y01.y);
     b[2 * i] = (T)(-fx);
     b[2 * i + 1] = (T)(-fy);
-    d2[i] = (double)jx * (double)jx + (double)jy * (double)jy;
-    T* Si = S + 16 * i;   // 2 x 8, column-major
-    const int64_t col = t.c0[k] + 2 * seg;
-    start[i] = (int32_t)col;
-    double* dS = d2 + t.NP + col;
+    start[i] = (int32_t)(c0 + 2 * seg);
+    double B[4];
+    bspline_values(u, B);
+    T* Si = S + 16 * i;   // 2 x 8, column-major: (B_q, 0) for column 2 q, (0, B_q) for column 2 q + 1
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const T v = (T)Bv[q];
-      Si[4 * q + 0] = v;      // (row x, column 2q)
-      Si[4 * q + 1] = T(0);   // (row y, column 2q)
-      Si[4 * q + 2] = T(0);   // (row x, column 2q + 1)
-      Si[4 * q + 3] = v;      // (row y, column 2q + 1)
-      const double v2 = (double)v * (double)v;
-      if (v2 != 0.0) {
-        if (tile_sum) {
-          atomicAdd(&scol[2 * seg + 2 * q], v2);
-          atomicAdd(&scol[2 * seg + 2 * q + 1], v2);
-        } else {
-          atomicAdd(dS + 2 * q, v2);
-          atomicAdd(dS + 2 * q + 1, v2);
-        }
+      const T v = (T)B[q];
+      if constexpr (sizeof(T) == 4) {
+        reinterpret_cast<float4*>(Si)[q] = make_float4(v, 0.f, 0.f, v);
+      } else {
+        reinterpret_cast<double2*>(Si)[2 * q] = make_double2(v, 0.0);
+        reinterpret_cast<double2*>(Si)[2 * q + 1] = make_double2(0.0, v);
       }
     }
   }
-  const double s = block_sum(fsq, red);
+  const double s = tile_sum(fsq, red);
   if (threadIdx.x == 0) tile_cost[tile] = s;
-  if (tile_sum) {
-    __syncthreads();
-    double* dP = d2 + t.NP + t.c0[kt];
-    for (int c = threadIdx.x; c < ncol; c += blockDim.x)
-      if (scol[c] != 0.0) atomicAdd(dP + c, scol[c]);
-  }
 }
 
-// E_j = lambda_k^(1/2) D_j with D_j = ||column j of J|| (zero -> 1).
-__global__ void lm_damp_kernel(LMTables t, const double* d2, const qrkit_lm_state* st, double* E) {
-  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= t.N) return;
-  double d = sqrt(d2[j]);
-  if (d == 0.0) d = 1.0;
-  E[j] = sqrt(st[t.col_prob[j]].lambda) * d;
+// E_j = lambda_k^(1/2) D_j with D_j = ||column j of J|| (zero -> 1): a tile of points per CTA, then the shared
+// columns (squared norms d2) 256 at a time.  The norm of a float block column is a float pair: its two
+// squares summed exactly, and one Newton step on the float root.
+template <typename T>
+__global__ void __launch_bounds__(kTilePts) lm_damp_kernel(LMTables t, const T* J, const double* d2,
+                                                           const qrkit_lm_state* st, double* E) {
+  __shared__ double root;
+  if (blockIdx.x < t.num_tiles) {
+    const int64_t tile = blockIdx.x, i = t.tile_p0[tile] + threadIdx.x;
+    if (threadIdx.x == 0) root = sqrt(st[t.tile_prob[tile]].lambda);
+    __syncthreads();
+    if (i >= t.tile_p0[tile + 1]) return;
+    const T jx = J[2 * i], jy = J[2 * i + 1];
+    double d;
+    if constexpr (sizeof(T) == 4) {
+      const float a = __fmul_rn(jx, jx), b = __fmul_rn(jy, jy);
+      float h, l;
+      dev::two_sum(a, b, h, l);
+      l += __fmaf_rn(jx, jx, -a) + __fmaf_rn(jy, jy, -b);
+      const float r = sqrtf(h);
+      const float c = r > 0.f ? (__fmaf_rn(-r, r, h) + l) / (2.f * r) : 0.f;
+      d = (double)r + (double)c;
+    } else {
+      d = sqrt(jx * jx + jy * jy);
+    }
+    E[i] = root * (d == 0.0 ? 1.0 : d);
+    return;
+  }
+  const int64_t c = (blockIdx.x - t.num_tiles) * (int64_t)kTilePts + threadIdx.x;
+  if (c >= t.s) return;
+  const double d = sqrt(d2[c]);
+  E[t.NP + c] = sqrt(st[t.col_prob[t.NP + c]].lambda) * (d == 0.0 ? 1.0 : d);
 }
 
 // f = curve(t) - data per point (two values), double.
@@ -217,10 +222,9 @@ __global__ void cf_residual_kernel(LMTables t, const double* x, const double* da
   if (i >= t.tile_p0[tile + 1]) return;
   const int k = t.tile_prob[tile];
   const int64_t Kc = (t.c0[k + 1] - t.c0[k]) / 2;
-  const double ti = x[i];
-  const int64_t seg = segment_of(ti, Kc);
-  double Bv[4], dB[4];
-  bspline(ti - (double)seg, Bv, dB);
+  double u, Bv[4];
+  const int seg = segment_of(x[i], Kc, u);
+  bspline_values(u, Bv);
   const double* P = x + t.NP + t.c0[k] + 2 * seg;
   double cx = 0, cy = 0;
 #pragma unroll
@@ -232,41 +236,29 @@ __global__ void cf_residual_kernel(LMTables t, const double* x, const double* da
   f[2 * i + 1] = cy - data[2 * i + 1];
 }
 
-template <typename T>
-__global__ void lm_xnew_kernel(int64_t N, const double* x, const T* p, double* xnew) {
-  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (j < N) xnew[j] = x[j] + (double)p[j];
-}
-
 // Cost at x + p and the row part of the predicted decrease, (J p)^T b + E_t^2 p_t^2, per tile.
 template <typename T>
 __global__ void __launch_bounds__(kTilePts)
-cf_trial_kernel(LMTables t, const double* xnew, const double* data, const T* J, const T* S, const T* b,
+cf_trial_kernel(LMTables t, const double* x, const double* data, const double* coef, const T* J, const T* S, const T* b,
                 const T* p, const double* E, const int32_t* start, double* tile_new, double* tile_pred) {
-  __shared__ double red[kTilePts / 32];
+  __shared__ double red[2][kTilePts];
   const int64_t tile = blockIdx.x;
   const int64_t i = t.tile_p0[tile] + threadIdx.x;
   double fsq = 0.0, pr = 0.0;
   if (i < t.tile_p0[tile + 1]) {
     const int k = t.tile_prob[tile];
     const int64_t Kc = (t.c0[k + 1] - t.c0[k]) / 2;
-    const double ti = xnew[i];
-    const int64_t seg = segment_of(ti, Kc);
-    double Bv[4];
-    bspline_values(ti - (double)seg, Bv);
-    const double* P = xnew + t.NP + t.c0[k] + 2 * seg;
-    double cx = 0, cy = 0;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      cx += Bv[q] * P[2 * q];
-      cy += Bv[q] * P[2 * q + 1];
-    }
-    const double fx = cx - data[2 * i], fy = cy - data[2 * i + 1];
-    fsq = fx * fx + fy * fy;
+    const T pt = p[i];
+    double u;
+    const int seg = segment_of(x[i] + (double)pt, Kc, u);
+    const double2* c = reinterpret_cast<const double2*>(coef + (t.c0[k] / 2 + seg) * kCoef);   // of x + p
+    const double2 x01 = c[0], x23 = c[1], y01 = c[3], y23 = c[4];
+    const double fx = fma(fma(fma(x23.y, u, x23.x), u, x01.y), u, x01.x) - data[2 * i];
+    const double fy = fma(fma(fma(y23.y, u, y23.x), u, y01.y), u, y01.x) - data[2 * i + 1];
+    fsq = fma(fx, fx, fy * fy);
     // (J p) at the linearisation point, with the system's own J, S and b; in the context
     // precision (a relative error of the order of its rounding in the predicted decrease moves
     // the gain ratio by as little, far below what the damping rule resolves)
-    const T pt = p[i];
     T jx = J[2 * i] * pt, jy = J[2 * i + 1] * pt;
     const T* Si = S + 16 * i;
     const T* pS = p + t.NP + start[i];
@@ -278,36 +270,37 @@ cf_trial_kernel(LMTables t, const double* xnew, const double* data, const T* J, 
     const T e = (T)E[i];
     pr = (double)(jx * b[2 * i] + jy * b[2 * i + 1] + e * e * pt * pt);
   }
-  const double s1 = block_sum(fsq, red);
-  __syncthreads();
-  const double s2 = block_sum(pr, red);
+  const double s1 = tile_sum(fsq, red[0]);
+  const double s2 = tile_sum(pr, red[1]);
   if (threadIdx.x == 0) {
     tile_new[tile] = s1;
     tile_pred[tile] = s2;
   }
 }
 
+constexpr int kUpdateThreads = 256;
 constexpr int kHist = 12;   // rho, accepted, log cost ratio of the last 4 steps
 
 __device__ __forceinline__ float clampf(float v, float lo, float hi) { return fminf(fmaxf(v, lo), hi); }
 
-// One warp per problem: costs, predicted decrease, gain ratio, then the damping update:
+// One CTA per problem (a warp, or eight for few problems): costs, predicted decrease, gain ratio, then on its first
+// warp the damping update:
 // Nielsen's rule, or after an accepted step (when the policy is on) lambda * multiplier of the
 // MLP's class for the features of the step history; stop rule.
 template <typename T>
 __global__ void lm_update_kernel(LMTables t, const double* tile_cost, const double* tile_new,
                                  const double* tile_pred, const double* E, const T* p, qrkit_lm_state* st,
                                  double ftol, int* ndone, MlpDev w, float* hist, float* feat) {
-  const int64_t k = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (k >= t.B) return;
+  __shared__ double part[3][kUpdateThreads / 32];
+  const int64_t k = blockIdx.x;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   double c = 0, cn = 0, pr = 0;
-  for (int64_t q = t.prob_tile0[k] + lane; q < t.prob_tile0[k + 1]; q += 32) {
+  for (int64_t q = t.prob_tile0[k] + threadIdx.x; q < t.prob_tile0[k + 1]; q += blockDim.x) {
     c += tile_cost[q];
     cn += tile_new[q];
     pr += tile_pred[q];
   }
-  for (int64_t j = t.NP + t.c0[k] + lane; j < t.NP + t.c0[k + 1]; j += 32) {
+  for (int64_t j = t.NP + t.c0[k] + threadIdx.x; j < t.NP + t.c0[k + 1]; j += blockDim.x) {
     const double pj = (double)p[j];
     pr += E[j] * E[j] * pj * pj;
   }
@@ -316,6 +309,21 @@ __global__ void lm_update_kernel(LMTables t, const double* tile_cost, const doub
     c += __shfl_xor_sync(0xffffffffu, c, d);
     cn += __shfl_xor_sync(0xffffffffu, cn, d);
     pr += __shfl_xor_sync(0xffffffffu, pr, d);
+  }
+  if (nw > 1) {
+    if (lane == 0) {
+      part[0][warp] = c;
+      part[1][warp] = cn;
+      part[2][warp] = pr;
+    }
+    __syncthreads();
+    if (warp > 0) return;
+    c = cn = pr = 0.0;
+    for (int q = 0; q < nw; ++q) {
+      c += part[0][q];
+      cn += part[1][q];
+      pr += part[2][q];
+    }
   }
   qrkit_lm_state s = st[k];
   if (s.done) {
@@ -384,10 +392,11 @@ __global__ void lm_update_kernel(LMTables t, const double* tile_cost, const doub
   if (s.done) atomicAdd(ndone, 1);
 }
 
-__global__ void lm_accept_kernel(LMTables t, const double* xnew, double* x, const qrkit_lm_state* st) {
+template <typename T>
+__global__ void lm_accept_kernel(LMTables t, const T* p, double* x, const qrkit_lm_state* st) {
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= t.N) return;
-  if (st[t.col_prob[j]].accepted) x[j] = xnew[j];
+  if (st[t.col_prob[j]].accepted) x[j] += (double)p[j];
 }
 
 inline unsigned nblk(int64_t n, int th) { return (unsigned)((n + th - 1) / th); }
@@ -412,30 +421,34 @@ qrkit_status lm_iteration(qrkit_ctx* ctx, double* x, int refine_steps, double ft
   T* p = (T*)L.p.ptr;
   double* d2 = (double*)L.d2.ptr;
   double* E = (double*)L.E.ptr;
-  QRKIT_CUDA_TRY(ctx, cudaMemsetAsync(d2 + t.NP, 0, (size_t)t.s * sizeof(double), st));
+  double* coef = (double*)L.coef.ptr;
+  int32_t* start = (int32_t*)ctx->plan.d_start.ptr;   // the model's starts lie in their segments
   QRKIT_CUDA_TRY(ctx, cudaMemsetAsync(L.ndone.ptr, 0, sizeof(int), st));
-  LM_LAUNCH(ctx, cf_eval_kernel<T><<<(unsigned)t.num_tiles, kTilePts, (size_t)L.sum_cols * sizeof(double), st>>>(
-                     t, x, L.data, J, Sv, b, (int32_t*)L.start.ptr, d2, (double*)L.tile_cost.ptr, L.sum_cols));
-  LM_LAUNCH(ctx, lm_damp_kernel<<<nblk(t.N, 256), 256, 0, st>>>(t, d2, S, E));
-  qrkit_status rc = window_start_copy(ctx, (const int32_t*)L.start.ptr);
+  LM_LAUNCH(ctx, cf_coef_kernel<T><<<nblk(t.s, 128), 128, 0, st>>>(t, x, (const T*)nullptr, coef));
+  LM_LAUNCH(ctx, cf_eval_kernel<T><<<(unsigned)t.num_tiles, kTilePts, 0, st>>>(t, x, L.data, coef, J, Sv, b, start,
+                                                                             (double*)L.tile_cost.ptr));
+  bool sorted = false;
+  qrkit_status rc = composed_sort_blocks(ctx, &sorted);
   if (rc != QRKIT_OK) return rc;
-  if ((rc = composed_factor_scaled(ctx, J, Sv, E, false)) != QRKIT_OK) return rc;
+  if (!sorted) return fail(ctx, QRKIT_ESTATE, "the LM plan has no block sort");
+  if ((rc = composed_window_sums(ctx, Sv, d2)) != QRKIT_OK) return rc;
+  LM_LAUNCH(ctx, lm_damp_kernel<T><<<(unsigned)(t.num_tiles + (t.s + kTilePts - 1) / kTilePts), kTilePts, 0, st>>>(
+                     t, J, d2, S, E));
+  if ((rc = composed_factor_scaled(ctx, J, Sv, E, true)) != QRKIT_OK) return rc;
   if ((rc = composed_solve(ctx, J, Sv, b, p, refine_steps)) != QRKIT_OK) return rc;
-  double* xn = (double*)L.xnew.ptr;
-  LM_LAUNCH(ctx, lm_xnew_kernel<T><<<nblk(t.N, 256), 256, 0, st>>>(t.N, x, p, xn));
+  LM_LAUNCH(ctx, cf_coef_kernel<T><<<nblk(t.s, 128), 128, 0, st>>>(t, x, p, coef));
   LM_LAUNCH(ctx, cf_trial_kernel<T><<<(unsigned)t.num_tiles, kTilePts, 0, st>>>(
-                     t, xn, L.data, J, Sv, b, p, E, (const int32_t*)L.start.ptr, (double*)L.tile_new.ptr,
-                     (double*)L.tile_pred.ptr));
+                     t, x, L.data, coef, J, Sv, b, p, E, start, (double*)L.tile_new.ptr, (double*)L.tile_pred.ptr));
   MlpDev w{};
   if (L.policy && ctx->mlp) {
     w.theta = (const float*)ctx->mlp->theta.ptr;
     w.wbf = (const __nv_bfloat16*)ctx->mlp->wbf.ptr;
   }
-  LM_LAUNCH(ctx, lm_update_kernel<T><<<nblk(t.B * 32, 128), 128, 0, st>>>(
+  LM_LAUNCH(ctx, lm_update_kernel<T><<<(unsigned)t.B, t.B >= 2 * ctx->num_sms ? 32 : kUpdateThreads, 0, st>>>(
                      t, (const double*)L.tile_cost.ptr, (const double*)L.tile_new.ptr,
                      (const double*)L.tile_pred.ptr, E, p, S, ftol, (int*)L.ndone.ptr, w, (float*)L.hist.ptr,
                      (float*)L.feat.ptr));
-  LM_LAUNCH(ctx, lm_accept_kernel<<<nblk(t.N, 256), 256, 0, st>>>(t, xn, x, S));
+  LM_LAUNCH(ctx, lm_accept_kernel<T><<<nblk(t.N, 256), 256, 0, st>>>(t, p, x, S));
   return QRKIT_OK;
 }
 
@@ -537,11 +550,6 @@ qrkit_status qrkit_lm_plan(qrkit_ctx* ctx, const qrkit_lm_problem* pr) {
   L.t.N = NP + s;
   L.h_p0 = p0;
   L.h_c0 = c0;
-  {
-    int64_t widest = 0;
-    for (size_t k = 0; k + 1 < c0.size(); ++k) widest = std::max<int64_t>(widest, c0[k + 1] - c0[k]);
-    L.sum_cols = widest <= kEvalSumCols ? (int)widest : 0;
-  }
   L.h_tile_p0.clear();
   L.h_prob_tile0.assign(B + 1, 0);
   std::vector<int32_t> tile_prob;
@@ -586,9 +594,9 @@ qrkit_status qrkit_lm_plan(qrkit_ctx* ctx, const qrkit_lm_problem* pr) {
   if ((rc = ensure(ctx, L.b, (size_t)2 * NP * es, "LM b")) != QRKIT_OK) return rc;
   if ((rc = ensure(ctx, L.p, (size_t)N * es, "LM p")) != QRKIT_OK) return rc;
   if ((rc = ensure(ctx, L.start, (size_t)NP * sizeof(int32_t), "LM starts")) != QRKIT_OK) return rc;
-  if ((rc = ensure(ctx, L.d2, (size_t)N * sizeof(double), "LM norms")) != QRKIT_OK) return rc;
+  if ((rc = ensure(ctx, L.d2, (size_t)s * sizeof(double), "LM norms")) != QRKIT_OK) return rc;
   if ((rc = ensure(ctx, L.E, (size_t)N * sizeof(double), "LM damping")) != QRKIT_OK) return rc;
-  if ((rc = ensure(ctx, L.xnew, (size_t)N * sizeof(double), "LM trial point")) != QRKIT_OK) return rc;
+  if ((rc = ensure(ctx, L.coef, (size_t)(s / 2) * kCoef * sizeof(double), "LM segments")) != QRKIT_OK) return rc;
   for (DevBuf* d : {&L.tile_cost, &L.tile_new, &L.tile_pred})
     if ((rc = ensure(ctx, *d, (size_t)nt * sizeof(double), "LM partial sums")) != QRKIT_OK) return rc;
   if ((rc = ensure(ctx, L.state, (size_t)B * sizeof(qrkit_lm_state), "LM state")) != QRKIT_OK) return rc;
@@ -608,17 +616,19 @@ qrkit_status qrkit_lm_linearize(qrkit_ctx* ctx, const double* x, void* J, void* 
   LM& L = *ctx->lm;
   const LMTables& t = L.t;
   cudaStream_t st = ctx->stream;
-  double* d2 = (double*)L.d2.ptr;
-  QRKIT_CUDA_TRY(ctx, cudaMemsetAsync(d2 + t.NP, 0, (size_t)t.s * sizeof(double), st));
-  if (ctx->precision == QRKIT_FP64)
-    cf_eval_kernel<double><<<(unsigned)t.num_tiles, kTilePts, (size_t)L.sum_cols * sizeof(double), st>>>(
-        t, x, L.data, (double*)L.J.ptr, (double*)L.S.ptr, (double*)L.b.ptr, (int32_t*)L.start.ptr, d2,
-        (double*)L.tile_cost.ptr, L.sum_cols);
-  else
-    cf_eval_kernel<float><<<(unsigned)t.num_tiles, kTilePts, (size_t)L.sum_cols * sizeof(double), st>>>(
-        t, x, L.data, (float*)L.J.ptr, (float*)L.S.ptr, (float*)L.b.ptr, (int32_t*)L.start.ptr, d2,
-        (double*)L.tile_cost.ptr, L.sum_cols);
-  ctx->launches += 1;
+  const double* coef = (const double*)L.coef.ptr;
+  if (ctx->precision == QRKIT_FP64) {
+    cf_coef_kernel<double><<<nblk(t.s, 128), 128, 0, st>>>(t, x, (const double*)nullptr, (double*)L.coef.ptr);
+    cf_eval_kernel<double><<<(unsigned)t.num_tiles, kTilePts, 0, st>>>(
+        t, x, L.data, coef, (double*)L.J.ptr, (double*)L.S.ptr, (double*)L.b.ptr, (int32_t*)L.start.ptr,
+        (double*)L.tile_cost.ptr);
+  } else {
+    cf_coef_kernel<float><<<nblk(t.s, 128), 128, 0, st>>>(t, x, (const float*)nullptr, (double*)L.coef.ptr);
+    cf_eval_kernel<float><<<(unsigned)t.num_tiles, kTilePts, 0, st>>>(
+        t, x, L.data, coef, (float*)L.J.ptr, (float*)L.S.ptr, (float*)L.b.ptr, (int32_t*)L.start.ptr,
+        (double*)L.tile_cost.ptr);
+  }
+  ctx->launches += 2;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());
   const size_t es = elem_size(ctx);
   if (J) QRKIT_CUDA_TRY(ctx, cudaMemcpyAsync(J, L.J.ptr, (size_t)2 * t.NP * es, cudaMemcpyDeviceToDevice, st));
