@@ -22,7 +22,6 @@ namespace {
 constexpr int kMaxRows = 16;   // augmented rows per block
 constexpr int kMaxCols = 8;    // columns per block
 constexpr int kChunk = 8;      // coupled columns processed per pass
-constexpr int kTileThreads = 256;
 
 __device__ __forceinline__ void record(int* status, int code) {
   if (status) atomicCAS(status, 0, code);
@@ -388,117 +387,6 @@ __global__ void reduced_damping_kernel(T* X0, int64_t ld0, int64_t row0, int s, 
   if (e >= (int64_t)count * s) return;
   const int c = (int)(e / count), j = (int)(e % count);
   X0[(int64_t)c * ld0 + row0 + j] = (damp && c == j) ? (T)(lam_half * D[nb + j]) : T(0);
-}
-
-// ---- TSQR tile factor: one CTA per row tile of a level matrix (column-major, ld) ----
-// Householder QR of the tile in shared memory; V below / R on and above the diagonal are
-// written back in place, tau to taus[tile * s + k], and the tile's R rows (upper
-// triangle, zeros below) to the next level's rows [tile * s, tile * s + min(r, s)).
-template <typename T>
-__global__ void __launch_bounds__(kTileThreads)
-tsqr_tile_kernel(T* X, int64_t ld, int64_t M, int s, int tile_rows, T* taus, T* Xn, int64_t ldn,
-                 int* status) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* A = reinterpret_cast<T*>(smem_raw);                 // tile_rows x s, ld = tile_rows
-  T* red = A + (size_t)tile_rows * s;                    // 32 partials
-  T* sh = red + 32;                                      // [0] tau, [1] beta, [2] scale
-  const int64_t r0 = (int64_t)blockIdx.x * tile_rows;
-  const int r = (int)(M - r0 < (int64_t)tile_rows ? M - r0 : (int64_t)tile_rows);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int nwarps = blockDim.x >> 5;
-  for (int e = tid; e < r * s; e += blockDim.x) {
-    const int c = e / r, i = e % r;
-    A[c * tile_rows + i] = X[(int64_t)c * ld + r0 + i];
-  }
-  __syncthreads();
-  const int kmax = min(r, s);
-  for (int k = 0; k < kmax; ++k) {
-    T* x = A + k * tile_rows;
-    if (warp == 0) {
-      T sq = 0;
-      for (int i = k + 1 + lane; i < r; i += 32) sq += x[i] * x[i];
-      for (int d = 16; d >= 1; d >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, d);
-      if (lane == 0) {
-        const T alpha = x[k];
-        const T norm = sqrt(alpha * alpha + sq);
-        T beta = 0, t = 0, scale = 0;
-        if (norm != T(0)) {
-          beta = alpha >= T(0) ? -norm : norm;
-          t = (beta - alpha) / beta;
-          scale = T(1) / (alpha - beta);
-        }
-        // a zero column inside a tile is not a singular R: a tile of stacked R rows can
-        // start below the diagonal; the final R_S is checked by the back-substitution
-        sh[0] = t;
-        sh[1] = beta;
-        sh[2] = scale;
-      }
-      __syncwarp();
-      const T scale = sh[2];
-      for (int i = k + 1 + lane; i < r; i += 32) x[i] *= scale;
-    }
-    __syncthreads();
-    const T t = sh[0];
-    for (int j = k + 1 + warp; j < s; j += nwarps) {
-      T* y = A + j * tile_rows;
-      T w = 0;
-      for (int i = k + 1 + lane; i < r; i += 32) w += x[i] * y[i];
-      for (int d = 16; d >= 1; d >>= 1) w += __shfl_xor_sync(0xffffffffu, w, d);
-      w = (w + y[k]) * t;
-      if (lane == 0) y[k] -= w;
-      for (int i = k + 1 + lane; i < r; i += 32) y[i] -= w * x[i];
-    }
-    if (tid == 0) {
-      x[k] = sh[1];
-      taus[(int64_t)blockIdx.x * s + k] = t;
-    }
-    __syncthreads();
-  }
-  for (int e = tid; e < r * s; e += blockDim.x) {
-    const int c = e / r, i = e % r;
-    X[(int64_t)c * ld + r0 + i] = A[c * tile_rows + i];
-  }
-  if (Xn) {
-    const int64_t n0 = (int64_t)blockIdx.x * s;
-    for (int e = tid; e < kmax * s; e += blockDim.x) {
-      const int c = e / kmax, i = e % kmax;
-      Xn[(int64_t)c * ldn + n0 + i] = (c >= i) ? A[c * tile_rows + i] : T(0);
-    }
-  }
-}
-
-// Q_tile^T applied to a level's rhs segment; the top min(r, s) entries go to the next level.
-template <typename T>
-__global__ void __launch_bounds__(kTileThreads)
-tsqr_apply_qt_kernel(const T* X, int64_t ld, int64_t M, int s, int tile_rows, const T* taus,
-                     T* rhs, T* rhs_next) {
-  __shared__ T red[32];
-  const int64_t r0 = (int64_t)blockIdx.x * tile_rows;
-  const int r = (int)(M - r0 < (int64_t)tile_rows ? M - r0 : (int64_t)tile_rows);
-  const int kmax = min(r, s);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  T* y = rhs + r0;
-  for (int k = 0; k < kmax; ++k) {
-    const T* x = X + (int64_t)k * ld + r0;
-    T w = 0;
-    for (int i = k + 1 + tid; i < r; i += blockDim.x) w += x[i] * y[i];
-    for (int d = 16; d >= 1; d >>= 1) w += __shfl_xor_sync(0xffffffffu, w, d);
-    if (lane == 0) red[warp] = w;
-    __syncthreads();
-    if (warp == 0) {
-      T v = lane < (int)(blockDim.x >> 5) ? red[lane] : T(0);
-      for (int d = 16; d >= 1; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-      if (lane == 0) red[0] = v;
-    }
-    __syncthreads();
-    const T wt = (red[0] + y[k]) * taus[(int64_t)blockIdx.x * s + k];
-    __syncthreads();
-    if (tid == 0) y[k] -= wt;
-    for (int i = k + 1 + tid; i < r; i += blockDim.x) y[i] -= wt * x[i];
-    __syncthreads();
-  }
-  if (rhs_next)
-    for (int i = tid; i < kmax; i += blockDim.x) rhs_next[(int64_t)blockIdx.x * s + i] = y[i];
 }
 
 // Per-block Q_i^T [b_i; 0]: top m -> ctop, bottom -> reduced rhs rows.  NA > 0: every block has
@@ -1287,11 +1175,8 @@ static qrkit_status factor_typed(qrkit_ctx* ctx, const void* J, const void* S, c
       TsqrLevel& L = C.levels[l];
       T* Xn = l + 1 < C.levels.size() ? (T*)C.levels[l + 1].X.ptr : nullptr;
       const int64_t ldn = l + 1 < C.levels.size() ? C.levels[l + 1].ld : 0;
-      const size_t smem = ((size_t)C.tile_rows * s + 64) * sizeof(T);
-      auto k = tsqr_tile_kernel<T>;
-      QRKIT_CUDA_TRY(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      LAUNCH(ctx, k<<<(unsigned)L.tiles, kTileThreads, smem, st>>>((T*)L.X.ptr, L.ld, L.M, s, C.tile_rows,
-                                                                  (T*)L.tau.ptr, Xn, ldn, ctx->d_status));
+      if ((rc = tsqr_tile<T>(ctx, (T*)L.X.ptr, L.ld, L.M, s, C.tile_rows, (T*)L.tau.ptr, Xn, ldn, L.tiles)) != QRKIT_OK)
+        return rc;
     }
   }
   return QRKIT_OK;
@@ -1338,8 +1223,9 @@ static qrkit_status solve_typed(qrkit_ctx* ctx, const void* J, const void* S, co
     for (size_t l = 0; l < C.levels.size() && !done; ++l) {
       TsqrLevel& L = C.levels[l];
       T* rn = l + 1 < C.levels.size() ? (T*)C.levels[l + 1].rhs.ptr : nullptr;
-      LAUNCH(ctx, tsqr_apply_qt_kernel<T><<<(unsigned)L.tiles, kTileThreads, 0, st>>>(
-                      (const T*)L.X.ptr, L.ld, L.M, s, C.tile_rows, (const T*)L.tau.ptr, (T*)L.rhs.ptr, rn));
+      qrkit_status rc = tsqr_qt<T>(ctx, (const T*)L.X.ptr, L.ld, L.M, s, C.tile_rows, (const T*)L.tau.ptr,
+                                   (T*)L.rhs.ptr, rn, L.tiles);
+      if (rc != QRKIT_OK) return rc;
     }
   }
   if (V.coupled == QRKIT_COUPLED_WINDOW && qt_only)
@@ -1739,7 +1625,7 @@ qrkit_status composed_layout(qrkit_ctx* ctx, size_t elem) {
     if (elem == sizeof(float) &&
         (rc = ensure(ctx, C.dref, dense_refine_bytes(P.rows, P.cols, s), "refinement sums")) != QRKIT_OK)
       return rc;
-    C.tile_rows = 256;
+    C.tile_rows = tsqr_rows(ctx, M0, s);
     const int tr = panels ? kPanelRows : C.tile_rows;
     if (panels) M0 = (M0 + 3) & ~int64_t(3);   // zero rows: every row count below is then a multiple of 4
     // the TSQR levels of a panel of pw columns over M rows, w columns wide (panel + trailing);

@@ -374,6 +374,15 @@ qrkit_status window_refine_gradient(qrkit_ctx* ctx, const ComposedView<T>& V, co
 // column sums of its S (s doubles, written); false in *done if the plan has no block sort.
 qrkit_status composed_sort_blocks(qrkit_ctx* ctx, bool* done);
 qrkit_status composed_window_sums(qrkit_ctx* ctx, const void* S, double* sq);
+// TSQR of a reduced block without column panels (tsqr.cu; s <= 64): rows of a tile for M rows; one level's tiles
+// (reflectors and R in place, tau, the R rows to Xn); and their Q^T on a right-hand side.
+int tsqr_rows(const qrkit_ctx* ctx, int64_t M, int s);
+template <typename T>
+qrkit_status tsqr_tile(qrkit_ctx* ctx, T* X, int64_t ld, int64_t M, int s, int rows, T* taus, T* Xn, int64_t ldn,
+                       int64_t tiles);
+template <typename T>
+qrkit_status tsqr_qt(qrkit_ctx* ctx, const T* X, int64_t ld, int64_t M, int s, int rows, const T* taus, T* rhs,
+                     T* rhs_next, int64_t tiles);
 // Column-panel TSQR (float; tsqr_tc.cu), one level of a 32-column panel in tiles of kPanelRows rows;
 // every pointer 16-byte aligned, every ld, row count and row offset a multiple of 4.
 // tsqr_panel_tile: reflectors and R in place, each tile's 32 x 32 T and G = Y^T Y (strict upper part,
