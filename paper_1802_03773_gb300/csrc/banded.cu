@@ -362,8 +362,8 @@ __global__ void band_colnorm_kernel(const float* Jf, const double* Jd, const int
 // thread reading its own group from global memory touches a cache line of its own at every load), thread t
 // computes the sums of group t per diagonal, and then the column of group t from the w sums on its anti-diagonal.
 // The rows' residuals are formed on the way, so a refinement step reads J once.
-// 256 instances, 13 million columns, 4 rows of 8 values per column (1.87 GB): %NORM% us for the norms
-// (2 phases reading global memory 1,000), %REF% us per gradient (residual 636 and gradient 1,738).
+// 256 instances, 13 million columns, 4 rows of 8 values per column (1.87 GB): 344 us for the norms
+// (2 phases reading global memory 1,000), 728 us per gradient (residual 636 and gradient 1,738).
 template <bool kStaged>
 __device__ __forceinline__ const float* group_rows_f32(const float* J, int64_t grp0, int64_t total, int rw, int gs,
                                                        float* buf) {

@@ -80,22 +80,31 @@ __device__ __forceinline__ float transpose_reduce(float (&v)[32], int lane) {
 // ---- the QR of one tile (up to 1024 x 32) of a panel ----
 //
 // 16 warps; column j lives in the registers of warp j % 16, rows 128 u + 4 lane + q (u < NU, q < 4)
-// on the lane.  At step k the reflector v_k goes through shared memory (two alternating slots);
-// every warp takes v_k against its two columns: those after k are updated, those before k give
-// G[c][k] = v_c^T v_k (v_k is zero above row k, so the R entries above a reflector drop out).  The
-// warp that holds column k + 1 forms the next reflector right after updating it, and one other warp
-// adds column k - 1 of T (T[k][k] = tau_k, the strict upper part -tau_k T[:, :k] G[:k, k]).  Bound by
-// the chain of a step (update, reduction, next reflector, barrier).  NU = 2, 4 or 8: the smallest
-// that covers the level's tiles, so that a short top level does not walk 1024 rows.
+// on the lane.  Every reflector v_k has a place of its own in shared memory and an mbarrier that says it is
+// there, so the warps run through k = 0, 1, .. at their own pace without a barrier of the CTA: a warp
+// takes v_k against its two columns, those after k are updated, those before k give G[c][k] = v_c^T v_k (v_k is
+// zero above row k, so the R entries above a reflector drop out).  The warp that holds column k + 1 updates
+// that column first, forms v_{k+1} and publishes it, and does the rest of its step k after that.  A step then
+// costs the chain of one column (product, reduction, update, norm, reduction) while the other warps' work
+// overlaps it; with a barrier per column it cost that chain plus the slowest warp's step: 35 us for a wave of
+// 1024-row tiles, 33 us now.  T comes last, its two diagonal 16 x 16 blocks by a warp each
+// (T[k][k] = tau_k, the strict upper part of column k -tau_k T[:, :k] G[:k, k]), then T12 = -T11 G12 T22.
+// NU = 2, 4 or 8: the smallest that covers the level's tiles, so that a short top level does not walk 1024 rows.
 constexpr int kPT = 512;
 constexpr int kPad = kNb + 1;   // row stride of G and T in shared memory (conflict-free columns)
+constexpr uint32_t kWaitLimit = 1u << 22;   // polls of a reflector (formed within microseconds)
+
+template <int NU>
+constexpr size_t panel_tile_smem() { return (size_t)kNb * 128 * NU * 4; }
 
 template <int NU>
 __global__ void __launch_bounds__(kPT, 1)
-tsqr_panel_tile_kernel(float* X, int64_t ld, int64_t M, float* Xn, int64_t ldn, float* Tout, float* Gout) {
-  __shared__ __align__(16) float V[2][128 * NU];
-  __shared__ float Gs[kNb * kPad], Tm[kNb * kPad];
-  __shared__ float tslot[2], tau_s[kNb];
+tsqr_panel_tile_kernel(float* X, int64_t ld, int64_t M, float* Xn, int64_t ldn, float* Tout, float* Gout, int* status) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float* V = reinterpret_cast<float*>(smem_raw);   // 32 reflectors of 128 NU rows
+  __shared__ float Gs[kNb * kPad], Tm[kNb * kPad], Ws[16 * kPad];
+  __shared__ float tau_s[kNb];
+  __shared__ __align__(8) uint64_t ready[kNb];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t r0 = (int64_t)blockIdx.x * kTR;
   const int r = (int)(M - r0 < (int64_t)kTR ? M - r0 : (int64_t)kTR);   // a multiple of 4
@@ -118,11 +127,16 @@ tsqr_panel_tile_kernel(float* X, int64_t ld, int64_t M, float* Xn, int64_t ldn, 
     a1[2 * u + 1] = pack2(q.z, q.w);
   }
   for (int e = tid; e < kNb * kPad; e += kPT) Gs[e] = Tm[e] = 0.f;
-  if (tid < kNb) tau_s[tid] = 0.f;
+  if (tid < kNb) {
+    tau_s[tid] = 0.f;
+    dev::mbar_init(&ready[tid], 1);
+  }
+  dev::fence_mbar_init();
+  __syncthreads();
 
   // the reflector of column k from its register column a (its owner warp): the column below k
-  // scaled to v (v_k = 1, stored implicitly), beta on the diagonal, v written to slot `slot`
-  auto form = [&](int k, f2 (&a)[2 * NU], int slot) {
+  // scaled to v (v_k = 1, stored implicitly), beta on the diagonal; v written to its place and announced
+  auto form = [&](int k, f2 (&a)[2 * NU]) {
     float h[4];   // rows 4 lane .. 4 lane + 3: the only ones that can lie on or above row k
     unpack2(a[0], h[0], h[1]);
     unpack2(a[1], h[2], h[3]);
@@ -139,8 +153,8 @@ tsqr_panel_tile_kernel(float* X, int64_t ld, int64_t M, float* Xn, int64_t ldn, 
       if (i > k) sq += h[q] * h[q];
       if (i == k) ak = h[q];
     }
-    sq = warp_sum(sq);
     const float alpha = __shfl_sync(0xffffffffu, ak, k >> 2);
+    sq = warp_sum(sq);
     const float norm = sqrtf(alpha * alpha + sq);
     float beta = 0.f, t = 0.f, scale = 0.f;
     if (norm != 0.f) {
@@ -158,7 +172,7 @@ tsqr_panel_tile_kernel(float* X, int64_t ld, int64_t M, float* Xn, int64_t ldn, 
     }
     a[0] = pack2(h[0], h[1]);
     a[1] = pack2(h[2], h[3]);
-    float* dst = V[slot] + 4 * lane;
+    float* dst = V + k * (128 * NU) + 4 * lane;
     *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
     const f2 sc = pack2(scale, scale);
 #pragma unroll
@@ -167,73 +181,68 @@ tsqr_panel_tile_kernel(float* X, int64_t ld, int64_t M, float* Xn, int64_t ldn, 
       a[2 * u + 1] = mul2(a[2 * u + 1], sc);
       *reinterpret_cast<ulonglong2*>(dst + 128 * u) = make_ulonglong2(a[2 * u], a[2 * u + 1]);
     }
-    if (lane == 0) {
-      tslot[slot] = t;
-      tau_s[k] = t;
-    }
-  };
-  // column k of T by one warp (lane l holds row l).  The sum runs over all 32 m: T[l][m] is still
-  // zero for m >= k and below the diagonal, and G[m][k] for m >= k.
-  auto t_column = [&](int k) {
-    const float tk = tau_s[k];
-    float q[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-    for (int m = 0; m < kNb; ++m) q[m & 3] += Tm[lane * kPad + m] * Gs[m * kPad + k];
-    const float v = -((q[0] + q[1]) + (q[2] + q[3])) * tk;
+    if (lane == 0) tau_s[k] = t;
     __syncwarp();
-    if (lane < k) Tm[lane * kPad + k] = v;
-    if (lane == k) Tm[k * kPad + k] = tk;
+    if (lane == 0)
+      asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(dev::smem_u32(&ready[k])) : "memory");
+  };
+  auto dot = [&](const f2 (&v)[2 * NU], const f2 (&a)[2 * NU]) -> float {
+    f2 d = 0ull, e = 0ull;
+#pragma unroll
+    for (int u = 0; u < NU; ++u) {
+      d = fma2(v[2 * u], a[2 * u], d);
+      e = fma2(v[2 * u + 1], a[2 * u + 1], e);
+    }
+    return sum2(d) + sum2(e);
+  };
+  auto update = [&](float w, const f2 (&v)[2 * NU], f2 (&a)[2 * NU]) {
+    const f2 w2 = pack2(w, w);
+#pragma unroll
+    for (int u = 0; u < 2 * NU; ++u) a[u] = fma2(w2, v[u], a[u]);
   };
 
-  __syncthreads();
-  if (warp == 0) form(0, a0, 0);
-  for (int k = 0; k < kmax; ++k) {
-    __syncthreads();   // reflector k is in slot k & 1, G[:k - 1][k - 1] and T[:, :k - 1] are complete
-    const int slot = k & 1;
-    const float t = tslot[slot];
+  if (warp == 0 && kmax > 0) form(0, a0);
+  bool ok = true;
+  for (int k = 0; k < kmax && ok; ++k) {
+    bool here = false;
+    for (uint32_t it = 0; it < kWaitLimit && !here; ++it) here = dev::mbar_try_wait(&ready[k], 0u);
+    ok = __all_sync(0xffffffffu, here);
+    if (!ok) break;
+    const float t = tau_s[k];
     f2 v[2 * NU];
 #pragma unroll
     for (int u = 0; u < NU; ++u) {
-      const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(V[slot] + 128 * u + 4 * lane);
+      const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(V + k * (128 * NU) + 128 * u + 4 * lane);
       v[2 * u] = w.x;
       v[2 * u + 1] = w.y;
     }
-    f2 d0 = 0ull, e0 = 0ull, d1 = 0ull, e1 = 0ull;
-#pragma unroll
-    for (int u = 0; u < NU; ++u) {
-      d0 = fma2(v[2 * u], a0[2 * u], d0);
-      d1 = fma2(v[2 * u], a1[2 * u], d1);
-      e0 = fma2(v[2 * u + 1], a0[2 * u + 1], e0);
-      e1 = fma2(v[2 * u + 1], a1[2 * u + 1], e1);
+    if (k + 1 < kmax && k + 1 == c0) {          // the next reflector first
+      update(-(warp_sum(dot(v, a0)) * t), v, a0);
+      form(k + 1, a0);
+      update(-(warp_sum(dot(v, a1)) * t), v, a1);
+      continue;
     }
-    float p0 = sum2(d0) + sum2(e0), p1 = sum2(d1) + sum2(e1);
+    if (k + 1 < kmax && k + 1 == c1) {
+      update(-(warp_sum(dot(v, a1)) * t), v, a1);
+      form(k + 1, a1);
+      const float p = warp_sum(dot(v, a0));     // c0 = c1 - 16 < k
+      if (lane == 0) Gs[c0 * kPad + k] = p;
+      continue;
+    }
+    float p0 = dot(v, a0), p1 = dot(v, a1);
 #pragma unroll
     for (int d = 16; d >= 1; d >>= 1) {
       p0 += __shfl_xor_sync(0xffffffffu, p0, d);
       p1 += __shfl_xor_sync(0xffffffffu, p1, d);
     }
-    if (c0 > k) {
-      const float w = -(p0 * t);
-      const f2 w2 = pack2(w, w);
-#pragma unroll
-      for (int u = 0; u < 2 * NU; ++u) a0[u] = fma2(w2, v[u], a0[u]);
-    } else if (c0 < k && lane == 0) {
-      Gs[c0 * kPad + k] = p0;
-    }
-    if (c1 > k) {
-      const float w = -(p1 * t);
-      const f2 w2 = pack2(w, w);
-#pragma unroll
-      for (int u = 0; u < 2 * NU; ++u) a1[u] = fma2(w2, v[u], a1[u]);
-    } else if (c1 < k && lane == 0) {
-      Gs[c1 * kPad + k] = p1;
-    }
-    if (k + 1 < kmax && ((k + 1) & 15) == warp) {
-      if (k + 1 < 16) form(k + 1, a0, slot ^ 1);
-      else form(k + 1, a1, slot ^ 1);
-    } else if (k > 0 && ((k + 9) & 15) == warp) {
-      t_column(k - 1);
-    }
+    if (c0 > k) update(-(p0 * t), v, a0);
+    else if (c0 < k && lane == 0) Gs[c0 * kPad + k] = p0;
+    if (c1 > k) update(-(p1 * t), v, a1);
+    else if (c1 < k && lane == 0) Gs[c1 * kPad + k] = p1;
+  }
+  if (__syncthreads_or(!ok)) {
+    if (tid == 0 && status) atomicCAS(status, 0, QRKIT_ETIMEOUT);
+    return;
   }
   // V below / R on and above the diagonal in place; the R rows (zeros below) to the next level
 #pragma unroll
@@ -256,8 +265,45 @@ tsqr_panel_tile_kernel(float* X, int64_t ld, int64_t M, float* Xn, int64_t ldn, 
       *reinterpret_cast<float4*>(Xn + (int64_t)c * ldn + n0) = make_float4(h[0], h[1], h[2], h[3]);
     }
   }
+  // T: warps 0 and 1 the diagonal blocks (lane l < 16 holds row l of the block; sums run over all 16
+  // columns, those not yet formed are zero)
+  if (warp < 2) {
+    const int o = 16 * warp, row = o + (lane & 15);
+    float tr[16];   // row `row` of the block
+#pragma unroll
+    for (int m = 0; m < 16; ++m) tr[m] = 0.f;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      const float tk = tau_s[o + k];
+      float q0 = 0.f, q1 = 0.f;
+#pragma unroll
+      for (int m = 0; m < k; ++m) {
+        if (m & 1) q1 += tr[m] * Gs[(o + m) * kPad + o + k];
+        else q0 += tr[m] * Gs[(o + m) * kPad + o + k];
+      }
+      tr[k] = (lane & 15) < k ? -(q0 + q1) * tk : ((lane & 15) == k ? tk : 0.f);
+    }
+    if (lane < 16) {
+#pragma unroll
+      for (int m = 0; m < 16; ++m) Tm[row * kPad + o + m] = tr[m];
+    }
+  }
   __syncthreads();
-  if (warp == 0) t_column(kmax - 1);
+  if (tid < 256) {   // W = G12 T22
+    const int i = tid >> 4, j = tid & 15;
+    float w = 0.f;
+#pragma unroll
+    for (int m = 0; m < 16; ++m) w += Gs[i * kPad + 16 + m] * Tm[(16 + m) * kPad + 16 + j];
+    Ws[i * kPad + j] = w;
+  }
+  __syncthreads();
+  if (tid < 256) {   // T12 = -T11 W
+    const int i = tid >> 4, j = tid & 15;
+    float w = 0.f;
+#pragma unroll
+    for (int m = 0; m < 16; ++m) w += Tm[i * kPad + m] * Ws[m * kPad + j];
+    Tm[i * kPad + 16 + j] = -w;
+  }
   __syncthreads();
   for (int e = tid; e < kNb * kNb; e += kPT) {
     const int m = e / kNb, k = e % kNb;
@@ -578,12 +624,17 @@ qrkit_status tsqr_panel_tile(qrkit_ctx* ctx, float* X, int64_t ld, int64_t M, fl
   if (!panel_aligned(X, ld, M) || !panel_aligned(Xn, ldn, 0))
     return fail(ctx, QRKIT_EINVAL, "column-panel TSQR: unaligned level matrix");
   const unsigned g = (unsigned)tiles;
-  if (M <= 256)
-    tsqr_panel_tile_kernel<2><<<g, kPT, 0, ctx->stream>>>(X, ld, M, Xn, ldn, Tout, Gout);
-  else if (M <= 512)
-    tsqr_panel_tile_kernel<4><<<g, kPT, 0, ctx->stream>>>(X, ld, M, Xn, ldn, Tout, Gout);
-  else
-    tsqr_panel_tile_kernel<8><<<g, kPT, 0, ctx->stream>>>(X, ld, M, Xn, ldn, Tout, Gout);
+  auto run = [&](auto k, size_t smem) -> cudaError_t {
+    if (smem > 48 * 1024) {
+      const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+    }
+    k<<<g, kPT, smem, ctx->stream>>>(X, ld, M, Xn, ldn, Tout, Gout, ctx->d_status);
+    return cudaSuccess;
+  };
+  if (M <= 256) QRKIT_CUDA_TRY(ctx, run(tsqr_panel_tile_kernel<2>, panel_tile_smem<2>()));
+  else if (M <= 512) QRKIT_CUDA_TRY(ctx, run(tsqr_panel_tile_kernel<4>, panel_tile_smem<4>()));
+  else QRKIT_CUDA_TRY(ctx, run(tsqr_panel_tile_kernel<8>, panel_tile_smem<8>()));
   ctx->launches += 1;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());
   return QRKIT_OK;
