@@ -77,20 +77,34 @@ __device__ __forceinline__ float transpose_reduce(float (&v)[32], int lane) {
   return v[0];
 }
 
+// Sums over the warp of four values per lane: lane l ends with the sum of v[l >> 3] (6 shuffles).
+__device__ __forceinline__ float sum4(const float (&v)[4], int lane) {
+  const bool up = (lane & 16) != 0, odd = (lane & 8) != 0;
+  float x = up ? v[2] : v[0], y = up ? v[3] : v[1];
+  x += __shfl_xor_sync(0xffffffffu, up ? v[0] : v[2], 16);
+  y += __shfl_xor_sync(0xffffffffu, up ? v[1] : v[3], 16);
+  float z = (odd ? y : x) + __shfl_xor_sync(0xffffffffu, odd ? x : y, 8);
+#pragma unroll
+  for (int d = 4; d >= 1; d >>= 1) z += __shfl_xor_sync(0xffffffffu, z, d);
+  return z;
+}
+
 // ---- the QR of one tile (up to 1024 x 32) of a panel ----
 //
-// 16 warps; column j lives in the registers of warp j % 16, rows 128 u + 4 lane + q (u < NU, q < 4)
-// on the lane.  Every reflector v_k has a place of its own in shared memory and an mbarrier that says it is
-// there, so the warps run through k = 0, 1, .. at their own pace without a barrier of the CTA: a warp
-// takes v_k against its two columns, those after k are updated, those before k give G[c][k] = v_c^T v_k (v_k is
-// zero above row k, so the R entries above a reflector drop out).  The warp that holds column k + 1 updates
-// that column first, forms v_{k+1} and publishes it, and does the rest of its step k after that.  A step then
-// costs the chain of one column (product, reduction, update, norm, reduction) while the other warps' work
-// overlaps it; with a barrier per column it cost that chain plus the slowest warp's step: 35 us for a wave of
-// 1024-row tiles, 33 us now.  T comes last, its two diagonal 16 x 16 blocks by a warp each
+// 8 warps; columns 4 w .. 4 w + 3 live in the registers of warp w, rows 128 u + 4 lane + q (u < NU, q < 4) on
+// the lane.  Every reflector v_k has a place of its own in shared memory and an mbarrier that says it is there, so
+// the warps run through k = 0, 1, .. at their own pace without a barrier of the CTA.  Reflectors before a
+// warp's columns update them; its own four it forms one after the other straight from its registers; against
+// those after them its columns give G[c][k] = v_c^T v_k (v_k is zero above row k, so the R entries above a
+// reflector drop out).  Bound by the chain from one reflector to the next.  With one column per warp and turn
+// (16 warps, column j on warp j % 16) that was 2,200 cycles: 340 until the next warp saw the reflector, 500 to load
+// it beside 15 others, 160 for the product, 200 and 190 for the two reductions, 250 for update and norm, 360 for
+// a root and two divisions, 260 to store; with four columns on a warp three of four reflectors skip the first two,
+// and one reciprocal root serves norm and tau.  A wave of 1024-row tiles of cold input: 38 us then, 30 us now.
+// T comes last, its two diagonal 16 x 16 blocks by a warp each
 // (T[k][k] = tau_k, the strict upper part of column k -tau_k T[:, :k] G[:k, k]), then T12 = -T11 G12 T22.
 // NU = 2, 4 or 8: the smallest that covers the level's tiles, so that a short top level does not walk 1024 rows.
-constexpr int kPT = 512;
+constexpr int kPT = 256;
 constexpr int kPad = kNb + 1;   // row stride of G and T in shared memory (conflict-free columns)
 constexpr uint32_t kWaitLimit = 1u << 22;   // polls of a reflector (formed within microseconds)
 
@@ -108,24 +122,20 @@ tsqr_panel_tile_kernel(float* X, int64_t ld, int64_t M, float* Xn, int64_t ldn, 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t r0 = (int64_t)blockIdx.x * kTR;
   const int r = (int)(M - r0 < (int64_t)kTR ? M - r0 : (int64_t)kTR);   // a multiple of 4
-  const int kmax = r < kNb ? r : kNb;
-  const int c0 = warp, c1 = warp + 16;
-  float* x0 = X + (int64_t)c0 * ld + r0 + 4 * lane;
-  float* x1 = X + (int64_t)c1 * ld + r0 + 4 * lane;
+  const int kmax = r < kNb ? r : kNb;                                   // so this too
+  const int c0 = 4 * warp;
+  float* x = X + (int64_t)c0 * ld + r0 + 4 * lane;
 
-  f2 a0[2 * NU], a1[2 * NU];
+  f2 a[4][2 * NU];
 #pragma unroll
-  for (int u = 0; u < NU; ++u) {
-    float4 p = make_float4(0.f, 0.f, 0.f, 0.f), q = p;
-    if (128 * u + 4 * lane < r) {
-      p = *reinterpret_cast<const float4*>(x0 + 128 * u);
-      q = *reinterpret_cast<const float4*>(x1 + 128 * u);
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int u = 0; u < NU; ++u) {
+      float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (128 * u + 4 * lane < r) p = *reinterpret_cast<const float4*>(x + (int64_t)j * ld + 128 * u);
+      a[j][2 * u] = pack2(p.x, p.y);
+      a[j][2 * u + 1] = pack2(p.z, p.w);
     }
-    a0[2 * u] = pack2(p.x, p.y);
-    a0[2 * u + 1] = pack2(p.z, p.w);
-    a1[2 * u] = pack2(q.x, q.y);
-    a1[2 * u + 1] = pack2(q.z, q.w);
-  }
   for (int e = tid; e < kNb * kPad; e += kPT) Gs[e] = Tm[e] = 0.f;
   if (tid < kNb) {
     tau_s[tid] = 0.f;
@@ -134,17 +144,18 @@ tsqr_panel_tile_kernel(float* X, int64_t ld, int64_t M, float* Xn, int64_t ldn, 
   dev::fence_mbar_init();
   __syncthreads();
 
-  // the reflector of column k from its register column a (its owner warp): the column below k
-  // scaled to v (v_k = 1, stored implicitly), beta on the diagonal; v written to its place and announced
-  auto form = [&](int k, f2 (&a)[2 * NU]) {
+  // the reflector of column k from its register column c: the column below k scaled to v (v_k = 1, stored
+  // implicitly), beta on the diagonal; v written to its place and announced; rows 4 lane .. + 3 of v to
+  // head, tau returned.  The root of n2 = norm^2 is n2 y with one Newton step, y = 1 / sqrt(n2).
+  auto form = [&](int k, f2 (&c)[2 * NU], f2 (&head)[2]) -> float {
     float h[4];   // rows 4 lane .. 4 lane + 3: the only ones that can lie on or above row k
-    unpack2(a[0], h[0], h[1]);
-    unpack2(a[1], h[2], h[3]);
+    unpack2(c[0], h[0], h[1]);
+    unpack2(c[1], h[2], h[3]);
     f2 s2 = 0ull, s3 = 0ull;
 #pragma unroll
     for (int u = 1; u < NU; ++u) {
-      s2 = fma2(a[2 * u], a[2 * u], s2);
-      s3 = fma2(a[2 * u + 1], a[2 * u + 1], s3);
+      s2 = fma2(c[2 * u], c[2 * u], s2);
+      s3 = fma2(c[2 * u + 1], c[2 * u + 1], s3);
     }
     float sq = sum2(s2) + sum2(s3), ak = 0.f;
 #pragma unroll
@@ -155,13 +166,15 @@ tsqr_panel_tile_kernel(float* X, int64_t ld, int64_t M, float* Xn, int64_t ldn, 
     }
     const float alpha = __shfl_sync(0xffffffffu, ak, k >> 2);
     sq = warp_sum(sq);
-    const float norm = sqrtf(alpha * alpha + sq);
-    float beta = 0.f, t = 0.f, scale = 0.f;
-    if (norm != 0.f) {
-      beta = alpha >= 0.f ? -norm : norm;
-      t = (beta - alpha) / beta;
-      scale = 1.f / (alpha - beta);
-    }
+    const float n2 = fmaf(alpha, alpha, sq);
+    const bool some = n2 != 0.f;
+    float y = rsqrtf(some ? n2 : 1.f);
+    float norm = n2 * y;
+    norm = fmaf(fmaf(-norm, norm, n2), 0.5f * y, norm);
+    y = fmaf(fmaf(-norm, y, 1.f), y, y);
+    const float beta = some ? (alpha >= 0.f ? -norm : norm) : 0.f;
+    const float t = some ? fmaf(fabsf(alpha), y, 1.f) : 0.f;        // (beta - alpha) / beta
+    const float scale = some ? __frcp_rn(alpha - beta) : 0.f;
     float v[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -170,75 +183,92 @@ tsqr_panel_tile_kernel(float* X, int64_t ld, int64_t M, float* Xn, int64_t ldn, 
       else if (i == k) h[q] = beta;
       v[q] = i > k ? h[q] : (i == k ? 1.f : 0.f);
     }
-    a[0] = pack2(h[0], h[1]);
-    a[1] = pack2(h[2], h[3]);
+    c[0] = pack2(h[0], h[1]);
+    c[1] = pack2(h[2], h[3]);
+    head[0] = pack2(v[0], v[1]);
+    head[1] = pack2(v[2], v[3]);
     float* dst = V + k * (128 * NU) + 4 * lane;
-    *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+    *reinterpret_cast<ulonglong2*>(dst) = make_ulonglong2(head[0], head[1]);
     const f2 sc = pack2(scale, scale);
 #pragma unroll
     for (int u = 1; u < NU; ++u) {
-      a[2 * u] = mul2(a[2 * u], sc);
-      a[2 * u + 1] = mul2(a[2 * u + 1], sc);
-      *reinterpret_cast<ulonglong2*>(dst + 128 * u) = make_ulonglong2(a[2 * u], a[2 * u + 1]);
+      c[2 * u] = mul2(c[2 * u], sc);
+      c[2 * u + 1] = mul2(c[2 * u + 1], sc);
+      *reinterpret_cast<ulonglong2*>(dst + 128 * u) = make_ulonglong2(c[2 * u], c[2 * u + 1]);
     }
     if (lane == 0) tau_s[k] = t;
     __syncwarp();
     if (lane == 0)
       asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(dev::smem_u32(&ready[k])) : "memory");
+    return t;
   };
-  auto dot = [&](const f2 (&v)[2 * NU], const f2 (&a)[2 * NU]) -> float {
+  // products with v (its first two pairs in head, the others in v) and its update of a column
+  auto dot = [&](const f2 (&head)[2], const f2 (&v)[2 * NU], const f2 (&c)[2 * NU]) -> float {
     f2 d = 0ull, e = 0ull;
 #pragma unroll
-    for (int u = 0; u < NU; ++u) {
-      d = fma2(v[2 * u], a[2 * u], d);
-      e = fma2(v[2 * u + 1], a[2 * u + 1], e);
+    for (int u = 1; u < NU; ++u) {
+      d = fma2(v[2 * u], c[2 * u], d);
+      e = fma2(v[2 * u + 1], c[2 * u + 1], e);
     }
+    d = fma2(head[0], c[0], d);
+    e = fma2(head[1], c[1], e);
     return sum2(d) + sum2(e);
   };
-  auto update = [&](float w, const f2 (&v)[2 * NU], f2 (&a)[2 * NU]) {
+  auto update = [&](float w, const f2 (&head)[2], const f2 (&v)[2 * NU], f2 (&c)[2 * NU]) {
     const f2 w2 = pack2(w, w);
+    c[0] = fma2(w2, head[0], c[0]);
+    c[1] = fma2(w2, head[1], c[1]);
 #pragma unroll
-    for (int u = 0; u < 2 * NU; ++u) a[u] = fma2(w2, v[u], a[u]);
+    for (int u = 2; u < 2 * NU; ++u) c[u] = fma2(w2, v[u], c[u]);
   };
-
-  if (warp == 0 && kmax > 0) form(0, a0);
-  bool ok = true;
-  for (int k = 0; k < kmax && ok; ++k) {
+  f2 v[2 * NU], head[2];
+  // waits for reflector k and loads it; false if it did not come
+  auto take = [&](int k) -> bool {
     bool here = false;
     for (uint32_t it = 0; it < kWaitLimit && !here; ++it) here = dev::mbar_try_wait(&ready[k], 0u);
-    ok = __all_sync(0xffffffffu, here);
-    if (!ok) break;
-    const float t = tau_s[k];
-    f2 v[2 * NU];
+    if (!__all_sync(0xffffffffu, here)) return false;
 #pragma unroll
     for (int u = 0; u < NU; ++u) {
       const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(V + k * (128 * NU) + 128 * u + 4 * lane);
       v[2 * u] = w.x;
       v[2 * u + 1] = w.y;
     }
-    if (k + 1 < kmax && k + 1 == c0) {          // the next reflector first
-      update(-(warp_sum(dot(v, a0)) * t), v, a0);
-      form(k + 1, a0);
-      update(-(warp_sum(dot(v, a1)) * t), v, a1);
-      continue;
-    }
-    if (k + 1 < kmax && k + 1 == c1) {
-      update(-(warp_sum(dot(v, a1)) * t), v, a1);
-      form(k + 1, a1);
-      const float p = warp_sum(dot(v, a0));     // c0 = c1 - 16 < k
-      if (lane == 0) Gs[c0 * kPad + k] = p;
-      continue;
-    }
-    float p0 = dot(v, a0), p1 = dot(v, a1);
+    head[0] = v[0];
+    head[1] = v[1];
+    return true;
+  };
+
+  bool ok = true;
+  for (int k = 0; k < kmax && k < c0; ++k) {
+    if (!(ok = take(k))) break;
+    const float t = -tau_s[k];
+    float p[4];
 #pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) {
-      p0 += __shfl_xor_sync(0xffffffffu, p0, d);
-      p1 += __shfl_xor_sync(0xffffffffu, p1, d);
+    for (int j = 0; j < 4; ++j) p[j] = dot(head, v, a[j]);
+    const float z = sum4(p, lane);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) update(__shfl_sync(0xffffffffu, z, 8 * j) * t, head, v, a[j]);
+  }
+  if (ok && c0 < kmax) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float t = -form(c0 + i, a[i], head);
+      float p[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) p[j] = j != i ? dot(head, a[i], a[j]) : 0.f;
+      const float z = sum4(p, lane);
+#pragma unroll
+      for (int j = i + 1; j < 4; ++j) update(__shfl_sync(0xffffffffu, z, 8 * j) * t, head, a[i], a[j]);
+      if ((lane & 7) == 0 && (lane >> 3) < i) Gs[(c0 + (lane >> 3)) * kPad + c0 + i] = z;
     }
-    if (c0 > k) update(-(p0 * t), v, a0);
-    else if (c0 < k && lane == 0) Gs[c0 * kPad + k] = p0;
-    if (c1 > k) update(-(p1 * t), v, a1);
-    else if (c1 < k && lane == 0) Gs[c1 * kPad + k] = p1;
+  }
+  for (int k = c0 + 4; k < kmax && ok; ++k) {
+    if (!(ok = take(k))) break;
+    float p[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) p[j] = dot(head, v, a[j]);
+    const float z = sum4(p, lane);
+    if ((lane & 7) == 0) Gs[(c0 + (lane >> 3)) * kPad + k] = z;
   }
   if (__syncthreads_or(!ok)) {
     if (tid == 0 && status) atomicCAS(status, 0, QRKIT_ETIMEOUT);
@@ -246,23 +276,22 @@ tsqr_panel_tile_kernel(float* X, int64_t ld, int64_t M, float* Xn, int64_t ldn, 
   }
   // V below / R on and above the diagonal in place; the R rows (zeros below) to the next level
 #pragma unroll
-  for (int u = 0; u < NU; ++u)
-    if (128 * u + 4 * lane < r) {
-      *reinterpret_cast<ulonglong2*>(x0 + 128 * u) = make_ulonglong2(a0[2 * u], a0[2 * u + 1]);
-      *reinterpret_cast<ulonglong2*>(x1 + 128 * u) = make_ulonglong2(a1[2 * u], a1[2 * u + 1]);
-    }
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int u = 0; u < NU; ++u)
+      if (128 * u + 4 * lane < r)
+        *reinterpret_cast<ulonglong2*>(x + (int64_t)j * ld + 128 * u) = make_ulonglong2(a[j][2 * u], a[j][2 * u + 1]);
   if (4 * lane < kmax) {
     const int64_t n0 = (int64_t)blockIdx.x * kNb + 4 * lane;
 #pragma unroll
-    for (int cc = 0; cc < 2; ++cc) {
-      const int c = cc ? c1 : c0;
+    for (int j = 0; j < 4; ++j) {
       float h[4];
-      unpack2(cc ? a1[0] : a0[0], h[0], h[1]);
-      unpack2(cc ? a1[1] : a0[1], h[2], h[3]);
+      unpack2(a[j][0], h[0], h[1]);
+      unpack2(a[j][1], h[2], h[3]);
 #pragma unroll
       for (int q = 0; q < 4; ++q)
-        if (4 * lane + q > c) h[q] = 0.f;
-      *reinterpret_cast<float4*>(Xn + (int64_t)c * ldn + n0) = make_float4(h[0], h[1], h[2], h[3]);
+        if (4 * lane + q > c0 + j) h[q] = 0.f;
+      *reinterpret_cast<float4*>(Xn + (int64_t)(c0 + j) * ldn + n0) = make_float4(h[0], h[1], h[2], h[3]);
     }
   }
   // T: warps 0 and 1 the diagonal blocks (lane l < 16 holds row l of the block; sums run over all 16
@@ -289,7 +318,7 @@ tsqr_panel_tile_kernel(float* X, int64_t ld, int64_t M, float* Xn, int64_t ldn, 
     }
   }
   __syncthreads();
-  if (tid < 256) {   // W = G12 T22
+  {   // W = G12 T22
     const int i = tid >> 4, j = tid & 15;
     float w = 0.f;
 #pragma unroll
@@ -297,7 +326,7 @@ tsqr_panel_tile_kernel(float* X, int64_t ld, int64_t M, float* Xn, int64_t ldn, 
     Ws[i * kPad + j] = w;
   }
   __syncthreads();
-  if (tid < 256) {   // T12 = -T11 W
+  {   // T12 = -T11 W
     const int i = tid >> 4, j = tid & 15;
     float w = 0.f;
 #pragma unroll
