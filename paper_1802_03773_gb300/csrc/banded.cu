@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "device_util.cuh"
+#include "f32x2.cuh"
 #include "internal.h"
 
 namespace qrkit {
@@ -363,7 +364,8 @@ __global__ void band_colnorm_kernel(const float* Jf, const double* Jd, const int
 // computes the sums of group t per diagonal, and then the column of group t from the w sums on its anti-diagonal.
 // The rows' residuals are formed on the way, so a refinement step reads J once.
 // 256 instances, 13 million columns, 4 rows of 8 values per column (1.87 GB): 344 us for the norms
-// (2 phases reading global memory 1,000), 728 us per gradient (residual 636 and gradient 1,738).
+// (2 phases reading global memory 1,000), 633 us per gradient (residual 636 and gradient 1,738; 728 with
+// scalar sums), bound by the additions of the pair sums.
 template <bool kStaged>
 __device__ __forceinline__ const float* group_rows_f32(const float* J, int64_t grp0, int64_t total, int rw, int gs,
                                                        float* buf) {
@@ -523,31 +525,74 @@ __global__ void __launch_bounds__(256) band_grad_f32_kernel(BandGroups B, const 
     float xv[8];
 #pragma unroll
     for (int t = 0; t < 8; ++t) xv[t] = t < nx ? -xs[tid + t] : 0.f;
-    for (int q = 0; q < B.rpc; ++q) {
-      float a[8];
-      row_f32<kW8, 8>(a, rows + (int64_t)q * w, w);
-      float sh = b[grp * B.rpc + q], sl = 0.f;
+    if constexpr (kW8) {
+      // two entries at a time; the even and the odd entries' residual sums are added at the end of the row
+      dev::f2 x2[4], nx2[4], h2[4], l2[4];
 #pragma unroll
-      for (int t = 0; t < 8; ++t) {
-        if (t < nx) {
-          const float pr = __fmul_rn(a[t], xv[t]);
-          const float pe = __fmaf_rn(a[t], xv[t], -pr);
-          float tt, e;
-          dev::two_sum(sh, pr, tt, e);
-          sh = tt;
-          sl = __fadd_rn(sl, __fadd_rn(e, pe));
+      for (int t = 0; t < 4; ++t) {
+        x2[t] = dev::pack2(xv[2 * t], xv[2 * t + 1]);
+        nx2[t] = dev::pack2(-xv[2 * t], -xv[2 * t + 1]);
+        h2[t] = l2[t] = 0ull;
+      }
+      for (int q = 0; q < B.rpc; ++q) {
+        dev::f2 a[4];
+        const ulonglong2* row = reinterpret_cast<const ulonglong2*>(rows + 8 * q);
+        const ulonglong2 lo = row[0], hi = row[1];
+        a[0] = lo.x;
+        a[1] = lo.y;
+        a[2] = hi.x;
+        a[3] = hi.y;
+        if (nx < 8) {   // an entry past the instance's last column belongs to no column
+#pragma unroll
+          for (int t = 0; t < 4; ++t) {
+            float u, v;
+            dev::unpack2(a[t], u, v);
+            a[t] = dev::pack2(2 * t < nx ? u : 0.f, 2 * t + 1 < nx ? v : 0.f);
+          }
         }
+        dev::f2 sh = dev::pack2(b[grp * B.rpc + q], 0.f), sl = 0ull;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) dev::dot2_add2(sh, sl, a[t], x2[t], nx2[t]);
+        float he, ho, s, e;
+        dev::unpack2(sh, he, ho);
+        dev::two_sum(he, ho, s, e);
+        const float c = dev::sum2(sl) + e;
+        const dev::f2 s2 = dev::pack2(s, s), ns2 = dev::pack2(-s, -s), c2 = dev::pack2(c, c);
+#pragma unroll
+        for (int t = 0; t < 4; ++t) dev::dot2_add2(h2[t], l2[t], a[t], s2, ns2, c2);
       }
 #pragma unroll
-      for (int t = 0; t < 8; ++t) {
-        if (t < nx) {   // an entry past the instance's last column belongs to no column
-          const float pr = __fmul_rn(a[t], sh);
-          float pe = __fmaf_rn(a[t], sh, -pr);
-          pe = __fmaf_rn(a[t], sl, pe);
-          float tt, e;
-          dev::two_sum(hs[t], pr, tt, e);
-          hs[t] = tt;
-          hc[t] = __fadd_rn(hc[t], __fadd_rn(e, pe));
+      for (int t = 0; t < 4; ++t) {
+        dev::unpack2(h2[t], hs[2 * t], hs[2 * t + 1]);
+        dev::unpack2(l2[t], hc[2 * t], hc[2 * t + 1]);
+      }
+    } else {
+      for (int q = 0; q < B.rpc; ++q) {
+        float a[8];
+        row_f32<kW8, 8>(a, rows + (int64_t)q * w, w);
+        float sh = b[grp * B.rpc + q], sl = 0.f;
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+          if (t < nx) {
+            const float pr = __fmul_rn(a[t], xv[t]);
+            const float pe = __fmaf_rn(a[t], xv[t], -pr);
+            float tt, e;
+            dev::two_sum(sh, pr, tt, e);
+            sh = tt;
+            sl = __fadd_rn(sl, __fadd_rn(e, pe));
+          }
+        }
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+          if (t < nx) {   // an entry past the instance's last column belongs to no column
+            const float pr = __fmul_rn(a[t], sh);
+            float pe = __fmaf_rn(a[t], sh, -pr);
+            pe = __fmaf_rn(a[t], sl, pe);
+            float tt, e;
+            dev::two_sum(hs[t], pr, tt, e);
+            hs[t] = tt;
+            hc[t] = __fadd_rn(hc[t], __fadd_rn(e, pe));
+          }
         }
       }
     }
@@ -559,12 +604,18 @@ __global__ void __launch_bounds__(256) band_grad_f32_kernel(BandGroups B, const 
   if (tid < w - 1 || !have) return;
   const int64_t j = grp - B.inst_col0[k];
   float s = 0.f, c = 0.f;
-  for (int t = 0; t < w && t <= j; ++t) {
+  auto diagonal = [&](int t) {
     const float2 v = S[(tid - t) * (w + 1) + t];
     float tt, e;
     dev::two_sum(s, v.x, tt, e);
     s = tt;
     c = __fadd_rn(c, __fadd_rn(e, v.y));
+  };
+  if (kW8 && j >= 7) {
+#pragma unroll
+    for (int t = 0; t < 8; ++t) diagonal(t);
+  } else {
+    for (int t = 0; t < w && t <= j; ++t) diagonal(t);
   }
   if (lam_h > 0.f) {   // - lambda D^2 x, all factors but x pairs
     const float2 d2 = D2[grp];

@@ -20,6 +20,7 @@
 #include <algorithm>
 
 #include "device_util.cuh"
+#include "f32x2.cuh"
 #include "internal.h"
 
 namespace qrkit {
@@ -29,31 +30,12 @@ constexpr int kTR = kPanelRows;   // tile rows
 constexpr int kNb = kPanelCols;   // panel width
 static_assert(kTR == 1024 && kNb == 32, "the kernels' thread layouts");
 
-// Two floats at a time (fma.rn.f32x2 and mul.rn.f32x2): half the instructions of the scalar forms.
-using f2 = unsigned long long;
-__device__ __forceinline__ f2 pack2(float x, float y) {
-  f2 d;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
-  return d;
-}
-__device__ __forceinline__ void unpack2(f2 d, float& x, float& y) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(d));
-}
-__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
-  f2 d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
-  f2 d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ float sum2(f2 d) {
-  float x, y;
-  unpack2(d, x, y);
-  return x + y;
-}
+using dev::f2;
+using dev::fma2;
+using dev::mul2;
+using dev::pack2;
+using dev::sum2;
+using dev::unpack2;
 
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
