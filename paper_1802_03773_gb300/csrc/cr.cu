@@ -33,6 +33,7 @@
 #include <vector>
 
 #include "device_util.cuh"
+#include "f32x2.cuh"
 #include "internal.h"
 
 namespace qrkit {
@@ -563,34 +564,111 @@ __device__ __forceinline__ void decode(int64_t it, int64_t& k, int64_t& i, int& 
 //   2. rows 0..7 of B' into A, which makes A the 8 rows of R    -> rows on left and right
 //   3. those rows triangular in the left columns, and the right-only rows of step 1 into rows 8..15 of B:
 //      the new 16-row block row on (left, right).
-// About 650 instructions per front and lane group of four fronts' warp, where a 32-row front on a whole warp with
-// its sums reduced by shuffles took 4,000.
+// Rows are taken two at a time (f32x2): 13 million columns of 256 instances spend 1,505 us on the fronts against 1,641
+// with scalar rows.  A 32-row front on a whole warp with
+// its sums reduced by shuffles took six times the instructions.
 constexpr int kItemThreads = kCB;
 
+// Eight rows of a column on a lane: two rows per operation for float.  The ranges [r0, r1) are known at compile time
+// once the loops are unrolled; a range that begins or ends inside a pair takes the pair, whose other row is
+// zero in v.
+template <typename T>
+struct Rows;
+template <>
+struct Rows<float> {
+  dev::f2 p[4];
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) p[i] = 0ull;
+  }
+  __device__ __forceinline__ float get(int r) const {
+    float x, y;
+    dev::unpack2(p[r >> 1], x, y);
+    return r & 1 ? y : x;
+  }
+  __device__ __forceinline__ void set(int r, float v) {
+    float x, y;
+    dev::unpack2(p[r >> 1], x, y);
+    p[r >> 1] = r & 1 ? dev::pack2(x, v) : dev::pack2(v, y);
+  }
+  __device__ __forceinline__ void scale(const Rows& x, float f, int r0, int r1) {
+    const dev::f2 f2v = dev::pack2(f, f);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (2 * i + 1 >= r0 && 2 * i < r1) p[i] = dev::mul2(x.p[i], f2v);
+  }
+  __device__ __forceinline__ float dot(const Rows& x, int r0, int r1) const {
+    dev::f2 d = 0ull;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (2 * i + 1 >= r0 && 2 * i < r1) d = dev::fma2(p[i], x.p[i], d);
+    return dev::sum2(d);
+  }
+  __device__ __forceinline__ void add(float w, const Rows& v, int r0, int r1) {   // += w v
+    const dev::f2 w2 = dev::pack2(w, w);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (2 * i + 1 >= r0 && 2 * i < r1) p[i] = dev::fma2(w2, v.p[i], p[i]);
+  }
+};
+template <>
+struct Rows<double> {
+  double v[8];
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int r = 0; r < 8; ++r) v[r] = 0.0;
+  }
+  __device__ __forceinline__ double get(int r) const { return v[r]; }
+  __device__ __forceinline__ void set(int r, double x) { v[r] = x; }
+  __device__ __forceinline__ void scale(const Rows& x, double f, int r0, int r1) {
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+      if (r >= r0 && r < r1) v[r] = x.v[r] * f;
+  }
+  __device__ __forceinline__ double dot(const Rows& x, int r0, int r1) const {
+    double d = 0.0;
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+      if (r >= r0 && r < r1) d += v[r] * x.v[r];
+    return d;
+  }
+  __device__ __forceinline__ void add(double w, const Rows& x, int r0, int r1) {
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+      if (r >= r0 && r < r1) v[r] += w * x.v[r];
+  }
+};
+
 // Columns j of A (rows 0..7) and B (rows 0..7, 8..15) of block row `it`, and its rhs.
-template <typename T, bool kCompressed>
-__device__ __forceinline__ void load_block_row(const T* base, int64_t it, int j, T (&a)[8], T (&bl)[8], T (&bh)[8],
-                                               T (&cl)[8], T (&ch)[8]) {
+template <typename T, bool kCompressed, class RA, class RL, class RH, class RC, class RD>
+__device__ __forceinline__ void load_block_row(const T* base, int64_t it, int j, RA&& a, RL&& bl, RH&& bh, RC&& cl,
+                                               RD&& ch) {
+  T c0[8], c1[8];
   if constexpr (kCompressed) {
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
       const T v = base[e0_at<T>(it, 8 * r + ((j - r) & 7))];   // column j of A for j >= r, of B for j < r
-      a[r] = j >= r ? v : T(0);
-      bl[r] = j < r ? v : T(0);
-      bh[r] = base[e0_at<T>(it, 64 + 8 * r + j)];
+      a(r, j >= r ? v : T(0));
+      bl(r, j < r ? v : T(0));
+      bh(r, base[e0_at<T>(it, 64 + 8 * r + j)]);
     }
-    load_e0(cl, base, it, 128);
-    load_e0(ch, base, it, 136);
+    load_e0(c0, base, it, 128);
+    load_e0(c1, base, it, 136);
   } else {
     const T* F = base + it * kFW;
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
-      a[r] = F[8 * r + j];
-      bl[r] = F[64 + 8 * r + j];
-      bh[r] = F[128 + 8 * r + j];
+      a(r, F[8 * r + j]);
+      bl(r, F[64 + 8 * r + j]);
+      bh(r, F[128 + 8 * r + j]);
     }
-    load8(cl, F + 192);
-    load8(ch, F + 200);
+    load8(c0, F + 192);
+    load8(c1, F + 200);
+  }
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    cl(r, c0[r]);
+    ch(r, c1[r]);
   }
 }
 
@@ -602,115 +680,90 @@ __device__ __forceinline__ T lane_of(const T (&v)[8], int j) {   // v[j] for a l
     if (j == q) x = v[q];
   return x;
 }
-
 template <typename T>
-__device__ __forceinline__ void store_block_row(T* F, int j, const T (&a)[8], const T (&bl)[8], const T (&bh)[8],
-                                                const T (&cl)[8], const T (&ch)[8]) {
+__device__ __forceinline__ T lane_of(const Rows<T>& v, int j) {
+  T x = v.get(0);
 #pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    F[8 * r + j] = a[r];
-    F[64 + 8 * r + j] = bl[r];
-    F[128 + 8 * r + j] = bh[r];
-  }
-  F[192 + j] = lane_of(cl, j);
-  F[200 + j] = lane_of(ch, j);
-}
-
-// w = tau (p + sum_r v_r x_r); p -= w, x_r -= w v_r over M rows.
-template <typename T, int M>
-__device__ __forceinline__ void apply_reflector(T tau, const T (&v)[8], T& p, T (&x)[8], int from = 0) {
-  T w = p;
-#pragma unroll
-  for (int r = 0; r < 8; ++r)
-    if (r >= from && r < M) w += v[r] * x[r];
-  w *= tau;
-  p -= w;
-#pragma unroll
-  for (int r = 0; r < 8; ++r)
-    if (r >= from && r < M) x[r] -= w * v[r];
+  for (int q = 1; q < 8; ++q)
+    if (j == q) x = v.get(q);
+  return x;
 }
 
 // One item of level `level`: block i of instance k.  The lanes add their share of the residual it leaves to res.
+//
+// The rows that a step's reflectors meet one at a time (A; then pa, bh as pivots) are scalars or halves of a pair, the
+// rows below in Rows.  A reflector of column q must leave the columns before it alone; their entries below
+// the diagonal are not cleared one by one: tj, the factor of a lane's own column, is zero on lanes up to q.
 template <typename T, bool kCompressed>
 __device__ __forceinline__ void cr_item(const CRArgs<T>& A, int64_t k, int64_t i, int kind, int level, const T* Fc,
                                         T* Fn, int j, unsigned gmask, ResidualSum<T>& res) {
   const int64_t b0 = A.blk0[k];
   T a[8], bl[8], bh[8], cl[8], ch[8];
-  load_block_row<T, kCompressed>(Fc, b0 + i, j, a, bl, bh, cl, ch);
+  auto to = [](T (&x)[8]) { return [&x](int r, T v) { x[r] = v; }; };
+  load_block_row<T, kCompressed>(Fc, b0 + i, j, to(a), to(bl), to(bh), to(cl), to(ch));
   if (kind == 1) {   // unpaired last block row: moves up
-    store_block_row(Fn + (b0 + i / 2) * kFW, j, a, bl, bh, cl, ch);
+    T* F = Fn + (b0 + i / 2) * kFW;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      F[8 * r + j] = a[r];
+      F[64 + 8 * r + j] = bl[r];
+      F[128 + 8 * r + j] = bh[r];
+    }
+    F[192 + j] = lane_of(cl, j);
+    F[200 + j] = lane_of(ch, j);
     return;
   }
   T* R = A.Rb + (b0 + (i << level)) * kRW;
-  T rl[8];   // R's left part
-#pragma unroll
-  for (int r = 0; r < 8; ++r) rl[r] = T(0);
   if (kind == 0) {
-    T pa[8], pl[8], ph[8], dl[8], dh[8], rr[8], lr[8];
-    load_block_row<T, kCompressed>(Fc, b0 + i - 1, j, pa, pl, ph, dl, dh);
+    Rows<T> pa, pl, ph, dl, dh, rr, lr, v, x;
+    auto rows = [](Rows<T>& y) { return [&y](int r, T u) { y.set(r, u); }; };
+    load_block_row<T, kCompressed>(Fc, b0 + i - 1, j, rows(pa), rows(pl), rows(ph), rows(dl), rows(dh));
+    rr.zero();   // right parts of the rows of B'
+    lr.zero();
+    T rl[8];     // R's left part
+    // the reflector of column q: pivot `piv` and rows [r0, r1) of y, both of lane q; v's other rows of touched pairs zero
+    T tj, t, beta;
+    auto reflector = [&](int q, T piv, const Rows<T>& y, int r0, int r1) {
+      const T p = __shfl_sync(gmask, piv, q, kItemThreads);
+      x.zero();
 #pragma unroll
-    for (int r = 0; r < 8; ++r) rr[r] = lr[r] = T(0);   // right parts of the rows of B'
-    T v[8], x[8];
+      for (int r = 0; r < 8; ++r)
+        if (r >= r0 && r < r1) x.set(r, __shfl_sync(gmask, y.get(r), q, kItemThreads));
+      const Reflector<T> h(p, x.dot(x, r0, r1));
+      v.scale(x, h.scale, r0, r1);
+      t = -h.tau;
+      tj = j > q ? t : T(0);
+      beta = h.beta;
+    };
+    // y, and the pivot p of its column, with the factor f
+    auto apply = [&](T f, T& p, Rows<T>& y, int r0, int r1) {
+      const T w = f * (p + v.dot(y, r0, r1));
+      p += w;
+      y.add(w, v, r0, r1);
+    };
+    auto apply_at = [&](T f, int q, Rows<T>& y, int r0, int r1) {   // the pivot is row q of y itself
+      T p = y.get(q);
+      const T w = f * (p + v.dot(y, r0, r1));
+      y.add(w, v, r0, r1);
+      y.set(q, p + w);
+    };
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      T s2 = T(0);
-      const T p = __shfl_sync(gmask, a[q], q, kItemThreads);
-#pragma unroll
-      for (int r = 0; r <= q; ++r) {
-        x[r] = __shfl_sync(gmask, ph[r], q, kItemThreads);
-        s2 += x[r] * x[r];
-      }
-      const Reflector<T> h(p, s2);
-#pragma unroll
-      for (int r = 0; r < 8; ++r) v[r] = r <= q ? x[r] * h.scale : T(0);
-      {
-        T w = a[q], y = bl[q], c = cl[q];
-#pragma unroll
-        for (int r = 0; r <= q; ++r) {
-          w += v[r] * ph[r];
-          y += v[r] * rr[r];
-          c += v[r] * dh[r];
-        }
-        w *= h.tau;
-        y *= h.tau;
-        c *= h.tau;
-        a[q] -= w;
-        bl[q] -= y;
-        cl[q] -= c;
-#pragma unroll
-        for (int r = 0; r <= q; ++r) {
-          ph[r] -= w * v[r];
-          rr[r] -= y * v[r];
-          dh[r] -= c * v[r];
-        }
-      }
-      if (j == q) {
-        a[q] = h.beta;
-#pragma unroll
-        for (int r = 0; r <= q; ++r) ph[r] = T(0);
-      }
+      reflector(q, a[q], ph, 0, q + 1);
+      apply(tj, a[q], ph, 0, q + 1);
+      apply(t, bl[q], rr, 0, q + 1);
+      apply(t, cl[q], dh, 0, q + 1);
+      if (j == q) a[q] = beta;
     }
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      T s2 = T(0);
-      const T p = __shfl_sync(gmask, a[q], q, kItemThreads);
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        x[r] = __shfl_sync(gmask, pl[r], q, kItemThreads);
-        s2 += x[r] * x[r];
-      }
-      const Reflector<T> h(p, s2);
-#pragma unroll
-      for (int r = 0; r < 8; ++r) v[r] = x[r] * h.scale;
-      apply_reflector<T, 8>(h.tau, v, a[q], pl);
-      apply_reflector<T, 8>(h.tau, v, rl[q], pa);
-      apply_reflector<T, 8>(h.tau, v, bl[q], lr);
-      apply_reflector<T, 8>(h.tau, v, cl[q], dl);
-      if (j == q) {
-        a[q] = h.beta;
-#pragma unroll
-        for (int r = 0; r < 8; ++r) pl[r] = T(0);
-      }
+      reflector(q, a[q], pl, 0, 8);
+      rl[q] = T(0);
+      apply(tj, a[q], pl, 0, 8);
+      apply(t, rl[q], pa, 0, 8);
+      apply(t, bl[q], lr, 0, 8);
+      apply(t, cl[q], dl, 0, 8);
+      if (j == q) a[q] = beta;
     }
     // the rows of R go out here; what follows needs pa, lr, dl (left and right) and rr, dh, bh, ch
 #pragma unroll
@@ -722,61 +775,28 @@ __device__ __forceinline__ void cr_item(const CRArgs<T>& A, int64_t k, int64_t i
     R[192 + j] = lane_of(cl, j);
 #pragma unroll
     for (int q = 0; q < 7; ++q) {
-      T s2 = T(0);
-      const T p = __shfl_sync(gmask, pa[q], q, kItemThreads);
-#pragma unroll
-      for (int r = q + 1; r < 8; ++r) {
-        x[r] = __shfl_sync(gmask, pa[r], q, kItemThreads);
-        s2 += x[r] * x[r];
-      }
-      const Reflector<T> h(p, s2);
-      T w = pa[q], y = lr[q], c = dl[q];
-#pragma unroll
-      for (int r = q + 1; r < 8; ++r) {
-        v[r] = x[r] * h.scale;
-        w += v[r] * pa[r];
-        y += v[r] * lr[r];
-        c += v[r] * dl[r];
-      }
-      w *= h.tau;
-      y *= h.tau;
-      c *= h.tau;
-      pa[q] -= w;
-      lr[q] -= y;
-      dl[q] -= c;
-#pragma unroll
-      for (int r = q + 1; r < 8; ++r) {
-        pa[r] -= w * v[r];
-        lr[r] -= y * v[r];
-        dl[r] -= c * v[r];
-      }
-      if (j == q) {
-        pa[q] = h.beta;
-#pragma unroll
-        for (int r = q + 1; r < 8; ++r) pa[r] = T(0);
-      }
+      reflector(q, pa.get(q), pa, q + 1, 8);
+      apply_at(tj, q, pa, q + 1, 8);
+      apply_at(t, q, lr, q + 1, 8);
+      apply_at(t, q, dl, q + 1, 8);
+      if (j == q) pa.set(q, beta);
     }
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      T s2 = T(0);
-      const T p = __shfl_sync(gmask, bh[q], q, kItemThreads);
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        x[r] = __shfl_sync(gmask, rr[r], q, kItemThreads);
-        s2 += x[r] * x[r];
-      }
-      const Reflector<T> h(p, s2);
-#pragma unroll
-      for (int r = 0; r < 8; ++r) v[r] = x[r] * h.scale;
-      apply_reflector<T, 8>(h.tau, v, bh[q], rr);
-      apply_reflector<T, 8>(h.tau, v, ch[q], dh);
-      if (j == q) {
-        bh[q] = h.beta;
-#pragma unroll
-        for (int r = 0; r < 8; ++r) rr[r] = T(0);
-      }
+      reflector(q, bh[q], rr, 0, 8);
+      apply(tj, bh[q], rr, 0, 8);
+      apply(t, ch[q], dh, 0, 8);
+      if (j == q) bh[q] = beta;
     }
-    store_block_row(Fn + (b0 + (i - 1) / 2) * kFW, j, pa, lr, bh, dl, ch);
+    T* F = Fn + (b0 + (i - 1) / 2) * kFW;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      F[8 * r + j] = r <= j ? pa.get(r) : T(0);
+      F[64 + 8 * r + j] = lr.get(r);
+      F[128 + 8 * r + j] = bh[r];
+    }
+    F[192 + j] = lane_of(dl, j);
+    F[200 + j] = lane_of(ch, j);
     res.square(lane_of(dh, j));
   } else {   // the last block: its A is triangular, nothing is to its right
 #pragma unroll
