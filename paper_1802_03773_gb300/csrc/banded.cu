@@ -22,6 +22,7 @@
 #include <string>
 #include <vector>
 
+#include "chain.cuh"
 #include "device_util.cuh"
 #include "f32x2.cuh"
 #include "internal.h"
@@ -441,6 +442,7 @@ struct BandGroups {   // what both kernels are told
 
 template <bool kW8, bool kStaged, int MW>
 __global__ void __launch_bounds__(256) band_norm_f32_kernel(BandGroups B, double* D, float2* D2) {
+  dev::chain_wait();
   extern __shared__ __align__(16) float sm_f[];
   const int nt = blockDim.x, tid = threadIdx.x, w = B.w;
   const int64_t grp0 = (int64_t)blockIdx.x * (nt - (w - 1)) - (w - 1), grp = grp0 + tid;
@@ -504,6 +506,7 @@ template <bool kW8, bool kStaged, int MW>
 __global__ void __launch_bounds__(256) band_grad_f32_kernel(BandGroups B, const float* b, const float* x,
                                                             const float2* D2, float lam_h, float lam_l,
                                                             const int64_t* blk0, float* gp) {
+  dev::chain_wait();
   extern __shared__ __align__(16) float sm_f[];
   const int nt = blockDim.x, tid = threadIdx.x, w = B.w;
   const int64_t grp0 = (int64_t)blockIdx.x * (nt - (w - 1)) - (w - 1), grp = grp0 + tid;
@@ -668,8 +671,7 @@ static BandLaunch band_launch(const BandGroups& B, size_t per_thread, size_t fix
                                                     (int)(L).smem);                                            \
         if (e_ != cudaSuccess) return e_;                                                                      \
       }                                                                                                        \
-      k_<<<(L).grid, (L).nt, (L).smem, (ctx)->stream>>>(__VA_ARGS__);                                          \
-      return cudaGetLastError();                                                                               \
+      return chain_launch((ctx)->stream, (L).grid, (L).nt, (L).smem, k_, __VA_ARGS__);                             \
     };                                                                                                         \
     QRKIT_CUDA_TRY(ctx, (L).w8 ? ((L).staged ? launch_(KERNEL<true, true, 8>) : launch_(KERNEL<true, false, 8>))  \
                                : ((L).staged ? launch_(KERNEL<false, true, MW>) : launch_(KERNEL<false, false, MW>))); \

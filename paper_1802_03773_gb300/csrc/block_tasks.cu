@@ -43,9 +43,11 @@ qrkit_status resident(qrkit_ctx* ctx, F setup, int threads, size_t smem, int slo
   return QRKIT_OK;
 }
 
-// One launch of the factor kernel of class CLS over tasks [t0, t1) of the plan.
+// One launch of the factor kernel of class CLS over tasks [t0, t1) of the plan.  `beside`: it may run beside the factor
+// kernel launched before it, whose tasks are others (and waits for it before it ends).
 template <typename T, bool SEL, int CLS>
-qrkit_status launch_class(qrkit_ctx* ctx, TaskArgs<T> A, int64_t t0, int64_t t1, int slot) {
+qrkit_status launch_class(qrkit_ctx* ctx, TaskArgs<T> A, int64_t t0, int64_t t1, int slot, bool few = false,
+                          bool beside = false) {
   const Plan& P = ctx->plan;
   if (t1 <= t0) return QRKIT_OK;
   const int es = (int)sizeof(T);
@@ -62,7 +64,7 @@ qrkit_status launch_class(qrkit_ctx* ctx, TaskArgs<T> A, int64_t t0, int64_t t1,
   const int64_t want = (A.num_tasks + wpc - 1) / wpc;
   const int64_t full = (int64_t)ctx->num_sms * per_sm;
   const unsigned grid = (unsigned)std::max<int64_t>(1, std::min(want, full));
-  QRKIT_CUDA_TRY(ctx, (kernel_launch<T, SEL, CLS>(A, grid, threads, smem, ctx->stream)));
+  QRKIT_CUDA_TRY(ctx, (kernel_launch<T, SEL, CLS>(A, grid, threads, smem, ctx->stream, few, beside)));
   ctx->launches += 1;
   return QRKIT_OK;
 }
@@ -93,6 +95,8 @@ qrkit_status launch_tasks_typed(qrkit_ctx* ctx, const void* J, const void* b, vo
   A.rec = nullptr;
   A.rec_off = (const int64_t*)P.d_rec_off.ptr;
   qrkit_status st;
+  // the two factor kernels side by side where one CTA per SM holds all tasks of both
+  const bool few = SEL && P.num_tasks <= (int64_t)ctx->num_sms * P.task_warps;
   if (SEL) {
     if ((st = ensure(ctx, ctx->ws.tlist, (size_t)std::max<int64_t>(P.K, 1) * sizeof(RefEntry), "refinement lists")) !=
         QRKIT_OK)
@@ -115,8 +119,10 @@ qrkit_status launch_tasks_typed(qrkit_ctx* ctx, const void* J, const void* b, vo
   } else {
     // float with the selection: a refined plan puts the tasks of blocks with at most 4 columns
     // first; each class runs in the kernel compiled for it
-    if ((st = launch_class<T, SEL, 1>(ctx, A, 0, P.narrow_tasks, 9)) != QRKIT_OK) return st;
-    if ((st = launch_class<T, SEL, 2>(ctx, A, P.narrow_tasks, P.num_tasks, 14)) != QRKIT_OK) return st;
+    if ((st = launch_class<T, SEL, 1>(ctx, A, 0, P.narrow_tasks, 9, few)) != QRKIT_OK) return st;
+    if ((st = launch_class<T, SEL, 2>(ctx, A, P.narrow_tasks, P.num_tasks, 14, few,
+                                      few && P.narrow_tasks > 0)) != QRKIT_OK)
+      return st;
   }
   if constexpr (SEL && sizeof(T) == sizeof(float)) {
     RefineTaskArgs R;
@@ -140,8 +146,8 @@ qrkit_status launch_tasks_typed(qrkit_ctx* ctx, const void* J, const void* b, vo
     const int64_t want2 = (P.max_refine_tasks + kRefineWarps - 1) / kRefineWarps;
     const int64_t full2 = (int64_t)ctx->num_sms * per_sm2;
     const unsigned grid2 = (unsigned)std::max<int64_t>(1, std::min(want2, full2));
-    QRKIT_CUDA_TRY(ctx, res64 ? refine_launch<1>(R, grid2, threads2, 0, ctx->stream)
-                              : refine_launch<0>(R, grid2, threads2, 0, ctx->stream));
+    QRKIT_CUDA_TRY(ctx, res64 ? refine_launch<1>(R, grid2, threads2, 0, ctx->stream, few)
+                              : refine_launch<0>(R, grid2, threads2, 0, ctx->stream, few));
     ctx->launches += 1;
   }
   return QRKIT_OK;

@@ -13,6 +13,7 @@
 #include <string>
 #include <vector>
 
+#include "chain.cuh"
 #include "device_util.cuh"
 #include "internal.h"
 
@@ -43,6 +44,7 @@ __device__ __forceinline__ void dot2_acc(float& sh, float& sl, float a, float x)
 // 819 MB) ----
 template <typename T>
 __global__ void colnorm_blocks_kernel(ComposedView<T> V, double* sq) {
+  dev::chain_wait();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= V.K) return;
   const int n = V.n[i], m = V.m[i];
@@ -66,6 +68,7 @@ constexpr int kNormThreads = 256;
 template <typename T>
 __global__ void __launch_bounds__(kNormThreads) colnorm_dense_part_kernel(ComposedView<T> V, double* part,
                                                                           int64_t nchunk) {
+  dev::chain_wait();
   __shared__ double ws[kNormThreads / 32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t r0 = (int64_t)blockIdx.x * kNormRows;
@@ -98,6 +101,7 @@ __global__ void __launch_bounds__(kNormThreads) colnorm_dense_part_kernel(Compos
 }
 
 __global__ void colnorm_dense_sum_kernel(const double* part, int64_t nchunk, int64_t s, double* sq) {
+  dev::chain_wait();
   const int64_t col = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (col >= s) return;
   double t = 0;
@@ -107,6 +111,7 @@ __global__ void colnorm_dense_sum_kernel(const double* part, int64_t nchunk, int
 
 template <typename T>
 __global__ void colnorm_window_kernel(ComposedView<T> V, double* sq) {
+  dev::chain_wait();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= V.K) return;
   const int n = V.n[i];
@@ -123,6 +128,7 @@ __global__ void colnorm_window_kernel(ComposedView<T> V, double* sq) {
 }
 
 __global__ void finalize_norms_kernel(const double* sq, double* D, int64_t N) {
+  dev::chain_wait();
   const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (j >= N) return;
   const double d = sqrt(sq[j]);
@@ -295,6 +301,7 @@ __device__ __forceinline__ void block_factor_small(const ComposedView<T>& V, con
 // small blocks only).
 template <typename T, int NA, int MM>
 __global__ void block_factor_small_kernel(ComposedView<T> V, FactorOut<T> O) {
+  dev::chain_wait();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= V.K) return;
   block_factor_small<T, NA, MM>(V, O, i, V.n[i], V.m[i]);
@@ -302,6 +309,7 @@ __global__ void block_factor_small_kernel(ComposedView<T> V, FactorOut<T> O) {
 
 template <typename T>
 __global__ void block_factor_kernel(ComposedView<T> V, FactorOut<T> O) {
+  dev::chain_wait();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= V.K) return;
   const int n = V.n[i], m = V.m[i];
@@ -383,6 +391,7 @@ __global__ void block_factor_kernel(ComposedView<T> V, FactorOut<T> O) {
 template <typename T>
 __global__ void reduced_damping_kernel(T* X0, int64_t ld0, int64_t row0, int s, int count, bool damp, const double* D,
                                        int64_t nb, double lam_half) {
+  dev::chain_wait();
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= (int64_t)count * s) return;
   const int c = (int)(e / count), j = (int)(e % count);
@@ -393,6 +402,7 @@ __global__ void reduced_damping_kernel(T* X0, int64_t ld0, int64_t row0, int s, 
 // at most NA augmented rows and MM columns (loops unrolled to those bounds, registers only).
 template <typename T, int NA = 0, int MM = 0>
 __global__ void block_apply_qt_kernel(ComposedView<T> V, FactorOut<T> O, const T* b, T* rhs0) {
+  dev::chain_wait();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= V.K) return;
   if constexpr (NA > 0) {
@@ -449,6 +459,7 @@ __global__ void block_apply_qt_kernel(ComposedView<T> V, FactorOut<T> O, const T
 template <typename T, int NA = 0, int MM = 0>
 __global__ void block_backsub_kernel(ComposedView<T> V, FactorOut<T> O, const T* rhs_t,
                                      const T* xS, T* x, int accumulate) {
+  dev::chain_wait();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= V.K) return;
   if constexpr (NA > 0) {
@@ -766,6 +777,7 @@ __device__ __forceinline__ bool window_range(const ComposedView<T>& V, int64_t i
 template <typename T, int NA = 0, int MM = 0>
 __global__ void resid_g_kernel(ComposedView<T> V, const T* b, const T* p, const double* D,
                                double lam, double* g, double* gS, int win_cols) {
+  dev::chain_wait();
   // dense S: every block adds to all s shared columns; the CTA's sums are gathered in shared
   // memory and leave with one global atomic per column
   extern __shared__ double sgS[];
@@ -802,6 +814,7 @@ __global__ void resid_g_kernel(ComposedView<T> V, const T* b, const T* p, const 
 
 __global__ void gS_damping_kernel(double* gS, const float* pf, const double* pd, const double* D,
                                   int64_t nb, int s, double lam) {
+  dev::chain_wait();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= s) return;
   const double pv = pf ? (double)pf[nb + c] : pd[nb + c];
@@ -888,6 +901,7 @@ __device__ __forceinline__ void fwdsub_rt_small(const ComposedView<T>& V, const 
 template <typename T, int NA = 0, int MM = 0>
 __global__ void block_fwdsub_rt_kernel(ComposedView<T> V, FactorOut<T> O, const double* g, T* h,
                                        double* gS, int win_cols) {
+  dev::chain_wait();
   extern __shared__ double sgS[];
   const bool cta_sum = V.coupled == QRKIT_COUPLED_DENSE && V.s <= kCtaSumCols;
   if (cta_sum) {
@@ -922,17 +936,20 @@ __global__ void block_fwdsub_rt_kernel(ComposedView<T> V, FactorOut<T> O, const 
 
 template <typename T>
 __global__ void gS_to_T_kernel(const double* gS, T* out, int s) {
+  dev::chain_wait();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c < s) out[c] = (T)gS[c];
 }
 
 template <typename T>
 __global__ void axpy_kernel(T* x, const T* d, int64_t n) {
+  dev::chain_wait();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i < n) x[i] += d[i];
 }
 
 __global__ void widen_kernel(const float* in, double* out, int64_t n) {
+  dev::chain_wait();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i < n) out[i] = (double)in[i];
 }
@@ -1014,9 +1031,9 @@ int small_class(const Plan& P, bool damp) {
 // A per-block kernel template KERNEL<T, NA, MM> launched in the instantiation of the class.
 #define LAUNCH_SHAPED(ctx, cls, KERNEL, grid, threads, smem, stream, ...)                      \
   do {                                                                                         \
-    if ((cls) == 1) LAUNCH(ctx, (KERNEL<T, 3, 1><<<grid, threads, smem, stream>>>(__VA_ARGS__))); \
-    else if ((cls) == 2) LAUNCH(ctx, (KERNEL<T, 6, 2><<<grid, threads, smem, stream>>>(__VA_ARGS__))); \
-    else LAUNCH(ctx, (KERNEL<T><<<grid, threads, smem, stream>>>(__VA_ARGS__)));                \
+    if ((cls) == 1) LAUNCH(ctx, (chain_launch(stream, grid, threads, smem, (KERNEL<T, 3, 1>), __VA_ARGS__))); \
+    else if ((cls) == 2) LAUNCH(ctx, (chain_launch(stream, grid, threads, smem, (KERNEL<T, 6, 2>), __VA_ARGS__))); \
+    else LAUNCH(ctx, (chain_launch(stream, grid, threads, smem, KERNEL<T>, __VA_ARGS__)));                \
   } while (0)
 
 // R_i x_i = rhs_i - R12_i x_S for every block.  From 16 shared columns on a warp takes a block (the
@@ -1064,19 +1081,20 @@ static qrkit_status norms_typed(qrkit_ctx* ctx, const ComposedView<T>& V, double
   if ((rc = ensure(ctx, C.sq, sq_bytes, "column sums")) != QRKIT_OK) return rc;
   double* sq = (double*)C.sq.ptr;
   QRKIT_CUDA_TRY(ctx, cudaMemsetAsync(sq, 0, (size_t)N * sizeof(double), st));
-  LAUNCH(ctx, colnorm_blocks_kernel<T><<<blocks_for(P.K, 128), 128, 0, st>>>(V, sq));
+  LAUNCH(ctx, chain_launch(st, blocks_for(P.K, 128), 128, 0, colnorm_blocks_kernel<T>, V, sq));
   if (V.coupled == QRKIT_COUPLED_DENSE) {
     if (nchunk > (int64_t)INT32_MAX) return fail(ctx, QRKIT_EUNSUPPORTED, "too many rows for the column norms");
     const dim3 grid((unsigned)nchunk, (unsigned)std::min<int64_t>(V.s, 65535));
-    LAUNCH(ctx, colnorm_dense_part_kernel<T><<<grid, kNormThreads, 0, st>>>(V, sq + N, nchunk));
-    LAUNCH(ctx, colnorm_dense_sum_kernel<<<blocks_for(V.s, 128), 128, 0, st>>>(sq + N, nchunk, V.s, sq + V.nb));
+    LAUNCH(ctx, chain_launch(st, grid, kNormThreads, 0, colnorm_dense_part_kernel<T>, V, sq + N, nchunk));
+    LAUNCH(ctx, chain_launch(st, blocks_for(V.s, 128), 128, 0, colnorm_dense_sum_kernel, sq + N, nchunk, V.s,
+                             sq + V.nb));
   } else if (V.coupled == QRKIT_COUPLED_WINDOW && sorted) {
     const WindowSums<T> A = window_sums<T>(ctx, V, sq + V.nb);
     if ((rc = window_square_sums<T>(ctx, A)) != QRKIT_OK) return rc;
   } else if (V.coupled == QRKIT_COUPLED_WINDOW) {
-    LAUNCH(ctx, colnorm_window_kernel<T><<<blocks_for(P.K, 128), 128, 0, st>>>(V, sq));
+    LAUNCH(ctx, chain_launch(st, blocks_for(P.K, 128), 128, 0, colnorm_window_kernel<T>, V, sq));
   }
-  LAUNCH(ctx, finalize_norms_kernel<<<blocks_for(N, 256), 256, 0, st>>>(sq, D, N));
+  LAUNCH(ctx, chain_launch(st, blocks_for(N, 256), 256, 0, finalize_norms_kernel, sq, D, N));
   return QRKIT_OK;
 }
 
@@ -1146,11 +1164,11 @@ static qrkit_status factor_typed(qrkit_ctx* ctx, const void* J, const void* S, c
   // the small-block kernels when every block fits them (e.g. 2 x 1 blocks of curve fits)
   const int cls = small_class(P, O.damp);
   if (cls == 1)
-    LAUNCH(ctx, (block_factor_small_kernel<T, 3, 1><<<blocks_for(P.K, 128), 128, 0, st>>>(V, O)));
+    LAUNCH(ctx, (chain_launch(st, blocks_for(P.K, 128), 128, 0, (block_factor_small_kernel<T, 3, 1>), V, O)));
   else if (cls == 2)
-    LAUNCH(ctx, (block_factor_small_kernel<T, 6, 2><<<blocks_for(P.K, 128), 128, 0, st>>>(V, O)));
+    LAUNCH(ctx, (chain_launch(st, blocks_for(P.K, 128), 128, 0, (block_factor_small_kernel<T, 6, 2>), V, O)));
   else
-    LAUNCH(ctx, block_factor_kernel<T><<<blocks_for(P.K, 64), 64, 0, st>>>(V, O));
+    LAUNCH(ctx, chain_launch(st, blocks_for(P.K, 64), 64, 0, block_factor_kernel<T>, V, O));
   if (V.coupled == QRKIT_COUPLED_DENSE && (rc = dense_apply_blocks<T>(ctx, V, O)) != QRKIT_OK) return rc;
   if (V.coupled == QRKIT_COUPLED_WINDOW && !C.bins) {
     // P_r of the reduced block: its rows sorted by leading column per segment (Sec. 4.3)
@@ -1163,13 +1181,13 @@ static qrkit_status factor_typed(qrkit_ctx* ctx, const void* J, const void* S, c
     const int s = V.s;
     T* X0 = (T*)C.levels[0].X.ptr;
     if (C.damp)
-      LAUNCH(ctx, reduced_damping_kernel<T><<<blocks_for((int64_t)s * s, 256), 256, 0, st>>>(
-                      X0, C.levels[0].ld, C.panels.empty() ? C.red_rows : 0, s, s, true, (const double*)C.D.ptr, P.cols,
-                      C.lam_half));
+      LAUNCH(ctx, chain_launch(st, blocks_for((int64_t)s * s, 256), 256, 0, reduced_damping_kernel<T>, X0,
+                               C.levels[0].ld, C.panels.empty() ? C.red_rows : 0, s, s, true, (const double*)C.D.ptr,
+                               P.cols, C.lam_half));
     const int64_t used = C.red_rows + (C.damp ? s : 0);
     if (C.levels[0].M > used)
-      LAUNCH(ctx, reduced_damping_kernel<T><<<blocks_for((C.levels[0].M - used) * s, 256), 256, 0, st>>>(
-                      X0, C.levels[0].ld, used, s, (int)(C.levels[0].M - used), false, nullptr, 0, 0.0));
+      LAUNCH(ctx, chain_launch(st, blocks_for((C.levels[0].M - used) * s, 256), 256, 0, reduced_damping_kernel<T>, X0,
+                               C.levels[0].ld, used, s, (int)(C.levels[0].M - used), false, nullptr, 0, 0.0));
     if (!C.panels.empty()) return factor_panels(ctx, s);
     for (size_t l = 0; l < C.levels.size(); ++l) {
       TsqrLevel& L = C.levels[l];
@@ -1285,9 +1303,9 @@ static qrkit_status solve_typed(qrkit_ctx* ctx, const void* J, const void* S, co
       QRKIT_CUDA_TRY(ctx, cudaMemsetAsync(gS, 0, (size_t)s * sizeof(double), st));
       WindowSums<T> A = window_sums<T>(ctx, V, gS);
       if ((rc = window_refine_gradient<T>(ctx, V, O, (const T*)b, x, C.lam, A)) != QRKIT_OK) return rc;
-      LAUNCH(ctx, gS_damping_kernel<<<blocks_for(s, 128), 128, 0, st>>>(
-                      gS, sizeof(T) == 4 ? (const float*)x : nullptr, sizeof(T) == 8 ? (const double*)x : nullptr, O.D,
-                      nb, s, C.lam));
+      LAUNCH(ctx, chain_launch(st, blocks_for(s, 128), 128, 0, gS_damping_kernel, gS,
+                               sizeof(T) == 4 ? (const float*)x : nullptr,
+                               sizeof(T) == 8 ? (const double*)x : nullptr, O.D, nb, s, C.lam));
       have_g = true;
     }
     if (!have_g) {
@@ -1302,9 +1320,9 @@ static qrkit_status solve_typed(qrkit_ctx* ctx, const void* J, const void* S, co
       LAUNCH_SHAPED(ctx, small_class(P, O.damp), resid_g_kernel, blocks_for(P.K, rthreads), rthreads, sum_smem, st, V,
                     (const T*)b, x, O.D, C.lam, g, gS, win_cols);
       if (s > 0)
-        LAUNCH(ctx, gS_damping_kernel<<<blocks_for(s, 128), 128, 0, st>>>(
-                        gS, sizeof(T) == 4 ? (const float*)x : nullptr,
-                        sizeof(T) == 8 ? (const double*)x : nullptr, O.D, nb, s, C.lam));
+        LAUNCH(ctx, chain_launch(st, blocks_for(s, 128), 128, 0, gS_damping_kernel, gS,
+                                 sizeof(T) == 4 ? (const float*)x : nullptr,
+                                 sizeof(T) == 8 ? (const double*)x : nullptr, O.D, nb, s, C.lam));
       LAUNCH_SHAPED(ctx, small_class(P, O.damp), block_fwdsub_rt_kernel, blocks_for(P.K, rthreads), rthreads, sum_smem,
                     st, V, O, g, h, gS, win_cols);
     }
@@ -1313,14 +1331,14 @@ static qrkit_status solve_typed(qrkit_ctx* ctx, const void* J, const void* S, co
       if ((rc = cr_normal_solve(ctx, *C.cr, gS, h + nb, x + nb)) != QRKIT_OK) return rc;
     } else if (V.coupled == QRKIT_COUPLED_WINDOW) {
       // h_S = R_S^{-T} (g_S - R12^T h_B), then dp_S = R_S^{-1} h_S, both banded
-      LAUNCH(ctx, gS_to_T_kernel<T><<<blocks_for(s, 128), 128, 0, st>>>(gS, h + nb, s));
+      LAUNCH(ctx, chain_launch(st, blocks_for(s, 128), 128, 0, gS_to_T_kernel<T>, gS, h + nb, s));
       const int64_t nseg = (int64_t)P.seg_cols.size();
       const int64_t* inst = (const int64_t*)C.seg_inst.ptr;
       qrkit_status rc = banded_tri_solve(ctx, nseg, inst, C.RwS.ptr, V.w, h + nb, true);
       if (rc != QRKIT_OK) return rc;
       rc = banded_tri_solve(ctx, nseg, inst, C.RwS.ptr, V.w, h + nb, false);
       if (rc != QRKIT_OK) return rc;
-      LAUNCH(ctx, axpy_kernel<T><<<blocks_for(s, 128), 128, 0, st>>>(x + nb, h + nb, s));
+      LAUNCH(ctx, chain_launch(st, blocks_for(s, 128), 128, 0, axpy_kernel<T>, x + nb, h + nb, s));
     }
     if (V.coupled == QRKIT_COUPLED_DENSE) {
       // dp_S = R_S^{-1} R_S^{-T} (g_S - R12^T h_B), added to p_S and kept in h for the blocks
@@ -1386,6 +1404,7 @@ qrkit_status composed_apply_qt(qrkit_ctx* ctx, const void* b, void* qtb) {
 namespace qrkit {
 
 __global__ void multiples_kernel(int64_t* out, int64_t n, int64_t step) {
+  dev::chain_wait();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i < n) out[i] = i * step;
 }
@@ -1398,7 +1417,7 @@ static qrkit_status upload_i64(qrkit_ctx* ctx, DevBuf& buf, const std::vector<in
 }
 
 qrkit_status widen_to_double(qrkit_ctx* ctx, const float* in, double* out, int64_t n) {
-  widen_kernel<<<blocks_for(n, 256), 256, 0, ctx->stream>>>(in, out, n);
+  chain_launch(ctx->stream, blocks_for(n, 256), 256, 0, widen_kernel, in, out, n);
   ctx->launches += 1;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());
   return QRKIT_OK;
@@ -1447,7 +1466,8 @@ qrkit_status composed_layout(qrkit_ctx* ctx, size_t elem) {
     DevBuf* buf[4] = {&C.d_aug_off_d, &C.d_aug_off_u, &C.d_red_off_d, &C.d_red_off_u};
     for (int q = 0; q < 4; ++q) {
       if ((rc = ensure(ctx, *buf[q], (size_t)(K + 1) * sizeof(int64_t), "block offsets")) != QRKIT_OK) return rc;
-      multiples_kernel<<<blocks_for(K + 1, 256), 256, 0, ctx->stream>>>((int64_t*)buf[q]->ptr, K + 1, step[q]);
+      chain_launch(ctx->stream, blocks_for(K + 1, 256), 256, 0, multiples_kernel, (int64_t*)buf[q]->ptr, K + 1,
+                   step[q]);
       ctx->launches += 1;
       QRKIT_CUDA_TRY(ctx, cudaGetLastError());
     }
@@ -1729,6 +1749,7 @@ qrkit_status composed_column_sumsq(qrkit_ctx* ctx, const void* J, const void* S,
 
 template <typename T>
 __global__ void norms_from_sumsq_kernel(const double* sq, T* D, int64_t n) {
+  dev::chain_wait();
   const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (j >= n) return;
   const double d = sqrt(sq[j]);
@@ -1737,14 +1758,17 @@ __global__ void norms_from_sumsq_kernel(const double* sq, T* D, int64_t n) {
 
 qrkit_status composed_norms_from_sumsq(qrkit_ctx* ctx, const double* sq, int64_t n, void* D) {
   if (ctx->precision == QRKIT_FP64)
-    LAUNCH(ctx, norms_from_sumsq_kernel<double><<<blocks_for(n, 256), 256, 0, ctx->stream>>>(sq, (double*)D, n));
+    LAUNCH(ctx, chain_launch(ctx->stream, blocks_for(n, 256), 256, 0, norms_from_sumsq_kernel<double>, sq, (double*)D,
+                             n));
   else
-    LAUNCH(ctx, norms_from_sumsq_kernel<float><<<blocks_for(n, 256), 256, 0, ctx->stream>>>(sq, (float*)D, n));
+    LAUNCH(ctx, chain_launch(ctx->stream, blocks_for(n, 256), 256, 0, norms_from_sumsq_kernel<float>, sq, (float*)D,
+                             n));
   return QRKIT_OK;
 }
 
 template <typename T>
 __global__ void copy_upper_kernel(const T* X, int64_t ld, int s, T* R) {
+  dev::chain_wait();
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= (int64_t)s * s) return;
   const int i = (int)(e % s), j = (int)(e / s);
@@ -1758,11 +1782,11 @@ qrkit_status composed_reduced_r(qrkit_ctx* ctx, void* R) {
   const void* src = C.panels.empty() ? top.X.ptr : C.Rs.ptr;
   const int64_t ld = C.panels.empty() ? top.ld : s;
   if (ctx->precision == QRKIT_FP64)
-    LAUNCH(ctx, copy_upper_kernel<double><<<blocks_for((int64_t)s * s, 256), 256, 0, ctx->stream>>>(
-                    (const double*)src, ld, s, (double*)R));
+    LAUNCH(ctx, chain_launch(ctx->stream, blocks_for((int64_t)s * s, 256), 256, 0, copy_upper_kernel<double>,
+                             (const double*)src, ld, s, (double*)R));
   else
-    LAUNCH(ctx, copy_upper_kernel<float><<<blocks_for((int64_t)s * s, 256), 256, 0, ctx->stream>>>(
-                    (const float*)src, ld, s, (float*)R));
+    LAUNCH(ctx, chain_launch(ctx->stream, blocks_for((int64_t)s * s, 256), 256, 0, copy_upper_kernel<float>,
+                             (const float*)src, ld, s, (float*)R));
   return QRKIT_OK;
 }
 

@@ -32,6 +32,7 @@
 #include <string>
 #include <vector>
 
+#include "chain.cuh"
 #include "device_util.cuh"
 #include "f32x2.cuh"
 #include "internal.h"
@@ -125,6 +126,7 @@ struct CRArgs {
 // First row of each block's group: lower bound of 8 g among the instance's sorted starts.
 template <typename T>
 __global__ void cr_ranges_kernel(CRArgs<T> A) {
+  dev::chain_wait();
   const int64_t gb = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (gb >= A.total_blocks) return;
   const int64_t k = A.binst[gb];
@@ -336,6 +338,7 @@ constexpr int stage_stride() { return 4 * kCB * (int)sizeof(T) + 16; }   // byte
 
 template <typename T, bool kStaged>
 __global__ void __launch_bounds__(kCompThreads, sizeof(T) == 4 ? 4 : 2) cr_compress_kernel(CRArgs<T> A) {
+  dev::chain_wait();
   extern __shared__ __align__(16) unsigned char stage[];   // two buffers of kCompThreads x stage_stride
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t item = (int64_t)blockIdx.x * kCompThreads + threadIdx.x;
@@ -495,6 +498,7 @@ struct MergeItem {
 template <typename T>
 __global__ void __launch_bounds__(kCompThreads) cr_merge_kernel(CRArgs<T> A, const MergeItem* items, int64_t nitems,
                                                                 const T* in, T* part) {
+  dev::chain_wait();
   const int64_t w = (int64_t)blockIdx.x * kCompThreads + threadIdx.x;
   if (w >= nitems) return;
   const MergeItem M = items[w];
@@ -815,6 +819,7 @@ constexpr int kLevelThreads = 128;
 template <typename T, bool kCompressed>
 __global__ void __launch_bounds__(kLevelThreads, sizeof(T) == 4 ? 4 : 2)
 cr_level_kernel(CRArgs<T> A, const int64_t* items, int64_t nitems, int level, const T* Fc, T* Fn) {
+  dev::chain_wait();
   const int64_t w = ((int64_t)blockIdx.x * kLevelThreads + threadIdx.x) / kItemThreads;
   const int j = threadIdx.x % kItemThreads;
   const unsigned gmask = 0xffu << (threadIdx.x & 24);
@@ -876,6 +881,7 @@ __device__ __forceinline__ void cr_backsub_item(const CRArgs<T>& A, int64_t k, i
 template <typename T>
 __global__ void cr_backsub_kernel(CRArgs<T> A, const int64_t* items, int64_t nitems, int level, int use_hp, T* x,
                                   T* xadd) {
+  dev::chain_wait();
   const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kItemThreads;
   if (w >= nitems) return;
   int64_t k, i;
@@ -933,6 +939,7 @@ __device__ __forceinline__ void cr_rt_level_item(const CRArgs<T>& A, int64_t k, 
 
 template <typename T>
 __global__ void cr_rt_level_kernel(CRArgs<T> A, const int64_t* items, int64_t nitems, int level) {
+  dev::chain_wait();
   const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kItemThreads;
   if (w >= nitems) return;
   cr_rt_level_item(A, items[w] >> 32, items[w] & 0xffffffff, level, (int)(threadIdx.x % kItemThreads),
@@ -967,6 +974,7 @@ __device__ __forceinline__ void tail_backsub(const CRArgs<T>& A, int64_t k, int6
 // Factor of the upper levels, then their back-substitution.
 template <typename T>
 __global__ void __launch_bounds__(tail_threads<T>(), 1) cr_tail_kernel(CRArgs<T> A, T* x) {
+  dev::chain_wait();
   const int64_t k = blockIdx.x;
   const int grp = threadIdx.x / kItemThreads, ng = blockDim.x / kItemThreads, j = threadIdx.x % kItemThreads;
   const unsigned gmask = 0xffu << (threadIdx.x & 24);
@@ -996,6 +1004,7 @@ __global__ void __launch_bounds__(tail_threads<T>(), 1) cr_tail_kernel(CRArgs<T>
 // R^T h = g through the upper levels, then their back-substitution.
 template <typename T>
 __global__ void __launch_bounds__(tail_threads<T>(), 1) cr_tail_normal_kernel(CRArgs<T> A, T* x, T* xadd) {
+  dev::chain_wait();
   const int64_t k = blockIdx.x;
   const int grp = threadIdx.x / kItemThreads, ng = blockDim.x / kItemThreads, q = threadIdx.x % kItemThreads;
   const unsigned gmask = 0xffu << (threadIdx.x & 24);
@@ -1023,6 +1032,7 @@ __global__ void __launch_bounds__(tail_threads<T>(), 1) cr_tail_normal_kernel(CR
 // g by global column into the padded layout (virtual columns 0).
 template <typename T>
 __global__ void cr_scatter_g_kernel(CRArgs<T> A, const double* g_in) {
+  dev::chain_wait();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= A.total_blocks * kCB) return;
   const int64_t gb = e / kCB;
@@ -1246,11 +1256,11 @@ static CRArgs<T> cr_args(qrkit_ctx* ctx, CRPlan& C) {
   return A;
 }
 
-#define CR_LAUNCH(ctx, ...)                         \
-  do {                                              \
-    __VA_ARGS__;                                    \
-    (ctx)->launches += 1;                           \
-    QRKIT_CUDA_TRY(ctx, cudaGetLastError());        \
+// CR_LAUNCH(ctx, grid, block, shared memory, kernel, arguments ..)
+#define CR_LAUNCH(ctx, ...)                                      \
+  do {                                                           \
+    QRKIT_CUDA_TRY(ctx, chain_launch((ctx)->stream, __VA_ARGS__)); \
+    (ctx)->launches += 1;                                        \
   } while (0)
 
 template <typename T>
@@ -1268,22 +1278,22 @@ static qrkit_status cr_solve_typed(qrkit_ctx* ctx, CRPlan& C, const int64_t* sta
   A.lam = lambda;
   A.res2 = res2;
   QRKIT_CUDA_TRY(ctx, cudaMemsetAsync(res2, 0, (size_t)C.num_inst * sizeof(double), st));
-  if (starts) CR_LAUNCH(ctx, cr_ranges_kernel<T><<<nblk(C.total_blocks, 256), 256, 0, st>>>(A));
+  if (starts) CR_LAUNCH(ctx, nblk(C.total_blocks, 256), 256, 0, cr_ranges_kernel<T>, A);
   const unsigned cgrid = nblk(C.num_items, kCompThreads);
   if (w == kCB && (reinterpret_cast<uintptr_t>(J) & 15) == 0) {
     const size_t smem = 2 * (size_t)kCompThreads * stage_stride<T>();
     auto kc = cr_compress_kernel<T, true>;
     if (smem > 48 * 1024)
       QRKIT_CUDA_TRY(ctx, cudaFuncSetAttribute(kc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    CR_LAUNCH(ctx, kc<<<cgrid, kCompThreads, smem, st>>>(A));
+    CR_LAUNCH(ctx, cgrid, kCompThreads, smem, kc, A);
   } else {
-    CR_LAUNCH(ctx, (cr_compress_kernel<T, false><<<cgrid, kCompThreads, 0, st>>>(A)));
+    CR_LAUNCH(ctx, cgrid, kCompThreads, 0, (cr_compress_kernel<T, false>), A);
   }
   T* in = A.P;
   T* other = (T*)C.P2.ptr;
   for (size_t q = 0; q < C.mg_n.size(); ++q) {
-    CR_LAUNCH(ctx, cr_merge_kernel<T><<<nblk(C.mg_n[q], kCompThreads), kCompThreads, 0, st>>>(
-                       A, (const MergeItem*)C.merges.ptr + C.mg_off[q], C.mg_n[q], in, other));
+    CR_LAUNCH(ctx, nblk(C.mg_n[q], kCompThreads), kCompThreads, 0, cr_merge_kernel<T>, A,
+              (const MergeItem*)C.merges.ptr + C.mg_off[q], C.mg_n[q], in, other);
     std::swap(in, other);
   }
   const int64_t* items = (const int64_t*)C.items.ptr;
@@ -1292,17 +1302,17 @@ static qrkit_status cr_solve_typed(qrkit_ctx* ctx, CRPlan& C, const int64_t* sta
     T* Fn = (l & 1) ? A.F0 : A.F1;
     const unsigned grid = nblk(C.lvl_n[l] * kItemThreads, kLevelThreads);
     if (l == 0)
-      CR_LAUNCH(ctx, (cr_level_kernel<T, true><<<grid, kLevelThreads, 0, st>>>(A, items + C.lvl_off[l], C.lvl_n[l], l,
-                                                                              Fc, Fn)));
+      CR_LAUNCH(ctx, grid, kLevelThreads, 0, (cr_level_kernel<T, true>), A, items + C.lvl_off[l],
+                C.lvl_n[l], l, Fc, Fn);
     else
-      CR_LAUNCH(ctx, (cr_level_kernel<T, false><<<grid, kLevelThreads, 0, st>>>(A, items + C.lvl_off[l], C.lvl_n[l], l,
-                                                                               Fc, Fn)));
+      CR_LAUNCH(ctx, grid, kLevelThreads, 0, (cr_level_kernel<T, false>), A, items + C.lvl_off[l],
+                C.lvl_n[l], l, Fc, Fn);
   }
   const int tt = C.num_inst >= 4 * ctx->num_sms ? 128 : tail_threads<T>();
-  CR_LAUNCH(ctx, cr_tail_kernel<T><<<(unsigned)C.num_inst, tt, 0, st>>>(A, x));
+  CR_LAUNCH(ctx, (unsigned)C.num_inst, tt, 0, cr_tail_kernel<T>, A, x);
   for (int l = C.levels - 1; l >= 0; --l)
-    CR_LAUNCH(ctx, cr_backsub_kernel<T><<<nblk(C.lvl_n[l] * kItemThreads, 128), 128, 0, st>>>(
-                       A, items + C.lvl_off[l], C.lvl_n[l], l, 0, x, (T*)nullptr));
+    CR_LAUNCH(ctx, nblk(C.lvl_n[l] * kItemThreads, 128), 128, 0, cr_backsub_kernel<T>, A, items + C.lvl_off[l],
+              C.lvl_n[l], l, 0, x, (T*)nullptr);
   return QRKIT_OK;
 }
 
@@ -1310,19 +1320,18 @@ static qrkit_status cr_solve_typed(qrkit_ctx* ctx, CRPlan& C, const int64_t* sta
 // padded layout), written to dx and added to xadd (either may be null).
 template <typename T>
 static qrkit_status cr_normal_typed(qrkit_ctx* ctx, CRPlan& C, const double* g, T* dx, T* xadd) {
-  cudaStream_t st = ctx->stream;
   CRArgs<T> A = cr_args<T>(ctx, C);
   const int64_t* items = (const int64_t*)C.items.ptr;
   const int64_t* evens = (const int64_t*)C.evens.ptr;
-  if (g) CR_LAUNCH(ctx, cr_scatter_g_kernel<T><<<nblk(C.total_blocks * kCB, 256), 256, 0, st>>>(A, g));
+  if (g) CR_LAUNCH(ctx, nblk(C.total_blocks * kCB, 256), 256, 0, cr_scatter_g_kernel<T>, A, g);
   for (int l = 0; l < C.levels; ++l)
-    CR_LAUNCH(ctx, cr_rt_level_kernel<T><<<nblk(C.ev_n[l] * kItemThreads, 128), 128, 0, st>>>(
-                       A, evens + C.ev_off[l], C.ev_n[l], l));
+    CR_LAUNCH(ctx, nblk(C.ev_n[l] * kItemThreads, 128), 128, 0, cr_rt_level_kernel<T>, A, evens + C.ev_off[l],
+              C.ev_n[l], l);
   const int tt = C.num_inst >= 4 * ctx->num_sms ? 128 : tail_threads<T>();
-  CR_LAUNCH(ctx, cr_tail_normal_kernel<T><<<(unsigned)C.num_inst, tt, 0, st>>>(A, dx, xadd));
+  CR_LAUNCH(ctx, (unsigned)C.num_inst, tt, 0, cr_tail_normal_kernel<T>, A, dx, xadd);
   for (int l = C.levels - 1; l >= 0; --l)
-    CR_LAUNCH(ctx, cr_backsub_kernel<T><<<nblk(C.lvl_n[l] * kItemThreads, 128), 128, 0, st>>>(
-                       A, items + C.lvl_off[l], C.lvl_n[l], l, 1, dx, xadd));
+    CR_LAUNCH(ctx, nblk(C.lvl_n[l] * kItemThreads, 128), 128, 0, cr_backsub_kernel<T>, A, items + C.lvl_off[l],
+              C.lvl_n[l], l, 1, dx, xadd);
   return QRKIT_OK;
 }
 

@@ -14,6 +14,7 @@
 
 #include <algorithm>
 
+#include "chain.cuh"
 #include "device_util.cuh"
 #include "internal.h"
 
@@ -31,6 +32,7 @@ __device__ __forceinline__ void cp_async_small(void* dst, const void* src) {
 template <typename T, int NA, int MM, int CC>
 __global__ void __launch_bounds__(kThreads) dense_apply_kernel(ComposedView<T> V, FactorOut<T> O, int cols_per_cta,
                                                                int ldr) {
+  dev::chain_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* buf = reinterpret_cast<T*>(smem_raw);   // two buffers of CC columns x ldr rows
   const int tid = threadIdx.x;
@@ -155,7 +157,7 @@ qrkit_status launch_apply(qrkit_ctx* ctx, const ComposedView<T>& V, const Factor
   const int groups = (V.s + CC - 1) / CC;
   const int per = (int)((groups + std::min<int64_t>(want, groups) - 1) / std::min<int64_t>(want, groups));
   const dim3 grid((unsigned)bx, (unsigned)((groups + per - 1) / per));
-  k<<<grid, kThreads, smem, ctx->stream>>>(V, O, per * CC, ldr);
+  chain_launch(ctx->stream, grid, kThreads, smem, k, V, O, per * CC, ldr);
   ctx->launches += 1;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());
   return QRKIT_OK;

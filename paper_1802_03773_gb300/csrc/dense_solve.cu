@@ -15,6 +15,7 @@
 
 #include <algorithm>
 
+#include "chain.cuh"
 #include "device_util.cuh"
 #include "internal.h"
 
@@ -141,6 +142,7 @@ __device__ __forceinline__ T tri_fwdsub(const T* R, int64_t ld, int s, T g, T* x
 template <typename T>
 __global__ void __launch_bounds__(kTriThreads) tri_backsub_kernel(const T* R, int64_t ld, int s, const T* c, T* x,
                                                                   int* status) {
+  dev::chain_wait();
   __shared__ T xs[32];
   const int i = threadIdx.x;
   const T y = tri_backsub<T>(R, ld, s, i < s ? c[i] : T(0), xs, status);
@@ -151,6 +153,7 @@ __global__ void __launch_bounds__(kTriThreads) tri_backsub_kernel(const T* R, in
 template <typename T>
 __global__ void __launch_bounds__(kTriThreads) tri_normal_kernel(const T* R, int64_t ld, int s, const double* g, T* dp,
                                                                  T* x, int* status) {
+  dev::chain_wait();
   __shared__ T xs[32];
   const int i = threadIdx.x;
   const T h = tri_fwdsub<T>(R, ld, s, i < s ? (T)g[i] : T(0), xs);
@@ -170,6 +173,7 @@ template <typename T>
 __global__ void __launch_bounds__(kWarpBackThreads) block_backsub_warp_kernel(ComposedView<T> V, FactorOut<T> O,
                                                                               const T* rhs, const T* xS, T* x,
                                                                               int accumulate) {
+  dev::chain_wait();
   __shared__ __align__(16) T xs[kMaxDenseS];
   const int s = V.s;
   for (int t = threadIdx.x; t < s; t += kWarpBackThreads) xs[t] = xS[t];
@@ -232,6 +236,7 @@ constexpr int kRowWarps = 8;
 template <int V>
 __global__ void __launch_bounds__(32 * kRowWarps) dense_rows_kernel(const float* S, int64_t rows, int s, const float* b,
                                                                     const float* pS, float* rh, float* rl) {
+  dev::chain_wait();
   __shared__ float sh_s[kRowWarps][32 * V], sl_s[kRowWarps][32 * V];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t row0 = (int64_t)blockIdx.x * (32 * V);
@@ -280,6 +285,7 @@ __global__ void __launch_bounds__(32 * kRowWarps) dense_rows_kernel(const float*
 // 2. blocks (one thread each): r -= J p, g_B = J^T r - lambda D^2 p, h_B = R_i^{-T} g_B.
 __global__ void __launch_bounds__(128) dense_blocks_kernel(ComposedView<float> V, FactorOut<float> O, const float* p,
                                                            double lam, float* rh, float* rl, float* h) {
+  dev::chain_wait();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= V.K) return;
   const int n = V.n[i], m = V.m[i];
@@ -336,6 +342,7 @@ constexpr int kSumCols = 2;    // columns per warp
 template <int V>
 __global__ void __launch_bounds__(32 * kSumWarps) dense_cols_kernel(const float* S, int64_t rows, int s, const float* rh,
                                                                     const float* rl, double* part) {
+  dev::chain_wait();
   __shared__ __align__(16) float rh_s[kSumRows], rl_s[kSumRows];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t row0 = (int64_t)blockIdx.x * kSumRows;
@@ -377,6 +384,7 @@ constexpr int kR12Threads = 256;
 template <int V>
 __global__ void __launch_bounds__(kR12Threads) dense_r12_kernel(const float* R12, int64_t nb, int s, const float* h,
                                                                 double* part) {
+  dev::chain_wait();
   __shared__ float h_s[kR12Rows];
   __shared__ double sum_s[kR12Threads * V];
   const int64_t j0 = (int64_t)blockIdx.x * kR12Rows;
@@ -415,6 +423,7 @@ __global__ void __launch_bounds__(kR12Threads) dense_r12_kernel(const float* R12
 __global__ void __launch_bounds__(256) dense_gsum_kernel(const double* part_s, int64_t ns, const double* part_r,
                                                          int64_t nr, int s, const double* DS, const float* pS,
                                                          double lam, double* gS) {
+  dev::chain_wait();
   const int c = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (c >= s) return;
   double t = 0;
@@ -441,7 +450,7 @@ inline unsigned nblk(int64_t n, int64_t t) { return (unsigned)((n + t - 1) / t);
 
 template <typename T>
 qrkit_status dense_backsub(qrkit_ctx* ctx, const T* R, int64_t ld, int s, const T* c, T* x) {
-  DS_LAUNCH(ctx, tri_backsub_kernel<T><<<1, tri_cta(s), 0, ctx->stream>>>(R, ld, s, c, x, ctx->d_status));
+  DS_LAUNCH(ctx, chain_launch(ctx->stream, 1, tri_cta(s), 0, tri_backsub_kernel<T>, R, ld, s, c, x, ctx->d_status));
   return QRKIT_OK;
 }
 template qrkit_status dense_backsub<float>(qrkit_ctx*, const float*, int64_t, int, const float*, float*);
@@ -449,7 +458,8 @@ template qrkit_status dense_backsub<double>(qrkit_ctx*, const double*, int64_t, 
 
 template <typename T>
 qrkit_status dense_normal(qrkit_ctx* ctx, const T* R, int64_t ld, int s, const double* g, T* dp, T* x) {
-  DS_LAUNCH(ctx, tri_normal_kernel<T><<<1, tri_cta(s), 0, ctx->stream>>>(R, ld, s, g, dp, x, ctx->d_status));
+  DS_LAUNCH(ctx, chain_launch(ctx->stream, 1, tri_cta(s), 0, tri_normal_kernel<T>, R, ld, s, g, dp, x,
+                              ctx->d_status));
   return QRKIT_OK;
 }
 template qrkit_status dense_normal<float>(qrkit_ctx*, const float*, int64_t, int, const double*, float*, float*);
@@ -458,8 +468,8 @@ template qrkit_status dense_normal<double>(qrkit_ctx*, const double*, int64_t, i
 template <typename T>
 qrkit_status dense_block_backsub(qrkit_ctx* ctx, const ComposedView<T>& V, const FactorOut<T>& O, const T* rhs,
                                  const T* xS, T* x, int accumulate) {
-  DS_LAUNCH(ctx, block_backsub_warp_kernel<T><<<nblk(V.K * 32, kWarpBackThreads), kWarpBackThreads, 0, ctx->stream>>>(
-                     V, O, rhs, xS, x, accumulate));
+  DS_LAUNCH(ctx, chain_launch(ctx->stream, nblk(V.K * 32, kWarpBackThreads), kWarpBackThreads, 0,
+                              block_backsub_warp_kernel<T>, V, O, rhs, xS, x, accumulate));
   return QRKIT_OK;
 }
 template qrkit_status dense_block_backsub<float>(qrkit_ctx*, const ComposedView<float>&, const FactorOut<float>&,
@@ -484,23 +494,25 @@ qrkit_status dense_refine_gradient(qrkit_ctx* ctx, const ComposedView<float>& V,
   // 16-byte loads where every column of the caller's S is 16-byte aligned
   const bool v4 = (V.rows & 3) == 0 && (reinterpret_cast<uintptr_t>(V.S) & 15) == 0;
   if (v4)
-    DS_LAUNCH(ctx, dense_rows_kernel<4><<<nblk(V.rows, 128), 32 * kRowWarps, 0, st>>>(V.S, V.rows, s, b, p + V.nb, rh, rl));
+    DS_LAUNCH(ctx, chain_launch(st, nblk(V.rows, 128), 32 * kRowWarps, 0, dense_rows_kernel<4>, V.S, V.rows, s, b,
+                                p + V.nb, rh, rl));
   else
-    DS_LAUNCH(ctx, dense_rows_kernel<1><<<nblk(V.rows, 32), 32 * kRowWarps, 0, st>>>(V.S, V.rows, s, b, p + V.nb, rh, rl));
-  DS_LAUNCH(ctx, dense_blocks_kernel<<<nblk(V.K, 128), 128, 0, st>>>(V, O, p, lam, rh, rl, h));
+    DS_LAUNCH(ctx, chain_launch(st, nblk(V.rows, 32), 32 * kRowWarps, 0, dense_rows_kernel<1>, V.S, V.rows, s, b,
+                                p + V.nb, rh, rl));
+  DS_LAUNCH(ctx, chain_launch(st, nblk(V.K, 128), 128, 0, dense_blocks_kernel, V, O, p, lam, rh, rl, h));
   const dim3 gs((unsigned)ns, nblk(s, kSumWarps * kSumCols));
   if (v4)
-    DS_LAUNCH(ctx, dense_cols_kernel<4><<<gs, 32 * kSumWarps, 0, st>>>(V.S, V.rows, s, rh, rl, part_s));
+    DS_LAUNCH(ctx, chain_launch(st, gs, 32 * kSumWarps, 0, dense_cols_kernel<4>, V.S, V.rows, s, rh, rl, part_s));
   else
-    DS_LAUNCH(ctx, dense_cols_kernel<1><<<gs, 32 * kSumWarps, 0, st>>>(V.S, V.rows, s, rh, rl, part_s));
+    DS_LAUNCH(ctx, chain_launch(st, gs, 32 * kSumWarps, 0, dense_cols_kernel<1>, V.S, V.rows, s, rh, rl, part_s));
   if ((s & 3) == 0)
-    DS_LAUNCH(ctx, dense_r12_kernel<4><<<dim3((unsigned)nr, nblk(s / 4, kR12Threads)), kR12Threads, 0, st>>>(
-                       O.R12, V.nb, s, h, part_r));
+    DS_LAUNCH(ctx, chain_launch(st, dim3((unsigned)nr, nblk(s / 4, kR12Threads)), kR12Threads, 0, dense_r12_kernel<4>,
+                                O.R12, V.nb, s, h, part_r));
   else
-    DS_LAUNCH(ctx, dense_r12_kernel<1><<<dim3((unsigned)nr, nblk(s, kR12Threads)), kR12Threads, 0, st>>>(
-                       O.R12, V.nb, s, h, part_r));
-  DS_LAUNCH(ctx, dense_gsum_kernel<<<nblk((int64_t)s * 32, 256), 256, 0, st>>>(part_s, ns, part_r, nr, s, O.D + V.nb,
-                                                                             p + V.nb, lam, gS));
+    DS_LAUNCH(ctx, chain_launch(st, dim3((unsigned)nr, nblk(s, kR12Threads)), kR12Threads, 0, dense_r12_kernel<1>,
+                                O.R12, V.nb, s, h, part_r));
+  DS_LAUNCH(ctx, chain_launch(st, nblk((int64_t)s * 32, 256), 256, 0, dense_gsum_kernel, part_s, ns, part_r, nr, s,
+                              O.D + V.nb, p + V.nb, lam, gS));
   return QRKIT_OK;
 }
 

@@ -29,6 +29,7 @@
 #include <string>
 #include <vector>
 
+#include "chain.cuh"
 #include "device_util.cuh"
 #include "internal.h"
 #include "mlp_policy.cuh"
@@ -86,6 +87,7 @@ constexpr int kCoef = 12;
 
 template <typename T>
 __global__ void cf_coef_kernel(LMTables t, const double* x, const T* p, double* coef) {
+  dev::chain_wait();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // shared column: control point e / 2, coordinate e % 2
   if (e + 6 >= t.s) return;
   // a segment that starts in the last three control points of a problem mixes two problems' and is never used
@@ -144,6 +146,7 @@ template <typename T>
 __global__ void __launch_bounds__(kTilePts)
 cf_eval_kernel(LMTables t, const double* x, const double* data, const double* coef, T* J, T* S, T* b, int32_t* start,
                double* tile_cost) {
+  dev::chain_wait();
   __shared__ double red[kTilePts];
   const int64_t tile = blockIdx.x;
   const int64_t i = t.tile_p0[tile] + threadIdx.x;
@@ -187,6 +190,7 @@ cf_eval_kernel(LMTables t, const double* x, const double* data, const double* co
 template <typename T>
 __global__ void __launch_bounds__(kTilePts) lm_damp_kernel(LMTables t, const T* J, const double* d2,
                                                            const qrkit_lm_state* st, double* E) {
+  dev::chain_wait();
   __shared__ double root;
   if (blockIdx.x < t.num_tiles) {
     const int64_t tile = blockIdx.x, i = t.tile_p0[tile] + threadIdx.x;
@@ -217,6 +221,7 @@ __global__ void __launch_bounds__(kTilePts) lm_damp_kernel(LMTables t, const T* 
 
 // f = curve(t) - data per point (two values), double.
 __global__ void cf_residual_kernel(LMTables t, const double* x, const double* data, double* f) {
+  dev::chain_wait();
   const int64_t tile = blockIdx.x;
   const int64_t i = t.tile_p0[tile] + threadIdx.x;
   if (i >= t.tile_p0[tile + 1]) return;
@@ -241,6 +246,7 @@ template <typename T>
 __global__ void __launch_bounds__(kTilePts)
 cf_trial_kernel(LMTables t, const double* x, const double* data, const double* coef, const T* J, const T* S, const T* b,
                 const T* p, const double* E, const int32_t* start, double* tile_new, double* tile_pred) {
+  dev::chain_wait();
   __shared__ double red[2][kTilePts];
   const int64_t tile = blockIdx.x;
   const int64_t i = t.tile_p0[tile] + threadIdx.x;
@@ -291,6 +297,7 @@ template <typename T>
 __global__ void lm_update_kernel(LMTables t, const double* tile_cost, const double* tile_new,
                                  const double* tile_pred, const double* E, const T* p, qrkit_lm_state* st,
                                  double ftol, int* ndone, MlpDev w, float* hist, float* feat) {
+  dev::chain_wait();
   __shared__ double part[3][kUpdateThreads / 32];
   const int64_t k = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -394,6 +401,7 @@ __global__ void lm_update_kernel(LMTables t, const double* tile_cost, const doub
 
 template <typename T>
 __global__ void lm_accept_kernel(LMTables t, const T* p, double* x, const qrkit_lm_state* st) {
+  dev::chain_wait();
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= t.N) return;
   if (st[t.col_prob[j]].accepted) x[j] += (double)p[j];
@@ -424,31 +432,31 @@ qrkit_status lm_iteration(qrkit_ctx* ctx, double* x, int refine_steps, double ft
   double* coef = (double*)L.coef.ptr;
   int32_t* start = (int32_t*)ctx->plan.d_start.ptr;   // the model's starts lie in their segments
   QRKIT_CUDA_TRY(ctx, cudaMemsetAsync(L.ndone.ptr, 0, sizeof(int), st));
-  LM_LAUNCH(ctx, cf_coef_kernel<T><<<nblk(t.s, 128), 128, 0, st>>>(t, x, (const T*)nullptr, coef));
-  LM_LAUNCH(ctx, cf_eval_kernel<T><<<(unsigned)t.num_tiles, kTilePts, 0, st>>>(t, x, L.data, coef, J, Sv, b, start,
-                                                                             (double*)L.tile_cost.ptr));
+  LM_LAUNCH(ctx, chain_launch(st, nblk(t.s, 128), 128, 0, cf_coef_kernel<T>, t, x, (const T*)nullptr, coef));
+  LM_LAUNCH(ctx, chain_launch(st, (unsigned)t.num_tiles, kTilePts, 0, cf_eval_kernel<T>, t, x, L.data, coef, J, Sv, b,
+                              start, (double*)L.tile_cost.ptr));
   bool sorted = false;
   qrkit_status rc = composed_sort_blocks(ctx, &sorted);
   if (rc != QRKIT_OK) return rc;
   if (!sorted) return fail(ctx, QRKIT_ESTATE, "the LM plan has no block sort");
   if ((rc = composed_window_sums(ctx, Sv, d2)) != QRKIT_OK) return rc;
-  LM_LAUNCH(ctx, lm_damp_kernel<T><<<(unsigned)(t.num_tiles + (t.s + kTilePts - 1) / kTilePts), kTilePts, 0, st>>>(
-                     t, J, d2, S, E));
+  LM_LAUNCH(ctx, chain_launch(st, (unsigned)(t.num_tiles + (t.s + kTilePts - 1) / kTilePts), kTilePts, 0,
+                              lm_damp_kernel<T>, t, J, d2, S, E));
   if ((rc = composed_factor_scaled(ctx, J, Sv, E, true)) != QRKIT_OK) return rc;
   if ((rc = composed_solve(ctx, J, Sv, b, p, refine_steps)) != QRKIT_OK) return rc;
-  LM_LAUNCH(ctx, cf_coef_kernel<T><<<nblk(t.s, 128), 128, 0, st>>>(t, x, p, coef));
-  LM_LAUNCH(ctx, cf_trial_kernel<T><<<(unsigned)t.num_tiles, kTilePts, 0, st>>>(
-                     t, x, L.data, coef, J, Sv, b, p, E, start, (double*)L.tile_new.ptr, (double*)L.tile_pred.ptr));
+  LM_LAUNCH(ctx, chain_launch(st, nblk(t.s, 128), 128, 0, cf_coef_kernel<T>, t, x, p, coef));
+  LM_LAUNCH(ctx, chain_launch(st, (unsigned)t.num_tiles, kTilePts, 0, cf_trial_kernel<T>, t, x, L.data, coef, J, Sv,
+                              b, p, E, start, (double*)L.tile_new.ptr, (double*)L.tile_pred.ptr));
   MlpDev w{};
   if (L.policy && ctx->mlp) {
     w.theta = (const float*)ctx->mlp->theta.ptr;
     w.wbf = (const __nv_bfloat16*)ctx->mlp->wbf.ptr;
   }
-  LM_LAUNCH(ctx, lm_update_kernel<T><<<(unsigned)t.B, t.B >= 2 * ctx->num_sms ? 32 : kUpdateThreads, 0, st>>>(
-                     t, (const double*)L.tile_cost.ptr, (const double*)L.tile_new.ptr,
-                     (const double*)L.tile_pred.ptr, E, p, S, ftol, (int*)L.ndone.ptr, w, (float*)L.hist.ptr,
-                     (float*)L.feat.ptr));
-  LM_LAUNCH(ctx, lm_accept_kernel<T><<<nblk(t.N, 256), 256, 0, st>>>(t, p, x, S));
+  LM_LAUNCH(ctx, chain_launch(st, (unsigned)t.B, t.B >= 2 * ctx->num_sms ? 32 : kUpdateThreads, 0,
+                              lm_update_kernel<T>, t, (const double*)L.tile_cost.ptr, (const double*)L.tile_new.ptr,
+                              (const double*)L.tile_pred.ptr, E, p, S, ftol, (int*)L.ndone.ptr, w, (float*)L.hist.ptr,
+                              (float*)L.feat.ptr));
+  LM_LAUNCH(ctx, chain_launch(st, nblk(t.N, 256), 256, 0, lm_accept_kernel<T>, t, p, x, S));
   return QRKIT_OK;
 }
 
@@ -618,15 +626,14 @@ qrkit_status qrkit_lm_linearize(qrkit_ctx* ctx, const double* x, void* J, void* 
   cudaStream_t st = ctx->stream;
   const double* coef = (const double*)L.coef.ptr;
   if (ctx->precision == QRKIT_FP64) {
-    cf_coef_kernel<double><<<nblk(t.s, 128), 128, 0, st>>>(t, x, (const double*)nullptr, (double*)L.coef.ptr);
-    cf_eval_kernel<double><<<(unsigned)t.num_tiles, kTilePts, 0, st>>>(
-        t, x, L.data, coef, (double*)L.J.ptr, (double*)L.S.ptr, (double*)L.b.ptr, (int32_t*)L.start.ptr,
-        (double*)L.tile_cost.ptr);
+    chain_launch(st, nblk(t.s, 128), 128, 0, cf_coef_kernel<double>, t, x, (const double*)nullptr,
+                 (double*)L.coef.ptr);
+    chain_launch(st, (unsigned)t.num_tiles, kTilePts, 0, cf_eval_kernel<double>, t, x, L.data, coef, (double*)L.J.ptr,
+                 (double*)L.S.ptr, (double*)L.b.ptr, (int32_t*)L.start.ptr, (double*)L.tile_cost.ptr);
   } else {
-    cf_coef_kernel<float><<<nblk(t.s, 128), 128, 0, st>>>(t, x, (const float*)nullptr, (double*)L.coef.ptr);
-    cf_eval_kernel<float><<<(unsigned)t.num_tiles, kTilePts, 0, st>>>(
-        t, x, L.data, coef, (float*)L.J.ptr, (float*)L.S.ptr, (float*)L.b.ptr, (int32_t*)L.start.ptr,
-        (double*)L.tile_cost.ptr);
+    chain_launch(st, nblk(t.s, 128), 128, 0, cf_coef_kernel<float>, t, x, (const float*)nullptr, (double*)L.coef.ptr);
+    chain_launch(st, (unsigned)t.num_tiles, kTilePts, 0, cf_eval_kernel<float>, t, x, L.data, coef, (float*)L.J.ptr,
+                 (float*)L.S.ptr, (float*)L.b.ptr, (int32_t*)L.start.ptr, (double*)L.tile_cost.ptr);
   }
   ctx->launches += 2;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());
@@ -645,7 +652,7 @@ qrkit_status qrkit_lm_residual(qrkit_ctx* ctx, const double* x, double* f) {
   if (!x || !f) return fail(ctx, QRKIT_EINVAL, "x and f are required");
   QRKIT_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
   LM& L = *ctx->lm;
-  cf_residual_kernel<<<(unsigned)L.t.num_tiles, kTilePts, 0, ctx->stream>>>(L.t, x, L.data, f);
+  chain_launch(ctx->stream, (unsigned)L.t.num_tiles, kTilePts, 0, cf_residual_kernel, L.t, x, L.data, f);
   ctx->launches += 1;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());
   return QRKIT_OK;

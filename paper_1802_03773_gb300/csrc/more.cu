@@ -18,6 +18,7 @@
 #include <algorithm>
 
 #include "block_tasks.cuh"
+#include "chain.cuh"
 #include "internal.h"
 
 namespace qrkit {
@@ -150,6 +151,7 @@ __device__ __forceinline__ void load_d(const MoreArgs<T>& A, const T (&R)[kM][kM
 // Warp-task factor: one thread per task slot.
 template <typename T, bool SUMS>
 __global__ void __launch_bounds__(128) more_planes_kernel(MoreArgs<T> A) {
+  dev::chain_wait();
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t t = gid >> 5;
   const int slot = (int)(gid & 31);
@@ -179,6 +181,7 @@ __global__ void __launch_bounds__(128) more_planes_kernel(MoreArgs<T> A) {
 // Tile-mapping factor (J's packing): one thread per block.
 template <typename T, bool SUMS>
 __global__ void __launch_bounds__(128) more_packed_kernel(MoreArgs<T> A) {
+  dev::chain_wait();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   double part[3] = {0.0, 0.0, 0.0};
   if (i < A.K) {
@@ -215,9 +218,9 @@ qrkit_status more_typed(qrkit_ctx* ctx, const void* qtb, const void* D, double l
     A.tF = (const T*)ctx->ws.tfactor.ptr;
     const int64_t threads = P.num_tasks * 32;
     if (sums)
-      more_planes_kernel<T, true><<<(unsigned)((threads + 127) / 128), 128, 0, ctx->stream>>>(A);
+      chain_launch(ctx->stream, (unsigned)((threads + 127) / 128), 128, 0, (more_planes_kernel<T, true>), A);
     else
-      more_planes_kernel<T, false><<<(unsigned)((threads + 127) / 128), 128, 0, ctx->stream>>>(A);
+      chain_launch(ctx->stream, (unsigned)((threads + 127) / 128), 128, 0, (more_planes_kernel<T, false>), A);
   } else {
     A.F = (const T*)ctx->ws.factor.ptr;
     A.val_off = (const int64_t*)P.d_val_off.ptr;
@@ -227,9 +230,9 @@ qrkit_status more_typed(qrkit_ctx* ctx, const void* qtb, const void* D, double l
     A.m = (const uint8_t*)P.d_m.ptr;
     A.K = P.K;
     if (sums)
-      more_packed_kernel<T, true><<<(unsigned)((P.K + 127) / 128), 128, 0, ctx->stream>>>(A);
+      chain_launch(ctx->stream, (unsigned)((P.K + 127) / 128), 128, 0, (more_packed_kernel<T, true>), A);
     else
-      more_packed_kernel<T, false><<<(unsigned)((P.K + 127) / 128), 128, 0, ctx->stream>>>(A);
+      chain_launch(ctx->stream, (unsigned)((P.K + 127) / 128), 128, 0, (more_packed_kernel<T, false>), A);
   }
   ctx->launches += 1;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());

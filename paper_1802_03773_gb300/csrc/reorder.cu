@@ -25,6 +25,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "chain.cuh"
 #include "internal.h"
 
 namespace qrkit {
@@ -46,6 +47,7 @@ __device__ __forceinline__ int64_t clamp_key(int64_t start, int64_t col0, int64_
 }
 
 __global__ void rsort_count_kernel(RowSortTables t, const int64_t* Xstart, int* hist, int* status) {
+  dev::chain_wait();
   const int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (c >= t.num_chunks) return;
@@ -63,6 +65,7 @@ constexpr int kBinThreads = 256;
 // Pass 1 of the scan: bin b of segment blockIdx.x; chunk-minor exclusive prefixes in place,
 // the bin's total to tot (indexed by global shared column).
 __global__ void __launch_bounds__(kBinThreads) rsort_bin_prefix_kernel(RowSortTables t, int* hist, int* tot) {
+  dev::chain_wait();
   const int64_t seg = blockIdx.x;
   const int64_t c0 = t.seg_chunk0[seg], c1 = t.seg_chunk0[seg + 1];
   if (c0 == c1) return;
@@ -80,6 +83,7 @@ __global__ void __launch_bounds__(kBinThreads) rsort_bin_prefix_kernel(RowSortTa
 
 // Pass 2: exclusive scan of a segment's bin totals (one CTA per segment), in place.
 __global__ void __launch_bounds__(kScanThreads) rsort_bin_scan_kernel(RowSortTables t, int* tot) {
+  dev::chain_wait();
   __shared__ int warp_tot[kScanThreads / 32];
   __shared__ int carry_s;
   const int64_t seg = blockIdx.x;
@@ -121,6 +125,7 @@ __global__ void __launch_bounds__(kScanThreads) rsort_bin_scan_kernel(RowSortTab
 
 // Pass 3: the bin's base added to its chunk entries.
 __global__ void __launch_bounds__(kBinThreads) rsort_bin_add_kernel(RowSortTables t, int* hist, const int* tot) {
+  dev::chain_wait();
   const int64_t seg = blockIdx.x;
   const int64_t c0 = t.seg_chunk0[seg], c1 = t.seg_chunk0[seg + 1];
   if (c0 == c1) return;
@@ -134,6 +139,7 @@ template <typename T>
 __global__ void rsort_scatter_kernel(RowSortTables t, const int64_t* Xstart, const T* Xw, int w,
                                      int* hist, int64_t* spos, int64_t* order, int64_t* Xstart_s,
                                      T* Xw_s) {
+  dev::chain_wait();
   const int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (c >= t.num_chunks) return;
@@ -181,6 +187,7 @@ __global__ void rsort_scatter_kernel(RowSortTables t, const int64_t* Xstart, con
 
 template <typename T>
 __global__ void rsort_rhs_kernel(const int64_t* spos, const T* rhs, T* rhs_s, int64_t rows) {
+  dev::chain_wait();
   const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (r < rows) rhs_s[spos[r]] = rhs[r];
 }
@@ -188,6 +195,7 @@ __global__ void rsort_rhs_kernel(const int64_t* spos, const T* rhs, T* rhs_s, in
 // ---- blocks of one shape ----
 __global__ void __launch_bounds__(256) bsort_count_kernel(BlockSortTables t, const int32_t* start, int* hist,
                                                           int* status) {
+  dev::chain_wait();
   const int64_t c = blockIdx.x;
   const int64_t k = t.chunk_seg[c], b0 = t.chunk_blk0[c], b1 = t.chunk_blk0[c + 1];
   const int64_t col0 = t.seg_col0[k], cols = t.seg_col0[k + 1] - col0, nch = t.seg_chunk0[k + 1] - t.seg_chunk0[k];
@@ -197,6 +205,7 @@ __global__ void __launch_bounds__(256) bsort_count_kernel(BlockSortTables t, con
 
 // Bin of shared column j: its chunk counts to exclusive prefixes in place, the total to colptr[j].
 __global__ void __launch_bounds__(256) bsort_prefix_kernel(BlockSortTables t, int64_t s, int* hist, int32_t* colptr) {
+  dev::chain_wait();
   const int64_t j = ((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (j >= s) return;
@@ -220,6 +229,7 @@ __global__ void __launch_bounds__(256) bsort_prefix_kernel(BlockSortTables t, in
 // Per segment (one CTA): bin totals to first sorted blocks, in place; colptr[s] = all blocks.
 __global__ void __launch_bounds__(kScanThreads) bsort_scan_kernel(BlockSortTables t, int64_t s, int64_t K,
                                                                   int32_t* colptr) {
+  dev::chain_wait();
   __shared__ int warp_tot[kScanThreads / 32];
   __shared__ int carry_s;
   const int64_t k = blockIdx.x;
@@ -263,6 +273,7 @@ __global__ void __launch_bounds__(kScanThreads) bsort_scan_kernel(BlockSortTable
 // One warp per chunk, its blocks in order: bpos[i] = sorted position of block i, bord its inverse.
 __global__ void __launch_bounds__(128) bsort_scatter_kernel(BlockSortTables t, const int32_t* start, int* hist,
                                                             const int32_t* colptr, int32_t* bpos, int32_t* bord) {
+  dev::chain_wait();
   const int64_t c = ((int64_t)blockIdx.x * 128 + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (c >= t.num_chunks) return;
@@ -295,6 +306,7 @@ __global__ void __launch_bounds__(128) bsort_scatter_kernel(BlockSortTables t, c
 
 // The order of the reduced rows from that of the blocks, q rows each.
 __global__ void rows_of_blocks_kernel(const int32_t* bord, int64_t K, int q, int64_t* order) {
+  dev::chain_wait();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= K * q) return;
   order[e] = (int64_t)bord[e / q] * q + e % q;
@@ -305,6 +317,7 @@ __global__ void rows_of_blocks_kernel(const int32_t* bord, int64_t K, int q, int
 // is recorded as QRKIT_EINVAL and clamped.
 __global__ void start_copy_kernel(const int32_t* in, int32_t* out, int64_t K, const int64_t* seg, int64_t nseg,
                                   int* status) {
+  dev::chain_wait();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= K) return;
   const int64_t* blk0 = seg;
@@ -329,8 +342,8 @@ inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 qrkit_status window_start_copy(qrkit_ctx* ctx, const int32_t* in) {
   Plan& P = ctx->plan;
   const int64_t nseg = (int64_t)P.seg_cols.size();
-  start_copy_kernel<<<nblk(P.K, 256), 256, 0, ctx->stream>>>(in, (int32_t*)P.d_start.ptr, P.K,
-                                                              (const int64_t*)P.d_seg.ptr, nseg, ctx->d_status);
+  chain_launch(ctx->stream, nblk(P.K, 256), 256, 0, start_copy_kernel, in, (int32_t*)P.d_start.ptr, P.K,
+               (const int64_t*)P.d_seg.ptr, nseg, ctx->d_status);
   ctx->launches += 1;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());
   return QRKIT_OK;
@@ -342,7 +355,7 @@ qrkit_status reduced_row_sort(qrkit_ctx* ctx, const RowSortTables& t, int64_t ns
   cudaStream_t st = ctx->stream;
   if (t.num_chunks == 0) return QRKIT_OK;
   QRKIT_CUDA_TRY(ctx, cudaMemsetAsync(hist, 0, (size_t)hist_entries * sizeof(int), st));
-  rsort_count_kernel<<<nblk(t.num_chunks * 32, 128), 128, 0, st>>>(t, Xstart, hist, ctx->d_status);
+  chain_launch(st, nblk(t.num_chunks * 32, 128), 128, 0, rsort_count_kernel, t, Xstart, hist, ctx->d_status);
   ctx->launches += 1;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());
   {
@@ -351,18 +364,18 @@ qrkit_status reduced_row_sort(qrkit_ctx* ctx, const RowSortTables& t, int64_t ns
     for (const int64_t c : ctx->plan.seg_cols) maxcols = c > maxcols ? c : maxcols;
     int* tot = hist + hist_entries;
     const dim3 grid((unsigned)nseg, (unsigned)((maxcols + kBinThreads - 1) / kBinThreads));
-    rsort_bin_prefix_kernel<<<grid, kBinThreads, 0, st>>>(t, hist, tot);
-    rsort_bin_scan_kernel<<<(unsigned)nseg, kScanThreads, 0, st>>>(t, tot);
-    rsort_bin_add_kernel<<<grid, kBinThreads, 0, st>>>(t, hist, tot);
+    chain_launch(st, grid, kBinThreads, 0, rsort_bin_prefix_kernel, t, hist, tot);
+    chain_launch(st, (unsigned)nseg, kScanThreads, 0, rsort_bin_scan_kernel, t, tot);
+    chain_launch(st, grid, kBinThreads, 0, rsort_bin_add_kernel, t, hist, tot);
     ctx->launches += 3;
     QRKIT_CUDA_TRY(ctx, cudaGetLastError());
   }
   if (ctx->precision == QRKIT_FP64)
-    rsort_scatter_kernel<double><<<nblk(t.num_chunks * 32, 128), 128, 0, st>>>(
-        t, Xstart, (const double*)Xw, w, hist, spos, order, Xstart_s, (double*)Xw_s);
+    chain_launch(st, nblk(t.num_chunks * 32, 128), 128, 0, rsort_scatter_kernel<double>, t, Xstart, (const double*)Xw,
+                 w, hist, spos, order, Xstart_s, (double*)Xw_s);
   else
-    rsort_scatter_kernel<float><<<nblk(t.num_chunks * 32, 128), 128, 0, st>>>(
-        t, Xstart, (const float*)Xw, w, hist, spos, order, Xstart_s, (float*)Xw_s);
+    chain_launch(st, nblk(t.num_chunks * 32, 128), 128, 0, rsort_scatter_kernel<float>, t, Xstart, (const float*)Xw,
+                 w, hist, spos, order, Xstart_s, (float*)Xw_s);
   ctx->launches += 1;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());
   return QRKIT_OK;
@@ -374,10 +387,11 @@ qrkit_status block_sort(qrkit_ctx* ctx, const BlockSortTables& t, const int32_t*
   cudaStream_t st = ctx->stream;
   const int64_t s = P.s.shared_cols, nseg = (int64_t)P.seg_cols.size();
   QRKIT_CUDA_TRY(ctx, cudaMemsetAsync(hist, 0, (size_t)hist_entries * sizeof(int), st));
-  bsort_count_kernel<<<(unsigned)t.num_chunks, 256, 0, st>>>(t, start, hist, ctx->d_status);
-  bsort_prefix_kernel<<<nblk(s * 32, 256), 256, 0, st>>>(t, s, hist, colptr);
-  bsort_scan_kernel<<<(unsigned)nseg, nseg >= 2 * ctx->num_sms ? 128 : kScanThreads, 0, st>>>(t, s, P.K, colptr);
-  bsort_scatter_kernel<<<nblk(t.num_chunks * 32, 128), 128, 0, st>>>(t, start, hist, colptr, bpos, bord);
+  chain_launch(st, (unsigned)t.num_chunks, 256, 0, bsort_count_kernel, t, start, hist, ctx->d_status);
+  chain_launch(st, nblk(s * 32, 256), 256, 0, bsort_prefix_kernel, t, s, hist, colptr);
+  chain_launch(st, (unsigned)nseg, nseg >= 2 * ctx->num_sms ? 128 : kScanThreads, 0, bsort_scan_kernel, t, s, P.K,
+               colptr);
+  chain_launch(st, nblk(t.num_chunks * 32, 128), 128, 0, bsort_scatter_kernel, t, start, hist, colptr, bpos, bord);
   ctx->launches += 4;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());
   return QRKIT_OK;
@@ -386,7 +400,7 @@ qrkit_status block_sort(qrkit_ctx* ctx, const BlockSortTables& t, const int32_t*
 qrkit_status block_row_order(qrkit_ctx* ctx, const int32_t* bord, int q, int64_t* order) {
   const int64_t K = ctx->plan.K;
   if (K * q == 0) return QRKIT_OK;
-  rows_of_blocks_kernel<<<nblk(K * q, 256), 256, 0, ctx->stream>>>(bord, K, q, order);
+  chain_launch(ctx->stream, nblk(K * q, 256), 256, 0, rows_of_blocks_kernel, bord, K, q, order);
   ctx->launches += 1;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());
   return QRKIT_OK;
@@ -395,11 +409,11 @@ qrkit_status block_row_order(qrkit_ctx* ctx, const int32_t* bord, int q, int64_t
 qrkit_status reduced_rhs_sort(qrkit_ctx* ctx, const int64_t* spos, const void* rhs, void* rhs_s, int64_t rows) {
   if (rows == 0) return QRKIT_OK;
   if (ctx->precision == QRKIT_FP64)
-    rsort_rhs_kernel<double><<<nblk(rows, 256), 256, 0, ctx->stream>>>(spos, (const double*)rhs,
-                                                                         (double*)rhs_s, rows);
+    chain_launch(ctx->stream, nblk(rows, 256), 256, 0, rsort_rhs_kernel<double>, spos, (const double*)rhs,
+                 (double*)rhs_s, rows);
   else
-    rsort_rhs_kernel<float><<<nblk(rows, 256), 256, 0, ctx->stream>>>(spos, (const float*)rhs,
-                                                                        (float*)rhs_s, rows);
+    chain_launch(ctx->stream, nblk(rows, 256), 256, 0, rsort_rhs_kernel<float>, spos, (const float*)rhs,
+                 (float*)rhs_s, rows);
   ctx->launches += 1;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());
   return QRKIT_OK;

@@ -13,6 +13,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include "chain.cuh"
 #include "device_util.cuh"
 #include "internal.h"
 
@@ -86,6 +87,7 @@ __device__ __forceinline__ void reflector(float alpha, float sq, float& beta, fl
 template <typename T, int RPL, int CPW>
 __global__ void __launch_bounds__(kThreads) tsqr_tile_kernel(T* X, int64_t ld, int64_t M, int s, int rows, T* taus,
                                                              T* Xn, int64_t ldn) {
+  dev::chain_wait();
   constexpr int kRows = 32 * RPL;
   __shared__ T V[2][kRows];
   __shared__ T tslot[2];
@@ -191,6 +193,7 @@ constexpr int kQtThreads = 128;
 template <typename T, int RPT>
 __global__ void __launch_bounds__(kQtThreads) tsqr_qt_kernel(const T* X, int64_t ld, int64_t M, int s, const T* taus,
                                                              T* rhs, T* rhs_next) {
+  dev::chain_wait();
   constexpr int kRows = kQtThreads * RPT;
   __shared__ T part[2][kQtThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -236,10 +239,10 @@ __global__ void __launch_bounds__(kQtThreads) tsqr_qt_kernel(const T* X, int64_t
 template <typename T, int RPL>
 void launch_tile(unsigned g, cudaStream_t st, T* X, int64_t ld, int64_t M, int s, int rows, T* taus, T* Xn,
                  int64_t ldn) {
-  if (s <= 8) tsqr_tile_kernel<T, RPL, 1><<<g, kThreads, 0, st>>>(X, ld, M, s, rows, taus, Xn, ldn);
-  else if (s <= 16) tsqr_tile_kernel<T, RPL, 2><<<g, kThreads, 0, st>>>(X, ld, M, s, rows, taus, Xn, ldn);
-  else if (s <= 32) tsqr_tile_kernel<T, RPL, 4><<<g, kThreads, 0, st>>>(X, ld, M, s, rows, taus, Xn, ldn);
-  else tsqr_tile_kernel<T, RPL, 8><<<g, kThreads, 0, st>>>(X, ld, M, s, rows, taus, Xn, ldn);
+  if (s <= 8) chain_launch(st, g, kThreads, 0, (tsqr_tile_kernel<T, RPL, 1>), X, ld, M, s, rows, taus, Xn, ldn);
+  else if (s <= 16) chain_launch(st, g, kThreads, 0, (tsqr_tile_kernel<T, RPL, 2>), X, ld, M, s, rows, taus, Xn, ldn);
+  else if (s <= 32) chain_launch(st, g, kThreads, 0, (tsqr_tile_kernel<T, RPL, 4>), X, ld, M, s, rows, taus, Xn, ldn);
+  else chain_launch(st, g, kThreads, 0, (tsqr_tile_kernel<T, RPL, 8>), X, ld, M, s, rows, taus, Xn, ldn);
 }
 
 }  // namespace
@@ -267,9 +270,11 @@ template <typename T>
 qrkit_status tsqr_qt(qrkit_ctx* ctx, const T* X, int64_t ld, int64_t M, int s, int rows, const T* taus, T* rhs,
                      T* rhs_next, int64_t tiles) {
   if (rows == 128)
-    tsqr_qt_kernel<T, 1><<<(unsigned)tiles, kQtThreads, 0, ctx->stream>>>(X, ld, M, s, taus, rhs, rhs_next);
+    chain_launch(ctx->stream, (unsigned)tiles, kQtThreads, 0, (tsqr_qt_kernel<T, 1>), X, ld, M, s, taus, rhs,
+                 rhs_next);
   else
-    tsqr_qt_kernel<T, 2><<<(unsigned)tiles, kQtThreads, 0, ctx->stream>>>(X, ld, M, s, taus, rhs, rhs_next);
+    chain_launch(ctx->stream, (unsigned)tiles, kQtThreads, 0, (tsqr_qt_kernel<T, 2>), X, ld, M, s, taus, rhs,
+                 rhs_next);
   ctx->launches += 1;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());
   return QRKIT_OK;

@@ -19,6 +19,7 @@
 
 #include <algorithm>
 
+#include "chain.cuh"
 #include "device_util.cuh"
 #include "f32x2.cuh"
 #include "internal.h"
@@ -96,6 +97,7 @@ constexpr size_t panel_tile_smem() { return (size_t)kNb * 128 * NU * 4; }
 template <int NU>
 __global__ void __launch_bounds__(kPT, 1)
 tsqr_panel_tile_kernel(float* X, int64_t ld, int64_t M, float* Xn, int64_t ldn, float* Tout, float* Gout, int* status) {
+  dev::chain_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* V = reinterpret_cast<float*>(smem_raw);   // 32 reflectors of 128 NU rows
   __shared__ float Gs[kNb * kPad], Tm[kNb * kPad], Ws[16 * kPad];
@@ -378,6 +380,7 @@ __device__ __forceinline__ void team_sync(int team) {
 __global__ void __launch_bounds__(kAT, 1)
 tsqr_panel_apply_kernel(const float* X, int64_t ld, int64_t M, const float* Tin, int n, int chunk, float* up,
                         int64_t ldu, float* down, int64_t ldd, int64_t down0) {
+  dev::chain_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* Y = reinterpret_cast<float*>(smem_raw);   // 32 reflectors x 1024 rows, ypos()
   float* Tm = Y + kNb * kTR;                       // 32 x 32: T[l][i] at l * 32 + i
@@ -559,6 +562,7 @@ constexpr int kQT = kTR / 4;
 __global__ void __launch_bounds__(kQT, 1)
 tsqr_panel_qt_kernel(const float* X, int64_t ld, int64_t M, const float* Gin, const float* rhs, float* rhs_next,
                      float* rhs_down, int64_t down0) {
+  dev::chain_wait();
   __shared__ float ws[kQT / 32][kNb];
   __shared__ float zs[kNb];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -640,7 +644,7 @@ qrkit_status tsqr_panel_tile(qrkit_ctx* ctx, float* X, int64_t ld, int64_t M, fl
       const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
     }
-    k<<<g, kPT, smem, ctx->stream>>>(X, ld, M, Xn, ldn, Tout, Gout, ctx->d_status);
+    chain_launch(ctx->stream, g, kPT, smem, k, X, ld, M, Xn, ldn, Tout, Gout, ctx->d_status);
     return cudaSuccess;
   };
   if (M <= 256) QRKIT_CUDA_TRY(ctx, run(tsqr_panel_tile_kernel<2>, panel_tile_smem<2>()));
@@ -678,7 +682,8 @@ qrkit_status tsqr_panel_apply(qrkit_ctx* ctx, const float* X, int64_t ld, int64_
     }
   }
   const dim3 grid((unsigned)tiles, (unsigned)((n + chunk - 1) / chunk));
-  tsqr_panel_apply_kernel<<<grid, kAT, smem, ctx->stream>>>(X, ld, M, T, n, chunk, up, ldu, down, ldd, down0);
+  chain_launch(ctx->stream, grid, kAT, smem, tsqr_panel_apply_kernel, X, ld, M, T, n, chunk, up, ldu, down, ldd,
+               down0);
   ctx->launches += 1;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());
   return QRKIT_OK;
@@ -689,7 +694,8 @@ qrkit_status tsqr_panel_qt(qrkit_ctx* ctx, const float* X, int64_t ld, int64_t M
   if (!panel_aligned(X, ld, M) || !panel_aligned(rhs, 0, 0) || !panel_aligned(rhs_next, 0, 0) ||
       !panel_aligned(rhs_down, 0, down0))
     return fail(ctx, QRKIT_EINVAL, "column-panel TSQR: unaligned right-hand side");
-  tsqr_panel_qt_kernel<<<(unsigned)tiles, kQT, 0, ctx->stream>>>(X, ld, M, G, rhs, rhs_next, rhs_down, down0);
+  chain_launch(ctx->stream, (unsigned)tiles, kQT, 0, tsqr_panel_qt_kernel, X, ld, M, G, rhs, rhs_next, rhs_down,
+               down0);
   ctx->launches += 1;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());
   return QRKIT_OK;

@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "chain.cuh"
 #include "device_util.cuh"
 #include "internal.h"
 
@@ -47,6 +48,7 @@ struct Sum {
 // Eight lanes per run of kRun sorted blocks.  kGrad: sum of S^T r - R12^T h; else of the squares of S.
 template <typename T, bool kGrad, int NR, int MM>
 __global__ void __launch_bounds__(kThreads) window_sums_kernel(WindowSums<T> A) {
+  dev::chain_wait();
   const int64_t run = ((int64_t)blockIdx.x * kThreads + threadIdx.x) / kLanes;
   const int t = threadIdx.x % kLanes;
   const int64_t p0 = run * kRun, p1 = p0 + kRun < A.K ? p0 + kRun : A.K;
@@ -123,6 +125,7 @@ __global__ void __launch_bounds__(kThreads) window_sums_kernel(WindowSums<T> A) 
 template <typename T, int NR, int MM>
 __global__ void __launch_bounds__(128) window_blocks_kernel(ComposedView<T> V, FactorOut<T> O, const T* b, const T* p,
                                                             double lam, int n, int m, T* r, T* h) {
+  dev::chain_wait();
   const int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x;
   if (i >= V.K) return;
   const int na = n + (O.damp ? m : 0), w = V.w;
@@ -213,9 +216,9 @@ inline unsigned nblk(int64_t n, int64_t t) { return (unsigned)((n + t - 1) / t);
 template <typename T>
 qrkit_status window_square_sums(qrkit_ctx* ctx, const WindowSums<T>& A) {
   const unsigned g = nblk((A.K + kRun - 1) / kRun * kLanes, kThreads);
-  WS_SHAPED(ctx, A.n, A.m, (window_sums_kernel<T, false, 2, 1><<<g, kThreads, 0, ctx->stream>>>(A)),
-            (window_sums_kernel<T, false, 6, 2><<<g, kThreads, 0, ctx->stream>>>(A)),
-            (window_sums_kernel<T, false, 16, 8><<<g, kThreads, 0, ctx->stream>>>(A)));
+  WS_SHAPED(ctx, A.n, A.m, (chain_launch(ctx->stream, g, kThreads, 0, (window_sums_kernel<T, false, 2, 1>), A)),
+            (chain_launch(ctx->stream, g, kThreads, 0, (window_sums_kernel<T, false, 6, 2>), A)),
+            (chain_launch(ctx->stream, g, kThreads, 0, (window_sums_kernel<T, false, 16, 8>), A)));
   return QRKIT_OK;
 }
 template qrkit_status window_square_sums<float>(qrkit_ctx*, const WindowSums<float>&);
@@ -227,12 +230,14 @@ qrkit_status window_refine_gradient(qrkit_ctx* ctx, const ComposedView<T>& V, co
   const unsigned gb = nblk(V.K, 128), g = nblk((A.K + kRun - 1) / kRun * kLanes, kThreads);
   T* r = const_cast<T*>(A.r);
   T* h = const_cast<T*>(A.h);
-  WS_SHAPED(ctx, A.n, A.m, (window_blocks_kernel<T, 2, 1><<<gb, 128, 0, ctx->stream>>>(V, O, b, p, lam, A.n, A.m, r, h)),
-            (window_blocks_kernel<T, 6, 2><<<gb, 128, 0, ctx->stream>>>(V, O, b, p, lam, A.n, A.m, r, h)),
-            (window_blocks_kernel<T, 16, 8><<<gb, 128, 0, ctx->stream>>>(V, O, b, p, lam, A.n, A.m, r, h)));
-  WS_SHAPED(ctx, A.n, A.m, (window_sums_kernel<T, true, 2, 1><<<g, kThreads, 0, ctx->stream>>>(A)),
-            (window_sums_kernel<T, true, 6, 2><<<g, kThreads, 0, ctx->stream>>>(A)),
-            (window_sums_kernel<T, true, 16, 8><<<g, kThreads, 0, ctx->stream>>>(A)));
+  WS_SHAPED(ctx, A.n, A.m, (chain_launch(ctx->stream, gb, 128, 0, (window_blocks_kernel<T, 2, 1>), V, O, b, p, lam,
+                                         A.n, A.m, r, h)),
+            (chain_launch(ctx->stream, gb, 128, 0, (window_blocks_kernel<T, 6, 2>), V, O, b, p, lam, A.n, A.m, r, h)),
+            (chain_launch(ctx->stream, gb, 128, 0, (window_blocks_kernel<T, 16, 8>), V, O, b, p, lam, A.n, A.m, r,
+                          h)));
+  WS_SHAPED(ctx, A.n, A.m, (chain_launch(ctx->stream, g, kThreads, 0, (window_sums_kernel<T, true, 2, 1>), A)),
+            (chain_launch(ctx->stream, g, kThreads, 0, (window_sums_kernel<T, true, 6, 2>), A)),
+            (chain_launch(ctx->stream, g, kThreads, 0, (window_sums_kernel<T, true, 16, 8>), A)));
   return QRKIT_OK;
 }
 template qrkit_status window_refine_gradient<float>(qrkit_ctx*, const ComposedView<float>&, const FactorOut<float>&,
