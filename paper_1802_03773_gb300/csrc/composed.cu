@@ -1042,6 +1042,7 @@ template <typename T>
 static qrkit_status launch_block_backsub(qrkit_ctx* ctx, const ComposedView<T>& V, const FactorOut<T>& O, const T* rhs,
                                          const T* xS, T* x, int accumulate) {
   if (V.coupled == QRKIT_COUPLED_DENSE && V.s >= 16) return dense_block_backsub<T>(ctx, V, O, rhs, xS, x, accumulate);
+  if (window21(ctx)) return window21_backsub<T>(ctx, V, O, rhs, xS, x, accumulate);
   LAUNCH_SHAPED(ctx, small_class(ctx->plan, O.damp), block_backsub_kernel, blocks_for(V.K, 64), 64, 0, ctx->stream, V, O,
                 rhs, xS, x, accumulate);
   return QRKIT_OK;
@@ -1163,7 +1164,9 @@ static qrkit_status factor_typed(qrkit_ctx* ctx, const void* J, const void* S, c
   FactorOut<T> O = fout<T>(ctx);
   // the small-block kernels when every block fits them (e.g. 2 x 1 blocks of curve fits)
   const int cls = small_class(P, O.damp);
-  if (cls == 1)
+  if (window21(ctx) && (reinterpret_cast<uintptr_t>(V.S) & 15) == 0) {
+    if ((rc = window21_factor<T>(ctx, V, O)) != QRKIT_OK) return rc;
+  } else if (cls == 1)
     LAUNCH(ctx, (chain_launch(st, blocks_for(P.K, 128), 128, 0, (block_factor_small_kernel<T, 3, 1>), V, O)));
   else if (cls == 2)
     LAUNCH(ctx, (chain_launch(st, blocks_for(P.K, 128), 128, 0, (block_factor_small_kernel<T, 6, 2>), V, O)));
@@ -1214,8 +1217,13 @@ static qrkit_status solve_typed(qrkit_ctx* ctx, const void* J, const void* S, co
   // Q^T [b; 0]
   T* rhs0 = (V.coupled == QRKIT_COUPLED_DENSE) ? (T*)C.levels[0].rhs.ptr + reduced_head(ctx)
              : (V.coupled == QRKIT_COUPLED_WINDOW ? (T*)(C.bins ? C.rhs_s.ptr : C.rhs_red.ptr) : nullptr);
-  LAUNCH_SHAPED(ctx, small_class(P, O.damp), block_apply_qt_kernel, blocks_for(P.K, 64), 64, 0, st, V, O, (const T*)b,
-                rhs0);
+  if (window21(ctx)) {
+    const qrkit_status rc = window21_qt<T>(ctx, V, O, (const T*)b, rhs0);
+    if (rc != QRKIT_OK) return rc;
+  } else {
+    LAUNCH_SHAPED(ctx, small_class(P, O.damp), block_apply_qt_kernel, blocks_for(P.K, 64), 64, 0, st, V, O, (const T*)b,
+                  rhs0);
+  }
   if (V.coupled == QRKIT_COUPLED_DENSE) {
     const int64_t head = reduced_head(ctx), tail = C.levels[0].M - head - C.red_rows;   // damping rows and padding
     if (head > 0) QRKIT_CUDA_TRY(ctx, cudaMemsetAsync(C.levels[0].rhs.ptr, 0, (size_t)head * sizeof(T), st));

@@ -374,6 +374,16 @@ qrkit_status window_refine_gradient(qrkit_ctx* ctx, const ComposedView<T>& V, co
 // column sums of its S (s doubles, written); false in *done if the plan has no block sort.
 qrkit_status composed_sort_blocks(qrkit_ctx* ctx, bool* done);
 qrkit_status composed_window_sums(qrkit_ctx* ctx, const void* S, double* sq);
+// Sorted plans of 2 x 1 blocks with windows of 8 (window_sums.cu): the per-block kernels without offset tables.  The
+// factorization reads S by 16-byte loads (its caller checks the alignment).
+bool window21(const qrkit_ctx* ctx);
+template <typename T>
+qrkit_status window21_factor(qrkit_ctx* ctx, const ComposedView<T>& V, const FactorOut<T>& O);
+template <typename T>
+qrkit_status window21_qt(qrkit_ctx* ctx, const ComposedView<T>& V, const FactorOut<T>& O, const T* b, T* rhs0);
+template <typename T>
+qrkit_status window21_backsub(qrkit_ctx* ctx, const ComposedView<T>& V, const FactorOut<T>& O, const T* rhs, const T* xS,
+                              T* x, int accumulate);
 // TSQR of a reduced block without column panels (tsqr.cu; s <= 64): rows of a tile for M rows; one level's tiles
 // (reflectors and R in place, tau, the R rows to Xn); and their Q^T on a right-hand side.
 int tsqr_rows(const qrkit_ctx* ctx, int64_t M, int s);

@@ -199,6 +199,120 @@ __global__ void __launch_bounds__(128) window_blocks_kernel(ComposedView<T> V, F
   }
 }
 
+// ---- 2 x 1 blocks with windows of 8, one thread each: factorization, Q^T b and back-substitution ----
+//
+// The general small-block kernels read six tables of offsets per block and touch a window entry by entry (a warp's
+// load spreads over 32 windows).  A plan of one shape needs no offsets, and rows of a window are whole 16-byte pieces:
+// 10.5 million blocks: factorization 634 -> 356 us, Q^T b 135 -> 105 us, back-substitution 140 -> 107 us.
+// The arithmetic is that of the general kernels.
+template <typename T, int N>
+__device__ __forceinline__ void load_wide(T (&v)[N], const T* src) {   // src 16-byte aligned
+  constexpr int E = 16 / (int)sizeof(T);
+  union Piece {
+    uint4 q;
+    T t[E];
+  };
+#pragma unroll
+  for (int k = 0; k < N / E; ++k) {
+    Piece p;
+    p.q = reinterpret_cast<const uint4*>(src)[k];
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[k * E + e] = p.t[e];
+  }
+}
+template <typename T, int N>
+__device__ __forceinline__ void store_wide(T* dst, const T (&v)[N]) {   // dst 16-byte aligned
+  constexpr int E = 16 / (int)sizeof(T);
+  union Piece {
+    uint4 q;
+    T t[E];
+  };
+#pragma unroll
+  for (int k = 0; k < N / E; ++k) {
+    Piece p;
+#pragma unroll
+    for (int e = 0; e < E; ++e) p.t[e] = v[k * E + e];
+    reinterpret_cast<uint4*>(dst)[k] = p.q;
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) window21_factor_kernel(ComposedView<T> V, FactorOut<T> O) {
+  dev::chain_wait();
+  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (i >= V.K) return;
+  const int64_t at = (int64_t)O.bpos[i] * O.q;   // the block's first reduced row
+  T S[16];
+  load_wide(S, V.S + 16 * i);
+  const T alpha = V.J[2 * i];
+  T b1 = V.J[2 * i + 1], b2 = O.damp ? (T)(O.lam_half * O.D[i]) : T(0);
+  T sq = b1 * b1;
+  if (O.damp) sq += b2 * b2;
+  const T norm = sqrt(alpha * alpha + sq);
+  T beta = 0, tau = 0, scale = 0;
+  if (norm != T(0)) {
+    beta = alpha >= T(0) ? -norm : norm;
+    tau = (beta - alpha) / beta;
+    scale = T(1) / (alpha - beta);
+  } else if (O.status) {
+    atomicCAS(O.status, 0, QRKIT_ESINGULAR);
+  }
+  b1 *= scale;
+  b2 *= scale;
+  const int na = O.damp ? 3 : 2;
+  T* F = O.Fa + na * i;
+  F[0] = beta;
+  F[1] = b1;
+  if (O.damp) F[2] = b2;
+  O.tau[i] = tau;
+  T r12[8], x0[8], x1[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const T w = (S[2 * c] + b1 * S[2 * c + 1]) * tau;
+    r12[c] = S[2 * c] - w;
+    x0[c] = S[2 * c + 1] - w * b1;
+    x1[c] = T(0) - w * b2;
+  }
+  store_wide(O.R12 + 8 * i, r12);
+  store_wide(O.Xw + 8 * at, x0);
+  if (O.damp) store_wide(O.Xw + 8 * (at + 1), x1);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) window21_qt_kernel(ComposedView<T> V, FactorOut<T> O, const T* b, T* rhs0) {
+  dev::chain_wait();
+  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (i >= V.K) return;
+  const int64_t at = (int64_t)O.bpos[i] * O.q;
+  const T y0 = b[2 * i], y1 = b[2 * i + 1];
+  const T* F = O.Fa + (O.damp ? 3 : 2) * i;
+  const T b1 = F[1], b2 = O.damp ? F[2] : T(0);
+  const T w = (y0 + b1 * y1) * O.tau[i];
+  O.ctop[i] = y0 - w;
+  if (!rhs0) return;
+  rhs0[at] = y1 - w * b1;
+  if (O.damp) rhs0[at + 1] = T(0) - w * b2;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) window21_backsub_kernel(ComposedView<T> V, FactorOut<T> O, const T* rhs,
+                                                               const T* xS, T* x, int accumulate) {
+  dev::chain_wait();
+  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (i >= V.K) return;
+  T y = rhs[i];
+  if (xS) {
+    const int64_t st = V.start[i];
+    T r12[8];
+    load_wide(r12, O.R12 + 8 * i);
+#pragma unroll
+    for (int t = 0; t < 8; ++t)
+      if (st + t < V.s) y -= r12[t] * xS[st + t];
+  }
+  y = y / O.Fa[(O.damp ? 3 : 2) * i];
+  x[i] = accumulate ? x[i] + y : y;
+}
+
 inline unsigned nblk(int64_t n, int64_t t) { return (unsigned)((n + t - 1) / t); }
 
 }  // namespace
@@ -244,5 +358,39 @@ template qrkit_status window_refine_gradient<float>(qrkit_ctx*, const ComposedVi
                                                     const float*, const float*, double, const WindowSums<float>&);
 template qrkit_status window_refine_gradient<double>(qrkit_ctx*, const ComposedView<double>&, const FactorOut<double>&,
                                                      const double*, const double*, double, const WindowSums<double>&);
+
+bool window21(const qrkit_ctx* ctx) {
+  const Plan& P = ctx->plan;
+  return ctx->comp.bins && P.max_n == 2 && P.max_m == 1 && ctx->plan.s.window == 8;
+}
+
+template <typename T>
+qrkit_status window21_factor(qrkit_ctx* ctx, const ComposedView<T>& V, const FactorOut<T>& O) {
+  QRKIT_CUDA_TRY(ctx, chain_launch(ctx->stream, nblk(V.K, 256), 256, 0, window21_factor_kernel<T>, V, O));
+  ctx->launches += 1;
+  return QRKIT_OK;
+}
+template <typename T>
+qrkit_status window21_qt(qrkit_ctx* ctx, const ComposedView<T>& V, const FactorOut<T>& O, const T* b, T* rhs0) {
+  QRKIT_CUDA_TRY(ctx, chain_launch(ctx->stream, nblk(V.K, 256), 256, 0, window21_qt_kernel<T>, V, O, b, rhs0));
+  ctx->launches += 1;
+  return QRKIT_OK;
+}
+template <typename T>
+qrkit_status window21_backsub(qrkit_ctx* ctx, const ComposedView<T>& V, const FactorOut<T>& O, const T* rhs, const T* xS,
+                              T* x, int accumulate) {
+  QRKIT_CUDA_TRY(ctx, chain_launch(ctx->stream, nblk(V.K, 256), 256, 0, window21_backsub_kernel<T>, V, O, rhs, xS, x,
+                                   accumulate));
+  ctx->launches += 1;
+  return QRKIT_OK;
+}
+#define WINDOW21_TYPES(T)                                                                                          \
+  template qrkit_status window21_factor<T>(qrkit_ctx*, const ComposedView<T>&, const FactorOut<T>&);              \
+  template qrkit_status window21_qt<T>(qrkit_ctx*, const ComposedView<T>&, const FactorOut<T>&, const T*, T*);    \
+  template qrkit_status window21_backsub<T>(qrkit_ctx*, const ComposedView<T>&, const FactorOut<T>&, const T*,    \
+                                            const T*, T*, int);
+WINDOW21_TYPES(float)
+WINDOW21_TYPES(double)
+#undef WINDOW21_TYPES
 
 }  // namespace qrkit
