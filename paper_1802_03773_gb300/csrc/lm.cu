@@ -105,25 +105,21 @@ __global__ void cf_coef_kernel(LMTables t, const double* x, const T* p, double* 
   c[5] = 3.0 * a3;
 }
 
-// The basis functions at u: 6 B_0 = (1-u)^3, 6 B_3 = u^3, B_1 = (u/2 - 1) u^2 + 2/3, and B_2 the rest of
-// their sum 1.
+// The basis functions at u, v = 1 - u: B_0 = v^3 / 6, B_1 = (u/2 - 1) u^2 + 2/3, and the same mirrored.
 __device__ __forceinline__ void bspline_values(double u, double B[4]) {
   const double sixth = 1.0 / 6.0;
-  const double v = 1.0 - u, u2 = u * u;
-  B[0] = v * v * v * sixth;
+  const double v = 1.0 - u, u2 = u * u, v2 = v * v;
+  B[0] = v2 * v * sixth;
   B[1] = fma(fma(0.5, u, -1.0), u2, 4.0 * sixth);
+  B[2] = fma(fma(0.5, v, -1.0), v2, 4.0 * sixth);
   B[3] = u2 * u * sixth;
-  B[2] = (1.0 - B[1]) - (B[0] + B[3]);
 }
 
 // Segment of parameter t and u = t - segment.
 __device__ __forceinline__ int segment_of(double t, int64_t Kc, double& u) {
-  const double hi = (double)(int)(Kc - 4);
-  double f = floor(t);
-  if (!(f >= 0.0)) f = 0.0;   // also NaN
-  if (f > hi) f = hi;
-  u = t - f;
-  return (int)f;
+  const int f = max(0, min(__double2int_rd(t), (int)(Kc - 4)));   // saturates; NaN becomes a negative number or 0
+  u = t - (double)f;
+  return f;
 }
 
 // Sum over the CTA of kTilePts threads, in thread 0: through shared memory, so that the FP64 additions are those of
