@@ -460,14 +460,14 @@ def other_workloads(dev, stream, only=None):
         flops = 2.0 * Mred * s * s   # useful flops of the reduced block's Householder QR (leading term)
         out["dense_hcat_100k_blocks_s128_fp32_refined"] = {
             "workload": "J = [blkdiag(100,000 blocks 4x2) | S 400,000 x 128], lambda 1e-2, D = norms; "
-                        "reduced block by 4 column panels of 32 (TSQR each, tcgen05 3xTF32 updates)",
+                        "reduced block by 4 column panels of 32 (TSQR each, 3xTF32 tensor-core updates)",
             "ms_factor": tf, "ms_solve_refined_1": ts, "value": 1000.0 / (tf + ts), "unit": "solves/s",
             "reduced_block_tflops_useful": flops / (tf * 1e-3) / 1e12}
         ctx.close()
         del J, S, b
     if want("dense_wide") or only == "dense_wide_small":
         # wider reduced blocks: s = 256 and 512 by 32-column panels, each a TSQR
-        # whose tiles' Q^T reaches the later columns through the tensor cores (tcgen05, 3xTF32).
+        # whose tiles' Q^T reaches the later columns through the tensor cores (3xTF32).
         # "dense_wide_small" (20,000 blocks, s = 512, asked for by name only) is the profiling case.
         small = only == "dense_wide_small"
         for s in ((512,) if small else (256, 512)):
@@ -493,7 +493,7 @@ def other_workloads(dev, stream, only=None):
             flops = 2.0 * Mred * s * s - 2.0 * s ** 3 / 3.0   # Householder QR of the Mred x s reduced block
             out[f"dense_wide_{K // 1000}k_blocks_s{s}_fp32_refined"] = {
                 "workload": f"J = [blkdiag({K:,} blocks 4x2) | S {K * n:,} x {s}], lambda 1e-2, D = norms; reduced "
-                            f"block by {s // 32} column panels of 32 (TSQR each, tcgen05 3xTF32 updates)",
+                            f"block by {s // 32} column panels of 32 (TSQR each, 3xTF32 tensor-core updates)",
                 "ms_factor": tf, "ms_solve_refined_1": ts, "value": 1000.0 / (tf + ts), "unit": "solves/s",
                 "reduced_block_tflops_useful": flops / (tf * 1e-3) / 1e12, "launches_per_factor": launches}
             ctx.close()

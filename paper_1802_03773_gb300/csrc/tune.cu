@@ -5,8 +5,8 @@
 // CTA) or tiles of consecutive blocks (blocks / values / rows / columns / padded working area
 // per tile, which set the tile count, the work per barrier phase and the shared memory per
 // CTA).  Banded plans: the
-// compression strategy of the parallel banded QR (one thread per column block, or warps with
-// a number of splits).  Every candidate is timed with CUDA events on the context's stream on
+// compression strategy of the parallel banded QR (one thread per column block, or a
+// number of threads per block whose triangles are merged).  Every candidate is timed with CUDA events on the context's stream on
 // the caller's inputs (one warm-up, three timed runs), the fastest is kept.  The cache holds
 // one line per structure key: "<key>\t<choice>"; a key already present is applied without
 // timing.
