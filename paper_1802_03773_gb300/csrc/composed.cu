@@ -1721,7 +1721,6 @@ static qrkit_status solve_r_typed(qrkit_ctx* ctx, const void* qtb, void* p) {
   if (P.s.coupled_kind == QRKIT_COUPLED_WINDOW)
     return fail(ctx, QRKIT_EUNSUPPORTED, "R of a windowed structure is formed in qrkit_solve");
   Composed& C = ctx->comp;
-  cudaStream_t st = ctx->stream;
   ComposedView<T> V = view<T>(ctx, nullptr, nullptr);
   FactorOut<T> O = fout<T>(ctx);
   const int s = V.s;

@@ -234,16 +234,6 @@ struct Window {
 };
 
 template <typename T>
-__device__ __forceinline__ void store8(T* dst, const T (&v)[8]) {   // dst 16-byte aligned
-  if constexpr (sizeof(T) == 4) {
-    reinterpret_cast<float4*>(dst)[0] = make_float4(v[0], v[1], v[2], v[3]);
-    reinterpret_cast<float4*>(dst)[1] = make_float4(v[4], v[5], v[6], v[7]);
-  } else {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) reinterpret_cast<double2*>(dst)[q] = make_double2(v[2 * q], v[2 * q + 1]);
-  }
-}
-template <typename T>
 __device__ __forceinline__ void load8(T (&v)[8], const T* src) {   // src 16-byte aligned
   if constexpr (sizeof(T) == 4) {
     const float4 a = reinterpret_cast<const float4*>(src)[0], b = reinterpret_cast<const float4*>(src)[1];
