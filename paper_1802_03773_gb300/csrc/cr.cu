@@ -559,8 +559,8 @@ __device__ __forceinline__ void decode(int64_t it, int64_t& k, int64_t& i, int& 
 //   3. those rows triangular in the left columns, and the right-only rows of step 1 into rows 8..15 of B:
 //      the new 16-row block row on (left, right).
 // Rows are taken two at a time (f32x2): 13 million columns of 256 instances spend 1,505 us on the fronts against 1,641
-// with scalar rows.  A 32-row front on a whole warp with
-// its sums reduced by shuffles took six times the instructions.
+// with scalar rows.  A 32-row front on a whole warp with its sums reduced by shuffles took six times the
+// instructions.
 constexpr int kItemThreads = kCB;
 
 // Eight rows of a column on a lane: two rows per operation for float.  The ranges [r0, r1) are known at compile time

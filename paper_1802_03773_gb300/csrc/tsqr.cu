@@ -80,9 +80,9 @@ __device__ __forceinline__ void reflector(float alpha, float sq, float& beta, fl
   scale = 1.f / (alpha - beta);
 }
 
-// One tile of at most 32 RPL rows (`rows` of the level each) and s <= 8 CPW columns: row lane + 32 u on the lane, column j on warp j % 8.  At step k the
-// reflector v_k is read from shared memory (two alternating slots) by every warp and applied to its
-// columns after k; the warp of column k + 1 forms the next reflector right after updating it.  V below / R
+// One tile of at most 32 RPL rows (`rows` of the level each) and s <= 8 CPW columns: row lane + 32 u on the lane,
+// column j on warp j % 8.  At step k the reflector v_k is read from shared memory (two alternating slots) by every
+// warp and applied to its columns after k; the warp of column k + 1 forms the next reflector right after updating it.  V below / R
 // on and above the diagonal in place, tau to taus[tile s + k], the R rows (zeros below) to the next level.
 template <typename T, int RPL, int CPW>
 __global__ void __launch_bounds__(kThreads) tsqr_tile_kernel(T* X, int64_t ld, int64_t M, int s, int rows, T* taus,
