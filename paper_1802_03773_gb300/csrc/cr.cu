@@ -1039,15 +1039,26 @@ inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 // ---------------------------------------------------------------------------------------
 // Host side: instance tables, level work lists, launches.
 
+// The compression's threads and the merges of their triangles.  Never changed once built, and kept as long as the
+// plan: a solve that is queued, or captured in a graph, holds the device addresses.
+struct CRSplits {
+  int each = 0;                            // threads of every block, or 0: per instance by its rows
+  int64_t num_items = 0;                   // threads of the compression
+  std::vector<int64_t> mg_off, mg_n;       // merge items per pass
+  DevBuf item_blk, blk_item0, merges;
+};
+
 struct CRPlan {
   int64_t num_inst = 0, total_blocks = 0;
   int levels = 0;                          // those run by launches of their own, before the tails
-  int64_t num_items = 0;                   // threads of the compression
+  int64_t total_rows = 0;
   std::vector<int64_t> h_blk0, h_rows;     // kept for the compression's strategy
-  std::vector<int64_t> mg_off, mg_n;       // merge items per pass
+  std::vector<CRSplits*> splits;           // the strategies asked for so far
+  const CRSplits* cur = nullptr;
+  std::vector<DevBuf> outgrown;            // partial triangles that a queued or captured solve may still use
   std::vector<int64_t> lvl_off, lvl_n;     // eliminate / move items per level
   std::vector<int64_t> ev_off, ev_n;       // staying (even) blocks per level
-  DevBuf tabs, items, evens, binst, item_blk, blk_item0, merges, grp_lo, P, P2, E0, F0, F1, Rb, xp, hp;
+  DevBuf tabs, items, evens, binst, grp_lo, P, P2, E0, F0, F1, Rb, xp, hp;
   const int64_t* d_cols = nullptr;
   const int64_t* d_col0 = nullptr;
   const int64_t* d_row0 = nullptr;
@@ -1056,9 +1067,16 @@ struct CRPlan {
   const int64_t* d_tail0 = nullptr;
 };
 
+static void release_splits(CRSplits* s) {
+  for (DevBuf* b : {&s->item_blk, &s->blk_item0, &s->merges}) release(*b);
+  delete s;
+}
+
 void release_cr(CRPlan*& p) {
   if (!p) return;
-  for (DevBuf* b : {&p->tabs, &p->items, &p->evens, &p->binst, &p->item_blk, &p->blk_item0, &p->merges, &p->grp_lo, &p->P, &p->P2, &p->E0, &p->F0, &p->F1, &p->Rb,
+  for (CRSplits* s : p->splits) release_splits(s);
+  for (DevBuf& b : p->outgrown) release(b);
+  for (DevBuf* b : {&p->tabs, &p->items, &p->evens, &p->binst, &p->grp_lo, &p->P, &p->P2, &p->E0, &p->F0, &p->F1, &p->Rb,
                     &p->xp, &p->hp})
     release(*b);
   delete p;
@@ -1072,15 +1090,25 @@ static qrkit_status upload(qrkit_ctx* ctx, DevBuf& d, const void* h, size_t byte
   return QRKIT_OK;
 }
 
-// The compression's threads: splits[k] per block of instance k, and the merges of their triangles.
-static qrkit_status cr_split(qrkit_ctx* ctx, CRPlan& C, const std::vector<int>& splits) {
-  C.num_items = 0;
-  C.mg_off.clear();
-  C.mg_n.clear();
-  for (int64_t k = 0; k < C.num_inst; ++k) C.num_items += (C.h_blk0[k + 1] - C.h_blk0[k]) * splits[k];
-  if (C.num_items >= ((int64_t)1 << 31)) return fail(ctx, QRKIT_EUNSUPPORTED, "too many column blocks");
-  if (C.num_items == C.total_blocks) return QRKIT_OK;   // one thread per block
-  std::vector<int32_t> item_blk((size_t)C.num_items), item0((size_t)C.total_blocks + 1);
+// A buffer of partial triangles of at least `parts`; an outgrown one is kept until the plan goes.  Strategies grow
+// it, so the kept ones are smaller than the current one.
+static qrkit_status cr_partials(qrkit_ctx* ctx, CRPlan& C, DevBuf& buf, int64_t parts) {
+  const size_t bytes = ((size_t)parts + 31) / 32 * 32 * kE0 * elem_size(ctx);
+  if (parts == 0 || buf.bytes >= bytes) return QRKIT_OK;
+  DevBuf grown;
+  const qrkit_status rc = ensure(ctx, grown, bytes, "banded partial triangles");
+  if (rc != QRKIT_OK) return rc;
+  if (buf.ptr) C.outgrown.push_back(buf);
+  buf = grown;
+  return QRKIT_OK;
+}
+
+// The tables of a strategy: splits[k] threads per block of instance k.
+static qrkit_status cr_split(qrkit_ctx* ctx, CRPlan& C, const std::vector<int>& splits, CRSplits& S) {
+  for (int64_t k = 0; k < C.num_inst; ++k) S.num_items += (C.h_blk0[k + 1] - C.h_blk0[k]) * splits[k];
+  if (S.num_items >= ((int64_t)1 << 31)) return fail(ctx, QRKIT_EUNSUPPORTED, "too many column blocks");
+  if (S.num_items == C.total_blocks) return QRKIT_OK;   // one thread per block
+  std::vector<int32_t> item_blk((size_t)S.num_items), item0((size_t)C.total_blocks + 1);
   std::vector<int32_t> first((size_t)C.total_blocks), n((size_t)C.total_blocks);   // a block's partials at this pass
   int64_t it = 0;
   for (int64_t k = 0; k < C.num_inst; ++k)
@@ -1094,7 +1122,7 @@ static qrkit_status cr_split(qrkit_ctx* ctx, CRPlan& C, const std::vector<int>& 
   int64_t parts2 = 0;
   for (bool more = true; more;) {
     more = false;
-    C.mg_off.push_back((int64_t)mg.size());
+    S.mg_off.push_back((int64_t)mg.size());
     int64_t out = 0;
     for (int64_t gb = 0; gb < C.total_blocks; ++gb) {
       if (n[gb] <= 1) continue;
@@ -1110,18 +1138,45 @@ static qrkit_status cr_split(qrkit_ctx* ctx, CRPlan& C, const std::vector<int>& 
       }
     }
     parts2 = std::max(parts2, out);
-    C.mg_n.push_back((int64_t)mg.size() - C.mg_off.back());
+    S.mg_n.push_back((int64_t)mg.size() - S.mg_off.back());
   }
-  const size_t es = elem_size(ctx);
   qrkit_status rc;
-  if ((rc = upload(ctx, C.item_blk, item_blk.data(), item_blk.size() * 4, "banded splits")) != QRKIT_OK) return rc;
-  if ((rc = upload(ctx, C.blk_item0, item0.data(), item0.size() * 4, "banded splits")) != QRKIT_OK) return rc;
-  if ((rc = upload(ctx, C.merges, mg.data(), mg.size() * sizeof(MergeItem), "banded merges")) != QRKIT_OK) return rc;
-  if ((rc = ensure(ctx, C.P, ((size_t)C.num_items + 31) / 32 * 32 * kE0 * es, "banded partial triangles")) != QRKIT_OK)
+  if ((rc = upload(ctx, S.item_blk, item_blk.data(), item_blk.size() * 4, "banded splits")) != QRKIT_OK) return rc;
+  if ((rc = upload(ctx, S.blk_item0, item0.data(), item0.size() * 4, "banded splits")) != QRKIT_OK) return rc;
+  if ((rc = upload(ctx, S.merges, mg.data(), mg.size() * sizeof(MergeItem), "banded merges")) != QRKIT_OK) return rc;
+  if ((rc = cr_partials(ctx, C, C.P, S.num_items)) != QRKIT_OK) return rc;
+  return cr_partials(ctx, C, C.P2, parts2);
+}
+
+// The current strategy becomes `each` threads per block, or (0) as many as each instance's rows call for; on
+// failure it stays what it was.
+static qrkit_status cr_use_splits(qrkit_ctx* ctx, CRPlan& C, int each) {
+  for (const CRSplits* s : C.splits)
+    if (s->each == each) {
+      C.cur = s;
+      return QRKIT_OK;
+    }
+  std::vector<int> n((size_t)C.num_inst, each);
+  if (each == 0) {
+    // About 120,000 threads in all where that leaves each at least 64 rows (16 steps of four, what a merge pass
+    // takes), at most 64 per block.  A batch's instances differ in rows per block (curve fits: 60 to 10,000), and
+    // the longest thread bounds the kernel.
+    const double target = std::max(64.0, (double)C.total_rows / 120000.0);
+    for (int64_t k = 0; k < C.num_inst; ++k) {
+      const double per = (double)C.h_rows[k] / (double)(C.h_blk0[k + 1] - C.h_blk0[k]);
+      n[k] = (int)std::min(64.0, std::max(1.0, std::floor(per / target + 0.5)));
+    }
+  }
+  CRSplits* s = new CRSplits();
+  s->each = each;
+  const qrkit_status rc = cr_split(ctx, C, n, *s);
+  if (rc != QRKIT_OK) {
+    release_splits(s);
     return rc;
-  if (parts2 > 0)
-    rc = ensure(ctx, C.P2, ((size_t)parts2 + 31) / 32 * 32 * kE0 * es, "banded partial triangles");
-  return rc;
+  }
+  C.splits.push_back(s);
+  C.cur = s;
+  return QRKIT_OK;
 }
 
 qrkit_status cr_build(qrkit_ctx* ctx, CRPlan*& out, const std::vector<int64_t>& cols,
@@ -1133,11 +1188,10 @@ qrkit_status cr_build(qrkit_ctx* ctx, CRPlan*& out, const std::vector<int64_t>& 
   const int64_t ni = (int64_t)cols.size();
   C.num_inst = ni;
   std::vector<int64_t> blk0(ni + 1, 0);
-  int64_t total_rows = 0;
   for (int64_t k = 0; k < ni; ++k) {
     if (cols[k] < 1) return fail(ctx, QRKIT_EINVAL, "banded instance without columns");
     blk0[k + 1] = blk0[k] + (cols[k] + kCB - 1) / kCB;
-    total_rows += rows[k];
+    C.total_rows += rows[k];
   }
   C.total_blocks = blk0[ni];
   if (C.total_blocks >= ((int64_t)1 << 30)) return fail(ctx, QRKIT_EUNSUPPORTED, "too many column blocks");
@@ -1192,18 +1246,7 @@ qrkit_status cr_build(qrkit_ctx* ctx, CRPlan*& out, const std::vector<int64_t>& 
   const size_t es = elem_size(ctx);
   const size_t TB = (size_t)C.total_blocks;
   if ((rc = ensure(ctx, C.grp_lo, TB * sizeof(int64_t), "banded group rows")) != QRKIT_OK) return rc;
-  // Threads per block of an instance: about 120,000 in all where that leaves each at least 64 rows (16 steps of
-  // four, what a merge pass takes), at most 64 per block.  A batch's instances differ in rows per block
-  // (curve fits: 60 to 10,000), and the longest thread bounds the kernel.
-  {
-    const double target = std::max(64.0, (double)total_rows / 120000.0);
-    std::vector<int> splits(ni);
-    for (int64_t k = 0; k < ni; ++k) {
-      const double per = (double)rows[k] / (double)(blk0[k + 1] - blk0[k]);
-      splits[k] = (int)std::min(64.0, std::max(1.0, std::floor(per / target + 0.5)));
-    }
-    if ((rc = cr_split(ctx, C, splits)) != QRKIT_OK) return rc;
-  }
+  if ((rc = cr_use_splits(ctx, C, 0)) != QRKIT_OK) return rc;
   if ((rc = ensure(ctx, C.E0, (TB + 31) / 32 * 32 * kE0 * es, "banded block rows")) != QRKIT_OK) return rc;
   if ((rc = ensure(ctx, C.F0, TB * kFW * es, "banded block rows")) != QRKIT_OK) return rc;
   if ((rc = ensure(ctx, C.F1, TB * kFW * es, "banded block rows")) != QRKIT_OK) return rc;
@@ -1215,7 +1258,7 @@ qrkit_status cr_build(qrkit_ctx* ctx, CRPlan*& out, const std::vector<int64_t>& 
 
 qrkit_status cr_set_strategy(qrkit_ctx* ctx, CRPlan& C, bool thread_rows, int splits) {
   if (splits < 1 || splits > 64) return fail(ctx, QRKIT_EINVAL, "splits must be in [1, 64]");
-  return cr_split(ctx, C, std::vector<int>((size_t)C.num_inst, thread_rows ? 1 : splits));
+  return cr_use_splits(ctx, C, thread_rows ? 1 : splits);
 }
 
 template <typename T>
@@ -1230,10 +1273,9 @@ static CRArgs<T> cr_args(qrkit_ctx* ctx, CRPlan& C) {
   A.tail0 = C.d_tail0;
   A.binst = (const int32_t*)C.binst.ptr;
   A.total_blocks = C.total_blocks;
-  A.num_items = C.num_items;
-  const bool split = C.num_items != C.total_blocks;
-  A.item_blk = split ? (const int32_t*)C.item_blk.ptr : nullptr;
-  A.blk_item0 = split ? (const int32_t*)C.blk_item0.ptr : nullptr;
+  A.num_items = C.cur->num_items;
+  A.item_blk = (const int32_t*)C.cur->item_blk.ptr;   // both null for one thread per block
+  A.blk_item0 = (const int32_t*)C.cur->blk_item0.ptr;
   A.grp_lo = (int64_t*)C.grp_lo.ptr;
   A.P = (T*)C.P.ptr;
   A.E0 = (T*)C.E0.ptr;
@@ -1269,7 +1311,8 @@ static qrkit_status cr_solve_typed(qrkit_ctx* ctx, CRPlan& C, const int64_t* sta
   A.res2 = res2;
   QRKIT_CUDA_TRY(ctx, cudaMemsetAsync(res2, 0, (size_t)C.num_inst * sizeof(double), st));
   if (starts) CR_LAUNCH(ctx, nblk(C.total_blocks, 256), 256, 0, cr_ranges_kernel<T>, A);
-  const unsigned cgrid = nblk(C.num_items, kCompThreads);
+  const CRSplits& S = *C.cur;
+  const unsigned cgrid = nblk(S.num_items, kCompThreads);
   if (w == kCB && (reinterpret_cast<uintptr_t>(J) & 15) == 0) {
     const size_t smem = 2 * (size_t)kCompThreads * stage_stride<T>();
     auto kc = cr_compress_kernel<T, true>;
@@ -1281,9 +1324,9 @@ static qrkit_status cr_solve_typed(qrkit_ctx* ctx, CRPlan& C, const int64_t* sta
   }
   T* in = A.P;
   T* other = (T*)C.P2.ptr;
-  for (size_t q = 0; q < C.mg_n.size(); ++q) {
-    CR_LAUNCH(ctx, nblk(C.mg_n[q], kCompThreads), kCompThreads, 0, cr_merge_kernel<T>, A,
-              (const MergeItem*)C.merges.ptr + C.mg_off[q], C.mg_n[q], in, other);
+  for (size_t q = 0; q < S.mg_n.size(); ++q) {
+    CR_LAUNCH(ctx, nblk(S.mg_n[q], kCompThreads), kCompThreads, 0, cr_merge_kernel<T>, A,
+              (const MergeItem*)S.merges.ptr + S.mg_off[q], S.mg_n[q], in, other);
     std::swap(in, other);
   }
   const int64_t* items = (const int64_t*)C.items.ptr;
