@@ -662,8 +662,8 @@ static BandLaunch band_launch(const BandGroups& B, size_t per_thread, size_t fix
   return L;
 }
 
-// KERNEL<w = 8 by 16-byte loads, staged, widest window>
-#define BAND_F32_LAUNCH(ctx, L, KERNEL, MW, ...)                                                                   \
+// KERNEL<w = 8 by 16-byte loads, staged, widest window>, launched by LAUNCH (start_launch or chain_launch)
+#define BAND_F32_LAUNCH(ctx, LAUNCH, L, KERNEL, MW, ...)                                                                   \
   do {                                                                                                         \
     auto launch_ = [&](auto k_) -> cudaError_t {                                                               \
       if ((L).smem > 48 * 1024) {                                                                              \
@@ -671,7 +671,7 @@ static BandLaunch band_launch(const BandGroups& B, size_t per_thread, size_t fix
                                                     (int)(L).smem);                                            \
         if (e_ != cudaSuccess) return e_;                                                                      \
       }                                                                                                        \
-      return chain_launch((ctx)->stream, (L).grid, (L).nt, (L).smem, k_, __VA_ARGS__);                             \
+      return LAUNCH((ctx)->stream, (L).grid, (L).nt, (L).smem, k_, __VA_ARGS__);                               \
     };                                                                                                         \
     QRKIT_CUDA_TRY(ctx, (L).w8 ? ((L).staged ? launch_(KERNEL<true, true, 8>) : launch_(KERNEL<true, false, 8>))  \
                                : ((L).staged ? launch_(KERNEL<false, true, MW>) : launch_(KERNEL<false, false, MW>))); \
@@ -965,8 +965,8 @@ static qrkit_status banded_run(qrkit_ctx* ctx, const void* J, const void* b, con
         const BandLaunch L = band_launch(G, (size_t)(B.w + 1) * sizeof(float), 0);
         BandGroups GL = G;
         GL.gs = L.gs;
-        if (B.w <= 8) BAND_F32_LAUNCH(ctx, L, band_norm_f32_kernel, 8, GL, D, (float2*)B.D2.ptr);
-        else BAND_F32_LAUNCH(ctx, L, band_norm_f32_kernel, kBW, GL, D, (float2*)B.D2.ptr);
+        if (B.w <= 8) BAND_F32_LAUNCH(ctx, start_launch, L, band_norm_f32_kernel, 8, GL, D, (float2*)B.D2.ptr);
+        else BAND_F32_LAUNCH(ctx, start_launch, L, band_norm_f32_kernel, kBW, GL, D, (float2*)B.D2.ptr);
       } else {
         band_colnorm_kernel<<<nblk(B.total_cols, 256), 256, 0, st>>>(nullptr, (const double*)J, dcols, dc0, dr0,
                                                                     B.num_inst, B.rows_per_col, B.w, D);
@@ -1023,7 +1023,7 @@ static qrkit_status banded_run(qrkit_ctx* ctx, const void* J, const void* b, con
         const int64_t* blk0;
         void* gp;
         cr_padded(*B.cr, &blk0, &gp);
-        BAND_F32_LAUNCH(ctx, L, band_grad_f32_kernel, 8, GL, (const float*)b, (const float*)p, (const float2*)B.D2.ptr,
+        BAND_F32_LAUNCH(ctx, chain_launch, L, band_grad_f32_kernel, 8, GL, (const float*)b, (const float*)p, (const float2*)B.D2.ptr,
                         (float)lambda, (float)(lambda - (double)(float)lambda), blk0, (float*)gp);
       } else {
         band_resid_kernel<T><<<nblk(B.total_rows, 256), 256, 0, st>>>(

@@ -1029,22 +1029,24 @@ int small_class(const Plan& P, bool damp) {
   return 0;
 }
 // A per-block kernel template KERNEL<T, NA, MM> launched in the instantiation of the class.
-#define LAUNCH_SHAPED(ctx, cls, KERNEL, grid, threads, smem, stream, ...)                      \
-  do {                                                                                         \
-    if ((cls) == 1) LAUNCH(ctx, (chain_launch(stream, grid, threads, smem, (KERNEL<T, 3, 1>), __VA_ARGS__))); \
-    else if ((cls) == 2) LAUNCH(ctx, (chain_launch(stream, grid, threads, smem, (KERNEL<T, 6, 2>), __VA_ARGS__))); \
-    else LAUNCH(ctx, (chain_launch(stream, grid, threads, smem, KERNEL<T>, __VA_ARGS__)));                \
+#define LAUNCH_SHAPED(ctx, chained, cls, KERNEL, grid, threads, smem, stream, ...)                                     \
+  do {                                                                                                                \
+    if ((cls) == 1) LAUNCH(ctx, (launch_kernel(chained, stream, grid, threads, smem, (KERNEL<T, 3, 1>), __VA_ARGS__))); \
+    else if ((cls) == 2)                                                                                              \
+      LAUNCH(ctx, (launch_kernel(chained, stream, grid, threads, smem, (KERNEL<T, 6, 2>), __VA_ARGS__)));              \
+    else LAUNCH(ctx, (launch_kernel(chained, stream, grid, threads, smem, KERNEL<T>, __VA_ARGS__)));                   \
   } while (0)
 
 // R_i x_i = rhs_i - R12_i x_S for every block.  From 16 shared columns on a warp takes a block (the
 // lanes read its rows of R12 together); below, and for windows of up to 8, a thread per block.
 template <typename T>
-static qrkit_status launch_block_backsub(qrkit_ctx* ctx, const ComposedView<T>& V, const FactorOut<T>& O, const T* rhs,
-                                         const T* xS, T* x, int accumulate) {
-  if (V.coupled == QRKIT_COUPLED_DENSE && V.s >= 16) return dense_block_backsub<T>(ctx, V, O, rhs, xS, x, accumulate);
+static qrkit_status launch_block_backsub(qrkit_ctx* ctx, bool chained, const ComposedView<T>& V, const FactorOut<T>& O,
+                                         const T* rhs, const T* xS, T* x, int accumulate) {
+  if (V.coupled == QRKIT_COUPLED_DENSE && V.s >= 16)
+    return dense_block_backsub<T>(ctx, chained, V, O, rhs, xS, x, accumulate);
   if (window21(ctx)) return window21_backsub<T>(ctx, V, O, rhs, xS, x, accumulate);
-  LAUNCH_SHAPED(ctx, small_class(ctx->plan, O.damp), block_backsub_kernel, blocks_for(V.K, 64), 64, 0, ctx->stream, V, O,
-                rhs, xS, x, accumulate);
+  LAUNCH_SHAPED(ctx, chained, small_class(ctx->plan, O.damp), block_backsub_kernel, blocks_for(V.K, 64), 64, 0,
+                ctx->stream, V, O, rhs, xS, x, accumulate);
   return QRKIT_OK;
 }
 
@@ -1204,7 +1206,7 @@ static qrkit_status factor_typed(qrkit_ctx* ctx, const void* J, const void* S, c
 }
 
 template <typename T>
-static qrkit_status solve_typed(qrkit_ctx* ctx, const void* J, const void* S, const void* b, void* p,
+static qrkit_status solve_typed(qrkit_ctx* ctx, bool chained, const void* J, const void* S, const void* b, void* p,
                                 int refine_steps, bool qt_only, void* qtb_out) {
   Plan& P = ctx->plan;
   Composed& C = ctx->comp;
@@ -1218,11 +1220,11 @@ static qrkit_status solve_typed(qrkit_ctx* ctx, const void* J, const void* S, co
   T* rhs0 = (V.coupled == QRKIT_COUPLED_DENSE) ? (T*)C.levels[0].rhs.ptr + reduced_head(ctx)
              : (V.coupled == QRKIT_COUPLED_WINDOW ? (T*)(C.bins ? C.rhs_s.ptr : C.rhs_red.ptr) : nullptr);
   if (window21(ctx)) {
-    const qrkit_status rc = window21_qt<T>(ctx, V, O, (const T*)b, rhs0);
+    const qrkit_status rc = window21_qt<T>(ctx, chained, V, O, (const T*)b, rhs0);
     if (rc != QRKIT_OK) return rc;
   } else {
-    LAUNCH_SHAPED(ctx, small_class(P, O.damp), block_apply_qt_kernel, blocks_for(P.K, 64), 64, 0, st, V, O, (const T*)b,
-                  rhs0);
+    LAUNCH_SHAPED(ctx, chained, small_class(P, O.damp), block_apply_qt_kernel, blocks_for(P.K, 64), 64, 0, st, V, O,
+                  (const T*)b, rhs0);
   }
   if (V.coupled == QRKIT_COUPLED_DENSE) {
     const int64_t head = reduced_head(ctx), tail = C.levels[0].M - head - C.red_rows;   // damping rows and padding
@@ -1271,7 +1273,7 @@ static qrkit_status solve_typed(qrkit_ctx* ctx, const void* J, const void* S, co
   const T* RS = pan ? (const T*)C.Rs.ptr : (top ? (const T*)top->X.ptr : nullptr);
   const int64_t ldRS = pan ? s : (top ? top->ld : 0);
   if (V.coupled == QRKIT_COUPLED_DENSE) {
-    qrkit_status rc = dense_backsub<T>(ctx, RS, ldRS, s, pan ? (const T*)C.cs.ptr : (const T*)top->rhs.ptr, x + nb);
+    qrkit_status rc = dense_backsub<T>(ctx, true, RS, ldRS, s, pan ? (const T*)C.cs.ptr : (const T*)top->rhs.ptr, x + nb);
     if (rc != QRKIT_OK) return rc;
   } else if (V.coupled == QRKIT_COUPLED_WINDOW) {
     // reduced banded block of every segment (Sec. 4.4), rows in P_r order, the shared
@@ -1289,7 +1291,7 @@ static qrkit_status solve_typed(qrkit_ctx* ctx, const void* J, const void* S, co
                                  C.damp ? C.lam : 0.0, C.RwS.ptr, C.cS.ptr, x + nb, (double*)C.res2.ptr);
     if (rc != QRKIT_OK) return rc;
   }
-  qrkit_status rc_b = launch_block_backsub<T>(ctx, V, O, (const T*)O.ctop, s ? x + nb : nullptr, x, 0);
+  qrkit_status rc_b = launch_block_backsub<T>(ctx, true, V, O, (const T*)O.ctop, s ? x + nb : nullptr, x, 0);
   if (rc_b != QRKIT_OK) return rc_b;
   // refinement (extended-precision residual, corrections through R only)
   for (int it = 0; it < refine_steps; ++it) {
@@ -1325,14 +1327,14 @@ static qrkit_status solve_typed(qrkit_ctx* ctx, const void* J, const void* S, co
       const size_t sum_smem = (V.coupled == QRKIT_COUPLED_DENSE && s <= kCtaSumCols) ? (size_t)s * sizeof(double)
                               : win ? (size_t)kWinSumCols * sizeof(double) : 0;
       const int win_cols = win ? kWinSumCols : 0;
-      LAUNCH_SHAPED(ctx, small_class(P, O.damp), resid_g_kernel, blocks_for(P.K, rthreads), rthreads, sum_smem, st, V,
+      LAUNCH_SHAPED(ctx, true, small_class(P, O.damp), resid_g_kernel, blocks_for(P.K, rthreads), rthreads, sum_smem, st, V,
                     (const T*)b, x, O.D, C.lam, g, gS, win_cols);
       if (s > 0)
         LAUNCH(ctx, chain_launch(st, blocks_for(s, 128), 128, 0, gS_damping_kernel, gS,
                                  sizeof(T) == 4 ? (const float*)x : nullptr,
                                  sizeof(T) == 8 ? (const double*)x : nullptr, O.D, nb, s, C.lam));
-      LAUNCH_SHAPED(ctx, small_class(P, O.damp), block_fwdsub_rt_kernel, blocks_for(P.K, rthreads), rthreads, sum_smem,
-                    st, V, O, g, h, gS, win_cols);
+      LAUNCH_SHAPED(ctx, true, small_class(P, O.damp), block_fwdsub_rt_kernel, blocks_for(P.K, rthreads), rthreads,
+                    sum_smem, st, V, O, g, h, gS, win_cols);
     }
     if (V.coupled == QRKIT_COUPLED_WINDOW && C.cr) {
       // dp_S = R_S^{-1} R_S^{-T} (g_S - R12^T h_B) with the parallel banded factor
@@ -1353,7 +1355,7 @@ static qrkit_status solve_typed(qrkit_ctx* ctx, const void* J, const void* S, co
       if ((rc = dense_normal<T>(ctx, RS, ldRS, s, gS, h + nb, x + nb)) != QRKIT_OK) return rc;
     }
     // dp_B = R_B^{-1} (h_B - R12 dp_S), accumulated into p
-    if ((rc = launch_block_backsub<T>(ctx, V, O, (const T*)h, s ? h + nb : nullptr, x, 1)) != QRKIT_OK) return rc;
+    if ((rc = launch_block_backsub<T>(ctx, true, V, O, (const T*)h, s ? h + nb : nullptr, x, 1)) != QRKIT_OK) return rc;
   }
   return QRKIT_OK;
 }
@@ -1395,16 +1397,16 @@ qrkit_status composed_window_sums(qrkit_ctx* ctx, const void* S, double* sq) {
   return window_square_sums<float>(ctx, window_sums<float>(ctx, view<float>(ctx, nullptr, S), sq));
 }
 
-qrkit_status composed_solve(qrkit_ctx* ctx, const void* J, const void* S, const void* b, void* p,
+qrkit_status composed_solve(qrkit_ctx* ctx, bool chained, const void* J, const void* S, const void* b, void* p,
                             int refine_steps) {
-  if (ctx->precision == QRKIT_FP64) return solve_typed<double>(ctx, J, S, b, p, refine_steps, false, nullptr);
+  if (ctx->precision == QRKIT_FP64) return solve_typed<double>(ctx, chained, J, S, b, p, refine_steps, false, nullptr);
   const int steps = ctx->precision == QRKIT_FP32 ? 0 : refine_steps;
-  return solve_typed<float>(ctx, J, S, b, p, steps, false, nullptr);
+  return solve_typed<float>(ctx, chained, J, S, b, p, steps, false, nullptr);
 }
 
 qrkit_status composed_apply_qt(qrkit_ctx* ctx, const void* b, void* qtb) {
-  if (ctx->precision == QRKIT_FP64) return solve_typed<double>(ctx, nullptr, nullptr, b, nullptr, 0, true, qtb);
-  return solve_typed<float>(ctx, nullptr, nullptr, b, nullptr, 0, true, qtb);
+  if (ctx->precision == QRKIT_FP64) return solve_typed<double>(ctx, false, nullptr, nullptr, b, nullptr, 0, true, qtb);
+  return solve_typed<float>(ctx, false, nullptr, nullptr, b, nullptr, 0, true, qtb);
 }
 
 }  // namespace qrkit
@@ -1425,7 +1427,7 @@ static qrkit_status upload_i64(qrkit_ctx* ctx, DevBuf& buf, const std::vector<in
 }
 
 qrkit_status widen_to_double(qrkit_ctx* ctx, const float* in, double* out, int64_t n) {
-  chain_launch(ctx->stream, blocks_for(n, 256), 256, 0, widen_kernel, in, out, n);
+  start_launch(ctx->stream, blocks_for(n, 256), 256, 0, widen_kernel, in, out, n);
   ctx->launches += 1;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());
   return QRKIT_OK;
@@ -1474,7 +1476,7 @@ qrkit_status composed_layout(qrkit_ctx* ctx, size_t elem) {
     DevBuf* buf[4] = {&C.d_aug_off_d, &C.d_aug_off_u, &C.d_red_off_d, &C.d_red_off_u};
     for (int q = 0; q < 4; ++q) {
       if ((rc = ensure(ctx, *buf[q], (size_t)(K + 1) * sizeof(int64_t), "block offsets")) != QRKIT_OK) return rc;
-      chain_launch(ctx->stream, blocks_for(K + 1, 256), 256, 0, multiples_kernel, (int64_t*)buf[q]->ptr, K + 1,
+      start_launch(ctx->stream, blocks_for(K + 1, 256), 256, 0, multiples_kernel, (int64_t*)buf[q]->ptr, K + 1,
                    step[q]);
       ctx->launches += 1;
       QRKIT_CUDA_TRY(ctx, cudaGetLastError());
@@ -1729,11 +1731,11 @@ static qrkit_status solve_r_typed(qrkit_ctx* ctx, const void* qtb, void* p) {
   if (V.coupled == QRKIT_COUPLED_DENSE) {
     const TsqrLevel& top = C.levels.back();
     const bool pan = !C.panels.empty();
-    qrkit_status rc = dense_backsub<T>(ctx, pan ? (const T*)C.Rs.ptr : (const T*)top.X.ptr, pan ? s : top.ld, s,
+    qrkit_status rc = dense_backsub<T>(ctx, false, pan ? (const T*)C.Rs.ptr : (const T*)top.X.ptr, pan ? s : top.ld, s,
                                        c + P.cols, x + P.cols);
     if (rc != QRKIT_OK) return rc;
   }
-  return launch_block_backsub<T>(ctx, V, O, c, s ? x + P.cols : nullptr, x, 0);
+  return launch_block_backsub<T>(ctx, V.coupled == QRKIT_COUPLED_DENSE, V, O, c, s ? x + P.cols : nullptr, x, 0);
 }
 
 qrkit_status composed_solve_r(qrkit_ctx* ctx, const void* qtb, void* p) {
@@ -1765,10 +1767,10 @@ __global__ void norms_from_sumsq_kernel(const double* sq, T* D, int64_t n) {
 
 qrkit_status composed_norms_from_sumsq(qrkit_ctx* ctx, const double* sq, int64_t n, void* D) {
   if (ctx->precision == QRKIT_FP64)
-    LAUNCH(ctx, chain_launch(ctx->stream, blocks_for(n, 256), 256, 0, norms_from_sumsq_kernel<double>, sq, (double*)D,
+    LAUNCH(ctx, start_launch(ctx->stream, blocks_for(n, 256), 256, 0, norms_from_sumsq_kernel<double>, sq, (double*)D,
                              n));
   else
-    LAUNCH(ctx, chain_launch(ctx->stream, blocks_for(n, 256), 256, 0, norms_from_sumsq_kernel<float>, sq, (float*)D,
+    LAUNCH(ctx, start_launch(ctx->stream, blocks_for(n, 256), 256, 0, norms_from_sumsq_kernel<float>, sq, (float*)D,
                              n));
   return QRKIT_OK;
 }
@@ -1789,10 +1791,10 @@ qrkit_status composed_reduced_r(qrkit_ctx* ctx, void* R) {
   const void* src = C.panels.empty() ? top.X.ptr : C.Rs.ptr;
   const int64_t ld = C.panels.empty() ? top.ld : s;
   if (ctx->precision == QRKIT_FP64)
-    LAUNCH(ctx, chain_launch(ctx->stream, blocks_for((int64_t)s * s, 256), 256, 0, copy_upper_kernel<double>,
+    LAUNCH(ctx, start_launch(ctx->stream, blocks_for((int64_t)s * s, 256), 256, 0, copy_upper_kernel<double>,
                              (const double*)src, ld, s, (double*)R));
   else
-    LAUNCH(ctx, chain_launch(ctx->stream, blocks_for((int64_t)s * s, 256), 256, 0, copy_upper_kernel<float>,
+    LAUNCH(ctx, start_launch(ctx->stream, blocks_for((int64_t)s * s, 256), 256, 0, copy_upper_kernel<float>,
                              (const float*)src, ld, s, (float*)R));
   return QRKIT_OK;
 }
@@ -1803,7 +1805,7 @@ static qrkit_status solve_blocks_typed(qrkit_ctx* ctx, const void* qtb, void* p)
   ComposedView<T> V = view<T>(ctx, nullptr, nullptr);
   FactorOut<T> O = fout<T>(ctx);
   T* x = (T*)p;
-  return launch_block_backsub<T>(ctx, V, O, (const T*)qtb, V.s ? x + P.cols : nullptr, x, 0);
+  return launch_block_backsub<T>(ctx, false, V, O, (const T*)qtb, V.s ? x + P.cols : nullptr, x, 0);
 }
 
 qrkit_status composed_solve_blocks(qrkit_ctx* ctx, const void* qtb, void* p) {

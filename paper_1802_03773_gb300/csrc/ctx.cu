@@ -346,7 +346,7 @@ qrkit_status qrkit_factor_solve(qrkit_ctx* ctx, const void* J, const void* b, co
     if (st != QRKIT_OK) return st;
     ctx->factored = true;
     ctx->factor_in_planes = ctx->plan.mapping == 0 && ctx->plan.num_tasks > 0;
-    return more_stage2(ctx, q, D, lambda, p);
+    return more_stage2(ctx, true, q, D, lambda, p);
   }
   qrkit_status st = launch_block_solve(ctx, J, b, D, p, qtb, refine_steps);
   if (st == QRKIT_OK) {
@@ -365,7 +365,7 @@ qrkit_status qrkit_more_solve(qrkit_ctx* ctx, const void* qtb, const void* D, do
   if (!qtb || !p) return fail(ctx, QRKIT_EINVAL, "qtb and p are required");
   if (!(lambda >= 0.0)) return fail(ctx, QRKIT_EINVAL, "lambda must be >= 0");
   QRKIT_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
-  return more_stage2(ctx, qtb, D, lambda, p);
+  return more_stage2(ctx, false, qtb, D, lambda, p);
 }
 
 qrkit_status qrkit_more_trust_region(qrkit_ctx* ctx, const void* qtb, const void* D, double delta, double sigma,
@@ -485,7 +485,7 @@ qrkit_status qrkit_solve(qrkit_ctx* ctx, const void* b, void* p, int refine_step
   if (!b || !p) return fail(ctx, QRKIT_EINVAL, "b and p are required");
   if (refine_steps < 0 || refine_steps > 8) return fail(ctx, QRKIT_EINVAL, "refine_steps must be in [0, 8]");
   QRKIT_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
-  return composed_solve(ctx, ctx->comp.J, ctx->comp.S, b, p, refine_steps);
+  return composed_solve(ctx, false, ctx->comp.J, ctx->comp.S, b, p, refine_steps);
 }
 
 qrkit_status qrkit_get_band_factor(qrkit_ctx* ctx, void* Rw, void* c, double* res2) {

@@ -449,12 +449,13 @@ inline unsigned nblk(int64_t n, int64_t t) { return (unsigned)((n + t - 1) / t);
   } while (0)
 
 template <typename T>
-qrkit_status dense_backsub(qrkit_ctx* ctx, const T* R, int64_t ld, int s, const T* c, T* x) {
-  DS_LAUNCH(ctx, chain_launch(ctx->stream, 1, tri_cta(s), 0, tri_backsub_kernel<T>, R, ld, s, c, x, ctx->d_status));
+qrkit_status dense_backsub(qrkit_ctx* ctx, bool chained, const T* R, int64_t ld, int s, const T* c, T* x) {
+  DS_LAUNCH(ctx, launch_kernel(chained, ctx->stream, 1, tri_cta(s), 0, tri_backsub_kernel<T>, R, ld, s, c, x,
+                               ctx->d_status));
   return QRKIT_OK;
 }
-template qrkit_status dense_backsub<float>(qrkit_ctx*, const float*, int64_t, int, const float*, float*);
-template qrkit_status dense_backsub<double>(qrkit_ctx*, const double*, int64_t, int, const double*, double*);
+template qrkit_status dense_backsub<float>(qrkit_ctx*, bool, const float*, int64_t, int, const float*, float*);
+template qrkit_status dense_backsub<double>(qrkit_ctx*, bool, const double*, int64_t, int, const double*, double*);
 
 template <typename T>
 qrkit_status dense_normal(qrkit_ctx* ctx, const T* R, int64_t ld, int s, const double* g, T* dp, T* x) {
@@ -466,15 +467,15 @@ template qrkit_status dense_normal<float>(qrkit_ctx*, const float*, int64_t, int
 template qrkit_status dense_normal<double>(qrkit_ctx*, const double*, int64_t, int, const double*, double*, double*);
 
 template <typename T>
-qrkit_status dense_block_backsub(qrkit_ctx* ctx, const ComposedView<T>& V, const FactorOut<T>& O, const T* rhs,
-                                 const T* xS, T* x, int accumulate) {
-  DS_LAUNCH(ctx, chain_launch(ctx->stream, nblk(V.K * 32, kWarpBackThreads), kWarpBackThreads, 0,
-                              block_backsub_warp_kernel<T>, V, O, rhs, xS, x, accumulate));
+qrkit_status dense_block_backsub(qrkit_ctx* ctx, bool chained, const ComposedView<T>& V, const FactorOut<T>& O,
+                                 const T* rhs, const T* xS, T* x, int accumulate) {
+  DS_LAUNCH(ctx, launch_kernel(chained, ctx->stream, nblk(V.K * 32, kWarpBackThreads), kWarpBackThreads, 0,
+                               block_backsub_warp_kernel<T>, V, O, rhs, xS, x, accumulate));
   return QRKIT_OK;
 }
-template qrkit_status dense_block_backsub<float>(qrkit_ctx*, const ComposedView<float>&, const FactorOut<float>&,
+template qrkit_status dense_block_backsub<float>(qrkit_ctx*, bool, const ComposedView<float>&, const FactorOut<float>&,
                                                  const float*, const float*, float*, int);
-template qrkit_status dense_block_backsub<double>(qrkit_ctx*, const ComposedView<double>&, const FactorOut<double>&,
+template qrkit_status dense_block_backsub<double>(qrkit_ctx*, bool, const ComposedView<double>&, const FactorOut<double>&,
                                                   const double*, const double*, double*, int);
 
 size_t dense_refine_bytes(int64_t rows, int64_t nb, int s) {

@@ -332,7 +332,7 @@ qrkit_status composed_factor_scaled(qrkit_ctx* ctx, const void* J, const void* S
 // D = column norms of the block structure's J (zero -> 1), N doubles.
 qrkit_status composed_column_norms(qrkit_ctx* ctx, const void* J, const void* S, double* D);
 template <typename T> ComposedView<T> composed_view(qrkit_ctx* ctx, const void* J, const void* S);
-qrkit_status composed_solve(qrkit_ctx* ctx, const void* J, const void* S, const void* b, void* p,
+qrkit_status composed_solve(qrkit_ctx* ctx, bool chained, const void* J, const void* S, const void* b, void* p,
                             int refine_steps);
 qrkit_status composed_apply_qt(qrkit_ctx* ctx, const void* b, void* qtb);
 qrkit_status composed_solve_r(qrkit_ctx* ctx, const void* qtb, void* p);
@@ -380,7 +380,8 @@ bool window21(const qrkit_ctx* ctx);
 template <typename T>
 qrkit_status window21_factor(qrkit_ctx* ctx, const ComposedView<T>& V, const FactorOut<T>& O);
 template <typename T>
-qrkit_status window21_qt(qrkit_ctx* ctx, const ComposedView<T>& V, const FactorOut<T>& O, const T* b, T* rhs0);
+qrkit_status window21_qt(qrkit_ctx* ctx, bool chained, const ComposedView<T>& V, const FactorOut<T>& O, const T* b,
+                         T* rhs0);
 template <typename T>
 qrkit_status window21_backsub(qrkit_ctx* ctx, const ComposedView<T>& V, const FactorOut<T>& O, const T* rhs, const T* xS,
                               T* x, int accumulate);
@@ -417,12 +418,12 @@ qrkit_status dense_apply_blocks(qrkit_ctx* ctx, const ComposedView<T>& V, const 
 // R_i x_i = rhs_i - R12_i x_S by a warp per block; and, for float plans, a refinement step's
 // h_B = R_i^{-T} g_B and g_S - R12^T h_B with g = J^T (b - J p) - lambda D^2 p (ws: dense_refine_bytes).
 template <typename T>
-qrkit_status dense_backsub(qrkit_ctx* ctx, const T* R, int64_t ld, int s, const T* c, T* x);
+qrkit_status dense_backsub(qrkit_ctx* ctx, bool chained, const T* R, int64_t ld, int s, const T* c, T* x);
 template <typename T>
 qrkit_status dense_normal(qrkit_ctx* ctx, const T* R, int64_t ld, int s, const double* g, T* dp, T* x);
 template <typename T>
-qrkit_status dense_block_backsub(qrkit_ctx* ctx, const ComposedView<T>& V, const FactorOut<T>& O, const T* rhs,
-                                 const T* xS, T* x, int accumulate);
+qrkit_status dense_block_backsub(qrkit_ctx* ctx, bool chained, const ComposedView<T>& V, const FactorOut<T>& O,
+                                 const T* rhs, const T* xS, T* x, int accumulate);
 size_t dense_refine_bytes(int64_t rows, int64_t nb, int s);
 qrkit_status dense_refine_gradient(qrkit_ctx* ctx, const ComposedView<float>& V, const FactorOut<float>& O,
                                    const float* b, const float* p, double lam, void* ws, float* h, double* gS);
@@ -439,7 +440,7 @@ qrkit_status launch_block_tasks(qrkit_ctx* ctx, const void* J, const void* b, vo
                                 int refine_steps);
 // Moré's stage 2 (Sec. 5.2) for the stored block factor: p from [R_i; lambda^(1/2) D_i] and the
 // top m_i entries of qtb per block (D null: column norms of R_i).
-qrkit_status more_stage2(qrkit_ctx* ctx, const void* qtb, const void* D, double lambda, void* p);
+qrkit_status more_stage2(qrkit_ctx* ctx, bool chained, const void* qtb, const void* D, double lambda, void* p);
 qrkit_status more_trust_region(qrkit_ctx* ctx, const void* qtb, const void* D, double delta, double sigma,
                                int max_iter, double* lambda, void* p, int* iterations);
 // The warp-task factor (task planes) copied into J's packing and tau into column order.

@@ -439,7 +439,7 @@ qrkit_status lm_iteration(qrkit_ctx* ctx, double* x, int refine_steps, double ft
   LM_LAUNCH(ctx, chain_launch(st, (unsigned)(t.num_tiles + (t.s + kTilePts - 1) / kTilePts), kTilePts, 0,
                               lm_damp_kernel<T>, t, J, d2, S, E));
   if ((rc = composed_factor_scaled(ctx, J, Sv, E, true)) != QRKIT_OK) return rc;
-  if ((rc = composed_solve(ctx, J, Sv, b, p, refine_steps)) != QRKIT_OK) return rc;
+  if ((rc = composed_solve(ctx, true, J, Sv, b, p, refine_steps)) != QRKIT_OK) return rc;
   LM_LAUNCH(ctx, chain_launch(st, nblk(t.s, 128), 128, 0, cf_coef_kernel<T>, t, x, p, coef));
   LM_LAUNCH(ctx, chain_launch(st, (unsigned)t.num_tiles, kTilePts, 0, cf_trial_kernel<T>, t, x, L.data, coef, J, Sv,
                               b, p, E, start, (double*)L.tile_new.ptr, (double*)L.tile_pred.ptr));
@@ -622,12 +622,12 @@ qrkit_status qrkit_lm_linearize(qrkit_ctx* ctx, const double* x, void* J, void* 
   cudaStream_t st = ctx->stream;
   const double* coef = (const double*)L.coef.ptr;
   if (ctx->precision == QRKIT_FP64) {
-    chain_launch(st, nblk(t.s, 128), 128, 0, cf_coef_kernel<double>, t, x, (const double*)nullptr,
+    start_launch(st, nblk(t.s, 128), 128, 0, cf_coef_kernel<double>, t, x, (const double*)nullptr,
                  (double*)L.coef.ptr);
     chain_launch(st, (unsigned)t.num_tiles, kTilePts, 0, cf_eval_kernel<double>, t, x, L.data, coef, (double*)L.J.ptr,
                  (double*)L.S.ptr, (double*)L.b.ptr, (int32_t*)L.start.ptr, (double*)L.tile_cost.ptr);
   } else {
-    chain_launch(st, nblk(t.s, 128), 128, 0, cf_coef_kernel<float>, t, x, (const float*)nullptr, (double*)L.coef.ptr);
+    start_launch(st, nblk(t.s, 128), 128, 0, cf_coef_kernel<float>, t, x, (const float*)nullptr, (double*)L.coef.ptr);
     chain_launch(st, (unsigned)t.num_tiles, kTilePts, 0, cf_eval_kernel<float>, t, x, L.data, coef, (float*)L.J.ptr,
                  (float*)L.S.ptr, (float*)L.b.ptr, (int32_t*)L.start.ptr, (double*)L.tile_cost.ptr);
   }
@@ -648,7 +648,7 @@ qrkit_status qrkit_lm_residual(qrkit_ctx* ctx, const double* x, double* f) {
   if (!x || !f) return fail(ctx, QRKIT_EINVAL, "x and f are required");
   QRKIT_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
   LM& L = *ctx->lm;
-  chain_launch(ctx->stream, (unsigned)L.t.num_tiles, kTilePts, 0, cf_residual_kernel, L.t, x, L.data, f);
+  start_launch(ctx->stream, (unsigned)L.t.num_tiles, kTilePts, 0, cf_residual_kernel, L.t, x, L.data, f);
   ctx->launches += 1;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());
   return QRKIT_OK;

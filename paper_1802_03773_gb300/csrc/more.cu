@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(128) more_packed_kernel(MoreArgs<T> A) {
 }
 
 template <typename T>
-qrkit_status more_typed(qrkit_ctx* ctx, const void* qtb, const void* D, double lambda, void* p, double* sums) {
+qrkit_status more_typed(qrkit_ctx* ctx, bool chained, const void* qtb, const void* D, double lambda, void* p, double* sums) {
   const Plan& P = ctx->plan;
   MoreArgs<T> A{};
   A.qtb = (const T*)qtb;
@@ -218,9 +218,9 @@ qrkit_status more_typed(qrkit_ctx* ctx, const void* qtb, const void* D, double l
     A.tF = (const T*)ctx->ws.tfactor.ptr;
     const int64_t threads = P.num_tasks * 32;
     if (sums)
-      chain_launch(ctx->stream, (unsigned)((threads + 127) / 128), 128, 0, (more_planes_kernel<T, true>), A);
+      launch_kernel(chained, ctx->stream, (unsigned)((threads + 127) / 128), 128, 0, (more_planes_kernel<T, true>), A);
     else
-      chain_launch(ctx->stream, (unsigned)((threads + 127) / 128), 128, 0, (more_planes_kernel<T, false>), A);
+      launch_kernel(chained, ctx->stream, (unsigned)((threads + 127) / 128), 128, 0, (more_planes_kernel<T, false>), A);
   } else {
     A.F = (const T*)ctx->ws.factor.ptr;
     A.val_off = (const int64_t*)P.d_val_off.ptr;
@@ -230,9 +230,9 @@ qrkit_status more_typed(qrkit_ctx* ctx, const void* qtb, const void* D, double l
     A.m = (const uint8_t*)P.d_m.ptr;
     A.K = P.K;
     if (sums)
-      chain_launch(ctx->stream, (unsigned)((P.K + 127) / 128), 128, 0, (more_packed_kernel<T, true>), A);
+      launch_kernel(chained, ctx->stream, (unsigned)((P.K + 127) / 128), 128, 0, (more_packed_kernel<T, true>), A);
     else
-      chain_launch(ctx->stream, (unsigned)((P.K + 127) / 128), 128, 0, (more_packed_kernel<T, false>), A);
+      launch_kernel(chained, ctx->stream, (unsigned)((P.K + 127) / 128), 128, 0, (more_packed_kernel<T, false>), A);
   }
   ctx->launches += 1;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());
@@ -241,9 +241,9 @@ qrkit_status more_typed(qrkit_ctx* ctx, const void* qtb, const void* D, double l
 
 }  // namespace
 
-qrkit_status more_stage2(qrkit_ctx* ctx, const void* qtb, const void* D, double lambda, void* p) {
-  if (ctx->precision == QRKIT_FP64) return more_typed<double>(ctx, qtb, D, lambda, p, nullptr);
-  return more_typed<float>(ctx, qtb, D, lambda, p, nullptr);
+qrkit_status more_stage2(qrkit_ctx* ctx, bool chained, const void* qtb, const void* D, double lambda, void* p) {
+  if (ctx->precision == QRKIT_FP64) return more_typed<double>(ctx, chained, qtb, D, lambda, p, nullptr);
+  return more_typed<float>(ctx, chained, qtb, D, lambda, p, nullptr);
 }
 
 // Moré's choice of lambda for a trust region of scaled radius delta (Moré 1977): stage 2 at
@@ -263,8 +263,8 @@ qrkit_status more_trust_region(qrkit_ctx* ctx, const void* qtb, const void* D, d
   double h[3];
   auto eval = [&](double lam) -> qrkit_status {
     QRKIT_CUDA_TRY(ctx, cudaMemsetAsync(sums, 0, 3 * sizeof(double), ctx->stream));
-    qrkit_status r = ctx->precision == QRKIT_FP64 ? more_typed<double>(ctx, qtb, D, lam, p, sums)
-                                                  : more_typed<float>(ctx, qtb, D, lam, p, sums);
+    qrkit_status r = ctx->precision == QRKIT_FP64 ? more_typed<double>(ctx, true, qtb, D, lam, p, sums)
+                                                  : more_typed<float>(ctx, true, qtb, D, lam, p, sums);
     if (r != QRKIT_OK) return r;
     QRKIT_CUDA_TRY(ctx, cudaMemcpyAsync(h, sums, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
     QRKIT_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));

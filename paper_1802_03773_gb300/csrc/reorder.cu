@@ -342,7 +342,7 @@ inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 qrkit_status window_start_copy(qrkit_ctx* ctx, const int32_t* in) {
   Plan& P = ctx->plan;
   const int64_t nseg = (int64_t)P.seg_cols.size();
-  chain_launch(ctx->stream, nblk(P.K, 256), 256, 0, start_copy_kernel, in, (int32_t*)P.d_start.ptr, P.K,
+  start_launch(ctx->stream, nblk(P.K, 256), 256, 0, start_copy_kernel, in, (int32_t*)P.d_start.ptr, P.K,
                (const int64_t*)P.d_seg.ptr, nseg, ctx->d_status);
   ctx->launches += 1;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());
@@ -400,7 +400,7 @@ qrkit_status block_sort(qrkit_ctx* ctx, const BlockSortTables& t, const int32_t*
 qrkit_status block_row_order(qrkit_ctx* ctx, const int32_t* bord, int q, int64_t* order) {
   const int64_t K = ctx->plan.K;
   if (K * q == 0) return QRKIT_OK;
-  chain_launch(ctx->stream, nblk(K * q, 256), 256, 0, rows_of_blocks_kernel, bord, K, q, order);
+  start_launch(ctx->stream, nblk(K * q, 256), 256, 0, rows_of_blocks_kernel, bord, K, q, order);
   ctx->launches += 1;
   QRKIT_CUDA_TRY(ctx, cudaGetLastError());
   return QRKIT_OK;

@@ -371,8 +371,9 @@ qrkit_status window21_factor(qrkit_ctx* ctx, const ComposedView<T>& V, const Fac
   return QRKIT_OK;
 }
 template <typename T>
-qrkit_status window21_qt(qrkit_ctx* ctx, const ComposedView<T>& V, const FactorOut<T>& O, const T* b, T* rhs0) {
-  QRKIT_CUDA_TRY(ctx, chain_launch(ctx->stream, nblk(V.K, 256), 256, 0, window21_qt_kernel<T>, V, O, b, rhs0));
+qrkit_status window21_qt(qrkit_ctx* ctx, bool chained, const ComposedView<T>& V, const FactorOut<T>& O, const T* b,
+                         T* rhs0) {
+  QRKIT_CUDA_TRY(ctx, launch_kernel(chained, ctx->stream, nblk(V.K, 256), 256, 0, window21_qt_kernel<T>, V, O, b, rhs0));
   ctx->launches += 1;
   return QRKIT_OK;
 }
@@ -386,7 +387,7 @@ qrkit_status window21_backsub(qrkit_ctx* ctx, const ComposedView<T>& V, const Fa
 }
 #define WINDOW21_TYPES(T)                                                                                          \
   template qrkit_status window21_factor<T>(qrkit_ctx*, const ComposedView<T>&, const FactorOut<T>&);              \
-  template qrkit_status window21_qt<T>(qrkit_ctx*, const ComposedView<T>&, const FactorOut<T>&, const T*, T*);    \
+  template qrkit_status window21_qt<T>(qrkit_ctx*, bool, const ComposedView<T>&, const FactorOut<T>&, const T*, T*); \
   template qrkit_status window21_backsub<T>(qrkit_ctx*, const ComposedView<T>&, const FactorOut<T>&, const T*,    \
                                             const T*, T*, int);
 WINDOW21_TYPES(float)
