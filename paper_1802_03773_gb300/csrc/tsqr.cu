@@ -16,6 +16,7 @@
 #include "chain.cuh"
 #include "device_util.cuh"
 #include "internal.h"
+#include "roots.cuh"
 
 namespace qrkit {
 namespace {
@@ -64,8 +65,7 @@ __device__ __forceinline__ void reflector(double alpha, double sq, double& beta,
   beta = tau = scale = 0.0;
   if (n2 == 0.0) return;
   const double y = rsqrt(n2);
-  double norm = n2 * y;
-  norm = fma(fma(-norm, norm, n2), 0.5 * y, norm);   // the root to its last place
+  const double norm = dev::newton_root(n2, y);
   const double a = fabs(alpha);
   beta = alpha >= 0.0 ? -norm : norm;
   tau = fma(a, y, 1.0);

@@ -23,6 +23,7 @@
 #include "device_util.cuh"
 #include "f32x2.cuh"
 #include "internal.h"
+#include "roots.cuh"
 
 namespace qrkit {
 namespace {
@@ -130,7 +131,7 @@ tsqr_panel_tile_kernel(float* X, int64_t ld, int64_t M, float* Xn, int64_t ldn, 
 
   // the reflector of column k from its register column c: the column below k scaled to v (v_k = 1, stored
   // implicitly), beta on the diagonal; v written to its place and announced; rows 4 lane .. + 3 of v to
-  // head, tau returned.  The root of n2 = norm^2 is n2 y with one Newton step, y = 1 / sqrt(n2).
+  // head, tau returned.
   auto form = [&](int k, f2 (&c)[2 * NU], f2 (&head)[2]) -> float {
     float h[4];   // rows 4 lane .. 4 lane + 3: the only ones that can lie on or above row k
     unpack2(c[0], h[0], h[1]);
@@ -152,10 +153,8 @@ tsqr_panel_tile_kernel(float* X, int64_t ld, int64_t M, float* Xn, int64_t ldn, 
     sq = warp_sum(sq);
     const float n2 = fmaf(alpha, alpha, sq);
     const bool some = n2 != 0.f;
-    float y = rsqrtf(some ? n2 : 1.f);
-    float norm = n2 * y;
-    norm = fmaf(fmaf(-norm, norm, n2), 0.5f * y, norm);
-    y = fmaf(fmaf(-norm, y, 1.f), y, y);
+    const float seed = rsqrtf(some ? n2 : 1.f);
+    const float norm = dev::newton_root(n2, seed), y = dev::newton_inverse(norm, seed);
     const float beta = some ? (alpha >= 0.f ? -norm : norm) : 0.f;
     const float t = some ? fmaf(fabsf(alpha), y, 1.f) : 0.f;        // (beta - alpha) / beta
     const float scale = some ? __frcp_rn(alpha - beta) : 0.f;
