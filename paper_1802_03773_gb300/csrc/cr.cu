@@ -37,6 +37,7 @@
 #include "f32x2.cuh"
 #include "internal.h"
 #include "roots.cuh"
+#include "sums.cuh"
 
 namespace qrkit {
 namespace {
@@ -96,10 +97,11 @@ struct ExactReflector {
       if (!(n2 < 1.17549435e-38f)) {   // below: the column is dropped from the reflector, as its norm underflows
         float y;
         asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(n2));
+        const float seed = qr_rcp(p >= 0.f ? p + n2 * y : p - n2 * y);   // of the scale, while the root is refined
         const float norm = dev::newton_root(n2, y);
         beta = p >= 0.f ? -norm : norm;
         tau = fma(fabsf(p), dev::newton_inverse(norm, y), 1.f);
-        scale = dev::newton_inverse(p - beta, qr_rcp(p - beta));
+        scale = dev::newton_inverse(p - beta, seed);
       }
     } else {
       const T norm = sqrt(n2);
@@ -308,47 +310,76 @@ __device__ __forceinline__ void load_e0(T (&v)[8], const T* base, int64_t it, in
   }
 }
 
-// A thread's squared residual: a float pair (Dot2) for float, a double for double.  (A warp's FP64 instruction
+// A thread's squared residual: a float pair for float, a double for double.  (A warp's FP64 instruction
 // occupies the SM's FP64 unit for 16 cycles here: summing every square in double took a quarter of the
-// compression's and of the fronts' time.)
+// compression's and of the fronts' time.)  A right-hand side may have any
+// scale: an entry whose square or its rounding error would leave the float range goes to res2 in double by itself.
 template <typename T>
-struct ResidualSum {
-  T h = T(0), l = T(0);
-  __device__ __forceinline__ void square(T x) {
-    if constexpr (sizeof(T) == 4) {
-      const T p = __fmul_rn(x, x), pe = __fmaf_rn(x, x, -p);
-      add(p, pe);
-    } else {
-      h += x * x;
-    }
-  }
-  __device__ __forceinline__ void add(T ph, T pl) {
-    if constexpr (sizeof(T) == 4) {
-      T t, e;
-      dev::two_sum(h, ph, t, e);
-      h = t;
-      l = __fadd_rn(l, __fadd_rn(e, pl));
-    } else {
-      h += ph;
-    }
-  }
-  // into res2 of the thread's instance: one atomic per warp where all its threads work on one instance
-  __device__ __forceinline__ void flush(double* res2, int64_t k) {
-    __syncwarp();
-    const unsigned m = __activemask();
-    const int64_t k0 = __shfl_sync(m, k, __ffs(m) - 1);
-    if (m == 0xffffffffu && __all_sync(m, k == k0)) {
+struct ResidualSum;
+template <>
+struct ResidualSum<float> {
+  dev::Pair s;
+  template <int N>
+  __device__ __forceinline__ void squares(const float (&x)[N], double* res2) {
+    bool all = true;
+    float p[N], e[N];   // the squares and their rounding errors, added up pairwise
 #pragma unroll
-      for (int d = 16; d >= 1; d >>= 1) {
-        const T ph = __shfl_xor_sync(m, h, d), pl = __shfl_xor_sync(m, l, d);
-        add(ph, pl);
+    for (int q = 0; q < N; ++q) {
+      const bool ok = dev::square_exact(x[q]);
+      const float y = ok ? x[q] : 0.f;
+      p[q] = __fmul_rn(y, y);
+      e[q] = __fmaf_rn(y, y, -p[q]);
+      all = all && ok;
+    }
+#pragma unroll
+    for (int w = N / 2; w >= 1; w /= 2)
+#pragma unroll
+      for (int q = 0; q < w; ++q) {
+        float t, d;
+        dev::two_sum(p[q], p[q + w], t, d);
+        p[q] = t;
+        e[q] = __fadd_rn(__fadd_rn(e[q], e[q + w]), d);
       }
-      if ((threadIdx.x & 31) == 0 && h != T(0)) atomicAdd(res2 + k, (double)h + (double)l);
-    } else if (h != T(0)) {
-      atomicAdd(res2 + k, (double)h + (double)l);
+    s.add(p[0], e[0]);
+    if (!all) {
+#pragma unroll
+      for (int q = 0; q < N; ++q)
+        if (!dev::square_exact(x[q])) atomicAdd(res2, (double)x[q] * (double)x[q]);
     }
   }
+  __device__ __forceinline__ void add_lane(unsigned m, int d) {
+    const float ph = __shfl_xor_sync(m, s.h, d), pl = __shfl_xor_sync(m, s.l, d);
+    s.add(ph, pl);
+  }
+  __device__ __forceinline__ double value() const { return s.value(); }
 };
+template <>
+struct ResidualSum<double> {
+  double s = 0.0;
+  template <int N>
+  __device__ __forceinline__ void squares(const double (&x)[N], double*) {
+#pragma unroll
+    for (int q = 0; q < N; ++q) s += x[q] * x[q];
+  }
+  __device__ __forceinline__ void add_lane(unsigned m, int d) { s += __shfl_xor_sync(m, s, d); }
+  __device__ __forceinline__ double value() const { return s; }
+};
+// into res2 of the thread's instance: one atomic per warp where all its threads work on one instance
+template <typename T>
+__device__ __forceinline__ void flush_residual(ResidualSum<T>& r, double* res2, int64_t k) {
+  __syncwarp();
+  const unsigned m = __activemask();
+  const int64_t k0 = __shfl_sync(m, k, __ffs(m) - 1);
+  const bool one = m == 0xffffffffu && __all_sync(m, k == k0);
+  if (one) {
+#pragma unroll
+    for (int d = 16; d >= 1; d >>= 1) r.add_lane(m, d);
+  }
+  if (!one || (threadIdx.x & 31) == 0) {
+    const double v = r.value();
+    if (v != 0.0) atomicAdd(res2 + k, v);
+  }
+}
 
 // Rows of 8 aligned values (kStaged) arrive through shared memory: the lanes of a warp fetch each thread's next
 // four rows together (8 or 16 lanes a thread, whole lines, where a thread's own 16-byte loads touch a line of
@@ -479,8 +510,7 @@ __global__ void __launch_bounds__(kCompThreads, sizeof(T) == 4 ? 4 : 2) cr_compr
         for (int q = 0; q < 4; ++q) ahead[q] = r + q < r_end ? A.starts[r + q] - c0 : -1;
       }
       W.insert(a, b);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) res.square(b[q]);
+      res.squares(b, A.res2 + k);
     } else if (c < kCB) {
       T row[8];
 #pragma unroll
@@ -504,7 +534,7 @@ __global__ void __launch_bounds__(kCompThreads, sizeof(T) == 4 ? 4 : 2) cr_compr
     }
     store_e0(dst, at, 136, W.z);
   }
-  res.flush(A.res2, k);
+  flush_residual(res, A.res2, k);
 }
 
 // 1b. merge of up to kMergeFan partial triangles of a block into one, by the same window; 16 columns.
@@ -523,7 +553,7 @@ __global__ void __launch_bounds__(kCompThreads) cr_merge_kernel(CRArgs<T> A, con
   if (w >= nitems) return;
   const MergeItem M = items[w];
   const int n = M.n;
-  const int64_t first = M.first, gb = M.blk, item = M.out < 0 ? gb : M.out;
+  const int64_t first = M.first, gb = M.blk, item = M.out < 0 ? gb : M.out, k = A.binst[gb];
   T* out = M.out < 0 ? A.E0 : part;
   Window<T> W;
 #pragma unroll
@@ -551,8 +581,7 @@ __global__ void __launch_bounds__(kCompThreads) cr_merge_kernel(CRArgs<T> A, con
       }
     }
     W.insert(a, b);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) res.square(b[q]);
+    res.squares(b, A.res2 + k);
     if (c < 8) {
       T row[8];
 #pragma unroll
@@ -568,7 +597,7 @@ __global__ void __launch_bounds__(kCompThreads) cr_merge_kernel(CRArgs<T> A, con
     out[e0_at<T>(item, 128 + c)] = W.z[0];
     W.shift();
   }
-  res.flush(A.res2, A.binst[gb]);
+  flush_residual(res, A.res2, k);
 }
 
 // Work items of a level: inst << 32 | i << 2 | kind (0 eliminate odd i, 1 move up, 2 last).
@@ -821,7 +850,8 @@ __device__ __forceinline__ void cr_item(const CRArgs<T>& A, int64_t k, int64_t i
     }
     F[192 + j] = lane_of(dl, j);
     F[200 + j] = lane_of(ch, j);
-    res.square(lane_of(dh, j));
+    const T left[1] = {lane_of(dh, j)};
+    res.squares(left, A.res2 + k);
   } else {   // the last block: its A is triangular, nothing is to its right
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
@@ -830,7 +860,8 @@ __device__ __forceinline__ void cr_item(const CRArgs<T>& A, int64_t k, int64_t i
       R[128 + 8 * r + j] = bl[r];
     }
     R[192 + j] = lane_of(cl, j);
-    res.square(lane_of(ch, j));
+    const T left[1] = {lane_of(ch, j)};
+    res.squares(left, A.res2 + k);
   }
 }
 
@@ -852,7 +883,7 @@ cr_level_kernel(CRArgs<T> A, const int64_t* items, int64_t nitems, int level, co
   } else if (nitems > 0) {
     decode(items[nitems - 1], k, i, kind);   // adds nothing, to the last item's instance
   }
-  res.flush(A.res2, k);
+  flush_residual(res, A.res2, k);
 }
 
 // ---- 3. back-substitution of one block, eight lanes: lane q owns row q of the block's R (own | left |
@@ -1017,7 +1048,7 @@ __global__ void __launch_bounds__(tail_threads<T>(), 1) cr_tail_kernel(CRArgs<T>
     __syncthreads();
     if (Gl == 1) break;
   }
-  res.flush(A.res2, k);
+  flush_residual(res, A.res2, k);
   tail_backsub(A, k, G, lt, l, false, x, (T*)nullptr);
 }
 
