@@ -67,6 +67,14 @@ __device__ __forceinline__ float qr_rcp(float x) {
 }
 __device__ __forceinline__ double qr_rcp(double x) { return 1.0 / x; }
 
+// Squared norms of float columns below 2^-90 lose bits, and vanish below 2^-149: the column is then squared again times
+// kLift.  (A reflector of few rows meets pivots far below the scale of the data.)
+constexpr float kLift = 0x1p80f;
+template <typename T>
+__device__ __forceinline__ bool faint(T n2) {
+  return sizeof(T) == 4 && n2 < T(0x1p-90f);
+}
+
 // The Householder reflector of a column with pivot p and squared norm s2 below it (Sec. 2):
 // v = (1, scale x), H = I - tau v v^T, the pivot becomes beta.
 template <typename T>
@@ -228,10 +236,23 @@ struct Window {
       T s2 = T(0);
 #pragma unroll
       for (int q = 0; q < 4; ++q) s2 += a[q][k] * a[q][k];
-      const ExactReflector<T> h(t[tri(k, k)], s2);
+      const T p = t[tri(k, k)];
+      ExactReflector<T> h(p, s2);
       T v[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) v[q] = a[q][k] * h.scale;
+      if (faint(p * p + s2)) {
+        s2 = T(0);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          v[q] = a[q][k] * T(kLift);
+          s2 += v[q] * v[q];
+        }
+        h = ExactReflector<T>(p * T(kLift), s2);
+        h.beta *= T(1) / T(kLift);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] *= h.scale;
+      }
       t[tri(k, k)] = h.beta;
 #pragma unroll
       for (int j = k + 1; j < 8; ++j) {

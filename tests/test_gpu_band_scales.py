@@ -35,3 +35,29 @@ def test_squared_residual_of_scaled_rhs(scale, tuning):
     got = p.cpu().numpy().astype(np.float64) / scale
     assert np.linalg.norm(got - x) <= 1e-5 * np.linalg.norm(x)
     np.testing.assert_allclose(res2 / scale / scale, want, rtol=2e-6)
+
+
+# A power of two scales every operation exactly, so the solution of a scaled J is the inversely scaled one, but for
+# the entries that underflow against the others: rounding errors of plain float
+@pytest.mark.parametrize("rpc,tuning", [(4, None), (4, "compress 0 3"), (25, None)])
+@pytest.mark.parametrize("power", [-62, -60, -57, -52, 50, 56])
+def test_scaled_matrix(power, rpc, tuning):
+    torch = cuda_or_skip()
+    from paper_1802_03773_gb300 import Context
+    N = 200
+    inst, vals, b = batch([N], rpc, 8, np.float32, seed=7)
+    J, rhs = torch.from_numpy(np.ascontiguousarray(vals.reshape(-1))).cuda(), torch.from_numpy(b).cuda()
+
+    def solve(factor):
+        ctx = Context(0, precision="fp32")
+        ctx.plan_banded([N], rows_per_col=rpc, window=8, solver=2)
+        if tuning:
+            ctx.apply_tuning(tuning)
+        p = torch.empty(N, device="cuda")
+        ctx.factor_solve(J * factor, rhs, p, lam=0.5, refine_steps=0)
+        ctx.sync_status()
+        ctx.close()
+        return p.cpu().numpy().astype(np.float64) * factor
+
+    want = solve(1.0)
+    assert np.abs(solve(2.0 ** power) - want).max() <= 1e-6 * np.abs(want).max()
