@@ -16,6 +16,7 @@
 #include "chain.cuh"
 #include "device_util.cuh"
 #include "internal.h"
+#include "sums.cuh"
 
 namespace qrkit {
 namespace {
@@ -40,7 +41,7 @@ __device__ __forceinline__ void dot2_acc(float& sh, float& sl, float a, float x)
 }
 
 // ---- column norms D = diag(J^T J)^(1/2) (Sec. 5.2): sums in double, those of a float dense S as
-// float pairs per thread first (FP64 runs at 1/73 of the FP32 rate: 811 us in FP64 for an S of
+// sums of three floats per thread first (FP64 runs at 1/73 of the FP32 rate: 811 us in FP64 for an S of
 // 819 MB) ----
 template <typename T>
 __global__ void colnorm_blocks_kernel(ComposedView<T> V, double* sq) {
@@ -77,11 +78,14 @@ __global__ void __launch_bounds__(kNormThreads) colnorm_dense_part_kernel(Compos
     const T* c = V.S + col * V.rows;
     double s = 0;
     if constexpr (sizeof(T) == sizeof(float)) {
-      // at most 32 squares per thread as a float pair (Dot2)
-      float sh = 0.f, sl = 0.f;
-#pragma unroll 8
-      for (int64_t r = r0 + threadIdx.x; r < r1; r += kNormThreads) dot2_acc(sh, sl, c[r], c[r]);
-      s = (double)sh + (double)sl;
+      dev::Squares sum;
+      for (int64_t r = r0 + threadIdx.x; r < r1; r += 8 * kNormThreads) {
+        float x[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) x[q] = r + q * kNormThreads < r1 ? c[r + q * kNormThreads] : 0.f;
+        sum.add(x);
+      }
+      s = sum.value();
     } else {
       for (int64_t r = r0 + threadIdx.x; r < r1; r += kNormThreads) {
         const double x = (double)c[r];

@@ -15,6 +15,7 @@
 #include "chain.cuh"
 #include "device_util.cuh"
 #include "internal.h"
+#include "sums.cuh"
 
 namespace qrkit {
 namespace {
@@ -45,6 +46,29 @@ struct Sum {
   __device__ __forceinline__ double value() const { return (double)h + (double)l; }
 };
 
+// What a lane of a run adds up: products (kGrad), or squares.
+template <typename T, bool kGrad>
+struct RunSum {
+  Sum<T> s;
+  template <int N>
+  __device__ __forceinline__ void squares(const T (&x)[N]) {
+#pragma unroll
+    for (int r = 0; r < N; ++r) s.fma(x[r], x[r]);
+  }
+  __device__ __forceinline__ void fma(T a, T x) { s.fma(a, x); }
+  __device__ __forceinline__ void fma(T a, T xh, T xl) { s.fma(a, xh, xl); }
+  __device__ __forceinline__ double value() const { return s.value(); }
+};
+template <>
+struct RunSum<float, false> {
+  dev::Squares s;
+  template <int N>
+  __device__ __forceinline__ void squares(const float (&x)[N]) {
+    s.add(x);
+  }
+  __device__ __forceinline__ double value() const { return s.value(); }
+};
+
 // Eight lanes per run of kRun sorted blocks.  kGrad: sum of S^T r - R12^T h; else of the squares of S.
 template <typename T, bool kGrad, int NR, int MM>
 __global__ void __launch_bounds__(kThreads) window_sums_kernel(WindowSums<T> A) {
@@ -54,14 +78,14 @@ __global__ void __launch_bounds__(kThreads) window_sums_kernel(WindowSums<T> A) 
   const int64_t p0 = run * kRun, p1 = p0 + kRun < A.K ? p0 + kRun : A.K;
   if (p0 >= A.K || t >= A.w) return;
   const int n = A.n, m = A.m, w = A.w;
-  Sum<T> acc;
+  RunSum<T, kGrad> acc;
   int64_t cur = -1;
   auto flush = [&]() {
     if (cur >= 0 && cur + t < A.s) {
       const double v = acc.value();
       if (v != 0.0) atomicAdd(A.out + cur + t, v);
     }
-    acc = Sum<T>();
+    acc = RunSum<T, kGrad>();
   };
   constexpr int U = NR * MM <= 2 ? 4 : 1;   // blocks whose loads are in flight together
   for (int64_t q0 = p0; q0 < p1; q0 += U) {
@@ -105,13 +129,11 @@ __global__ void __launch_bounds__(kThreads) window_sums_kernel(WindowSums<T> A) 
         flush();
         cur = st[u];
       }
-#pragma unroll
-      for (int r = 0; r < NR; ++r)
-        if (r < n) {
-          if constexpr (kGrad) acc.fma(sv[u][r], rh[u][r], rl[u][r]);
-          else acc.fma(sv[u][r], sv[u][r]);
-        }
+      if constexpr (!kGrad) acc.squares(sv[u]);   // zeros past row n
       if constexpr (kGrad) {
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+          if (r < n) acc.fma(sv[u][r], rh[u][r], rl[u][r]);
 #pragma unroll
         for (int k = 0; k < MM; ++k)
           if (k < m) acc.fma(rv[u][k], hv[u][k]);
