@@ -33,6 +33,7 @@
 #include "device_util.cuh"
 #include "internal.h"
 #include "mlp_policy.cuh"
+#include "roots.cuh"
 
 namespace qrkit {
 
@@ -181,8 +182,7 @@ cf_eval_kernel(LMTables t, const double* x, const double* data, const double* co
 }
 
 // E_j = lambda_k^(1/2) D_j with D_j = ||column j of J|| (zero -> 1): a tile of points per CTA, then the shared
-// columns (squared norms d2) 256 at a time.  The norm of a float block column is a float pair: its two
-// squares summed exactly, and one Newton step on the float root.
+// columns (squared norms d2) 256 at a time.
 template <typename T>
 __global__ void __launch_bounds__(kTilePts) lm_damp_kernel(LMTables t, const T* J, const double* d2,
                                                            const qrkit_lm_state* st, double* E) {
@@ -195,17 +195,8 @@ __global__ void __launch_bounds__(kTilePts) lm_damp_kernel(LMTables t, const T* 
     if (i >= t.tile_p0[tile + 1]) return;
     const T jx = J[2 * i], jy = J[2 * i + 1];
     double d;
-    if constexpr (sizeof(T) == 4) {
-      const float a = __fmul_rn(jx, jx), b = __fmul_rn(jy, jy);
-      float h, l;
-      dev::two_sum(a, b, h, l);
-      l += __fmaf_rn(jx, jx, -a) + __fmaf_rn(jy, jy, -b);
-      const float r = sqrtf(h);
-      const float c = r > 0.f ? (__fmaf_rn(-r, r, h) + l) / (2.f * r) : 0.f;
-      d = (double)r + (double)c;
-    } else {
-      d = sqrt(jx * jx + jy * jy);
-    }
+    if constexpr (sizeof(T) == 4) d = dev::norm_of_two(jx, jy);
+    else d = sqrt(jx * jx + jy * jy);
     E[i] = root * (d == 0.0 ? 1.0 : d);
     return;
   }

@@ -9,6 +9,8 @@
 
 #include <cuda_runtime.h>
 
+#include "sums.cuh"
+
 namespace qrkit {
 namespace dev {
 
@@ -20,6 +22,28 @@ __device__ __forceinline__ T newton_root(T x, T y) {
   if (x < tiny) return sqrt(x);
   const T r = x * y;
   return y == T(0) ? x : fma(fma(-r, r, x), T(0.5) * y, r);
+}
+// The root of a sum h + l + m of floats (h the sum rounded, normal) in double: the float root of h, its remainder, which
+// is a float, and two quotients of what is left.
+__device__ __forceinline__ double root_of_sum(float h, float l, float m) {
+  const float r = sqrtf(h);
+  const float e = fmaf(-r, r, h);              // exact
+  const float a = e + l, b = a - e;            // a + al = e + l (TwoSum)
+  const float al = (e - (a - b)) + (l - b) + m;
+  const float c = a / (2.f * r);
+  const float d = (fmaf(-2.f * r, c, a) + fmaf(-c, c, al)) / (2.f * r);
+  return (double)r + ((double)c + (double)d);
+}
+// sqrt(x^2 + y^2) of floats in double, to its last bits, with a quarter of the FP64 instructions (their squares as a sum
+// of floats); in double where a square leaves the float range.
+__device__ __forceinline__ double norm_of_two(float x, float y) {
+  if (square_exact(x) && square_exact(y) && (x != 0.f || y != 0.f)) {
+    Triple s;
+    s.fma(x, x);
+    s.fma(y, y);
+    return root_of_sum(s.h, s.l, s.m);
+  }
+  return sqrt((double)x * (double)x + (double)y * (double)y);
 }
 // 1 / x from a seed y: y + (1 - x y) y, within one unit in the last place (and 1 / infinity = 0).
 template <typename T>
