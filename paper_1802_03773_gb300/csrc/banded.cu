@@ -440,8 +440,30 @@ struct BandGroups {   // what both kernels are told
   int rpc, w, gs;   // gs: stride of a staged group
 };
 
+// lambda D^2 of a column as a float pair, for the gradient: float arithmetic while lambda and D^2 are of a size whose
+// products stay exact, double otherwise (a given D may balance a lambda of any size).
+struct BandDamping {
+  double lam;
+  float h, l;       // lambda as a pair
+  bool ordinary;    // 2^-60 <= lambda <= 2^60
+  explicit BandDamping(double x)
+      : lam(x), h((float)x), l((float)(x - (double)(float)x)), ordinary(x >= 0x1p-60 && x <= 0x1p60) {}
+  // times D^2 = s + e; dd: D^2 in double
+  template <class F>
+  __device__ __forceinline__ float2 times(float s, float e, F&& dd) const {
+    if (ordinary && s >= 0x1p-40f && s <= 0x1p60f) {
+      const float p = __fmul_rn(h, s);
+      return make_float2(p, __fmaf_rn(h, e, __fmaf_rn(l, s, __fmaf_rn(h, s, -p))));
+    }
+    const double v = lam * dd();
+    return make_float2((float)v, (float)(v - (double)(float)v));
+  }
+};
+
+// The group sums are floats, as accurate as the entries' squares; what follows them is done in float pairs and adds
+// nothing to their error.
 template <bool kW8, bool kStaged, int MW>
-__global__ void __launch_bounds__(256) band_norm_f32_kernel(BandGroups B, double* D, float2* D2) {
+__global__ void __launch_bounds__(256) band_norm_f32_kernel(BandGroups B, BandDamping damp, double* D, float2* E2) {
   dev::chain_wait();
   extern __shared__ __align__(16) float sm_f[];
   const int nt = blockDim.x, tid = threadIdx.x, w = B.w;
@@ -475,28 +497,26 @@ __global__ void __launch_bounds__(256) band_norm_f32_kernel(BandGroups B, double
   }
   const float s = h + l;
   l = (h - s) + l;
-  float r = 1.f, c = 0.f;
-  if (s > 0.f) {
+  float r = s, c = 0.f;   // NaN and infinity are their own root
+  if (s > 0.f && s <= 3.4e38f) {
     r = sqrtf(s);
     c = (__fmaf_rn(-r, r, s) + l) / (2.f * r);   // one Newton step for the root of s + l
-  } else if (s == 0.f) {
-    D2[grp] = make_float2(1.f, 0.f);   // zero norm -> 1
+  } else if (s == 0.f) {   // zero norm -> 1
+    E2[grp] = damp.times(1.f, 0.f, [] { return 1.0; });
     D[grp] = 1.0;
     return;
-  } else {
-    r = s;   // NaN
   }
-  D2[grp] = make_float2(s, l);
+  E2[grp] = damp.times(s, l, [&] { return (double)s + (double)l; });
   D[grp] = (double)r + (double)c;
 }
 
-// D and D^2 (a float pair) of a given float D.
-__global__ void band_given_d_kernel(const float* in, double* D, float2* D2, int64_t n) {
+// D and lambda D^2 (a float pair) of a given float D.
+__global__ void band_given_d_kernel(const float* in, BandDamping damp, double* D, float2* E2, int64_t n) {
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
   const float d = in[j], p = __fmul_rn(d, d);
   D[j] = (double)d;
-  D2[j] = make_float2(p, __fmaf_rn(d, d, -p));
+  E2[j] = damp.times(p, __fmaf_rn(d, d, -p), [&] { return (double)d * (double)d; });
 }
 
 // g = J^T (b - J x) - lambda D^2 x into the parallel QR's padded layout: the residual of a row as an
@@ -504,7 +524,7 @@ __global__ void band_given_d_kernel(const float* in, double* D, float2* D2, int6
 // without GB300's slow FP64 pipe), the column sums as pairs too.
 template <bool kW8, bool kStaged, int MW>
 __global__ void __launch_bounds__(256) band_grad_f32_kernel(BandGroups B, const float* b, const float* x,
-                                                            const float2* D2, float lam_h, float lam_l,
+                                                            const float2* E2, bool damped,
                                                             const int64_t* blk0, float* gp) {
   dev::chain_wait();
   extern __shared__ __align__(16) float sm_f[];
@@ -620,14 +640,11 @@ __global__ void __launch_bounds__(256) band_grad_f32_kernel(BandGroups B, const 
   } else {
     for (int t = 0; t < w && t <= j; ++t) diagonal(t);
   }
-  if (lam_h > 0.f) {   // - lambda D^2 x, all factors but x pairs
-    const float2 d2 = D2[grp];
-    float p = __fmul_rn(lam_h, d2.x);
-    float pe = __fmaf_rn(lam_h, d2.x, -p);
-    pe = __fmaf_rn(lam_h, d2.y, __fmaf_rn(lam_l, d2.x, pe));
+  if (damped) {   // - lambda D^2 x
+    const float2 e2 = E2[grp];
     const float xj = -xs[tid];
-    const float q = __fmul_rn(p, xj);
-    const float qe = __fmaf_rn(pe, xj, __fmaf_rn(p, xj, -q));
+    const float q = __fmul_rn(e2.x, xj);
+    const float qe = __fmaf_rn(e2.y, xj, __fmaf_rn(e2.x, xj, -q));
     float tt, e;
     dev::two_sum(s, q, tt, e);
     s = tt;
@@ -896,7 +913,7 @@ qrkit_status banded_plan(qrkit_ctx* ctx, const qrkit_structure* s) {
   if ((st = ensure(ctx, B.Rw, (size_t)cc * B.w * es, "banded R")) != QRKIT_OK) return st;
   if ((st = ensure(ctx, B.c, (size_t)cc * es, "banded c")) != QRKIT_OK) return st;
   if ((st = ensure(ctx, B.D, (size_t)cc * sizeof(double), "banded D")) != QRKIT_OK) return st;
-  if (es == sizeof(float) && (st = ensure(ctx, B.D2, (size_t)cc * sizeof(float2), "banded D")) != QRKIT_OK) return st;
+  if (es == sizeof(float) && (st = ensure(ctx, B.E2, (size_t)cc * sizeof(float2), "banded D")) != QRKIT_OK) return st;
   if ((st = ensure(ctx, B.res2, (size_t)B.num_inst * sizeof(double), "banded residual")) != QRKIT_OK) return st;
   if (B.parallel) {
     if ((st = cr_build(ctx, B.cr, cols, c0, r0, nrows)) != QRKIT_OK) return st;
@@ -948,8 +965,8 @@ static qrkit_status banded_run(qrkit_ctx* ctx, const void* J, const void* b, con
         QRKIT_CUDA_TRY(ctx, cudaMemcpyAsync(D, Dext, (size_t)B.total_cols * sizeof(double),
                                             cudaMemcpyDeviceToDevice, st));
       } else {
-        band_given_d_kernel<<<nblk(B.total_cols, 256), 256, 0, st>>>((const float*)Dext, D, (float2*)B.D2.ptr,
-                                                                    B.total_cols);
+        band_given_d_kernel<<<nblk(B.total_cols, 256), 256, 0, st>>>((const float*)Dext, BandDamping(lambda), D,
+                                                                    (float2*)B.E2.ptr, B.total_cols);
         ctx->launches += 1;
         QRKIT_CUDA_TRY(ctx, cudaGetLastError());
       }
@@ -965,8 +982,9 @@ static qrkit_status banded_run(qrkit_ctx* ctx, const void* J, const void* b, con
         const BandLaunch L = band_launch(G, (size_t)(B.w + 1) * sizeof(float), 0);
         BandGroups GL = G;
         GL.gs = L.gs;
-        if (B.w <= 8) BAND_F32_LAUNCH(ctx, start_launch, L, band_norm_f32_kernel, 8, GL, D, (float2*)B.D2.ptr);
-        else BAND_F32_LAUNCH(ctx, start_launch, L, band_norm_f32_kernel, kBW, GL, D, (float2*)B.D2.ptr);
+        const BandDamping damp(lambda);
+        if (B.w <= 8) BAND_F32_LAUNCH(ctx, start_launch, L, band_norm_f32_kernel, 8, GL, damp, D, (float2*)B.E2.ptr);
+        else BAND_F32_LAUNCH(ctx, start_launch, L, band_norm_f32_kernel, kBW, GL, damp, D, (float2*)B.E2.ptr);
       } else {
         band_colnorm_kernel<<<nblk(B.total_cols, 256), 256, 0, st>>>(nullptr, (const double*)J, dcols, dc0, dr0,
                                                                     B.num_inst, B.rows_per_col, B.w, D);
@@ -1023,8 +1041,8 @@ static qrkit_status banded_run(qrkit_ctx* ctx, const void* J, const void* b, con
         const int64_t* blk0;
         void* gp;
         cr_padded(*B.cr, &blk0, &gp);
-        BAND_F32_LAUNCH(ctx, chain_launch, L, band_grad_f32_kernel, 8, GL, (const float*)b, (const float*)p, (const float2*)B.D2.ptr,
-                        (float)lambda, (float)(lambda - (double)(float)lambda), blk0, (float*)gp);
+        BAND_F32_LAUNCH(ctx, chain_launch, L, band_grad_f32_kernel, 8, GL, (const float*)b, (const float*)p,
+                        (const float2*)B.E2.ptr, lambda > 0.0, blk0, (float*)gp);
       } else {
         band_resid_kernel<T><<<nblk(B.total_rows, 256), 256, 0, st>>>(
             (const T*)J, (const T*)b, (const T*)p, dcols, dc0, dr0, B.num_inst, B.total_rows, B.rows_per_col, B.w,
@@ -1167,7 +1185,7 @@ qrkit_status banded_get_factor(qrkit_ctx* ctx, void* Rw_out, void* c_out, double
 void release_band(Band& B) {
   release(B.d_cols); release(B.d_col0); release(B.d_row0); release(B.Rw); release(B.c);
   release(B.d_inst); release(B.d_rows); release(B.d_start);
-  release(B.D); release(B.D2); release(B.res2); release(B.g); release(B.h); release(B.r);
+  release(B.D); release(B.E2); release(B.res2); release(B.g); release(B.h); release(B.r);
   release_cr(B.cr);
   B = Band();
 }

@@ -182,7 +182,7 @@ struct Band {
   bool explicit_starts = false;   // rows carry explicit starts (band_row_start)
   CRPlan* cr = nullptr;
   DevBuf d_cols, d_col0, d_row0, Rw, c, D, res2, g, h, r;
-  DevBuf D2;                      // float plans: D^2 per column as a float pair
+  DevBuf E2;                      // float plans: lambda D^2 per column as a float pair
   DevBuf d_inst, d_rows, d_start;   // explicit starts: 4 x num_inst table, rows, global starts
 };
 
