@@ -18,26 +18,18 @@
 #include "chain.cuh"
 #include "device_util.cuh"
 #include "internal.h"
+#include "sums.cuh"
 
 namespace qrkit {
 namespace {
 
-// Compensated float accumulation (Dot2, Ogita-Rump-Oishi): (sh + sl) += a x.
-__device__ __forceinline__ void dot2(float& sh, float& sl, float a, float x) {
-  const float p = __fmul_rn(a, x);
-  const float pe = __fmaf_rn(a, x, -p);
-  float t, e;
-  dev::two_sum(sh, p, t, e);
-  sh = t;
-  sl = __fadd_rn(sl, __fadd_rn(e, pe));
-}
-
-// (sh + sl) += (bh + bl)
-__device__ __forceinline__ void add_pair(float& sh, float& sl, float bh, float bl) {
-  float t, e;
-  dev::two_sum(sh, bh, t, e);
-  sh = t;
-  sl = __fadd_rn(sl, __fadd_rn(e, bl));
+// A double as a sum of three floats, and back.
+__device__ __forceinline__ dev::Triple triple_of(double v) {
+  dev::Triple s;
+  s.h = (float)v;
+  s.l = (float)(v - (double)s.h);
+  s.m = (float)(v - (double)s.h - (double)s.l);
+  return s;
 }
 
 template <int V>
@@ -227,23 +219,22 @@ __global__ void __launch_bounds__(kWarpBackThreads) block_backsub_warp_kernel(Co
     if (k < m && lane == k) x[c0 + k] = accumulate ? x[c0 + k] + y[k] : y[k];
 }
 
-// ---- refinement of float plans: g = J^T (b - J p - S p_S) - lambda D^2 p with the residual and
-// its sums as unevaluated float pairs (Dot2) ----
+// ---- refinement of float plans: g = J^T (b - J p - S p_S) - lambda D^2 p with the residual and its sums as sums of
+// three floats, no less accurate than in double.  A product that overflows (right-hand sides have any scale) leaves a
+// sum that is not finite: that one is formed again in double. ----
 
-// 1. rows: b - S p_S as a pair per row.  A CTA takes 32 V rows; its 8 warps split the columns.
+// 1. rows: b - S p_S, three floats per row.  A CTA takes 32 V rows; its 8 warps split the columns.
 constexpr int kRowWarps = 8;
 
 template <int V>
 __global__ void __launch_bounds__(32 * kRowWarps) dense_rows_kernel(const float* S, int64_t rows, int s, const float* b,
-                                                                    const float* pS, float* rh, float* rl) {
+                                                                    const float* pS, float* rh, float* rl, float* rm) {
   dev::chain_wait();
-  __shared__ float sh_s[kRowWarps][32 * V], sl_s[kRowWarps][32 * V];
+  __shared__ float part[3][kRowWarps][32 * V];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t row0 = (int64_t)blockIdx.x * (32 * V);
   const int64_t row = row0 + lane * V;
-  float sh[V], sl[V];
-#pragma unroll
-  for (int q = 0; q < V; ++q) sh[q] = sl[q] = 0.f;
+  dev::Triple sum[V];
   if (row < rows) {   // V divides rows
     const float* src = S + row;
     int c = warp;
@@ -255,7 +246,7 @@ __global__ void __launch_bounds__(32 * kRowWarps) dense_rows_kernel(const float*
       for (int u = 0; u < 4; ++u) {
         const float p = -pS[c + u * kRowWarps];
 #pragma unroll
-        for (int q = 0; q < V; ++q) dot2(sh[q], sl[q], a[u].v[q], p);
+        for (int q = 0; q < V; ++q) sum[q].fma(a[u].v[q], p);
       }
     }
     for (; c < s; c += kRowWarps) {
@@ -263,28 +254,36 @@ __global__ void __launch_bounds__(32 * kRowWarps) dense_rows_kernel(const float*
       a.load(src + (int64_t)c * rows);
       const float p = -pS[c];
 #pragma unroll
-      for (int q = 0; q < V; ++q) dot2(sh[q], sl[q], a.v[q], p);
+      for (int q = 0; q < V; ++q) sum[q].fma(a.v[q], p);
     }
   }
 #pragma unroll
   for (int q = 0; q < V; ++q) {
-    sh_s[warp][lane * V + q] = sh[q];
-    sl_s[warp][lane * V + q] = sl[q];
+    part[0][warp][lane * V + q] = sum[q].h;
+    part[1][warp][lane * V + q] = sum[q].l;
+    part[2][warp][lane * V + q] = sum[q].m;
   }
   __syncthreads();
   const int t = threadIdx.x;
   if (t < 32 * V && row0 + t < rows) {
-    float h = b[row0 + t], l = 0.f;
+    dev::Triple r;
+    r.h = b[row0 + t];
 #pragma unroll
-    for (int w = 0; w < kRowWarps; ++w) add_pair(h, l, sh_s[w][t], sl_s[w][t]);
-    rh[row0 + t] = h;
-    rl[row0 + t] = l;
+    for (int w = 0; w < kRowWarps; ++w) r.add(part[0][w][t], part[1][w][t], part[2][w][t]);
+    if (!isfinite(r.h + r.l)) {
+      double v = (double)b[row0 + t];
+      for (int c = 0; c < s; ++c) v -= (double)S[(int64_t)c * rows + row0 + t] * (double)pS[c];
+      r = triple_of(v);
+    }
+    rh[row0 + t] = r.h;
+    rl[row0 + t] = r.l;
+    rm[row0 + t] = r.m;
   }
 }
 
 // 2. blocks (one thread each): r -= J p, g_B = J^T r - lambda D^2 p, h_B = R_i^{-T} g_B.
 __global__ void __launch_bounds__(128) dense_blocks_kernel(ComposedView<float> V, FactorOut<float> O, const float* p,
-                                                           double lam, float* rh, float* rl, float* h) {
+                                                           double lam, float* rh, float* rl, float* rm, float* h) {
   dev::chain_wait();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= V.K) return;
@@ -293,37 +292,47 @@ __global__ void __launch_bounds__(128) dense_blocks_kernel(ComposedView<float> V
   const int64_t c0 = V.col_off[i], r0 = V.row_off[i];
   const float* J = V.J + V.val_off[i];
   const float* F = O.Fa + O.aug_off[i];
-  float ph[16], pl[16], pj[8], hv[8];
+  float pj[8], hv[8];
+  dev::Triple res[16];
 #pragma unroll
   for (int j = 0; j < 8; ++j) pj[j] = j < m ? p[c0 + j] : 0.f;
 #pragma unroll
   for (int r = 0; r < 16; ++r) {
-    ph[r] = pl[r] = 0.f;
     if (r < n) {
-      float sh = rh[r0 + r], sl = rl[r0 + r];
+      const float sh = rh[r0 + r], sl = rl[r0 + r], sm = rm[r0 + r];
+      res[r].h = sh;
+      res[r].l = sl;
+      res[r].m = sm;
 #pragma unroll
       for (int j = 0; j < 8; ++j)
-        if (j < m) dot2(sh, sl, -J[j * n + r], pj[j]);
-      ph[r] = sh;
-      pl[r] = sl;
-      rh[r0 + r] = sh;
-      rl[r0 + r] = sl;
+        if (j < m) res[r].fma(-J[j * n + r], pj[j]);
+      if (!isfinite(res[r].h + res[r].l)) {
+        double v = (double)sh + ((double)sl + (double)sm);
+        for (int j = 0; j < m; ++j) v -= (double)J[j * n + r] * (double)p[c0 + j];
+        res[r] = triple_of(v);
+      }
+      rh[r0 + r] = res[r].h;
+      rl[r0 + r] = res[r].l;
+      rm[r0 + r] = res[r].m;
     }
   }
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     hv[k] = 0.f;
     if (k < m) {
-      float ah = 0.f, al = 0.f;
+      dev::Triple g;
 #pragma unroll
       for (int r = 0; r < 16; ++r)
-        if (r < n) {
-          const float a = J[k * n + r];
-          dot2(ah, al, a, ph[r]);
-          al = __fmaf_rn(a, pl[r], al);
-        }
+        if (r < n) g.fma(J[k * n + r], res[r].h, res[r].l, res[r].m);
+      double gv = g.value();
+      if (!isfinite(gv)) {
+        gv = 0.0;
+#pragma unroll
+        for (int r = 0; r < 16; ++r)
+          if (r < n) gv += (double)J[k * n + r] * res[r].value();
+      }
       const double d = O.D[c0 + k];
-      float v = (float)(((double)ah + (double)al) - lam * d * d * (double)pj[k]);
+      float v = (float)(gv - lam * d * d * (double)pj[k]);
 #pragma unroll
       for (int j = 0; j < 8; ++j)
         if (j < k) v -= F[k * na + j] * hv[j];
@@ -334,42 +343,45 @@ __global__ void __launch_bounds__(128) dense_blocks_kernel(ComposedView<float> V
 }
 
 // 3. shared columns, first part: S^T r per chunk of kSumRows rows.  A warp takes a column at a
-// time; the chunk's r pairs are in shared memory.
+// time; the chunk's r is in shared memory.
 constexpr int kSumRows = 2048;
 constexpr int kSumWarps = 8;
 constexpr int kSumCols = 2;    // columns per warp
 
 template <int V>
 __global__ void __launch_bounds__(32 * kSumWarps) dense_cols_kernel(const float* S, int64_t rows, int s, const float* rh,
-                                                                    const float* rl, double* part) {
+                                                                    const float* rl, const float* rm, double* part) {
   dev::chain_wait();
-  __shared__ __align__(16) float rh_s[kSumRows], rl_s[kSumRows];
+  __shared__ __align__(16) float rh_s[kSumRows], rl_s[kSumRows], rm_s[kSumRows];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t row0 = (int64_t)blockIdx.x * kSumRows;
   const int nr = (int)(rows - row0 < kSumRows ? rows - row0 : kSumRows);
   for (int e = threadIdx.x; e < nr; e += 32 * kSumWarps) {
     rh_s[e] = rh[row0 + e];
     rl_s[e] = rl[row0 + e];
+    rm_s[e] = rm[row0 + e];
   }
   __syncthreads();
   for (int u = 0; u < kSumCols; ++u) {
     const int c = ((int)blockIdx.y * kSumCols + u) * kSumWarps + warp;
     if (c >= s) return;
     const float* src = S + (int64_t)c * rows + row0;
-    float sh = 0.f, sl = 0.f;
+    dev::Triple sum;
 #pragma unroll 4
     for (int e = lane * V; e < nr; e += 32 * V) {   // V divides nr
-      Vec<V> a, h, l;
+      Vec<V> a, h, l, m;
       a.load(src + e);
       h.load(rh_s + e);
       l.load(rl_s + e);
+      m.load(rm_s + e);
 #pragma unroll
-      for (int q = 0; q < V; ++q) {
-        dot2(sh, sl, a.v[q], h.v[q]);
-        sl = __fmaf_rn(a.v[q], l.v[q], sl);
-      }
+      for (int q = 0; q < V; ++q) sum.fma(a.v[q], h.v[q], l.v[q], m.v[q]);
     }
-    double t = (double)sh + (double)sl;
+    double t = sum.value();
+    if (__any_sync(0xffffffffu, !isfinite(t))) {
+      t = 0.0;
+      for (int e = lane; e < nr; e += 32) t += (double)src[e] * ((double)rh_s[e] + ((double)rl_s[e] + (double)rm_s[e]));
+    }
 #pragma unroll
     for (int d = 16; d >= 1; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
     if (lane == 0) part[(int64_t)blockIdx.x * s + c] = t;
@@ -397,19 +409,24 @@ __global__ void __launch_bounds__(kR12Threads) dense_r12_kernel(const float* R12
   for (int e = threadIdx.x; e < nj; e += kR12Threads) h_s[e] = h[j0 + e];
   __syncthreads();
   if (g < groups) {
-    float sh[V], sl[V];
-#pragma unroll
-    for (int q = 0; q < V; ++q) sh[q] = sl[q] = 0.f;
+    dev::Triple sum[V];
     const float* src = R12 + j0 * s + (int64_t)(u0 + u) * V;
 #pragma unroll 4
     for (int j = g; j < nj; j += groups) {
       Vec<V> a;
       a.load(src + (int64_t)j * s);
 #pragma unroll
-      for (int q = 0; q < V; ++q) dot2(sh[q], sl[q], a.v[q], h_s[j]);
+      for (int q = 0; q < V; ++q) sum[q].fma(a.v[q], h_s[j]);
     }
 #pragma unroll
-    for (int q = 0; q < V; ++q) sum_s[(g * nu + u) * V + q] = (double)sh[q] + (double)sl[q];
+    for (int q = 0; q < V; ++q) {
+      double t = sum[q].value();
+      if (!isfinite(t)) {
+        t = 0.0;
+        for (int j = g; j < nj; j += groups) t += (double)src[(int64_t)j * s + q] * (double)h_s[j];
+      }
+      sum_s[(g * nu + u) * V + q] = t;
+    }
   }
   __syncthreads();
   for (int c = threadIdx.x; c < nu * V; c += kR12Threads) {
@@ -480,7 +497,7 @@ template qrkit_status dense_block_backsub<double>(qrkit_ctx*, bool, const Compos
 
 size_t dense_refine_bytes(int64_t rows, int64_t nb, int s) {
   const int64_t chunks = (rows + kSumRows - 1) / kSumRows + (nb + kR12Rows - 1) / kR12Rows;
-  return (size_t)chunks * s * sizeof(double) + 2 * (size_t)((rows + 3) & ~int64_t(3)) * sizeof(float);
+  return (size_t)chunks * s * sizeof(double) + 3 * (size_t)((rows + 3) & ~int64_t(3)) * sizeof(float);
 }
 
 qrkit_status dense_refine_gradient(qrkit_ctx* ctx, const ComposedView<float>& V, const FactorOut<float>& O,
@@ -492,20 +509,21 @@ qrkit_status dense_refine_gradient(qrkit_ctx* ctx, const ComposedView<float>& V,
   double* part_r = part_s + ns * s;
   float* rh = (float*)(part_r + nr * s);
   float* rl = rh + ((V.rows + 3) & ~int64_t(3));
+  float* rm = rl + ((V.rows + 3) & ~int64_t(3));
   // 16-byte loads where every column of the caller's S is 16-byte aligned
   const bool v4 = (V.rows & 3) == 0 && (reinterpret_cast<uintptr_t>(V.S) & 15) == 0;
   if (v4)
     DS_LAUNCH(ctx, chain_launch(st, nblk(V.rows, 128), 32 * kRowWarps, 0, dense_rows_kernel<4>, V.S, V.rows, s, b,
-                                p + V.nb, rh, rl));
+                                p + V.nb, rh, rl, rm));
   else
     DS_LAUNCH(ctx, chain_launch(st, nblk(V.rows, 32), 32 * kRowWarps, 0, dense_rows_kernel<1>, V.S, V.rows, s, b,
-                                p + V.nb, rh, rl));
-  DS_LAUNCH(ctx, chain_launch(st, nblk(V.K, 128), 128, 0, dense_blocks_kernel, V, O, p, lam, rh, rl, h));
+                                p + V.nb, rh, rl, rm));
+  DS_LAUNCH(ctx, chain_launch(st, nblk(V.K, 128), 128, 0, dense_blocks_kernel, V, O, p, lam, rh, rl, rm, h));
   const dim3 gs((unsigned)ns, nblk(s, kSumWarps * kSumCols));
   if (v4)
-    DS_LAUNCH(ctx, chain_launch(st, gs, 32 * kSumWarps, 0, dense_cols_kernel<4>, V.S, V.rows, s, rh, rl, part_s));
+    DS_LAUNCH(ctx, chain_launch(st, gs, 32 * kSumWarps, 0, dense_cols_kernel<4>, V.S, V.rows, s, rh, rl, rm, part_s));
   else
-    DS_LAUNCH(ctx, chain_launch(st, gs, 32 * kSumWarps, 0, dense_cols_kernel<1>, V.S, V.rows, s, rh, rl, part_s));
+    DS_LAUNCH(ctx, chain_launch(st, gs, 32 * kSumWarps, 0, dense_cols_kernel<1>, V.S, V.rows, s, rh, rl, rm, part_s));
   if ((s & 3) == 0)
     DS_LAUNCH(ctx, chain_launch(st, dim3((unsigned)nr, nblk(s / 4, kR12Threads)), kR12Threads, 0, dense_r12_kernel<4>,
                                 O.R12, V.nb, s, h, part_r));
