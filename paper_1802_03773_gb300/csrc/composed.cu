@@ -1542,7 +1542,8 @@ qrkit_status composed_layout(qrkit_ctx* ctx, size_t elem) {
       if ((rc = ensure(ctx, C.colptr, (size_t)(s + 1) * sizeof(int32_t), "block sort")) != QRKIT_OK) return rc;
       if ((rc = ensure(ctx, C.bpos, (size_t)P.K * sizeof(int32_t), "block sort")) != QRKIT_OK) return rc;
       if ((rc = ensure(ctx, C.bord, (size_t)P.K * sizeof(int32_t), "block sort")) != QRKIT_OK) return rc;
-      if ((rc = ensure(ctx, C.wres, (size_t)2 * P.rows * elem, "refinement residual")) != QRKIT_OK) return rc;
+      const size_t rv = (size_t)window_residual_values(P.max_n, P.max_m, elem);
+      if ((rc = ensure(ctx, C.wres, rv * P.rows * elem, "refinement residual")) != QRKIT_OK) return rc;
     }
     if ((rc = ensure(ctx, C.RwS, (size_t)s * w * elem, "reduced R")) != QRKIT_OK) return rc;
     if ((rc = ensure(ctx, C.cS, (size_t)s * elem, "reduced c")) != QRKIT_OK) return rc;

@@ -168,11 +168,16 @@ struct WindowSums {
   const int32_t* bord;    // block at each sorted position
   const int32_t* start;
   const T* S;
-  const T* R12;           // gradient: R12, the residual pairs (2 per row) and h_B
+  const T* R12;           // gradient: R12, the residuals (window_residual_values per row) and h_B
   const T* r;
   const T* h;
   double* out;            // s sums, added to
 };
+
+// Values that a row's residual takes: a double, or two floats for blocks up to 6 x 2, three for larger ones.
+inline int window_residual_values(int n, int m, size_t elem) {
+  return elem == sizeof(double) ? 1 : (m <= 2 && n <= 6 ? 2 : 3);
+}
 
 // Device state of a batch of banded instances (Sec. 4.4).
 struct Band {
@@ -221,7 +226,7 @@ struct Composed {
   bool bins = false;
   BlockSortTables bsort{};
   int64_t bsort_hist = 0;
-  DevBuf bs_tab, bs_colseg, colptr, bpos, bord, wres;   // colptr: s + 1 first sorted blocks; wres: residual pairs
+  DevBuf bs_tab, bs_colseg, colptr, bpos, bord, wres;   // colptr: s + 1 first sorted blocks; wres: residuals
   DevBuf seg_inst;                 // 4 x nseg: cols, col0, row0, rows of the segments' banded solves
   CRPlan* cr = nullptr;            // parallel banded QR of the segments (window <= 8)
   // normal-equations (Cholesky) comparison path

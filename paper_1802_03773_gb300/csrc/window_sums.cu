@@ -24,39 +24,98 @@ constexpr int kLanes = 8;     // lanes of a run: the widest window
 constexpr int kRun = 32;      // sorted blocks of a run
 constexpr int kThreads = 256;
 
-// A sum: an unevaluated float pair (Dot2) for float data, a double for double.
-template <typename T>
-struct Sum {
-  T h = T(0), l = T(0);
-  __device__ __forceinline__ void fma(T a, T x) {
-    if constexpr (sizeof(T) == 4) {
-      const T p = __fmul_rn(a, x), pe = __fmaf_rn(a, x, -p);
-      T t, e;
-      dev::two_sum(h, p, t, e);
-      h = t;
-      l = __fadd_rn(l, __fadd_rn(e, pe));
+// Sums over a block's rows: float pairs for blocks up to 6 x 2 of floats, three floats for larger ones, doubles for doubles;
+// a residual is kept as such a sum.
+struct DoubleSum {
+  double s = 0.0;
+  __device__ __forceinline__ void fma(double a, double x) { s += a * x; }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <typename T, int NR>
+struct BlockSum;
+template <int NR>
+struct BlockSum<double, NR> {
+  static constexpr int kValues = 1;
+  DoubleSum s;
+  __device__ __forceinline__ void start(double b) { s.s = b; }
+  __device__ __forceinline__ void fma(double a, double x) { s.fma(a, x); }
+  __device__ __forceinline__ void fma(double a, const double (&x)[1]) { s.fma(a, x[0]); }
+  __device__ __forceinline__ void get(double (&v)[1]) const { v[0] = s.s; }
+  __device__ __forceinline__ double value() const { return s.s; }
+};
+template <int NR>
+struct BlockSum<float, NR> {
+  static constexpr int kValues = NR > 6 ? 3 : 2;
+  dev::Triple s;   // of a pair, two of the three
+  __device__ __forceinline__ void start(float b) { s.h = b; }
+  __device__ __forceinline__ void fma(float a, float x) {
+    if constexpr (kValues == 3) {
+      s.fma(a, x);
     } else {
-      h += a * x;
+      dev::Pair p;
+      p.h = s.h;
+      p.l = s.l;
+      p.fma(a, x);
+      s.h = p.h;
+      s.l = p.l;
     }
   }
-  __device__ __forceinline__ void fma(T a, T xh, T xl) {   // a (xh + xl)
-    fma(a, xh);
-    if constexpr (sizeof(T) == 4) l = __fmaf_rn(a, xl, l);
+  __device__ __forceinline__ void fma(float a, const float (&x)[kValues]) {
+    if constexpr (kValues == 3) {
+      s.fma(a, x[0], x[1], x[2]);
+    } else {
+      fma(a, x[0]);
+      s.l = __fmaf_rn(a, x[1], s.l);
+    }
   }
-  __device__ __forceinline__ double value() const { return (double)h + (double)l; }
+  __device__ __forceinline__ void get(float (&v)[kValues]) const {
+    v[0] = s.h;
+    v[1] = s.l;
+    if constexpr (kValues == 3) v[2] = s.m;
+  }
+  __device__ __forceinline__ double value() const { return s.value(); }
+  __device__ __forceinline__ void set(double v) {
+    s.h = (float)v;
+    s.l = (float)(v - (double)s.h);
+    s.m = (float)(v - (double)s.h - (double)s.l);
+  }
 };
 
-// What a lane of a run adds up: products (kGrad), or squares.
+// What a lane of a run adds up over its blocks: products (kGrad), or squares; no less accurate than in double.
 template <typename T, bool kGrad>
 struct RunSum {
-  Sum<T> s;
+  DoubleSum s;
+  __device__ __forceinline__ void fma(T a, T x) { s.fma(a, x); }
+  __device__ __forceinline__ void fma(T a, const T (&x)[1]) { s.fma(a, x[0]); }
   template <int N>
   __device__ __forceinline__ void squares(const T (&x)[N]) {
 #pragma unroll
     for (int r = 0; r < N; ++r) s.fma(x[r], x[r]);
   }
-  __device__ __forceinline__ void fma(T a, T x) { s.fma(a, x); }
-  __device__ __forceinline__ void fma(T a, T xh, T xl) { s.fma(a, xh, xl); }
+  __device__ __forceinline__ double value() const { return s.value(); }
+};
+template <>
+struct RunSum<float, true> {
+  dev::Triple s;
+  __device__ __forceinline__ void fma(float a, float x) { s.fma(a, x); }
+  __device__ __forceinline__ void fma(float a, const float (&x)[3]) { s.fma(a, x[0], x[1], x[2]); }
+  // a small block's products (residuals of two floats; zeros past its rows and columns) as a pair of its own, then added
+  template <int NR, int MM>
+  __device__ __forceinline__ void block(const float (&a)[NR], const float (&x)[NR][2], const float (&b)[MM],
+                                        const float (&y)[MM]) {
+    dev::Pair p;
+    p.h = __fmul_rn(a[0], x[0][0]);
+    p.l = __fmaf_rn(a[0], x[0][1], __fmaf_rn(a[0], x[0][0], -p.h));
+#pragma unroll
+    for (int r = 1; r < NR; ++r) {
+      const float q = __fmul_rn(a[r], x[r][0]);
+      p.add(q, __fmaf_rn(a[r], x[r][1], __fmaf_rn(a[r], x[r][0], -q)));
+    }
+#pragma unroll
+    for (int k = 0; k < MM; ++k) p.fma(b[k], y[k]);
+    s.add(p.h);
+    s.low(p.l);
+  }
   __device__ __forceinline__ double value() const { return s.value(); }
 };
 template <>
@@ -78,27 +137,45 @@ __global__ void __launch_bounds__(kThreads) window_sums_kernel(WindowSums<T> A) 
   const int64_t p0 = run * kRun, p1 = p0 + kRun < A.K ? p0 + kRun : A.K;
   if (p0 >= A.K || t >= A.w) return;
   const int n = A.n, m = A.m, w = A.w;
+  constexpr int RV = BlockSum<T, NR>::kValues;
   RunSum<T, kGrad> acc;
-  int64_t cur = -1;
-  auto flush = [&]() {
+  int64_t cur = -1, first = p0;   // start of the blocks added up, and the first of them
+  auto flush = [&](int64_t end) {
     if (cur >= 0 && cur + t < A.s) {
-      const double v = acc.value();
+      double v = acc.value();
+      if (kGrad && sizeof(T) == 4 && !isfinite(v)) {   // a product left the float range: these blocks again in double
+        v = 0.0;
+        for (int64_t q = first; q < end; ++q) {
+          const int64_t i = A.bord[q];
+          for (int r = 0; r < n; ++r) {
+            double x = 0.0;
+            for (int e = RV - 1; e >= 0; --e) x += (double)A.r[RV * (i * n + r) + e];
+            v += (double)A.S[(i * w + t) * n + r] * x;
+          }
+          for (int k = 0; k < m; ++k) v -= (double)A.R12[(i * m + k) * w + t] * (double)A.h[i * m + k];
+        }
+      }
       if (v != 0.0) atomicAdd(A.out + cur + t, v);
     }
     acc = RunSum<T, kGrad>();
+    first = end;
   };
   constexpr int U = NR * MM <= 2 ? 4 : 1;   // blocks whose loads are in flight together
   for (int64_t q0 = p0; q0 < p1; q0 += U) {
     int64_t i[U];
     int32_t st[U];
-    T sv[U][NR], rh[U][NR], rl[U][NR], rv[U][MM], hv[U][MM];
+    T sv[U][NR], res[U][NR][RV], rv[U][MM], hv[U][MM];
 #pragma unroll
     for (int u = 0; u < U; ++u) i[u] = q0 + u < p1 ? A.bord[q0 + u] : -1;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       st[u] = 0;
 #pragma unroll
-      for (int r = 0; r < NR; ++r) sv[u][r] = rh[u][r] = rl[u][r] = T(0);
+      for (int r = 0; r < NR; ++r) {
+        sv[u][r] = T(0);
+#pragma unroll
+        for (int e = 0; e < RV; ++e) res[u][r][e] = T(0);
+      }
 #pragma unroll
       for (int k = 0; k < MM; ++k) rv[u][k] = hv[u][k] = T(0);
       if (i[u] < 0) continue;
@@ -111,8 +188,8 @@ __global__ void __launch_bounds__(kThreads) window_sums_kernel(WindowSums<T> A) 
 #pragma unroll
         for (int r = 0; r < NR; ++r)
           if (r < n) {
-            rh[u][r] = A.r[2 * (i[u] * n + r)];
-            rl[u][r] = A.r[2 * (i[u] * n + r) + 1];
+#pragma unroll
+            for (int e = 0; e < RV; ++e) res[u][r][e] = A.r[RV * (i[u] * n + r) + e];
           }
 #pragma unroll
         for (int k = 0; k < MM; ++k)
@@ -126,24 +203,26 @@ __global__ void __launch_bounds__(kThreads) window_sums_kernel(WindowSums<T> A) 
     for (int u = 0; u < U; ++u) {
       if (i[u] < 0) continue;
       if (st[u] != cur) {
-        flush();
+        flush(q0 + u);
         cur = st[u];
       }
       if constexpr (!kGrad) acc.squares(sv[u]);   // zeros past row n
-      if constexpr (kGrad) {
+      if constexpr (kGrad && RV == 2) {
+        acc.block(sv[u], res[u], rv[u], hv[u]);
+      } else if constexpr (kGrad) {
 #pragma unroll
         for (int r = 0; r < NR; ++r)
-          if (r < n) acc.fma(sv[u][r], rh[u][r], rl[u][r]);
+          if (r < n) acc.fma(sv[u][r], res[u][r]);
 #pragma unroll
         for (int k = 0; k < MM; ++k)
           if (k < m) acc.fma(rv[u][k], hv[u][k]);
       }
     }
   }
-  flush();
+  flush(p1);
 }
 
-// A block per thread: r = b - J p - S p_S as pairs, g_B = J^T r - lambda D^2 p, h_B = R_i^{-T} g_B.
+// A block per thread: r = b - J p - S p_S, g_B = J^T r - lambda D^2 p, h_B = R_i^{-T} g_B.
 template <typename T, int NR, int MM>
 __global__ void __launch_bounds__(128) window_blocks_kernel(ComposedView<T> V, FactorOut<T> O, const T* b, const T* p,
                                                             double lam, int n, int m, T* r, T* h) {
@@ -161,13 +240,15 @@ __global__ void __launch_bounds__(128) window_blocks_kernel(ComposedView<T> V, F
   for (int j = 0; j < MM; ++j) pj[j] = j < m ? -p[c0 + j] : T(0);
 #pragma unroll
   for (int t = 0; t < kLanes; ++t) ps[t] = t < w && st + t < V.s ? -p[V.nb + st + t] : T(0);
-  Sum<T> res[NR];
+  using Res = BlockSum<T, NR>;
+  constexpr int RV = Res::kValues;
+  Res res[NR];
   bool done = false;
   if constexpr (sizeof(T) == 4 && NR == 2) {
     if (w == 8 && n == 2 && (reinterpret_cast<uintptr_t>(V.S) & 15) == 0) {   // the window by 16-byte loads
       const float4* s4 = reinterpret_cast<const float4*>(S);
 #pragma unroll
-      for (int q = 0; q < 2; ++q) res[q].h = b[r0 + q];
+      for (int q = 0; q < 2; ++q) res[q].start(b[r0 + q]);
 #pragma unroll
       for (int q = 0; q < 2; ++q) res[q].fma(J[q], pj[0]);
 #pragma unroll
@@ -185,7 +266,7 @@ __global__ void __launch_bounds__(128) window_blocks_kernel(ComposedView<T> V, F
 #pragma unroll
     for (int q = 0; q < NR; ++q) {
       if (q < n) {
-        res[q].h = b[r0 + q];
+        res[q].start(b[r0 + q]);
 #pragma unroll
         for (int j = 0; j < MM; ++j)
           if (j < m) res[q].fma(J[j * n + q], pj[j]);
@@ -198,20 +279,44 @@ __global__ void __launch_bounds__(128) window_blocks_kernel(ComposedView<T> V, F
 #pragma unroll
   for (int q = 0; q < NR; ++q)
     if (q < n) {
-      r[2 * (r0 + q)] = res[q].h;
-      r[2 * (r0 + q) + 1] = res[q].l;
+      if constexpr (RV == 3) {
+        if (!isfinite(res[q].s.h + res[q].s.l)) {   // a product left the float range
+          double v = (double)b[r0 + q];
+          for (int j = 0; j < m; ++j) v -= (double)J[j * n + q] * (double)p[c0 + j];
+          for (int t = 0; t < w; ++t)
+            if (st + t < V.s) v -= (double)S[t * n + q] * (double)p[V.nb + st + t];
+          res[q].set(v);
+        }
+      }
+      T v[RV];
+      res[q].get(v);
+#pragma unroll
+      for (int e = 0; e < RV; ++e) r[RV * (r0 + q) + e] = v[e];
     }
   T hv[MM];
 #pragma unroll
   for (int k = 0; k < MM; ++k) {
     hv[k] = T(0);
     if (k < m) {
-      Sum<T> g;
+      Res g;
 #pragma unroll
       for (int q = 0; q < NR; ++q)
-        if (q < n) g.fma(J[k * n + q], res[q].h, res[q].l);
+        if (q < n) {
+          T x[RV];
+          res[q].get(x);
+          g.fma(J[k * n + q], x);
+        }
+      double gv = g.value();
+      if constexpr (RV == 3) {
+        if (!isfinite(gv)) {
+          gv = 0.0;
+#pragma unroll
+          for (int q = 0; q < NR; ++q)
+            if (q < n) gv += (double)J[k * n + q] * res[q].value();
+        }
+      }
       const double d = O.D[c0 + k];
-      T v = (T)(g.value() + lam * d * d * (double)pj[k]);
+      T v = (T)(gv + lam * d * d * (double)pj[k]);
 #pragma unroll
       for (int j = 0; j < MM; ++j)
         if (j < k) v -= F[k * na + j] * hv[j];

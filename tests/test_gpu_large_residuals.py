@@ -47,6 +47,7 @@ def refined(torch, n, m, K, s, w, J, S, start, b, lam, steps):
 
 def solution(A, b, lam):
     D = np.linalg.norm(A, axis=0)
+    D[D == 0] = 1.0   # an untouched shared column
     return np.linalg.solve(A.T @ A + lam * np.diag(D * D), A.T @ b)
 
 
