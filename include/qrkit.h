@@ -407,8 +407,9 @@ qrkit_status qrkit_get_row_order(qrkit_ctx* ctx, int64_t* order);
  * solve, "tasks <supertile> <warps per CTA> [<key-major 0/1>]" (shape-uniform warp tasks, the
  * default; see qrkit_task_layout) or
  * "budget <blocks> <values> <rows> <cols> <padded>" (tiles of consecutive blocks); parallel
- * banded plans: the compression strategy "compress <0/1> <splits>" (1: a thread per
- * column block; 0: 1-64 threads per block, their triangles merged).  cache_path (HOST string, may be NULL): a text file with one line per
+ * banded plans: the compression strategy, "compress auto" (the plan's default: as many threads per column block as
+ * each instance's rows call for) or "compress <0/1> <splits>" (1: a thread per column block; 0: 1-64 threads per
+ * block, their triangles merged).  cache_path (HOST string, may be NULL): a text file with one line per
  * structure key (GPU name, precision, shape signature) and its choice; a key found there is
  * applied without timing, a new choice is appended.  chosen (HOST, may be NULL): receives the
  * choice as text.  Synchronous. */

@@ -1230,30 +1230,33 @@ static qrkit_status cr_split(qrkit_ctx* ctx, CRPlan& C, const std::vector<int>& 
   return cr_partials(ctx, C, C.P2, parts2);
 }
 
-// The current strategy becomes `each` threads per block, or (0) as many as each instance's rows call for; on
-// failure it stays what it was.
+// Threads per block of each instance: about 120,000 in all where that leaves each at least 64 rows (16 steps of four,
+// what a merge pass takes), at most 64 per block.  A batch's instances differ in rows per block (curve fits: 60 to
+// 10,000), and the longest thread bounds the kernel.
+static std::vector<int> default_splits(const CRPlan& C) {
+  std::vector<int> n((size_t)C.num_inst);
+  const double target = std::max(64.0, (double)C.total_rows / 120000.0);
+  for (int64_t k = 0; k < C.num_inst; ++k) {
+    const double per = (double)C.h_rows[k] / (double)(C.h_blk0[k + 1] - C.h_blk0[k]);
+    n[k] = (int)std::min(64.0, std::max(1.0, std::floor(per / target + 0.5)));
+  }
+  return n;
+}
+
+// The current strategy becomes `each` threads per block, or (0) the default; on failure it stays what it was.
 static qrkit_status cr_use_splits(qrkit_ctx* ctx, CRPlan& C, int each) {
   for (const CRSplits* s : C.splits)
     if (s->each == each) {
       C.cur = s;
       return QRKIT_OK;
     }
-  std::vector<int> n((size_t)C.num_inst, each);
-  if (each == 0) {
-    // About 120,000 threads in all where that leaves each at least 64 rows (16 steps of four, what a merge pass
-    // takes), at most 64 per block.  A batch's instances differ in rows per block (curve fits: 60 to 10,000), and
-    // the longest thread bounds the kernel.
-    const double target = std::max(64.0, (double)C.total_rows / 120000.0);
-    for (int64_t k = 0; k < C.num_inst; ++k) {
-      const double per = (double)C.h_rows[k] / (double)(C.h_blk0[k + 1] - C.h_blk0[k]);
-      n[k] = (int)std::min(64.0, std::max(1.0, std::floor(per / target + 0.5)));
-    }
-  }
+  const std::vector<int> n = each ? std::vector<int>((size_t)C.num_inst, each) : default_splits(C);
   CRSplits* s = new CRSplits();
   s->each = each;
   const qrkit_status rc = cr_split(ctx, C, n, *s);
   if (rc != QRKIT_OK) {
     release_splits(s);
+    if (rc == QRKIT_ENOMEM) cudaGetLastError();   // reported; the next launch's check is not to find it
     return rc;
   }
   C.splits.push_back(s);
@@ -1338,9 +1341,43 @@ qrkit_status cr_build(qrkit_ctx* ctx, CRPlan*& out, const std::vector<int64_t>& 
   return QRKIT_OK;
 }
 
-qrkit_status cr_set_strategy(qrkit_ctx* ctx, CRPlan& C, bool thread_rows, int splits) {
-  if (splits < 1 || splits > 64) return fail(ctx, QRKIT_EINVAL, "splits must be in [1, 64]");
-  return cr_use_splits(ctx, C, thread_rows ? 1 : splits);
+qrkit_status cr_set_strategy(qrkit_ctx* ctx, CRPlan& C, int splits) {
+  if (splits < 0 || splits > 64) return fail(ctx, QRKIT_EINVAL, "splits must be in [1, 64]");
+  return cr_use_splits(ctx, C, splits);
+}
+
+std::vector<int> cr_candidates(const CRPlan& C) {
+  const std::vector<int> def = default_splits(C);
+  const bool uniform = std::all_of(def.begin(), def.end(), [&](int n) { return n == def[0]; });
+  double most = 0.0;   // rows per block
+  for (int64_t k = 0; k < C.num_inst; ++k)
+    most = std::max(most, (double)C.h_rows[k] / (double)(C.h_blk0[k + 1] - C.h_blk0[k]));
+  std::vector<int> c{0};
+  for (const int n : {1, 2, 4, 8, 16, 32, 64})
+    if ((n <= 8 || 4 * n <= most) && !(uniform && n == def[0])) c.push_back(n);   // a step is four rows
+  return c;
+}
+
+CRTuning cr_tuning_begin(const CRPlan& C) { return {C.splits.size(), C.outgrown.size(), C.P.ptr, C.P2.ptr}; }
+
+void cr_tuning_end(CRPlan& C, const CRTuning& before) {
+  // the timing has ended, and nothing else has been told of what it built
+  for (size_t q = before.strategies; q < C.splits.size();) {
+    if (C.splits[q] == C.cur) {
+      ++q;
+    } else {
+      release_splits(C.splits[q]);
+      C.splits.erase(C.splits.begin() + (int64_t)q);
+    }
+  }
+  for (size_t q = before.outgrown; q < C.outgrown.size();) {
+    if (C.outgrown[q].ptr == before.P || C.outgrown[q].ptr == before.P2) {
+      ++q;
+    } else {
+      release(C.outgrown[q]);
+      C.outgrown.erase(C.outgrown.begin() + (int64_t)q);
+    }
+  }
 }
 
 template <typename T>

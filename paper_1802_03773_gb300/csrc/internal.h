@@ -251,9 +251,17 @@ qrkit_status cr_build(qrkit_ctx* ctx, CRPlan*& out, const std::vector<int64_t>& 
 // rpc colptr[j] .. rpc colptr[j + 1] - 1.
 qrkit_status cr_solve(qrkit_ctx* ctx, CRPlan& C, const int64_t* starts, const int32_t* colptr, int rpc, int w,
                       const void* J, const void* b, const double* D, double lambda, void* x, double* res2);
-// Compression strategy of the parallel banded QR: one thread per column block, or `splits` threads
-// per block whose triangles are merged (autotuning).
-qrkit_status cr_set_strategy(qrkit_ctx* ctx, CRPlan& C, bool thread_rows, int splits);
+// Compression strategy of the parallel banded QR (autotuning): `splits` threads per block, 1 to 64, whose triangles are
+// merged, or 0: as many as each instance's rows call for, the default.  The candidates to time, without one that is
+// the same as the default; and the strategies that the timing built and dropped: CRTuning holds what was there before.
+qrkit_status cr_set_strategy(qrkit_ctx* ctx, CRPlan& C, int splits);
+std::vector<int> cr_candidates(const CRPlan& C);
+struct CRTuning {
+  size_t strategies = 0, outgrown = 0;
+  void *P = nullptr, *P2 = nullptr;
+};
+CRTuning cr_tuning_begin(const CRPlan& C);
+void cr_tuning_end(CRPlan& C, const CRTuning& before);
 // The padded layout of its right-hand sides: column j of instance k at 8 blk0[k] + j, zero past the instance's
 // last column.
 void cr_padded(const CRPlan& C, const int64_t** blk0, void** g);

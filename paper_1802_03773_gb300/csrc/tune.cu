@@ -4,12 +4,12 @@
 // solve: shape-uniform warp tasks (supertile of consecutive blocks sorted by shape, warps per
 // CTA) or tiles of consecutive blocks (blocks / values / rows / columns / padded working area
 // per tile, which set the tile count, the work per barrier phase and the shared memory per
-// CTA).  Banded plans: the
-// compression strategy of the parallel banded QR (one thread per column block, or a
-// number of threads per block whose triangles are merged).  Every candidate is timed with CUDA events on the context's stream on
-// the caller's inputs (one warm-up, three timed runs), the fastest is kept.  The cache holds
-// one line per structure key: "<key>\t<choice>"; a key already present is applied without
-// timing.
+// CTA).  Banded plans: the compression strategy of the parallel banded QR (the plan's own number of threads per
+// instance's blocks, or one number for all, whose triangles are merged).  Every candidate is timed
+// with CUDA events on the context's stream on the caller's inputs (one warm-up, three timed runs), the fastest
+// is kept.  The cache holds one line per structure key: "<key>\t<choice>"; a key already present is
+// applied without timing.  A key begins with the version of what its choices mean: v2 for blocks, v3 for banded plans,
+// whose "compress 0 n" meant n warps in v2.
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <stdio.h>
@@ -47,7 +47,7 @@ uint64_t shape_hash(const Plan& P) {
 std::string plan_key(const qrkit_ctx* ctx) {
   const Plan& P = ctx->plan;
   std::ostringstream k;
-  k << "v2:" << gpu_name(ctx->device) << ":prec" << ctx->precision << ":";
+  k << (P.s.kind == QRKIT_STRUCT_BANDED ? "v3:" : "v2:") << gpu_name(ctx->device) << ":prec" << ctx->precision << ":";
   if (P.s.kind == QRKIT_STRUCT_BANDED) {
     const Band& B = ctx->band;
     k << "banded:inst" << B.num_inst << ":cols" << B.total_cols << ":rpc" << B.rows_per_col << ":w" << B.w;
@@ -193,6 +193,23 @@ std::vector<BlockChoice> block_candidates(size_t elem) {
   return c;
 }
 
+// Compression choices: "compress auto", or "compress <0/1> <threads per block>" (1: one thread).
+std::string compress_str(int splits) {
+  if (splits == 0) return "compress auto";
+  return splits == 1 ? "compress 1 1" : "compress 0 " + std::to_string(splits);
+}
+
+bool parse_compress(const std::string& v, int& splits) {
+  if (v == "compress auto") {
+    splits = 0;
+    return true;
+  }
+  int tr = 1, sp = 1;
+  if (sscanf(v.c_str(), "compress %d %d", &tr, &sp) != 2) return false;
+  splits = sp < 1 || sp > 64 ? -1 : (tr != 0 ? 1 : sp);   // -1: parsed, refused
+  return true;
+}
+
 template <typename F>
 qrkit_status time_runs(qrkit_ctx* ctx, F run, float& ms) {
   qrkit_status st = run();
@@ -252,29 +269,28 @@ extern "C" qrkit_status qrkit_autotune(qrkit_ctx* ctx, const void* J, const void
   } else {
     Band& B = ctx->band;
     if (!B.parallel || !B.cr) return fail(ctx, QRKIT_EUNSUPPORTED, "qrkit_autotune: parallel banded plans only");
-    int tr = 1, sp = 1;
-    if (cache_lookup(cache_path, key, value) && sscanf(value.c_str(), "compress %d %d", &tr, &sp) == 2) {
-      if ((st = cr_set_strategy(ctx, *B.cr, tr != 0, sp)) != QRKIT_OK) return st;
+    int splits = 0;
+    if (cache_lookup(cache_path, key, value) && parse_compress(value, splits)) {
+      if ((st = cr_set_strategy(ctx, *B.cr, splits)) != QRKIT_OK) return st;
     } else {
+      const CRTuning before = cr_tuning_begin(*B.cr);
       float best = 1e30f;
-      int btr = 1, bsp = 1;
-      for (const int cand_tr : {1, 0})
-        for (const int cand_sp : {1, 2, 4, 8}) {
-          if (cand_tr && cand_sp != 1) continue;
-          if ((st = cr_set_strategy(ctx, *B.cr, cand_tr != 0, cand_sp)) != QRKIT_OK) return st;
-          float ms = 0.f;
+      int chosen_splits = 0;
+      for (const int cand : cr_candidates(*B.cr)) {
+        st = cr_set_strategy(ctx, *B.cr, cand);
+        if (st == QRKIT_ENOMEM) continue;   // no room for its triangles
+        float ms = 0.f;
+        if (st == QRKIT_OK)
           st = time_runs(ctx, [&] { return banded_factor_solve(ctx, J, b, nullptr, 1e-3, p, refine_steps); }, ms);
-          if (st != QRKIT_OK) return st;
-          if (ms < best) {
-            best = ms;
-            btr = cand_tr;
-            bsp = cand_sp;
-          }
+        if (st != QRKIT_OK) return st;
+        if (ms < best) {
+          best = ms;
+          chosen_splits = cand;
         }
-      if ((st = cr_set_strategy(ctx, *B.cr, btr != 0, bsp)) != QRKIT_OK) return st;
-      std::ostringstream v;
-      v << "compress " << btr << " " << bsp;
-      value = v.str();
+      }
+      if ((st = cr_set_strategy(ctx, *B.cr, chosen_splits)) != QRKIT_OK) return st;
+      cr_tuning_end(*B.cr, before);
+      value = compress_str(chosen_splits);
       cache_store(cache_path, key, value);
     }
     ctx->band_factored = false;
@@ -302,10 +318,9 @@ extern "C" qrkit_status qrkit_apply_tuning(qrkit_ctx* ctx, const char* choice) {
   }
   Band& B = ctx->band;
   if (!B.parallel || !B.cr) return fail(ctx, QRKIT_EUNSUPPORTED, "qrkit_apply_tuning: parallel banded plans only");
-  int tr = 1, sp = 1;
-  if (sscanf(v.c_str(), "compress %d %d", &tr, &sp) != 2)
-    return fail(ctx, QRKIT_EINVAL, "cannot parse compression strategy '" + v + "'");
-  const qrkit_status st = cr_set_strategy(ctx, *B.cr, tr != 0, sp);
+  int splits = 0;
+  if (!parse_compress(v, splits)) return fail(ctx, QRKIT_EINVAL, "cannot parse compression strategy '" + v + "'");
+  const qrkit_status st = cr_set_strategy(ctx, *B.cr, splits);
   ctx->band_factored = false;
   return st;
 }
