@@ -214,6 +214,7 @@ __global__ void __launch_bounds__(kWarpBackThreads) block_backsub_warp_kernel(Co
       y[k] = v / F[k * na + k];
     }
   }
+  __syncwarp();   // x may be rhs: every lane has read it
 #pragma unroll
   for (int k = 0; k < 8; ++k)
     if (k < m && lane == k) x[c0 + k] = accumulate ? x[c0 + k] + y[k] : y[k];
