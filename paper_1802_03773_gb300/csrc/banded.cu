@@ -26,6 +26,7 @@
 #include "device_util.cuh"
 #include "f32x2.cuh"
 #include "internal.h"
+#include "sums.cuh"
 
 namespace qrkit {
 namespace {
@@ -489,12 +490,7 @@ __global__ void __launch_bounds__(256) band_norm_f32_kernel(BandGroups B, BandDa
   if (tid < w - 1 || !have) return;
   const int64_t j = grp - B.inst_col0[k];
   float h = 0.f, l = 0.f;   // the sum, and then its root, as float pairs
-  for (int t = 0; t < w && t <= j; ++t) {
-    float tt, e;
-    dev::two_sum(h, S[(tid - t) * (w + 1) + t], tt, e);
-    h = tt;
-    l = __fadd_rn(l, e);
-  }
+  for (int t = 0; t < w && t <= j; ++t) dev::pair_add(h, l, S[(tid - t) * (w + 1) + t], 0.f);
   const float s = h + l;
   l = (h - s) + l;
   float r = s, c = 0.f;   // NaN and infinity are their own root
@@ -596,25 +592,13 @@ __global__ void __launch_bounds__(256) band_grad_f32_kernel(BandGroups B, const 
         float sh = b[grp * B.rpc + q], sl = 0.f;
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
-          if (t < nx) {
-            const float pr = __fmul_rn(a[t], xv[t]);
-            const float pe = __fmaf_rn(a[t], xv[t], -pr);
-            float tt, e;
-            dev::two_sum(sh, pr, tt, e);
-            sh = tt;
-            sl = __fadd_rn(sl, __fadd_rn(e, pe));
-          }
+          if (t < nx) dev::dot2(sh, sl, a[t], xv[t]);
         }
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
           if (t < nx) {   // an entry past the instance's last column belongs to no column
             const float pr = __fmul_rn(a[t], sh);
-            float pe = __fmaf_rn(a[t], sh, -pr);
-            pe = __fmaf_rn(a[t], sl, pe);
-            float tt, e;
-            dev::two_sum(hs[t], pr, tt, e);
-            hs[t] = tt;
-            hc[t] = __fadd_rn(hc[t], __fadd_rn(e, pe));
+            dev::pair_add(hs[t], hc[t], pr, __fmaf_rn(a[t], sl, __fmaf_rn(a[t], sh, -pr)));
           }
         }
       }
@@ -629,10 +613,7 @@ __global__ void __launch_bounds__(256) band_grad_f32_kernel(BandGroups B, const 
   float s = 0.f, c = 0.f;
   auto diagonal = [&](int t) {
     const float2 v = S[(tid - t) * (w + 1) + t];
-    float tt, e;
-    dev::two_sum(s, v.x, tt, e);
-    s = tt;
-    c = __fadd_rn(c, __fadd_rn(e, v.y));
+    dev::pair_add(s, c, v.x, v.y);
   };
   if (kW8 && j >= 7) {
 #pragma unroll
@@ -645,10 +626,7 @@ __global__ void __launch_bounds__(256) band_grad_f32_kernel(BandGroups B, const 
     const float xj = -xs[tid];
     const float q = __fmul_rn(e2.x, xj);
     const float qe = __fmaf_rn(e2.y, xj, __fmaf_rn(e2.x, xj, -q));
-    float tt, e;
-    dev::two_sum(s, q, tt, e);
-    s = tt;
-    c = __fadd_rn(c, __fadd_rn(e, qe));
+    dev::pair_add(s, c, q, qe);
   }
   float* out = gp + 8 * blk0[k];
   out[j] = s + c;

@@ -29,17 +29,6 @@ __device__ __forceinline__ void record(int* status, int code) {
   if (status) atomicCAS(status, 0, code);
 }
 
-// Compensated float accumulation (Dot2, Ogita-Rump-Oishi): (sh + sl) += a x with the product's
-// rounding error from an FMA and the sum's from TwoSum (Knuth).
-__device__ __forceinline__ void dot2_acc(float& sh, float& sl, float a, float x) {
-  const float p = __fmul_rn(a, x);
-  const float pe = __fmaf_rn(a, x, -p);
-  float t, e;
-  dev::two_sum(sh, p, t, e);
-  sh = t;
-  sl = __fadd_rn(sl, __fadd_rn(e, pe));
-}
-
 // ---- column norms D = diag(J^T J)^(1/2) (Sec. 5.2): sums in double, those of a float dense S as
 // sums of three floats per thread first (FP64 runs at 1/73 of the FP32 rate: 811 us in FP64 for an S of
 // 819 MB) ----
@@ -524,7 +513,9 @@ __global__ void block_backsub_kernel(ComposedView<T> V, FactorOut<T> O, const T*
   for (int k = 0; k < m; ++k) x[c0 + k] = accumulate ? x[c0 + k] + y[k] : y[k];
 }
 
-// ---- refinement: g = J^T (b - J p) - lambda D^2 p in double ----
+// ---- refinement: g = J^T (b - J p) - lambda D^2 p of double plans, and of float plans without a dense S whose blocks
+// differ in shape (a dense S: dense_solve.cu; blocks of one shape with windows: window_sums.cu).  In double; blocks of
+// floats up to 6 x 2 sum their rows in float pairs ----
 constexpr int kCtaSumCols = 4096;   // dense S: shared columns summed per CTA in shared memory
 constexpr int kWinSumCols = 2048;   // windowed S: the column range of a CTA summed in shared memory
 
@@ -535,11 +526,12 @@ __device__ __forceinline__ void resid_g_block(ComposedView<T> V, const T* b, con
   const int64_t c0 = V.col_off[i], r0 = V.row_off[i];
   const T* J = V.J + V.val_off[i];
   const int64_t st = V.coupled == QRKIT_COUPLED_WINDOW ? V.start[i] : 0;
+  const bool dense = sizeof(T) == sizeof(double) && V.coupled == QRKIT_COUPLED_DENSE;   // float: dense_solve.cu
   double res[kMaxRows];
   for (int r = 0; r < n; ++r) {
     double acc = (double)b[r0 + r];
     for (int j = 0; j < m; ++j) acc -= (double)J[j * n + r] * (double)p[c0 + j];
-    if (V.coupled == QRKIT_COUPLED_DENSE) {
+    if (dense) {
       for (int c = 0; c < V.s; ++c)
         acc -= (double)V.S[(int64_t)c * V.rows + r0 + r] * (double)p[V.nb + c];
     } else if (V.coupled == QRKIT_COUPLED_WINDOW) {
@@ -554,7 +546,7 @@ __device__ __forceinline__ void resid_g_block(ComposedView<T> V, const T* b, con
     const double d = D[c0 + j];
     g[c0 + j] = acc - lam * d * d * (double)p[c0 + j];
   }
-  if (V.coupled == QRKIT_COUPLED_DENSE) {
+  if (dense) {
     for (int c = 0; c < V.s; ++c) {
       double acc = 0;
       for (int r = 0; r < n; ++r) acc += (double)V.S[(int64_t)c * V.rows + r0 + r] * res[r];
@@ -604,9 +596,9 @@ __device__ __forceinline__ void resid_g_small_f32(const ComposedView<float>& V, 
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
         float sh = b[r0 + r], sl = 0.f;
-        dot2_acc(sh, sl, -J[r], p0);
+        dev::dot2(sh, sl, -J[r], p0);
 #pragma unroll
-        for (int t = 0; t < 8; ++t) dot2_acc(sh, sl, -sv[2 * t + r], ps[t]);
+        for (int t = 0; t < 8; ++t) dev::dot2(sh, sl, -sv[2 * t + r], ps[t]);
         rh2[r] = sh;
         rl2[r] = sl;
       }
@@ -614,7 +606,7 @@ __device__ __forceinline__ void resid_g_small_f32(const ComposedView<float>& V, 
         float ah = 0.f, al = 0.f;
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-          dot2_acc(ah, al, J[r], rh2[r]);
+          dev::dot2(ah, al, J[r], rh2[r]);
           al = __fmaf_rn(J[r], rl2[r], al);
         }
         const double d = D[c0];
@@ -625,7 +617,7 @@ __device__ __forceinline__ void resid_g_small_f32(const ComposedView<float>& V, 
         float ah = 0.f, al = 0.f;
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-          dot2_acc(ah, al, sv[2 * t + r], rh2[r]);
+          dev::dot2(ah, al, sv[2 * t + r], rh2[r]);
           al = __fmaf_rn(sv[2 * t + r], rl2[r], al);
         }
         const double acc = (double)ah + (double)al;
@@ -644,10 +636,10 @@ __device__ __forceinline__ void resid_g_small_f32(const ComposedView<float>& V, 
       sh = b[r0 + r];
 #pragma unroll
       for (int j = 0; j < MM; ++j)
-        if (j < m) dot2_acc(sh, sl, -J[j * n + r], pj[j]);
+        if (j < m) dev::dot2(sh, sl, -J[j * n + r], pj[j]);
       if (V.coupled == QRKIT_COUPLED_WINDOW) {
         for (int t = 0; t < V.w; ++t)
-          if (st + t < V.s) dot2_acc(sh, sl, -V.S[r0 * V.w + (int64_t)t * n + r], p[V.nb + st + t]);
+          if (st + t < V.s) dev::dot2(sh, sl, -V.S[r0 * V.w + (int64_t)t * n + r], p[V.nb + st + t]);
       }
     }
     rh[r] = sh;
@@ -662,7 +654,7 @@ __device__ __forceinline__ void resid_g_small_f32(const ComposedView<float>& V, 
       for (int r = 0; r < NR; ++r)
         if (r < n) {
           const float a = J[j * n + r];
-          dot2_acc(ah, al, a, rh[r]);
+          dev::dot2(ah, al, a, rh[r]);
           al = __fmaf_rn(a, rl[r], al);
         }
       const double d = D[c0 + j];
@@ -676,7 +668,7 @@ __device__ __forceinline__ void resid_g_small_f32(const ComposedView<float>& V, 
       for (int r = 0; r < NR; ++r)
         if (r < n) {
           const float a = V.S[r0 * V.w + (int64_t)t * n + r];
-          dot2_acc(ah, al, a, rh[r]);
+          dev::dot2(ah, al, a, rh[r]);
           al = __fmaf_rn(a, rl[r], al);
         }
       const double acc = (double)ah + (double)al;
@@ -785,7 +777,7 @@ __global__ void resid_g_kernel(ComposedView<T> V, const T* b, const T* p, const 
   // dense S: every block adds to all s shared columns; the CTA's sums are gathered in shared
   // memory and leave with one global atomic per column
   extern __shared__ double sgS[];
-  const bool cta_sum = V.coupled == QRKIT_COUPLED_DENSE && V.s <= kCtaSumCols;
+  const bool cta_sum = sizeof(T) == sizeof(double) && V.coupled == QRKIT_COUPLED_DENSE && V.s <= kCtaSumCols;
   if (cta_sum) {
     for (int c = threadIdx.x; c < V.s; c += blockDim.x) sgS[c] = 0.0;
     __syncthreads();
@@ -907,7 +899,7 @@ __global__ void block_fwdsub_rt_kernel(ComposedView<T> V, FactorOut<T> O, const 
                                        double* gS, int win_cols) {
   dev::chain_wait();
   extern __shared__ double sgS[];
-  const bool cta_sum = V.coupled == QRKIT_COUPLED_DENSE && V.s <= kCtaSumCols;
+  const bool cta_sum = sizeof(T) == sizeof(double) && V.coupled == QRKIT_COUPLED_DENSE && V.s <= kCtaSumCols;
   if (cta_sum) {
     for (int c = threadIdx.x; c < V.s; c += blockDim.x) sgS[c] = 0.0;
     __syncthreads();

@@ -23,19 +23,22 @@ __device__ __forceinline__ bool square_exact(float x) {
   return a - 1u >= ((127u - 50u) << 23) - 1u && a <= (127u + 50u) << 23;
 }
 
+// (h, l) += ph + pl, and += a x
+__device__ __forceinline__ void pair_add(float& h, float& l, float ph, float pl) {
+  float t, e;
+  two_sum(h, ph, t, e);
+  h = t;
+  l = __fadd_rn(l, __fadd_rn(e, pl));
+}
+__device__ __forceinline__ void dot2(float& h, float& l, float a, float x) {
+  const float p = __fmul_rn(a, x);
+  pair_add(h, l, p, __fmaf_rn(a, x, -p));
+}
+
 struct Pair {
   float h = 0.f, l = 0.f;
-  __device__ __forceinline__ void add(float ph, float pl) {   // += ph + pl
-    float t, e;
-    two_sum(h, ph, t, e);
-    h = t;
-    l = __fadd_rn(l, __fadd_rn(e, pl));
-  }
-  __device__ __forceinline__ void add(const Pair& o) { add(o.h, o.l); }
-  __device__ __forceinline__ void fma(float a, float x) {   // += a x
-    const float p = __fmul_rn(a, x);
-    add(p, __fmaf_rn(a, x, -p));
-  }
+  __device__ __forceinline__ void add(float ph, float pl) { pair_add(h, l, ph, pl); }
+  __device__ __forceinline__ void fma(float a, float x) { dot2(h, l, a, x); }
   __device__ __forceinline__ double value() const { return (double)h + (double)l; }
 };
 
