@@ -1230,12 +1230,14 @@ static qrkit_status cr_split(qrkit_ctx* ctx, CRPlan& C, const std::vector<int>& 
   return cr_partials(ctx, C, C.P2, parts2);
 }
 
-// Threads per block of each instance: about 120,000 in all where that leaves each at least 64 rows (16 steps of four,
+// Threads per block of each instance: about 800 per SM in all where that leaves each at least 64 rows (16 steps of four,
 // what a merge pass takes), at most 64 per block.  A batch's instances differ in rows per block (curve fits: 60 to
-// 10,000), and the longest thread bounds the kernel.
-static std::vector<int> default_splits(const CRPlan& C) {
+// 10,000), and the longest thread bounds the kernel.  One LM step of 1,024 curve fits: 4,696 us at 400 per SM, 4,678 at
+// 800, 4,711 at 1,600, 4,793 at 6,400; three steps of one curve fit of 200,000 points, which the rows bound: 1,570 us at
+// least 32 rows, 1,397 at 64, 1,438 at 128.
+static std::vector<int> default_splits(const qrkit_ctx* ctx, const CRPlan& C) {
   std::vector<int> n((size_t)C.num_inst);
-  const double target = std::max(64.0, (double)C.total_rows / 120000.0);
+  const double target = std::max(64.0, (double)C.total_rows / (800.0 * ctx->num_sms));
   for (int64_t k = 0; k < C.num_inst; ++k) {
     const double per = (double)C.h_rows[k] / (double)(C.h_blk0[k + 1] - C.h_blk0[k]);
     n[k] = (int)std::min(64.0, std::max(1.0, std::floor(per / target + 0.5)));
@@ -1250,7 +1252,7 @@ static qrkit_status cr_use_splits(qrkit_ctx* ctx, CRPlan& C, int each) {
       C.cur = s;
       return QRKIT_OK;
     }
-  const std::vector<int> n = each ? std::vector<int>((size_t)C.num_inst, each) : default_splits(C);
+  const std::vector<int> n = each ? std::vector<int>((size_t)C.num_inst, each) : default_splits(ctx, C);
   CRSplits* s = new CRSplits();
   s->each = each;
   const qrkit_status rc = cr_split(ctx, C, n, *s);
@@ -1346,8 +1348,8 @@ qrkit_status cr_set_strategy(qrkit_ctx* ctx, CRPlan& C, int splits) {
   return cr_use_splits(ctx, C, splits);
 }
 
-std::vector<int> cr_candidates(const CRPlan& C) {
-  const std::vector<int> def = default_splits(C);
+std::vector<int> cr_candidates(const qrkit_ctx* ctx, const CRPlan& C) {
+  const std::vector<int> def = default_splits(ctx, C);
   const bool uniform = std::all_of(def.begin(), def.end(), [&](int n) { return n == def[0]; });
   double most = 0.0;   // rows per block
   for (int64_t k = 0; k < C.num_inst; ++k)

@@ -255,7 +255,7 @@ qrkit_status cr_solve(qrkit_ctx* ctx, CRPlan& C, const int64_t* starts, const in
 // merged, or 0: as many as each instance's rows call for, the default.  The candidates to time, without one that is
 // the same as the default; and the strategies that the timing built and dropped: CRTuning holds what was there before.
 qrkit_status cr_set_strategy(qrkit_ctx* ctx, CRPlan& C, int splits);
-std::vector<int> cr_candidates(const CRPlan& C);
+std::vector<int> cr_candidates(const qrkit_ctx* ctx, const CRPlan& C);
 struct CRTuning {
   size_t strategies = 0, outgrown = 0;
   void *P = nullptr, *P2 = nullptr;

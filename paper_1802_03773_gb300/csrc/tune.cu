@@ -276,7 +276,7 @@ extern "C" qrkit_status qrkit_autotune(qrkit_ctx* ctx, const void* J, const void
       const CRTuning before = cr_tuning_begin(*B.cr);
       float best = 1e30f;
       int chosen_splits = 0;
-      for (const int cand : cr_candidates(*B.cr)) {
+      for (const int cand : cr_candidates(ctx, *B.cr)) {
         st = cr_set_strategy(ctx, *B.cr, cand);
         if (st == QRKIT_ENOMEM) continue;   // no room for its triangles
         float ms = 0.f;
