@@ -255,7 +255,8 @@ qrkit_status qrkit_set_refinement(qrkit_ctx* ctx, double select, int residual);
  * Sec. 5.2): J holds the instances' rows back to back, row-major with band_window values per
  * row; b one value per row; D (total columns, or NULL for column norms, zero -> 1) as above;
  * lambda >= 0; p one value per column; qtb must be NULL; refine_steps: steps of refinement
- * with a double residual (FP32 refined mode).  Q is not kept. */
+ * (FP32 refined mode) with the residual and the gradient as unevaluated float pairs (PARALLEL with implicit row
+ * starts) or in double.  Q is not kept. */
 
 /* Composed factorization (Sec. 3 composition; Sec. 4.1 block diagonal, Sec. 4.2 horizontal
  * concatenation, Sec. 4.5 vertical concatenation of the damping rows, Sec. 5.2 Backtrack LM):
@@ -284,9 +285,11 @@ qrkit_status qrkit_solve_r(qrkit_ctx* ctx, const void* qtb, void* p);
 
 /* Sec. 5.1 (Q^T b, then the R solve) with refinement (not in the paper):
  * p = argmin ||P_r [J; lambda^(1/2) D] p - P_r [b; 0]|| with the stored factor: Q^T b,
- * back-substitution, then `refine_steps` refinement steps (QRKIT_FP32_REFINED: residual
- * g = J^T (b - J p) - lambda D^2 p in double, correction R^{-1} R^{-T} g; ignored for
- * QRKIT_FP32, allowed but not useful for QRKIT_FP64). */
+ * back-substitution, then `refine_steps` refinement steps (QRKIT_FP32_REFINED: the gradient
+ * g = J^T (b - J p) - lambda D^2 p, correction R^{-1} R^{-T} g; ignored for
+ * QRKIT_FP32, allowed but not useful for QRKIT_FP64).  g is as accurate as if computed in double, by sums of three
+ * floats where S is dense or the blocks of a windowed plan have one shape, in double otherwise; the residual rows and
+ * the per-block sums of blocks up to 6 x 2 without a dense S are float pairs (about 48 bits). */
 qrkit_status qrkit_solve(qrkit_ctx* ctx, const void* b, void* p, int refine_steps);
 
 /* ---- A dense S split by rows over several contexts (one per GPU): the horizontal

@@ -5,7 +5,8 @@
 // (Sec. 4.5), and R'_i p_i = top of Q'_i^T [c_i; 0].  Since ||J_i p - b_i||^2 = ||R_i p - c_i||^2
 // + const, p_i is the minimiser of ||J_i p - b_i||^2 + lambda ||D_i p||^2 (Eq. 2).
 //
-// Mapping: one thread per block (m_i <= 8, the whole stack in registers).  The interleaved
+// Mapping: one thread per block (m_i <= 8; R and c are indexed by the block's own m_i and so live in local memory, a
+// stack of 288 bytes per thread in float, which bounds the kernel).  The interleaved
 // stack is reduced row by row: the damping row of column k has one non-zero, at column k, and
 // is merged into rows k .. m-1 of the triangle by 2 x 2 reflections (each zeroes the row's
 // leading entry against the diagonal of the triangle row, the row-merge form of a Householder

@@ -3,7 +3,9 @@
 //
 // FP64 runs at about 2 multiply-adds per cycle and SM here, so a warp's FP64 instruction holds its quarter
 // of the SM for 64 cycles, and a tile of 256 x 30 needs 60 us of that whatever is done around it.  The
-// kernel keeps everything else off that unit: columns in registers, one barrier per column, the sums
+// kernel keeps everything else off that unit: columns with their warp (in registers up to 16 columns; from 17 on
+// the loop over a warp's column groups, which holds a barrier, is not unrolled and they live in local memory, a stack
+// of 128 bytes per thread for 128-row tiles of doubles), one barrier per column, the sums
 // of a warp's columns reduced together by a transposed butterfly (1.5 additions per column instead of 5),
 // one reciprocal root and one reciprocal per reflector.  Few tiles of up to 32 columns are cut to 128 rows,
 // which spreads the work over more SMs.  FP64, 200 blocks 4 x 2 with 30 shared columns (830 rows): factor
