@@ -1172,13 +1172,18 @@ static qrkit_status upload(qrkit_ctx* ctx, DevBuf& d, const void* h, size_t byte
   return QRKIT_OK;
 }
 
-// A buffer of partial triangles of at least `parts`; an outgrown one is kept until the plan goes.  Strategies grow
-// it, so the kept ones are smaller than the current one.
+// A buffer of partial triangles of at least `parts`; an outgrown one is kept until the plan goes.  Each is at least twice
+// the one before (or as large as there is room for), so that the kept ones together are no larger than the current.
 static qrkit_status cr_partials(qrkit_ctx* ctx, CRPlan& C, DevBuf& buf, int64_t parts) {
   const size_t bytes = ((size_t)parts + 31) / 32 * 32 * kE0 * elem_size(ctx);
   if (parts == 0 || buf.bytes >= bytes) return QRKIT_OK;
   DevBuf grown;
-  const qrkit_status rc = ensure(ctx, grown, bytes, "banded partial triangles");
+  qrkit_status rc = QRKIT_ENOMEM;
+  if (2 * buf.bytes > bytes) {
+    rc = ensure(ctx, grown, 2 * buf.bytes, "banded partial triangles");
+    if (rc == QRKIT_ENOMEM) cudaGetLastError();
+  }
+  if (rc != QRKIT_OK) rc = ensure(ctx, grown, bytes, "banded partial triangles");
   if (rc != QRKIT_OK) return rc;
   if (buf.ptr) C.outgrown.push_back(buf);
   buf = grown;
