@@ -31,7 +31,7 @@ __device__ __forceinline__ void record(int* status, int code) {
 
 // ---- column norms D = diag(J^T J)^(1/2) (Sec. 5.2): sums in double, those of a float dense S as
 // sums of three floats per thread first (FP64 runs at 1/73 of the FP32 rate: 811 us in FP64 for an S of
-// 819 MB) ----
+// 819 MB, 237 us so) ----
 template <typename T>
 __global__ void colnorm_blocks_kernel(ComposedView<T> V, double* sq) {
   dev::chain_wait();

@@ -4,9 +4,11 @@
 // Every pass over S (column-major, rows of J) or R12 (row-major, one row of s values per block
 // column) is written for the memory system: a warp reads whole 128-byte lines, a CTA's warps split
 // the columns, sums leave through per-chunk partials that are added in a fixed order.  S and R12
-// are read twice and once per refinement step, so those passes are bound by HBM: at 100,000 blocks
-// 4 x 2 with s = 512 (S 819 MB, R12 410 MB) the row pass takes 126 us, the column pass 135 us, the
-// R12 pass 136 us and a block back-substitution 97 us.  A thread per block walking all s columns,
+// are read twice and once per refinement step; those passes are bound by HBM and by the additions of the
+// three-float sums (22 and 33 operations per value): at 100,000 blocks
+// 4 x 2 with s = 512 (S 819 MB, R12 410 MB) the row pass takes 186 us, the column pass 250 us, the
+// R12 pass 159 us (126, 135 and 136 with float pairs, which are not enough: see the refinement below) and a block
+// back-substitution 95 us.  A thread per block walking all s columns,
 // with a shared-memory FP64 atomic per column and block, took 4.33 ms for the two passes over S,
 // 4.04 ms for R12^T h and 0.38 ms per back-substitution.
 #include <cuda_runtime.h>
@@ -221,7 +223,8 @@ __global__ void __launch_bounds__(kWarpBackThreads) block_backsub_warp_kernel(Co
 }
 
 // ---- refinement of float plans: g = J^T (b - J p - S p_S) - lambda D^2 p with the residual and its sums as sums of
-// three floats, no less accurate than in double.  A product that overflows (right-hand sides have any scale) leaves a
+// three floats, no less accurate than in double: with a residual 1e9 times what the unknowns explain, float pairs left
+// the refined solution off by 1.3e-7 to 2.1e-7, sums in double and these by 2.5e-8.  A product that overflows (right-hand sides have any scale) leaves a
 // sum that is not finite: that one is formed again in double. ----
 
 // 1. rows: b - S p_S, three floats per row.  A CTA takes 32 V rows; its 8 warps split the columns.

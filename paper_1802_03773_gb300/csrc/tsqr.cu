@@ -9,7 +9,7 @@
 // of a warp's columns reduced together by a transposed butterfly (1.5 additions per column instead of 5),
 // one reciprocal root and one reciprocal per reflector.  Few tiles of up to 32 columns are cut to 128 rows,
 // which spreads the work over more SMs.  FP64, 200 blocks 4 x 2 with 30 shared columns (830 rows): factor
-// 294 us, Q^T b 63 us, against 378 and 95 us for a tile in shared memory with a warp per column and two
+// 302 us, Q^T b 63 us, against 378 and 95 us for a tile in shared memory with a warp per column and two
 // barriers; 100,000 blocks 2 x 1 with 5 shared columns: 80 and 31 us against 77 and 45 us.
 #include <cuda_runtime.h>
 #include <math.h>

@@ -4,11 +4,11 @@
 // A shared column's sum runs over the blocks whose windows hold it, which lie anywhere in memory.  The blocks
 // sorted by window start (block_sort) bring those of one start together: eight lanes take kRun
 // consecutive sorted blocks, lane t the window's column t, read the blocks' rows of S (a whole 64-byte
-// window at a time for 2 x 1 blocks of floats) and keep the sum in a register pair until the start changes.
+// window at a time for 2 x 1 blocks of floats) and keep the sum in registers, three floats, until the start changes.
 // One atomic per column and run then, where a thread per block added its eight columns to shared
 // memory by FP64 atomics: those retry as compare-and-swap loops around an FP64 add, and a warp's FP64
 // instruction holds the SM's FP64 unit for 16 cycles (83 % busy).  10.5 million blocks 2 x 1, windows of
-// 8: the gradient takes 674 us (residuals 269, sums 404) against 2.20 ms.
+// 8: the gradient takes 870 us (residuals 273, sums 597) against 2.20 ms.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(128) window_blocks_kernel(ComposedView<T> V, F
 //
 // The general small-block kernels read six tables of offsets per block and touch a window entry by entry (a warp's
 // load spreads over 32 windows).  A plan of one shape needs no offsets, and rows of a window are whole 16-byte pieces:
-// 10.5 million blocks: factorization 634 -> 356 us, Q^T b 135 -> 105 us, back-substitution 140 -> 107 us.
+// 10.5 million blocks: factorization 634 -> 354 us, Q^T b 135 -> 105 us, back-substitution 140 -> 106 us.
 // The arithmetic is that of the general kernels.
 template <typename T, int N>
 __device__ __forceinline__ void load_wide(T (&v)[N], const T* src) {   // src 16-byte aligned
