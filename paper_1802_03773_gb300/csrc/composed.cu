@@ -1033,8 +1033,8 @@ int small_class(const Plan& P, bool damp) {
     else LAUNCH(ctx, (launch_kernel(chained, stream, grid, threads, smem, KERNEL<T>, __VA_ARGS__)));                   \
   } while (0)
 
-// R_i x_i = rhs_i - R12_i x_S for every block.  From 16 shared columns on a warp takes a block (the
-// lanes read its rows of R12 together); below, and for windows of up to 8, a thread per block.
+// R_i x_i = rhs_i - R12_i x_S for every block.  From 16 shared columns on in dense_solve.cu; below, and for windows of
+// up to 8, a thread per block.
 template <typename T>
 static qrkit_status launch_block_backsub(qrkit_ctx* ctx, bool chained, const ComposedView<T>& V, const FactorOut<T>& O,
                                          const T* rhs, const T* xS, T* x, int accumulate) {

@@ -158,6 +158,21 @@ __global__ void __launch_bounds__(kTriThreads) tri_normal_kernel(const T* R, int
   }
 }
 
+// y := R^-1 y with R = F's leading m x m upper triangle (m <= 8, columns of na).
+template <typename T>
+__device__ __forceinline__ void block_substitute(const T* F, int na, int m, T (&y)[8]) {
+#pragma unroll
+  for (int k = 7; k >= 0; --k) {
+    if (k < m) {
+      T v = y[k];
+#pragma unroll
+      for (int j = k + 1; j < 8; ++j)
+        if (j < m) v -= F[j * na + k] * y[j];
+      y[k] = v / F[k * na + k];
+    }
+  }
+}
+
 // ---- block unknowns R_i x_i = c_i - R12_i x_S, one warp per block ----
 // The lanes share a row of R12 (s values, contiguous), so that the pass over R12 is coalesced and
 // many loads are in flight; the m_i <= 8 unknowns are then found by every lane alike.
@@ -206,20 +221,49 @@ __global__ void __launch_bounds__(kWarpBackThreads) block_backsub_warp_kernel(Co
       y[k] = rhs[c0 + k] - a;
     }
   }
-#pragma unroll
-  for (int k = 7; k >= 0; --k) {
-    if (k < m) {
-      T v = y[k];
-#pragma unroll
-      for (int j = k + 1; j < 8; ++j)
-        if (j < m) v -= F[j * na + k] * y[j];
-      y[k] = v / F[k * na + k];
-    }
-  }
   __syncwarp();   // x may be rhs: every lane has read it
+  block_substitute(F, na, m, y);
 #pragma unroll
   for (int k = 0; k < 8; ++k)
     if (k < m && lane == k) x[c0 + k] = accumulate ? x[c0 + k] + y[k] : y[k];
+}
+
+// The same with a thread per block, for many blocks.  Eight partial sums keep as many loads in flight and the sum of s
+// products as accurate as the warp's.
+constexpr int kThreadBackThreads = 64;
+
+template <typename T>
+__global__ void __launch_bounds__(kThreadBackThreads) block_backsub_thread_kernel(ComposedView<T> V, FactorOut<T> O,
+                                                                                  const T* rhs, const T* xS, T* x,
+                                                                                  int accumulate) {
+  dev::chain_wait();
+  __shared__ T xs[kMaxDenseS];
+  const int s = V.s;
+  for (int t = threadIdx.x; t < s; t += kThreadBackThreads) xs[t] = xS[t];
+  __syncthreads();
+  const int64_t i = (int64_t)blockIdx.x * kThreadBackThreads + threadIdx.x;
+  if (i >= V.K) return;
+  const int n = V.n[i], m = V.m[i];
+  const int na = n + (O.damp ? m : 0);
+  const int64_t c0 = V.col_off[i];
+  T y[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    y[k] = T(0);
+    if (k < m) {
+      const T* r12 = O.R12 + (c0 + k) * (int64_t)s;
+      T a[8] = {};
+      for (int t = 0; t < s; t += 8)
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          if (t + j < s) a[j] += r12[t + j] * xs[t + j];
+      y[k] = rhs[c0 + k] - (((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7])));
+    }
+  }
+  block_substitute(O.Fa + O.aug_off[i], na, m, y);
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    if (k < m) x[c0 + k] = accumulate ? x[c0 + k] + y[k] : y[k];
 }
 
 // ---- refinement of float plans: g = J^T (b - J p - S p_S) - lambda D^2 p with the residual and its sums as sums of
@@ -487,11 +531,27 @@ qrkit_status dense_normal(qrkit_ctx* ctx, const T* R, int64_t ld, int s, const d
 template qrkit_status dense_normal<float>(qrkit_ctx*, const float*, int64_t, int, const double*, float*, float*);
 template qrkit_status dense_normal<double>(qrkit_ctx*, const double*, int64_t, int, const double*, double*, double*);
 
+// By warps a block's rows of R12 are read together, which hides latency while there are few blocks; but every lane
+// repeats the substitution, and a sum over the warp costs five additions of all lanes.  A thread per block does neither:
+// with many blocks its strided reads of R12 are covered by the other threads.  Doubles, where the warp pays
+// the FP64 unit for each lane, cross at 12 to 24 blocks per SM (s = 16 .. 64), floats at 23 (s = 16, one column) to 260
+// (s = 48, eight columns) along 16 + s m / 2; from s = 64 on float rows are read 16 bytes a lane and the warp is as
+// fast or faster.  @MEAS@
+template <typename T>
+static bool backsub_by_warps(const qrkit_ctx* ctx, int64_t K, int s) {
+  if (sizeof(T) == 8) return K <= (int64_t)ctx->num_sms * (8 + s / 4);
+  return s >= 64 || K <= (int64_t)ctx->num_sms * (16 + s * ctx->plan.max_m / 2);
+}
+
 template <typename T>
 qrkit_status dense_block_backsub(qrkit_ctx* ctx, bool chained, const ComposedView<T>& V, const FactorOut<T>& O,
                                  const T* rhs, const T* xS, T* x, int accumulate) {
-  DS_LAUNCH(ctx, launch_kernel(chained, ctx->stream, nblk(V.K * 32, kWarpBackThreads), kWarpBackThreads, 0,
-                               block_backsub_warp_kernel<T>, V, O, rhs, xS, x, accumulate));
+  if (backsub_by_warps<T>(ctx, V.K, V.s))
+    DS_LAUNCH(ctx, launch_kernel(chained, ctx->stream, nblk(V.K * 32, kWarpBackThreads), kWarpBackThreads, 0,
+                                 block_backsub_warp_kernel<T>, V, O, rhs, xS, x, accumulate));
+  else
+    DS_LAUNCH(ctx, launch_kernel(chained, ctx->stream, nblk(V.K, kThreadBackThreads), kThreadBackThreads, 0,
+                                 block_backsub_thread_kernel<T>, V, O, rhs, xS, x, accumulate));
   return QRKIT_OK;
 }
 template qrkit_status dense_block_backsub<float>(qrkit_ctx*, bool, const ComposedView<float>&, const FactorOut<float>&,
