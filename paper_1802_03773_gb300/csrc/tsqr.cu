@@ -97,6 +97,7 @@ __global__ void __launch_bounds__(kThreads) tsqr_tile_kernel(T* X, int64_t ld, i
   const int64_t r0 = (int64_t)blockIdx.x * rows;
   const int r = (int)(M - r0 < (int64_t)rows ? M - r0 : (int64_t)rows);   // <= 32 RPL
   const int kmax = r < s ? r : s;
+  const int mine = sizeof(T) == 8 ? (s - warp + kWarps - 1) / kWarps : CPW;   // the warp's columns, without those of zeros
   T a[CPW][RPL];
 #pragma unroll
   for (int i = 0; i < CPW; ++i) {
@@ -145,19 +146,19 @@ __global__ void __launch_bounds__(kThreads) tsqr_tile_kernel(T* X, int64_t ld, i
 #pragma unroll
       for (int c = 0; c < CPW; ++c) {
         p[c] = T(0);
-        if (c > i || (c == i && warp > w)) {
+        if (c < mine && (c > i || (c == i && warp > w))) {
 #pragma unroll
           for (int u = 0; u < RPL; ++u) p[c] += v[u] * a[c][u];
         }
       }
-      if (i + 1 < CPW || warp > w) {
+      if (i + 1 < mine || (i < mine && warp > w)) {
         T q[CPW];
 #pragma unroll
         for (int c = 0; c < CPW; ++c) q[c] = c >= i ? p[c] : T(0);
         warp_sums<T, CPW>(q, lane);
 #pragma unroll
         for (int c = 0; c < CPW; ++c) {
-          if (c > i || (c == i && warp > w)) {
+          if (c < mine && (c > i || (c == i && warp > w))) {
             const T wt = q[c] * t;
 #pragma unroll
             for (int u = 0; u < RPL; ++u) a[c][u] -= wt * v[u];
@@ -238,13 +239,17 @@ __global__ void __launch_bounds__(kQtThreads) tsqr_qt_kernel(const T* X, int64_t
   }
 }
 
-template <typename T, int RPL>
+// CPW column groups of 8.  A double column of zeros costs the FP64 unit as much as any other, so doubles take as many
+// groups as s has (rounded up to the next power of two of groups, s = 33 was 1.1 to 1.4 times as slow over the whole
+// solve); floats take the next power of two.
+template <typename T, int RPL, int CPW = 1>
 void launch_tile(unsigned g, cudaStream_t st, T* X, int64_t ld, int64_t M, int s, int rows, T* taus, T* Xn,
                  int64_t ldn) {
-  if (s <= 8) chain_launch(st, g, kThreads, 0, (tsqr_tile_kernel<T, RPL, 1>), X, ld, M, s, rows, taus, Xn, ldn);
-  else if (s <= 16) chain_launch(st, g, kThreads, 0, (tsqr_tile_kernel<T, RPL, 2>), X, ld, M, s, rows, taus, Xn, ldn);
-  else if (s <= 32) chain_launch(st, g, kThreads, 0, (tsqr_tile_kernel<T, RPL, 4>), X, ld, M, s, rows, taus, Xn, ldn);
-  else chain_launch(st, g, kThreads, 0, (tsqr_tile_kernel<T, RPL, 8>), X, ld, M, s, rows, taus, Xn, ldn);
+  if constexpr (CPW < 8) {
+    if (s > kWarps * CPW)
+      return launch_tile<T, RPL, sizeof(T) == 8 ? CPW + 1 : 2 * CPW>(g, st, X, ld, M, s, rows, taus, Xn, ldn);
+  }
+  chain_launch(st, g, kThreads, 0, (tsqr_tile_kernel<T, RPL, CPW>), X, ld, M, s, rows, taus, Xn, ldn);
 }
 
 }  // namespace
