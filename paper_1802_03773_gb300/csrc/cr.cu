@@ -1240,11 +1240,22 @@ static qrkit_status cr_split(qrkit_ctx* ctx, CRPlan& C, const std::vector<int>& 
 // 10,000), and the longest thread bounds the kernel.  One LM step of 1,024 curve fits: 4,696 us at 400 per SM, 4,678 at
 // 800, 4,711 at 1,600, 4,793 at 6,400; three steps of one curve fit of 200,000 points, which the rows bound: 1,570 us at
 // least 32 rows, 1,397 at 64, 1,438 at 128.
+// In double a thread takes about 10 us per row and a merge pass of up to four partials 320 us whatever is in it, so
+// while the chip has room the powers of four are compared by rows per thread + 32 per pass (solve of 20,000 blocks 2 x 1
+// with windows of 8 in 500 columns: 1,906 us at 64 rows per thread, 1,778; 300 columns of 40 rows: 1,813 and 1,620).
 static std::vector<int> default_splits(const qrkit_ctx* ctx, const CRPlan& C) {
   std::vector<int> n((size_t)C.num_inst);
   const double target = std::max(64.0, (double)C.total_rows / (800.0 * ctx->num_sms));
   for (int64_t k = 0; k < C.num_inst; ++k) {
     const double per = (double)C.h_rows[k] / (double)(C.h_blk0[k + 1] - C.h_blk0[k]);
+    if (elem_size(ctx) == 8) {
+      const double least = (double)C.total_rows / (800.0 * ctx->num_sms);
+      n[k] = 1;
+      for (int m = 4, passes = 1; m <= 64 && per / m >= least; m *= 4, ++passes)
+        if (per / m + 32.0 * passes < per / n[k] + 32.0 * (passes - 1)) n[k] = m;
+        else break;
+      continue;
+    }
     n[k] = (int)std::min(64.0, std::max(1.0, std::floor(per / target + 0.5)));
   }
   return n;
