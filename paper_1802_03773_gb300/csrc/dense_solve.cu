@@ -532,12 +532,13 @@ template qrkit_status dense_normal<float>(qrkit_ctx*, const float*, int64_t, int
 template qrkit_status dense_normal<double>(qrkit_ctx*, const double*, int64_t, int, const double*, double*, double*);
 
 // By warps a block's rows of R12 are read together, which hides latency while there are few blocks; but every lane
-// repeats the substitution, and a sum over the warp costs five additions of all lanes.  A thread per block does neither:
-// with many blocks its strided reads of R12 are covered by the other threads.  Doubles, where the warp pays
+// repeats the substitution, and a sum over the warp costs five additions of all lanes.  A thread per block does
+// neither: with many blocks its strided reads of R12 are covered by the other threads.  Doubles, where the warp pays
 // the FP64 unit for each lane, cross at 9 to 22 blocks per SM (s = 16 .. 64), floats at 23 (s = 16, one column) to 260
-// (s = 48, eight columns) along 16 + s m / 2; from s = 64 on (one column: above)
-// float rows are read 16 bytes a lane and the warp is as fast or faster.  The whole R solve with s = 30 and blocks of 5 x 3: 8,000 in double 50 us by warps, 28 by threads;
-// 50,000 in float 40 and 18; 1,000 in double 24 and 27; 4,000 in float 12 and 15.
+// (s = 48, eight columns) along 16 + s m / 2; from s = 64 on, where float rows are read 16 bytes a lane, the warp is
+// as fast or faster, one column per block and s = 64 apart.  The whole R solve with s = 30 and blocks of 5 x 3: 8,000
+// in double 50 us by warps, 28 by threads; 50,000 in float 40 and 18; 1,000 in double 24 and 27; 4,000 in float 12
+// and 15.
 template <typename T>
 static bool backsub_by_warps(const qrkit_ctx* ctx, int64_t K, int s) {
   if (sizeof(T) == 8) return K <= (int64_t)ctx->num_sms * (5 + s / 4);
